@@ -10,12 +10,16 @@
 // transposes, a symmetric A read from its lower triangle, a lower-triangular
 // C, a fused second product (symmetric rank-2k update), split-K with atomics
 // and device-side batched descriptors.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "internal.cuh"
 
 namespace fraclap {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
 
@@ -293,6 +297,180 @@ __global__ void __launch_bounds__(SG_NT, 2) sgemm_big_batched_kernel(const GemmD
 // The large-tile FP32 kernel pays off once both output dimensions fill it.
 inline bool sg_big(int64_t M, int64_t N) { return M >= 256 && N >= 256; }
 
+// ---------------------------------------------------------------------------
+// FP64 products without padding.  The FP64 pipe retires about 1.7 FMAs per
+// clock and SM, so a warp's FMA occupies it for some 19 cycles and every
+// operand can come straight from L1 at no cost; what a narrow or small product
+// pays for on the 64 x 64 tile is the padding (5 columns cost 64) and the SMs
+// its few tiles leave idle.  These kernels skip the columns past N one by one,
+// and a cluster of CTAs along K splits the sum of a tile until the tiles cover
+// the SMs; the CTAs' partial sums meet in distributed shared memory and are
+// added in rank order, so the result does not depend on the schedule.
+// Bound: the FP64 pipe.  GB300, column counts as given, against the 64 x 64
+// tile: 2304 x 5 x 2304 (A^T B) 2409 -> 143 us and 2304 x 20 x 2304 2411 ->
+// 294 us (both with the caller's wait of some 50 us), 8835 x 128 x 8835 17.9
+// -> 16.6 ms (1.20 TFLOP/s); the apply at n = 2304 with 5 columns and 20 pairs
+// 4.80 -> 0.36 ms, at n = 144 0.31 -> 0.04 ms.
+constexpr int DG_NT = 256, DG_NC = 8, DG_ROWS = 32;
+
+// Adds the partial sums of the cluster's CTAs (one value per thread) and
+// writes C from rank 0.  Every thread of every CTA of the cluster calls it.
+template <int MODE>
+__device__ __forceinline__ void dg_finish(const GemmDescT<double>& d, double v, int64_t gm, int64_t gn) {
+  __shared__ double part[DG_NT];
+  cg::cluster_group cluster = cg::this_cluster();
+  const unsigned S = cluster.num_blocks();
+  if (S > 1) {
+    part[threadIdx.x] = v;
+    cluster.sync();
+    if (cluster.block_rank() == 0)
+      for (unsigned q = 1; q < S; ++q) v += *cluster.map_shared_rank(&part[threadIdx.x], q);
+    cluster.sync();  // a peer's partial sums stay until they are read
+    if (cluster.block_rank() != 0) return;
+  }
+  if (gm >= d.M || gn >= d.N) return;
+  double* c = d.C + gm + gn * d.ldc;
+  v *= d.alpha;
+  *c = (d.beta == 0.0) ? v : v + d.beta * *c;
+}
+
+// op(A) = A (or symmetric, lower triangle read): a lane per row, eight warps
+// interleaved over K, up to eight columns in registers; the reads of A are
+// coalesced along the rows (in the mirrored half of a symmetric A a lane walks
+// along its own column, whose lines L1 keeps), B is one address per warp.
+template <bool TB, int MODE>
+__global__ void __launch_bounds__(DG_NT) dgemm_rows_kernel(GemmDescT<double> d, int64_t kper, int ncol) {
+  __shared__ double red[DG_NC][DG_NC][DG_ROWS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t m0 = (int64_t)(blockIdx.x / cg::this_cluster().num_blocks()) * DG_ROWS, n0 = (int64_t)blockIdx.y * ncol;
+  const int nc = (int)((d.N - n0 < ncol) ? d.N - n0 : ncol);
+  const int64_t kbeg = (int64_t)cg::this_cluster().block_rank() * kper;
+  const int64_t kend = (kbeg + kper < d.K) ? kbeg + kper : d.K;
+  const int64_t row = m0 + lane;
+  const int64_t i = (row < d.M) ? row : d.M - 1;
+  const int64_t bk = TB ? d.ldb : 1, bj = TB ? 1 : d.ldb;
+  const double* Bp = d.B + n0 * bj;
+  auto a_at = [&](int64_t k) -> double {
+    if (MODE == kGemmSymA) return (i >= k) ? d.A[i + k * d.lda] : d.A[k + i * d.lda];
+    return d.A[i + k * d.lda];
+  };
+  double acc[DG_NC];
+#pragma unroll
+  for (int j = 0; j < DG_NC; ++j) acc[j] = 0.0;
+  constexpr int KU = 4;
+  for (int64_t k0 = kbeg + KU * warp; k0 < kend; k0 += KU * (DG_NT / 32)) {
+    if (k0 + KU <= kend) {
+      double a[KU];
+#pragma unroll
+      for (int u = 0; u < KU; ++u) a[u] = a_at(k0 + u);
+#pragma unroll
+      for (int j = 0; j < DG_NC; ++j)
+        if (j < nc) {
+          const double* b = Bp + j * bj + k0 * bk;
+#pragma unroll
+          for (int u = 0; u < KU; ++u) acc[j] = fma(a[u], b[u * bk], acc[j]);
+        }
+    } else {
+      for (int64_t k = k0; k < kend; ++k) {
+        const double a = a_at(k);
+#pragma unroll
+        for (int j = 0; j < DG_NC; ++j)
+          if (j < nc) acc[j] = fma(a, Bp[j * bj + k * bk], acc[j]);
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < DG_NC; ++j) red[warp][j][lane] = acc[j];
+  __syncthreads();
+  double v = 0.0;  // thread (warp, lane): column warp, row lane, the warps' sums in order
+#pragma unroll
+  for (int w = 0; w < DG_NT / 32; ++w) v += red[w][warp][lane];
+  dg_finish<MODE>(d, v, row, (warp < nc) ? n0 + warp : d.N);
+}
+
+// op(A) = A^T, op(B) = B (both contiguous along K): the lanes of a warp share
+// K, each warp holds four rows x eight columns, and a butterfly that halves
+// the 32 sums at every step leaves one output per lane.
+__global__ void __launch_bounds__(DG_NT) dgemm_dots_kernel(GemmDescT<double> d, int64_t kper, int ncol) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t m0 = (int64_t)(blockIdx.x / cg::this_cluster().num_blocks()) * DG_ROWS + 4 * warp;
+  const int64_t n0 = (int64_t)blockIdx.y * ncol;
+  const int nc = (int)((d.N - n0 < ncol) ? d.N - n0 : ncol);
+  const int64_t kbeg = (int64_t)cg::this_cluster().block_rank() * kper;
+  const int64_t kend = (kbeg + kper < d.K) ? kbeg + kper : d.K;
+  const double* Ap[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) Ap[r] = d.A + ((m0 + r < d.M) ? m0 + r : d.M - 1) * d.lda;
+  const double* Bp = d.B + n0 * d.ldb;
+  double acc[4 * DG_NC];
+#pragma unroll
+  for (int q = 0; q < 4 * DG_NC; ++q) acc[q] = 0.0;
+  for (int64_t k = kbeg + lane; k < kend; k += 32) {
+    double a[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) a[r] = Ap[r][k];
+#pragma unroll
+    for (int j = 0; j < DG_NC; ++j)
+      if (j < nc) {
+        const double b = Bp[j * d.ldb + k];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[r * DG_NC + j] = fma(a[r], b, acc[r * DG_NC + j]);
+      }
+  }
+  int idx = 0;  // output this lane ends with: row idx / 8, column idx % 8
+#pragma unroll
+  for (int half = 16; half >= 1; half >>= 1) {
+    const bool up = (lane & half) != 0;
+#pragma unroll
+    for (int q = 0; q < half; ++q) {
+      const double send = up ? acc[q] : acc[q + half];
+      const double keep = up ? acc[q + half] : acc[q];
+      acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+    }
+    if (up) idx += half;
+  }
+  const int j = idx % DG_NC;
+  dg_finish<kGemmPlain>(d, acc[0], m0 + idx / DG_NC, (j < nc) ? n0 + j : d.N);
+}
+
+// True when the FP64 product takes the kernels above: fewer than four 64 x 64
+// tiles per SM (a last wave of idle SMs costs more than a tile's reuse of its
+// operands saves; at 9 tiles per SM, 2304 x 2304 x 32, both take 357 us), or
+// more than a tenth of the tiles is padding.
+inline bool dg_narrow(const fraclap_ctx* ctx, int64_t M, int64_t N) {
+  const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
+  const int64_t tiles = cdiv(M, BM) * cdiv(N, BN);
+  return tiles < 4 * sms || (double)(tiles * BM * BN) > 1.1 * (double)M * (double)N;
+}
+
+template <bool TA, bool TB, int MODE>
+int launch_narrow(fraclap_ctx* ctx, const GemmDescT<double>& d, cudaStream_t st) {
+  const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
+  const int64_t gx = cdiv(d.M, DG_ROWS), gy = cdiv(d.N, DG_NC);
+  const int ncol = (int)cdiv(d.N, gy);  // the columns dealt evenly
+  FL_CHECK(ctx, gy <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm: N = %lld too large", (long long)d.N);
+  int S = 1;
+  while (S < 8 && gx * gy * S < 4 * sms && d.K >= 256 * (int64_t)S) S *= 2;
+  const int64_t kper = cdiv(cdiv(d.K > 0 ? d.K : 1, S), 32) * 32;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(gx * S), (unsigned)gy, 1);
+  cfg.blockDim = dim3(DG_NT);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)S;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if constexpr (TA)
+    FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, dgemm_dots_kernel, d, kper, ncol));
+  else
+    FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, dgemm_rows_kernel<TB, MODE>, d, kper, ncol));
+  count_launch(ctx);
+  return 0;
+}
+
 template <class T, bool TA, bool TB, int MODE>
 int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st) {
   if constexpr (std::is_same<T, float>::value && MODE != kGemmSymA) {
@@ -312,6 +490,9 @@ int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st
       FL_CUDA(ctx, cudaGetLastError());
       return 0;
     }
+  }
+  if constexpr (std::is_same<T, double>::value && MODE != kGemmLowerC && !(TA && TB)) {
+    if (d.K2 == 0 && dg_narrow(ctx, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
   }
   const int64_t gx = cdiv(d.M, BM), gy = cdiv(d.N, BN);
   FL_CHECK(ctx, gy <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm: N = %lld too large", (long long)d.N);
