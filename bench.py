@@ -226,11 +226,9 @@ def refine_slice_counts(iterations: int, cap: int, digit_bits: int = 7) -> list:
     return out
 
 
-# DRAM bytes per BF16 flop of ozaki_tc_kernel (128 x 192 tiles) from one ncu
-# capture of the 4096^3 product with the current kernel: (9.98 + 1.32) GB
-# over 4.95e12 flop; its tile re-streaming grows in proportion to the flops.
-# None whenever the kernel changes until it is captured again.
-OZAKI_DRAM_BYTES_PER_FLOP = 2.285e-3
+# DRAM bytes per BF16 flop of ozaki_tc_kernel from an ncu capture of the 4096^3
+# product; None whenever the kernel changes until it is captured again.
+OZAKI_DRAM_BYTES_PER_FLOP = None
 
 
 def run_path(F, ctx, p, path, args, mask, Fd, pf, pa, U, app_ws, barrier, steps=None, warmup=None):
@@ -388,7 +386,7 @@ def run_gpu(args, rank, world, local_rank):
         dur = g_ms / max(g_cnt, 1)
         # average over the launches of one step: 2 per refinement iteration
         # (fewer slices in the first two) and the apply's 2
-        digit_bits = R["ctx"].get_schedule("ozaki_bits")
+        digit_bits = 8  # balanced digits: s of 8 bits for s slices in the refinement and the apply
         per_iter = refine_slice_counts(len(R.get("refine", [])) or 3, REFINE_ITERS, digit_bits)
         total = sum(2 * ozaki_bf16_flops(n, sl) for sl in per_iter)
         launches_per_step = 2 * len(per_iter)

@@ -569,9 +569,10 @@ int fraclap_partition_spectrum(fraclap_ctx* ctx, int64_t n, const int64_t* rowpt
  *  FRACLAP_SCHED_OZAKI_GROUP: tile rows per raster group of the slice-product
  *    kernel (fraclap_dgemm_ozaki, the refinement's residual products, the
  *    sliced apply), 0..4096; 0 = every tile row in one group [8].
- *  FRACLAP_SCHED_OZAKI_BITS: digit width of the slices when K > 256: 7
- *    (exact chunks of 1024, ceil(8 s / 7) digits per operand) or 8 (exact
- *    chunks of 256, s digits: fewer slice pairs, more chunk sums) [7].
+ *  FRACLAP_SCHED_OZAKI_BITS: magnitude bits of the slices' balanced digits
+ *    when K > 256: 7 (digits of 8 bits in [-128, 128], exact chunks of 1024;
+ *    s digits per operand for s = 6 and 7, s + 1 otherwise) or 8 (digits of 9
+ *    bits, exact chunks of 256, s digits: more chunk sums) [7].
  *  FRACLAP_SCHED_FP32_STAGES: the FP32 products of eig_full_mixed's band
  *    reduction and first back-transformation: 0 on the FP32 FMA kernel, 1 on
  *    the tensor cores as three TF32 products (FP32-level accuracy, a few

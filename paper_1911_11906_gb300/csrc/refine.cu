@@ -486,6 +486,7 @@ constexpr double kConvergedR = 3e-9;
 constexpr int kRefineSlices = 7;
 constexpr int kRefineFirstSlices = 5;   // first iteration (40 bits)
 constexpr int kRefineSecondSlices = 6;  // second iteration (48 bits)
+// each slice is one digit of 8 bits: 15, 21 and 28 digit pairs a product
 
 __device__ void cluster_jacobi_body(const double* Sc, const double* Bc, int c, double* Q, double* w,
                                     int32_t* status) {
@@ -942,14 +943,14 @@ int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t
     {
       StageTimer tm(ctx, kStageResidualGemm, st);
       Arena oz = *ar;
-      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, -1.0, X, ldx, X, ldx, 0.0, R, n, slices_it, true, &oz, st));
+      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, -1.0, X, ldx, X, ldx, 0.0, R, n, slices_it, true, &oz, st, slices_it));
     }
     add_identity<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(R, n, n);
     count_launch(ctx);
     {
       StageTimer tm(ctx, kStageResidualGemm, st);
       Arena oz = *ar;
-      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, 1.0, X, ldx, AX, n, 0.0, S, n, slices_it, true, &oz, st));
+      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, 1.0, X, ldx, AX, n, 0.0, S, n, slices_it, true, &oz, st, slices_it));
     }
     span.start(kStageRefineNorms);
     ritz_values<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(S, n, R, n, n, lt);
