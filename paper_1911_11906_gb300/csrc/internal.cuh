@@ -277,6 +277,7 @@ struct Stage2T {
   T* refl;        // (n-1) * kmax * b
   double* rtau;   // (n-1) * kmax
   int* progress;  // 2 (n + 1): completed steps per sweep, then published subdiagonal values
+  T* ut;          // block factors of the back-transformation (b = 32, 64)
   int64_t kmax;
 };
 using Stage2 = Stage2T<double>;

@@ -428,6 +428,349 @@ q2t_apply_kernel(const T* __restrict__ refl, const double* __restrict__ rtau, in
   }
 }
 
+// ---------------------------------------------------------------------------
+// Y <- Y Q2^T in blocks (b = 32 and 64).  For one step k, B reflectors of
+// consecutive sweeps s = qB .. qB + B - 1 act on 2B - 1 rows from
+// base = 1 + kB + qB; their product H(qB) ... H(qB + B - 1) is I - V T V^T with
+// V(i + t, i) = v_i(t), a parallelogram, and T upper triangular.  The factor
+// -U = -V T (stored by columns of 2B rows) is formed once per block by
+// q2_factor_kernel; q2_block_kernel then streams the blocks: a CTA owns NCB
+// columns of Z, keeps the 2B rows of the window in shared memory, and for each
+// block forms W = V^T Z and Z += (-U) W as two small products in registers.
+// The next block's window is B rows higher: the upper half becomes the lower
+// one, the finished lower half goes to global memory and the rows that enter
+// (fetched a block ahead) take its place.
+//
+// Why: applied one by one, every reflector costs a dot product over the lanes
+// that share a column (three shuffles) and a one-row slide, a serial chain of
+// some 190 ns per reflector at n = 8810, 16 % of the FP32 pipe; in blocks the
+// FMAs are independent and run in packed pairs, for 1.4 times the flops (the
+// factor U fills the parallelogram; the loops skip its zero corners).  What
+// bounds them now is the shared-memory bandwidth (1.5 to 2 bytes per FMA at
+// 8 x 4 and 4 x 4 outputs a thread) and the latency of eight warps an SM.
+// GB300, the whole stage: FP32 n = 8810, b = 64 112 -> 68 ms (of which the
+// factors some 9), n = 3001 12.1 -> 5 ms; FP64 n = 2304, b = 32 79 -> 39 ms,
+// n = 751 8.6 -> 4.8 ms, bound by the FP64 pipe.
+// ---------------------------------------------------------------------------
+template <class T>
+struct Pair2;  // two values along the rows of an operand, multiplied by one broadcast value
+template <>
+struct Pair2<float> {
+  unsigned long long v;
+  static __device__ __forceinline__ Pair2 of(float a, float b) {
+    Pair2 p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p.v) : "f"(a), "f"(b));
+    return p;
+  }
+  __device__ __forceinline__ void get(float* a, float* b) const {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(*a), "=f"(*b) : "l"(v));
+  }
+  __device__ __forceinline__ void fma(const Pair2& x, const Pair2& y) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(v) : "l"(x.v), "l"(y.v));
+  }
+};
+template <>
+struct Pair2<double> {
+  double x, y;
+  static __device__ __forceinline__ Pair2 of(double a, double b) { return Pair2{a, b}; }
+  __device__ __forceinline__ void get(double* a, double* b) const { *a = x, *b = y; }
+  __device__ __forceinline__ void fma(const Pair2& p, const Pair2& q) {
+    x = ::fma(p.x, q.x, x);
+    y = ::fma(p.y, q.y, y);
+  }
+};
+
+// Blocks of step k start at k N0 - k (k - 1) / 2, N0 = ceil((n - 1) / B).
+__host__ __device__ inline int64_t q2_block_offset(int64_t k, int64_t N0) { return k * N0 - k * (k - 1) / 2; }
+
+template <int B>
+constexpr size_t q2_factor_smem() {
+  return sizeof(double) * (3 * B * (B + 1));
+}
+
+// One CTA per block: V from the reflectors, G = V^T V, T by the column
+// recurrence T(0:i, i) = -tau_i T(0:i, 0:i) G(0:i, i), and -U = -V T, all in FP64
+// (-U is rounded once, so the block is orthogonal to the rounding of its
+// factors; the FP64 work, some n^2 b / 8 FMAs, is a few per cent of the stage).
+template <class T, int B>
+__global__ void __launch_bounds__(256) q2_factor_kernel(const T* __restrict__ refl, const double* __restrict__ rtau,
+                                                        int64_t n, int64_t kmax, int64_t N0, T* __restrict__ ut) {
+  extern __shared__ __align__(128) unsigned char q2_smem[];
+  constexpr int LD = B + 1;
+  double* Ts = reinterpret_cast<double*>(q2_smem);
+  double* G = Ts + B * LD;
+  double* V = G + B * LD;  // V[i][t] (converted once: a conversion costs the FP64 pipe as much as an FMA)
+  __shared__ double tau[B];
+  const int tid = threadIdx.x;
+  // block index -> (k, q): row k of the triangle has N0 - k blocks
+  const int64_t blk = blockIdx.x;
+  int64_t k = (int64_t)((2.0 * N0 + 1.0 - sqrt((2.0 * N0 + 1.0) * (2.0 * N0 + 1.0) - 8.0 * (double)blk)) * 0.5);
+  if (k < 0) k = 0;
+  while (k > 0 && q2_block_offset(k, N0) > blk) --k;
+  while (q2_block_offset(k + 1, N0) <= blk) ++k;
+  const int64_t q = blk - q2_block_offset(k, N0), smax = n - 2 - k * B;
+  for (int e = tid; e < B * B; e += 256) {
+    const int64_t s = q * B + e / B;
+    V[(e / B) * LD + e % B] = (s <= smax) ? (double)refl[(s * kmax + k) * B + e % B] : 0.0;
+  }
+  if (tid < B) tau[tid] = (q * B + tid <= smax) ? rtau[(q * B + tid) * kmax + k] : 0.0;
+  __syncthreads();
+  for (int e = tid; e < B * B; e += 256) {
+    const int i = e % B, j = e / B, o = j - i;  // i < j: rows j .. i + B - 1
+    Ts[i * LD + j] = 0.0;
+    if (o <= 0) continue;
+    double sum = 0.0;
+    for (int t = 0; t < B - o; ++t) sum = ::fma(V[j * LD + t], V[i * LD + t + o], sum);
+    G[i * LD + j] = sum;
+  }
+  __syncthreads();
+  // row i of T by four lanes: T(i, j) = -tau_j sum_{i <= p < j} T(i, p) G(p, j)
+  if (tid < 4 * B) {
+    const int i = tid >> 2, part = tid & 3;
+    if (part == 0) Ts[i * LD + i] = tau[i];
+    for (int j = 1; j < B; ++j) {
+      double sum = 0.0;
+      __syncwarp();
+      if (i < j)
+        for (int p = i + part; p < j; p += 4) sum = ::fma(Ts[i * LD + p], G[p * LD + j], sum);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+      if (i < j && part == 0) Ts[i * LD + j] = -tau[j] * sum;
+    }
+  }
+  __syncthreads();
+  // -U(r, i) = -sum_{i' <= i, 0 <= r - i' < B} V(r, i') T(i', i), stored [i][r]
+  T* out = ut + blk * (2 * B * B);
+  for (int e = tid; e < 2 * B * B; e += 256) {
+    const int r = e % (2 * B), i = e / (2 * B);
+    const int lo = (r >= B) ? r - B + 1 : 0, hi = (r < i) ? r : i;
+    double sum = 0.0;
+    for (int p = lo; p <= hi; ++p) sum = ::fma(V[p * LD + r - p], Ts[p * LD + i], sum);
+    out[e] = (T)(-sum);
+  }
+}
+
+template <class T, int B, int NCB>
+struct Q2Shape {
+  static constexpr bool F32 = sizeof(T) == 4;
+  static constexpr int RT = F32 ? 4 : 2;                       // rows per thread of each half (and of W)
+  static constexpr int CT = F32 ? (NCB >= 32 ? 4 : 2) : 2;  // columns per thread
+  static constexpr int NT = (B / RT) * (NCB / CT);             // threads
+  static constexpr int LC = (NCB / CT < 8) ? NCB / CT : 8;     // lanes of a warp along the columns
+  static constexpr int LDV = B + 16 / sizeof(T);
+  static constexpr size_t SMEM = sizeof(T) * (2 * B * LDV + 2 * B * B + 2 * B * NCB + B * NCB);
+};
+
+template <class T, int N>
+struct alignas(sizeof(T) * N) Vec {
+  T v[N];
+};
+
+template <class T, int B, int NCB>
+__global__ void __launch_bounds__(Q2Shape<T, B, NCB>::NT)
+q2_block_kernel(const T* __restrict__ refl, const T* __restrict__ ut, int64_t n, int64_t kmax, int64_t N0, T* Y,
+                int64_t ldy, int64_t ncols) {
+  using Sh = Q2Shape<T, B, NCB>;
+  using P = Pair2<T>;
+  constexpr int RT = Sh::RT, CT = Sh::CT, NT = Sh::NT, LC = Sh::LC, LDV = Sh::LDV;
+  constexpr int WC = (NCB / CT) / LC, LG = 32 / LC;
+  constexpr int VPER = B * B / NT;
+  extern __shared__ __align__(128) unsigned char q2_smem[];
+  T* Us = reinterpret_cast<T*>(q2_smem);  // [B][2B]
+  T* Vs = Us + 2 * B * B;                 // [2B][LDV], V(r, i)
+  T* Zs = Vs + 2 * B * LDV;               // [2][B][NCB]
+  T* Ws = Zs + 2 * B * NCB;               // [B][NCB]
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g0 = (warp / WC) * LG, g = g0 + lane / LC;        // row group (warp's first, this thread's)
+  const int c0 = ((warp % WC) * LC + lane % LC) * CT;         // first column of this thread in the tile
+  const int64_t col = (int64_t)blockIdx.x * NCB + c0;
+  const int nc = (int)((ncols - col >= CT) ? CT : (ncols > col ? ncols - col : 0));
+
+  auto load_rows = [&](int64_t row0, T (&z)[RT][CT]) {  // rows row0 + g RT + q of the thread's columns
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+      const int64_t row = row0 + g * RT + q;
+#pragma unroll
+      for (int c = 0; c < CT; ++c) z[q][c] = (row < n && c < nc) ? Y[row * ldy + col + c] : T(0);
+    }
+  };
+  auto store_rows = [&](int64_t row0, const T (&z)[RT][CT]) {
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+      const int64_t row = row0 + g * RT + q;
+#pragma unroll
+      for (int c = 0; c < CT; ++c)
+        if (row < n && c < nc) Y[row * ldy + col + c] = z[q][c];
+    }
+  };
+  auto put_half = [&](int half, const T (&z)[RT][CT]) {
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+      Vec<T, CT> o;
+#pragma unroll
+      for (int c = 0; c < CT; ++c) o.v[c] = z[q][c];
+      *reinterpret_cast<Vec<T, CT>*>(&Zs[(half * B + g * RT + q) * NCB + c0]) = o;
+    }
+  };
+  auto get_half = [&](int half, T (&z)[RT][CT]) {
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+      const Vec<T, CT> o = *reinterpret_cast<const Vec<T, CT>*>(&Zs[(half * B + g * RT + q) * NCB + c0]);
+#pragma unroll
+      for (int c = 0; c < CT; ++c) z[q][c] = o.v[c];
+    }
+  };
+  auto fetch_v = [&](int64_t k, int64_t q, T (&v)[VPER]) {
+    const int64_t smax = n - 2 - k * B;
+#pragma unroll
+    for (int e = 0; e < VPER; ++e) {
+      const int p = tid + e * NT;
+      const int64_t s = q * B + p / B;
+      v[e] = (s <= smax) ? __ldg(refl + (s * kmax + k) * B + p % B) : T(0);
+    }
+  };
+  auto put_v = [&](const T (&v)[VPER]) {
+#pragma unroll
+    for (int e = 0; e < VPER; ++e) {
+      const int p = tid + e * NT, i = p / B, t = p % B;
+      Vs[(i + t) * LDV + i] = v[e];
+    }
+  };
+  auto fetch_u = [&](int64_t blk) {
+    const T* src = ut + blk * (2 * B * B);
+    T* dst = Us;
+    constexpr int E = 16 / sizeof(T);
+    for (int p = tid * E; p < 2 * B * B; p += NT * E)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst + p)),
+                   "l"(src + p)
+                   : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  for (int p = tid; p < 2 * B * LDV; p += NT) Vs[p] = T(0);  // the corners outside the parallelogram stay zero
+  for (int64_t k = 0; k < kmax; ++k) {
+    const int64_t N = N0 - k, row_k = 1 + k * B;  // blocks N - 1 .. 0, block q starts at row row_k + q B
+    if (N <= 0) break;
+    __syncthreads();  // the previous step's rows are in global memory, the buffers are free
+    T v[VPER], zn[RT][CT];
+    fetch_v(k, N - 1, v);
+    put_v(v);
+    int top = 0;
+    load_rows(row_k + (N - 1) * B, zn);
+    put_half(0, zn);
+    load_rows(row_k + N * B, zn);
+    put_half(1, zn);
+    for (int64_t q = N - 1; q >= 0; --q) {
+      const bool more = q > 0;
+      if (more) {
+        fetch_v(k, q - 1, v);
+        load_rows(row_k + (q - 1) * B, zn);
+      }
+      __syncthreads();
+      fetch_u(q2_block_offset(k, N0) + q);  // last read before this barrier; lands while W is formed
+      {  // W = V^T Z: rows i = g RT .. of W, over r = i .. i + B - 1 of the window
+        P acc[RT / 2][CT];
+#pragma unroll
+        for (int a = 0; a < RT / 2; ++a)
+#pragma unroll
+          for (int c = 0; c < CT; ++c) acc[a][c] = P::of(T(0), T(0));
+        const int lo = g0 * RT, hi = (g0 + LG) * RT + B - 1;  // r of the warp's rows
+        const T* vp = Vs + g * RT;
+        auto dot = [&](int r0, int r1, int half, int sub) {
+          const T* zp = Zs + (half * B - sub) * NCB + c0;
+#pragma unroll 4
+          for (int r = r0; r < r1; ++r) {
+            const Vec<T, RT> a = *reinterpret_cast<const Vec<T, RT>*>(vp + r * LDV);
+            const Vec<T, CT> z = *reinterpret_cast<const Vec<T, CT>*>(zp + r * NCB);
+#pragma unroll
+            for (int c = 0; c < CT; ++c) {
+              const P d = P::of(z.v[c], z.v[c]);
+#pragma unroll
+              for (int i = 0; i < RT / 2; ++i) acc[i][c].fma(P::of(a.v[2 * i], a.v[2 * i + 1]), d);
+            }
+          }
+        };
+        dot(lo, B, top, 0);
+        dot(B, hi < 2 * B ? hi : 2 * B, top ^ 1, B);
+#pragma unroll
+        for (int i = 0; i < RT / 2; ++i) {
+          Vec<T, CT> w0, w1;
+#pragma unroll
+          for (int c = 0; c < CT; ++c) acc[i][c].get(&w0.v[c], &w1.v[c]);
+          T* wp = Ws + (g * RT + 2 * i) * NCB + c0;
+          *reinterpret_cast<Vec<T, CT>*>(wp) = w0;
+          *reinterpret_cast<Vec<T, CT>*>(wp + NCB) = w1;
+        }
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      if (more) put_v(v);
+      {  // Z += (-U) W: rows g RT .. of either half; the lower half starts at i = row + 1
+        P at[RT / 2][CT], ab[RT / 2][CT];  // the change of Z, added to it once
+#pragma unroll
+        for (int i = 0; i < RT / 2; ++i)
+#pragma unroll
+          for (int c = 0; c < CT; ++c) at[i][c] = ab[i][c] = P::of(T(0), T(0));
+        const T* up = Us + g * RT;
+        const T* wp = Ws + c0;
+        const int lo = g0 * RT + 1;  // smaller i have zeros in every lower row of this warp
+        auto wdup = [&](int i, P (&d)[CT]) {
+          const Vec<T, CT> w = *reinterpret_cast<const Vec<T, CT>*>(wp + i * NCB);
+#pragma unroll
+          for (int c = 0; c < CT; ++c) d[c] = P::of(w.v[c], w.v[c]);
+        };
+#pragma unroll 4
+        for (int i = 0; i < lo; ++i) {
+          P d[CT];
+          wdup(i, d);
+          const Vec<T, RT> u = *reinterpret_cast<const Vec<T, RT>*>(up + i * (2 * B));
+#pragma unroll
+          for (int c = 0; c < CT; ++c)
+#pragma unroll
+            for (int r = 0; r < RT / 2; ++r) at[r][c].fma(P::of(u.v[2 * r], u.v[2 * r + 1]), d[c]);
+        }
+#pragma unroll 4
+        for (int i = lo; i < B; ++i) {
+          P d[CT];
+          wdup(i, d);
+          const Vec<T, RT> u = *reinterpret_cast<const Vec<T, RT>*>(up + i * (2 * B));
+          const Vec<T, RT> l = *reinterpret_cast<const Vec<T, RT>*>(up + i * (2 * B) + B);
+#pragma unroll
+          for (int c = 0; c < CT; ++c)
+#pragma unroll
+            for (int r = 0; r < RT / 2; ++r) {
+              at[r][c].fma(P::of(u.v[2 * r], u.v[2 * r + 1]), d[c]);
+              ab[r][c].fma(P::of(l.v[2 * r], l.v[2 * r + 1]), d[c]);
+            }
+        }
+        T zt[RT][CT], zb[RT][CT];
+        get_half(top, zt);
+        get_half(top ^ 1, zb);
+#pragma unroll
+        for (int i = 0; i < RT / 2; ++i)
+#pragma unroll
+          for (int c = 0; c < CT; ++c) {
+            T x, y;
+            at[i][c].get(&x, &y);
+            zt[2 * i][c] += x;
+            zt[2 * i + 1][c] += y;
+            ab[i][c].get(&x, &y);
+            zb[2 * i][c] += x;
+            zb[2 * i + 1][c] += y;
+          }
+        store_rows(row_k + (q + 1) * B, zb);
+        if (more) {
+          put_half(top, zt);
+          put_half(top ^ 1, zn);  // only this thread reads or writes these entries between the barriers
+        } else {
+          store_rows(row_k + q * B, zt);
+        }
+      }
+      top ^= 1;
+    }
+  }
+}
+
 // 32 x 32 tiled transpose: B(j, i) = A(i, j), A is rows x cols.
 template <class T>
 __global__ void transpose_kernel(const T* A, int64_t lda, T* Bm, int64_t ldb, int64_t rows,
@@ -454,6 +797,8 @@ int stage2_take(Arena* ar, int64_t n, int b, Stage2T<T>* s) {
   s->refl = ar->take<T>(nsw * s->kmax * b);
   s->rtau = ar->take<double>(nsw * s->kmax);
   s->progress = ar->take<int>(2 * (n + 1));  // completed steps, then published betas
+  // -U of every block of b reflectors (one step, b consecutive sweeps): 2b x b each
+  s->ut = (b == 32 || b == 64) ? ar->take<T>(s->kmax * (s->kmax + 1) / 2 * 2 * b * b) : nullptr;
   return 0;
 }
 
@@ -510,12 +855,55 @@ int transpose_run(fraclap_ctx* ctx, const T* A, int64_t lda, T* Bm, int64_t ldb,
   return 0;
 }
 
+// The block factors, then the blocks on CTAs of NCB columns each.
+template <class T, int B, int NCB>
+int q2_blocks_launch(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int64_t ncols, T* Yt, int64_t ldy,
+                     cudaStream_t st) {
+  using Sh = Q2Shape<T, B, NCB>;
+  const int64_t N0 = s->kmax, blocks = N0 * (N0 + 1) / 2;  // N0 = ceil((n - 1) / B) = kmax
+  FL_CHECK(ctx, blocks <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "q2 back-transformation: n too large");
+  constexpr size_t fsm = q2_factor_smem<B>();
+  FL_CUDA(ctx, cudaFuncSetAttribute(q2_factor_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+  q2_factor_kernel<T, B><<<(unsigned)blocks, 256, fsm, st>>>(s->refl, s->rtau, n, s->kmax, N0, s->ut);
+  count_launch(ctx);
+  FL_CUDA(ctx, cudaFuncSetAttribute(q2_block_kernel<T, B, NCB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)Sh::SMEM));
+  q2_block_kernel<T, B, NCB><<<(unsigned)cdiv(ncols, NCB), Sh::NT, Sh::SMEM, st>>>(s->refl, s->ut, n, s->kmax, N0, Yt,
+                                                                                   ldy, ncols);
+  count_launch(ctx);
+  FL_CUDA(ctx, cudaGetLastError());
+  return 0;
+}
+
 // Z <- Q2 Z (n x ncols, ld ldz), through the transposed copy Yt (ld >= ncols).
 template <class T>
 int q2_apply_run(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int b, T* Z, int64_t ldz,
                  int64_t ncols, T* Yt, int64_t ldy, cudaStream_t st) {
   if (n < 2 || ncols <= 0) return 0;
   FL_TRY(transpose_run<T>(ctx, Z, ldz, Yt, ldy, n, ncols, st));
+  if ((b == 64 && ctx->q2_parts == 0) || b == 32) {
+    // Columns per CTA: the fewest columns on the busiest SM, the wider CTA at a
+    // tie (it reuses the factors more).  FP32, b = 64, 64 / 32 / 16 columns: n =
+    // 7735 52.6 / 58.1 / 76.5 ms, 4741 20.3 / 15.1 / 16.3, 2740 6.8 / 5.1 / 5.5,
+    // 1200 1.47 / 1.14 / 0.91.
+    const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
+    const auto cost = [&](int ncb) { return cdiv(cdiv(ncols, ncb), sms) * ncb; };
+    int rc = 0;
+    if constexpr (sizeof(T) == 8) {
+      if (b == 64) rc = q2_blocks_launch<T, 64, 16>(ctx, s, n, ncols, Yt, ldy, st);
+      else if (cost(16) <= cost(8)) rc = q2_blocks_launch<T, 32, 16>(ctx, s, n, ncols, Yt, ldy, st);
+      else rc = q2_blocks_launch<T, 32, 8>(ctx, s, n, ncols, Yt, ldy, st);
+    } else if (b == 64) {
+      if (cost(64) <= cost(32) && cost(64) <= cost(16)) rc = q2_blocks_launch<T, 64, 64>(ctx, s, n, ncols, Yt, ldy, st);
+      else if (cost(32) <= cost(16)) rc = q2_blocks_launch<T, 64, 32>(ctx, s, n, ncols, Yt, ldy, st);
+      else rc = q2_blocks_launch<T, 64, 16>(ctx, s, n, ncols, Yt, ldy, st);
+    } else {
+      if (cost(32) <= cost(16)) rc = q2_blocks_launch<T, 32, 32>(ctx, s, n, ncols, Yt, ldy, st);
+      else rc = q2_blocks_launch<T, 32, 16>(ctx, s, n, ncols, Yt, ldy, st);
+    }
+    if (rc) return rc;
+    return transpose_run<T>(ctx, Yt, ldy, Z, ldz, ncols, n, st);
+  }
   int cpw = 0;
   // parts per window at b = 64: 4 (16 rows per lane, 8 columns per warp),
   // 8 or 16 (fewer rows per lane, more warps over the same columns: the
@@ -543,7 +931,6 @@ int q2_apply_run(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int b, T* Z, 
   FL_Q2T(4, 1)
   FL_Q2T(8, 2)
   FL_Q2T(16, 4)
-  FL_Q2T(32, 8)
   if (b == 64) {
     if constexpr (sizeof(T) == 4) {  // FP64 windows of 16 rows would not fit the registers
       if (parts64 == 4) FL_Q2T(64, 4)
