@@ -19,12 +19,17 @@
 // then B(i, k) -= l_i (l_k d) for the trailing triangle), with explicit
 // round-to-nearest intrinsics so the compiler fuses nothing: the pivots,
 // hence the counts, are the same bits as a sequential factorisation.
+#include <cooperative_groups.h>
+
 #include "internal.cuh"
 
 namespace fraclap {
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int SL_NT = 256;
+constexpr size_t kClusterWindowMax = 200 * 1024;  // a cluster CTA's share of the window
 constexpr int kSmemWindowMaxLd = 168;  // (b + 1)^2 doubles + 2 (b + 1) in 227 KB
 
 // Half-bandwidth of the lower triangle: max(i - col) over the entries.
@@ -139,6 +144,153 @@ band_inertia_kernel(const double* BK, const double* BM, int64_t n, int b, const 
     __syncthreads();
   }
   if (!STORE && tid == 0) count[s] = s_zero ? -1 : neg;
+}
+
+// The same counts with a cluster of CTAs per shift (few shifts leave most SMs
+// idle, and one SM's FP64 pipe bounds a pivot's b^2 / 2 multiplies and
+// subtractions).  The rows of the band are dealt to the CTAs in panels of NB;
+// row y keeps its entries W[y][y - x] in its owner's shared memory.  Step p
+// applies the NB pivots of panel p: every CTA gathers L's entries of the panel
+// (each formed by the owner of its row) from its peers, updates its rows' NB
+// columns of panel p + 1, and after a cluster barrier the first warps
+// factorise panel p + 1 -- each CTA its own rows, and all of them the NB x NB
+// diagonal block, so that no pivot is exchanged: a lane per row, the pivot and
+// the multipliers by shuffles -- while the other warps update the remaining
+// columns.  A second barrier ends the step.  Every entry sees the same
+// operations in the same order (ascending pivots, each product and difference
+// rounded), so the pivots and counts are the bits of band_inertia_kernel.
+// Bound: a step's chain (gather, barrier, four divisions, barrier) beside the
+// FP64 pipe.  n = 8810, b = 128, 15 shifts on clusters of 8: NB = 4 16.9 ms, NB
+// = 8 18.9, NB = 2 31.6 (before the integer divisions left the loops), one CTA
+// per shift 62 ms.
+constexpr int SL_NB = 4;
+template <int NB>
+__global__ void __launch_bounds__(SL_NT)
+band_inertia_cluster_kernel(const double* BK, const double* BM, int n, int b, const double* sigma, int64_t* count,
+                            int slots, int lg) {  // 2^lg CTAs per shift
+  extern __shared__ __align__(16) double sl_smem[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CL = 1 << lg, rank = (int)cluster.block_rank();
+  const int s = (int)(blockIdx.x >> lg);
+  const int ld = b + 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = SL_NT / 32;
+  const int MR = slots * NB;  // rows of this CTA at one time
+  double* win = sl_smem;                    // MR rows of ld entries; panel P at slot (P / CL) % slots of its owner
+  double* lp = win + (size_t)MR * ld;       // [NB][MR]: L's entries of the next panel in this CTA's rows
+  double* lc = lp + (size_t)NB * MR;        // [NB][ld]: L's entries of the current panel, row j1 + i at i
+  double* f = lc + (size_t)NB * ld;         // [NB][ld]: those times the pivot
+  __shared__ double dcur[NB];
+  __shared__ int s_zero;
+  const double sg = sigma[s];
+  const int np = (n + NB - 1) / NB;
+  // This CTA's rows from panel P on: local panel index and slot of the first, row number and window row of the m-th.
+  struct Rows {
+    int first, slot;
+  };
+  auto rows_from = [&](int P) -> Rows {
+    const int first = (P + ((rank - P) & (CL - 1))) >> lg;
+    return Rows{first, first % slots};
+  };
+  auto row_of = [&](const Rows& r, int m) { return (((r.first + m / NB) << lg) + rank) * NB + m % NB; };
+  auto row_ptr = [&](const Rows& r, int m) {
+    int u = r.slot + m / NB;
+    if (u >= slots) u -= slots;
+    return win + (u * NB + m % NB) * ld;
+  };
+  auto load_rows = [&](int y0, int y1, int t0, int nt) {  // the owned ones of rows y0 .. y1 - 1
+    const Rows r = rows_from(y0 / NB);
+    for (int m0 = 0; row_of(r, m0) < y1; m0 += NB)
+      for (int e = t0; e < NB * ld; e += nt) {  // consecutive threads: the NB rows of one column
+        const int y = row_of(r, m0 + e % NB), o = e / NB, x = y - o;
+        if (y >= y0 && y < y1 && y < n) row_ptr(r, m0 + e % NB)[o] = (x >= 0) ? band_entry(BK, BM, ld, x, o, sg) : 0.0;
+      }
+  };
+  const int rw = (MR + 31 - NB) / (32 - NB);  // factorising warps: NB diagonal lanes, 32 - NB rows each
+  const int segs = (b + 31) / 32;
+  int neg = 0;
+  if (tid == 0) s_zero = 0;
+  load_rows(0, b + 2 * NB, tid, SL_NT);
+  cluster.sync();
+  for (int p = -1; p + 1 < np; ++p) {
+    const int j1 = (p + 1) * NB;  // first pivot of panel p + 1
+    const int in = ((j1 - 1 + b < n - 1) ? j1 - 1 + b : n - 1) - j1;  // last row panel p reaches, from j1
+    const Rows r1 = rows_from(p + 1);
+    if (p >= 0) {
+      for (int e = tid; e < NB * (in + 1); e += SL_NT) {
+        const int q = e % NB, i = e / NB, k = i / NB;  // row j1 + i lies in panel p + 1 + k
+        const double l = cluster.map_shared_rank(lp, (p + 1 + k) & (CL - 1))[q * MR + (k >> lg) * NB + i % NB];
+        lc[q * ld + i] = l;
+        f[q * ld + i] = __dmul_rn(l, dcur[q]);
+      }
+      __syncthreads();
+      // rows of this CTA, columns of panel p + 1
+      for (int e = tid; e < MR * NB; e += SL_NT) {
+        const int c = e % NB, m = e / NB, i = row_of(r1, m) - j1;
+        if (i > in || i < c) continue;
+        double* w = row_ptr(r1, m) + (i - c);
+        double a = *w;
+#pragma unroll
+        for (int q = 0; q < NB; ++q)
+          if (i + NB - q <= b) a = __dsub_rn(a, __dmul_rn(lc[q * ld + i], f[q * ld + c]));
+        *w = a;
+      }
+      cluster.sync();
+    }
+    if (warp < rw) {
+      // panel p + 1: lanes 0 .. NB - 1 the diagonal rows, the others rows past the panel
+      const Rows r2 = rows_from(p + 2);
+      const int m = warp * (32 - NB) + lane - NB;
+      const bool diag = lane < NB;
+      const int i = diag ? lane : row_of(r2, m) - j1;
+      const bool live = j1 + i < n && (diag || (m < MR && i <= NB - 1 + b));
+      const double* src = win;
+      if (diag) src = cluster.map_shared_rank(win + (((p + 1) >> lg) % slots * NB + lane) * ld, (p + 1) & (CL - 1));
+      else if (live) src = row_ptr(r2, m);
+      double w[NB];
+#pragma unroll
+      for (int c = 0; c < NB; ++c) w[c] = (live && i >= c && i - c <= b) ? src[i - c] : 0.0;
+      bool zero = false;
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        const double d = __shfl_sync(0xffffffffu, w[q], q);
+        if (j1 + q >= n || zero) continue;  // the same for every lane
+        if (d == 0.0) {
+          zero = true;
+          continue;
+        }
+        neg += (d < 0.0);
+        const bool below = live && i > q && i - q <= b;
+        const double l = below ? __ddiv_rn(w[q], d) : 0.0;
+        const double ld_q = __dmul_rn(l, d);
+#pragma unroll
+        for (int c = q + 1; c < NB; ++c) {
+          const double fc = __shfl_sync(0xffffffffu, ld_q, c);
+          if (below && i >= c) w[c] = __dsub_rn(w[c], __dmul_rn(l, fc));
+        }
+        if (!diag && m < MR) lp[q * MR + m] = l;
+        if (warp == 0 && lane == 0) dcur[q] = d;
+      }
+      if (zero && warp == 0 && lane == 0) s_zero = 1;
+    } else if (p >= 0) {
+      load_rows(j1 + NB + b, j1 + 2 * NB + b, tid - rw * 32, SL_NT - rw * 32);  // for panel p + 2
+      // the remaining columns of this CTA's rows, 32 entries of a row at a time
+      for (int it = warp - rw; it < MR * segs; it += nwarp - rw) {
+        const int m = it / segs, i = row_of(r1, m) - j1, o = (it - m * segs) * 32 + lane;  // entry of column y - o
+        if (i > in) break;
+        if (o > i - NB) continue;
+        double* w = row_ptr(r1, m) + o;
+        const double* lq = lc + i;
+        const double* fx = f + i - o;
+        double a = *w;
+#pragma unroll
+        for (int q = 0; q < NB; ++q)
+          if (i + NB - q <= b) a = __dsub_rn(a, __dmul_rn(lq[q * ld], fx[q * ld]));
+        *w = a;
+      }
+    }
+    cluster.sync();
+    if (s_zero) break;  // every CTA factorised the same diagonal block
+  }
+  if (rank == 0 && tid == 0) count[s] = s_zero ? -1 : neg;
 }
 
 // Negative pivots of the Sturm recurrence of T - sigma I:
@@ -264,6 +416,36 @@ int launch_inertia(fraclap_ctx* ctx, int64_t n, int64_t b, const InertiaWork& w,
                    int64_t nsig, int64_t* count, cudaStream_t st) {
   if (nsig <= 0) return 0;
   FL_CHECK(ctx, nsig <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "inertia: too many shifts");
+  // CTAs per shift: as many as the SMs hold at once (at most 8, the portable
+  // cluster).  Below b = 16 a pivot is too little work to share.
+  int lg = 3;
+  while (lg > 0 && (nsig << lg) > ctx->sm_count) --lg;
+  const int CL = 1 << lg;
+  if (CL > 1 && b >= 16) {
+    const int64_t ld = b + 1;
+    const int64_t slots = cdiv((b + SL_NB - 1) / SL_NB + 3, CL) + 1, rows = slots * SL_NB;
+    const size_t smem = sizeof(double) * (size_t)(rows * (ld + SL_NB) + 2 * SL_NB * ld);
+    if (smem <= kClusterWindowMax && rows <= 4 * (32 - SL_NB)) {
+      auto kern = band_inertia_cluster_kernel<SL_NB>;
+      FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterWindowMax));
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(nsig * CL));
+      cfg.blockDim = dim3(SL_NT);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)CL;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, (const double*)w.BK, (const double*)w.BM, (int)n, (int)b, sigma, count, (int)slots,
+                                      lg));
+      count_launch(ctx);
+      return 0;
+    }
+  }
   if (smem_window(b)) {
     const size_t ld = (size_t)b + 1;
     const size_t smem = (ld * ld + 2 * ld) * sizeof(double);
