@@ -579,7 +579,7 @@ int fraclap_partition_spectrum(fraclap_ctx* ctx, int64_t n, const int64_t* rowpt
  *    2^-22 per product instead of 2^-24) [0].
  *  FRACLAP_SCHED_OZAKI_TILE_N: columns of the slice-product kernel's output
  *    tile, 128, 192 or 256 (rows are 128; outputs of at most 128 columns
- *    always take 128) [192].
+ *    always take 128) [256].
  *  FRACLAP_SCHED_Q2_PARTS: at half-bandwidth 64, the lanes that share one
  *    column's window of the stage-2 back-transformation: 4, 8 or 16 (16, 8 or
  *    4 rows per lane; more parts give more warps over the same columns; FP64

@@ -23,7 +23,7 @@ struct fraclap_ctx {
   int apply_slices = 0;          // frac_apply products: 0 = FP64 engine, s = s BF16 slices (tensor cores)
   int oz_group = 8;              // slice-product kernel: tile rows per raster group (0 = all rows)
   int oz_bits = 7;               // slice-product kernel: digit width for K > 256 (7 or 8)
-  int oz_tile_n = 192;           // slice-product kernel: tile columns (128, 192 or 256)
+  int oz_tile_n = 256;           // slice-product kernel: tile columns (128, 192 or 256)
   int oz_cluster = 1;            // slice-product kernel: CTAs per cluster sharing a B tile (1 or 2)
   int q2_parts = 0;              // stage-2 back-transformation at b = 64: lane parts per window (0: default 8)
   int fp32_stages_tc = 0;        // mixed route: FP32 band reduction and Q1 products on the tensor cores (TF32 x 3)
@@ -311,7 +311,7 @@ int cluster_eig(fraclap_ctx* ctx, double* S, int64_t c, double* w, double* Q, Ar
                 cudaStream_t st);
 
 // FP64-accurate GEMM through BF16 tensor-core slices (ozaki.cu).
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s);
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false);
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
                int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits = 0);

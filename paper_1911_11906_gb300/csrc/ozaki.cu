@@ -22,8 +22,7 @@
 // tcgen05.mma with operands brought into shared memory by TMA
 // (cp.async.bulk.tensor, 128-byte swizzle) and the FP32 chunk accumulators in
 // tensor memory (four buffers at 128 columns, two at 256), so that the
-// draining and FP64 folding of finished chunks overlap the products of the
-// next ones; a plain mma.sync m16n8k16 kernel is kept as the reference route
+// draining of finished chunks overlaps the products of the next ones; a plain mma.sync m16n8k16 kernel is kept as the reference route
 // for checking it.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -326,22 +325,26 @@ ozaki_kernel(const __nv_bfloat16* __restrict__ SA, const __nv_bfloat16* __restri
 
 
 // ----------------------------------------------------------------------------
-// tcgen05 route: CTA tile 128 (rows of op(A)) x 128 (columns of op(B)).
-// Warp 0: TMA producer; warp 1: TMEM owner and MMA issuer; warps 2-9:
-// epilogue, two warps per TMEM lane quarter (lanes 32 (w % 4) ..), each
-// thread one output row and 64 of the 128 columns.  Six 32 KB stages keep
-// enough bytes in flight to cover the L2 latency.
+// tcgen05 route.  A work item is one output tile (128 rows of op(A) x TCN
+// columns of op(B)) and one group of digit pairs of a diagonal p + q = dg (all
+// of them, or a few when the tiles alone do not fill the SMs): its CTA adds the
+// pairs' exact chunk sums in int32 and stores them to the item's plane of an
+// int32 array; combine_planes then forms C.  Warp 0: TMA producer; warp 1: TMEM
+// owner and MMA issuer; TCN / 16 epilogue warps, each one quarter of the TMEM
+// lanes and 64 columns: a thread keeps 64 sums, which fit its registers at
+// every tile width (folding each diagonal into C in FP64 here kept the
+// epilogue to 8 warps, whose 96 or 128 sums spilled, and held the MMAs up).
+//
+// Tiles: 128 x 256 moves 48 KB of slices per 4.2 MFLOP k-block against 32 KB
+// per 2.1 MFLOP at 128 x 128, with four stages instead of six and two
+// accumulators in the 512 TMEM columns instead of four.  Bound: the MMAs and
+// their shared-memory feed.  GB300, 8810 x 8810 x 8810 at 7 slices (28 pairs,
+// 3.83e13 flop): 256 columns 27.6 ms (1.39 PFLOP/s), 192 31.3 ms, against 38.9
+// at 192 with the folds; outputs of few columns, whose tiles now share the SMs
+// by diagonals: 2867 x 7 x 2867 0.44 -> 0.10 ms.
 // ----------------------------------------------------------------------------
-// The tile width TCN (128, 192 or 256 columns of op(B)) is a schedule
-// choice: a 128 x 256 tile moves 48 KB of slices per 4.2 MFLOP k-block
-// instead of 32 KB per 2.1 MFLOP (1.33x fewer L2 bytes per flop), with four
-// stages instead of six and the two accumulators filling all 512 TMEM
-// columns, but its epilogue threads keep 128 integer sums each, more than
-// their registers hold; 128 x 192 (40 KB per 3.1 MFLOP, five stages) keeps
-// 96 per thread.
 constexpr int TC_M = 128, TC_KB = 64;
-constexpr int TC_EPI_WARPS = 8;
-constexpr int TC_THREADS = 64 + 32 * TC_EPI_WARPS;
+constexpr int TC_EPI_COLS = 64;  // columns per epilogue thread
 constexpr int TC_A_BYTES = TC_M * TC_KB * 2;
 template <int TCN>
 struct OzTile {
@@ -349,11 +352,10 @@ struct OzTile {
   static constexpr int STAGES = (TCN == 256) ? 4 : (TCN == 192) ? 5 : 6;
   static constexpr int B_BYTES = TCN * TC_KB * 2;
   static constexpr int STAGE_BYTES = TC_A_BYTES + B_BYTES;
-  static constexpr int EPI_COLS = TCN * 4 / TC_EPI_WARPS;  // columns per epilogue thread
-  // FP32 chunk accumulators in the 512 TMEM columns: four at 128 columns
-  // (the MMA warp runs up to three chunks ahead of an epilogue that is
-  // folding a finished diagonal into C), two at 192 or 256; the allocation
-  // is the whole (power-of-two) 512 columns
+  static constexpr int EPI_WARPS = TCN / TC_EPI_COLS * 4;
+  static constexpr int THREADS = 64 + 32 * EPI_WARPS;
+  // FP32 chunk accumulators in the 512 TMEM columns: four at 128 columns,
+  // two at 192 or 256; the allocation is the whole (power-of-two) 512 columns
   static constexpr int NBUF = 512 / TCN;
   static constexpr uint32_t TMEM_COLS = 512;
   // kind::f16 instruction descriptor: D F32, A and B BF16, both K-major, M 128, N TCN.
@@ -363,6 +365,52 @@ struct OzTile {
 
 // 2^e for e in [-1022, 1023], from its bit pattern.
 __device__ __forceinline__ double pow2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// The digit pairs (p, q = dg - p) and the K-chunks of one item, for D digits,
+// nchunk chunks and at most U pairs per item: diagonals from the longest
+// (dg = D - 1) down, so that the longest items start first.  An item adds at
+// most 127 chunk sums (127 2^24 < 2^31): a K of more chunks is cut too.
+struct OzParts {
+  int D, U, nchunk, cper, kparts;
+  __host__ __device__ int of_diag(int dg) const { return (dg + U) / U * kparts; }
+  __host__ __device__ int count() const {
+    int t = 0;
+    for (int dg = 0; dg < D; ++dg) t += of_diag(dg);
+    return t;
+  }
+  __device__ void get(int part, int* dg, int* p0, int* p1, int* c0, int* c1) const {
+    int d = D - 1;
+    while (part >= of_diag(d)) part -= of_diag(d--);
+    *dg = d;
+    *p0 = part / kparts * U;
+    *p1 = (*p0 + U < d + 1) ? *p0 + U : d + 1;
+    *c0 = part % kparts * cper;
+    *c1 = (*c0 + cper < nchunk) ? *c0 + cper : nchunk;
+  }
+};
+// A plane: M x N column-major, or (lower, M >= N) its columns from the diagonal
+// down, packed.  plane_column(j) + i is entry (i, j).
+__host__ __device__ inline int64_t plane_size(int64_t M, int64_t N, bool lower) {
+  return lower ? M * N - N * (N - 1) / 2 : M * N;
+}
+__host__ __device__ inline int64_t plane_column(int64_t j, int64_t M, bool lower) {
+  return lower ? j * M - j * (j + 1) / 2 : j * M;
+}
+// U: all pairs of a diagonal, fewer when the longest item would then exceed an
+// even share of all pairs over the SMs (a function of the sizes alone, so that
+// the workspace and the sums do not depend on the context).
+inline OzParts oz_parts(int64_t M, int64_t N, int64_t Kp, int D, int w, bool lower) {
+  OzParts o;
+  const int64_t chunk = (int64_t)1 << (24 - 2 * w);
+  o.D = D;
+  o.nchunk = (int)cdiv(Kp, chunk);
+  const int64_t tiles = cdiv(M, TC_M) * cdiv(N, TC_M) / (lower ? 2 : 1);
+  const int64_t even = cdiv(std::max<int64_t>(tiles, 1) * (D * (D + 1) / 2), 152);
+  o.U = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(D, even), 127 / std::min(o.nchunk, 127)));
+  o.cper = std::min(o.nchunk, 127);
+  o.kparts = (int)cdiv(o.nchunk, o.cper);
+  return o;
+}
 
 // Order of the output tiles over the CTAs: groups of G consecutive tile rows;
 // inside a group, the G rows of one tile column are consecutive CTAs, then
@@ -418,20 +466,17 @@ __device__ __forceinline__ void ozaki_tile_of(int64_t idx, int TM, int TN, int G
 // lies past the last row or above the diagonal; its epilogue then writes
 // nothing.
 template <int TCN, int CS>
-__global__ void __launch_bounds__(TC_THREADS, 1)
-ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                const int* __restrict__ ea, const int* __restrict__ eb, int64_t M, int64_t N, int64_t Kp,
-                int s, int bits, int64_t chunk, double alpha, double beta, double* C, int64_t ldc,
-                int lower, int group, long long limit,
+__global__ void __launch_bounds__(OzTile<TCN>::THREADS, 1)
+ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int64_t M, int64_t N,
+                int64_t Kp, OzParts parts, int64_t chunk, int tiles, int32_t* P, int lower, int group, long long limit,
                 int32_t* status) {
-  constexpr int TC_N = TCN, TC_STAGES = OzTile<TCN>::STAGES, TC_B_BYTES = OzTile<TCN>::B_BYTES;
-  constexpr int TC_STAGE_BYTES = OzTile<TCN>::STAGE_BYTES, TC_EPI_COLS = OzTile<TCN>::EPI_COLS;
+  constexpr int TC_N = TCN, TC_STAGES = OzTile<TCN>::STAGES;
+  constexpr int TC_STAGE_BYTES = OzTile<TCN>::STAGE_BYTES, TC_EPI_WARPS = OzTile<TCN>::EPI_WARPS;
   constexpr uint32_t TC_TMEM_COLS = OzTile<TCN>::TMEM_COLS, TC_IDESC = OzTile<TCN>::IDESC;
   constexpr int NBUF = OzTile<TCN>::NBUF;
   constexpr int B_ROWS = TCN / CS;  // rows of the B tile this CTA loads (and multicasts)
   static_assert(CS == 1 || CS == 2 || CS == 4, "cluster of 1, 2 or 4 CTAs");
   static_assert((B_ROWS * 128) % 1024 == 0, "a B share starts on a 128-byte-swizzle atom");
-  (void)TC_B_BYTES;
   extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)tc_smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full_bar[TC_STAGES], empty_bar[TC_STAGES];
@@ -441,19 +486,22 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int TM = (int)((M + TC_M - 1) / TC_M), TN = (int)((N + TC_N - 1) / TC_N);
   const int rank = (CS > 1) ? (int)cluster_ctarank() : 0;
+  // items: all tiles (or clusters of tiles) of the first group of pairs, then of the next
+  const int unit = (int)(blockIdx.x / CS), part = unit / tiles, tile = unit - part * tiles;
+  int dg, pbeg, pend, cbeg, cend;
+  parts.get(part, &dg, &pbeg, &pend, &cbeg, &cend);
   int tm, tn;
   if (CS == 1) {
-    ozaki_tile_of((int64_t)blockIdx.x, TM, TN, group, lower != 0, TC_M, TC_N, &tm, &tn);
+    ozaki_tile_of(tile, TM, TN, group, lower != 0, TC_M, TC_N, &tm, &tn);
     if (tm >= TM || tn >= TN) return;
     if (lower && (int64_t)tm * TC_M + TC_M - 1 < (int64_t)tn * TC_N) return;  // tile above the diagonal
   } else {
     // the grid holds whole clusters of CS tile rows: no CTA leaves early
     int tc;
-    ozaki_tile_of((int64_t)(blockIdx.x / CS), (TM + CS - 1) / CS, TN, group, lower != 0, CS * TC_M, TC_N, &tc, &tn);
+    ozaki_tile_of(tile, (TM + CS - 1) / CS, TN, group, lower != 0, CS * TC_M, TC_N, &tc, &tn);
     tm = tc * CS + rank;
   }
   const int64_t m0 = (int64_t)tm * TC_M, n0 = (int64_t)tn * TC_N;
-  const int nchunk = (int)((Kp + chunk - 1) / chunk);
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < TC_STAGES; ++i) {
@@ -487,9 +535,8 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     if (lane == 0) {
       int it = 0;
       bool ok = true;
-      for (int dg = 0; dg < s && ok; ++dg)
-        for (int p = 0; p <= dg && ok; ++p)
-          for (int c = 0; c < nchunk && ok; ++c) {
+      for (int p = pbeg; p < pend && ok; ++p)
+          for (int c = cbeg; c < cend && ok; ++c) {
             const int q = dg - p;
             const int64_t c0 = (int64_t)c * chunk;
             const int nkb = (int)(((Kp - c0) < chunk ? (Kp - c0) : chunk) / TC_KB);
@@ -530,9 +577,8 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     if (lane == 0) {
       int it = 0, chunk_i = 0;
       bool ok = true;
-      for (int dg = 0; dg < s && ok; ++dg)
-        for (int p = 0; p <= dg && ok; ++p)
-          for (int c = 0; c < nchunk && ok; ++c, ++chunk_i) {
+      for (int p = pbeg; p < pend && ok; ++p)
+          for (int c = cbeg; c < cend && ok; ++c, ++chunk_i) {
             const int buf = chunk_i % NBUF;
             if (!mbar_wait(&acc_empty[buf], ((chunk_i / NBUF) & 1) ^ 1, limit) || *(volatile int*)&abort_sh) {
               ok = false;
@@ -570,77 +616,43 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
       mbar_wait(&done_bar, 0, limit);
     }
   } else {
-    // ---------------- epilogue: exact integer sums, FP64 once per diagonal ----------------
-    // Pairs are visited by diagonal p + q, which share one scale.  A chunk
-    // sum is an integer below 2^24 (exact in FP32), so it converts exactly
-    // to int32; up to 127 of them add exactly in an int32 accumulator, which
-    // is scaled (exactly, by a power of two) and added into C in FP64 at the
-    // end of the diagonal (or after 127 chunks).
+    // ---------------- epilogue: exact integer sums ----------------
+    // A chunk sum is an integer of at most 2^24 (exact in FP32), so it converts
+    // exactly to int32, and an item's at most 127 of them add exactly.
     const int lg = warp & 3;                          // TMEM lane quarter of this warp
     const int cbase = ((warp - 2) >> 2) * TC_EPI_COLS;  // this warp's columns of the tile
     const int64_t row = m0 + lg * 32 + lane;          // output row of this thread
-    const int er = (row < M) ? ea[row] : 0;
     int acc[TC_EPI_COLS];
 #pragma unroll
     for (int j = 0; j < TC_EPI_COLS; ++j) acc[j] = 0;
-    bool first = true;
-    int chunk_i = 0;
+    const int nacc = (pend - pbeg) * (cend - cbeg);
     bool ok = true;
-    for (int dg = 0; dg < s && ok; ++dg) {
-      int pending = 0;
-      for (int p = 0; p <= dg && ok; ++p) {
-        for (int c = 0; c < nchunk; ++c, ++chunk_i) {
-          const int buf = chunk_i % NBUF;
-          if (!mbar_wait(&acc_full[buf], (chunk_i / NBUF) & 1, limit) || *(volatile int*)&abort_sh) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * TC_N + cbase);
+    for (int chunk_i = 0; chunk_i < nacc; ++chunk_i) {
+      const int buf = chunk_i % NBUF;
+      if (!mbar_wait(&acc_full[buf], (chunk_i / NBUF) & 1, limit) || *(volatile int*)&abort_sh) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(buf * TC_N + cbase);
 #pragma unroll
-          for (int j0 = 0; j0 < TC_EPI_COLS; j0 += 16) {
-            uint32_t r[16];
-            tmem_ld16(taddr + j0, r);
-            tmem_wait_ld();
+      for (int j0 = 0; j0 < TC_EPI_COLS; j0 += 16) {
+        uint32_t r[16];
+        tmem_ld16(taddr + j0, r);
+        tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 16; ++j) acc[j0 + j] += __float2int_rz(__uint_as_float(r[j]));
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&acc_empty[buf]);
-          // one call site (the fold is inlined once): after 127 chunks, and
-          // after the last chunk of the diagonal
-          if (++pending == 127 || (p == dg && c == nchunk - 1)) {
-            // fold: acc 2^(e_i + f_j - sh) into C in FP64, then restart the sums
-            const int sh = 2 * digit_frac_bits(bits, s) - (bits + 1) * (2 * s - 2 - dg);
-            if (row < M) {
-              // opaque copies of the base pointers: the per-column addresses are
-              // formed here, not hoisted out of the diagonal loop into registers
-              const int* ebp;
-              double* cb;
-              asm volatile("mov.b64 %0, %1;" : "=l"(ebp) : "l"(eb + n0 + cbase));
-              asm volatile("mov.b64 %0, %1;" : "=l"(cb) : "l"(C + row + (n0 + cbase) * ldc));
+        for (int j = 0; j < 16; ++j) acc[j0 + j] += __float2int_rz(__uint_as_float(r[j]));
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_empty[buf]);
+    }
+    if (ok && row < M) {
+      int32_t* out = P + part * plane_size(M, N, lower != 0) + row;
 #pragma unroll
-              for (int j = 0; j < TC_EPI_COLS; ++j) {
-                const int64_t col = n0 + cbase + j;
-                if (col < N && !(lower && row < col)) {
-                  // acc 2^e in two exact power-of-two steps (each factor normal);
-                  // beyond |e| = 2044 the result is 0 or infinite either way
-                  int e = er + ebp[j] - sh;
-                  e = (e < -2044) ? -2044 : (e > 2044 ? 2044 : e);
-                  const int e1 = e / 2;
-                  const double v = alpha * (((double)acc[j] * pow2i(e1)) * pow2i(e - e1));
-                  double* cp = cb + j * ldc;
-                  *cp = first ? ((beta == 0.0) ? v : v + beta * *cp) : *cp + v;
-                }
-              }
-            }
-#pragma unroll
-            for (int j = 0; j < TC_EPI_COLS; ++j) acc[j] = 0;
-            first = false;
-            pending = 0;
-          }
-        }
+      for (int j = 0; j < TC_EPI_COLS; ++j) {
+        const int64_t col = n0 + cbase + j;
+        if (col < N && !(lower && row < col)) out[plane_column(col, M, lower != 0)] = acc[j];
       }
     }
     if (!ok) {
@@ -658,6 +670,45 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
   if (CS > 1) cluster_sync_all();  // no CTA leaves while a peer may still signal it
 }
 
+// C = alpha 2^(e_i + f_j - 2t + r (2D - 2)) sum_dg 2^(-r dg) P_dg + beta C from the
+// items' planes.  Up to four diagonals at a time are one exact 64-bit integer
+// (a diagonal's sum is below 2^31 times its items, and three shifts of at most
+// 9 bits follow), so an element costs a conversion and an FMA per four
+// diagonals; the lowest diagonals are added first.
+__global__ void combine_planes(const int32_t* __restrict__ P, const int* __restrict__ ea, const int* __restrict__ eb,
+                               int64_t M, int64_t N, OzParts parts, int w, double alpha, double beta, double* C,
+                               int64_t ldc, int lower) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = plane_size(M, N, lower != 0);
+  if (i >= M) return;
+  const int rb = w + 1, D = parts.D;
+  const int e0 = ea[i] - 2 * digit_frac_bits(w, D) + rb * (2 * D - 2);
+  for (int64_t j = blockIdx.y; j < N; j += gridDim.y) {
+    if (lower && i < j) break;
+    const int32_t* q = P + i + plane_column(j, M, lower != 0);
+    double v = 0.0;
+    int plane = 0;
+    for (int d = D - 1; d >= 0;) {  // planes from the highest dg (lowest weight) up
+      const int lo = (d >= 4) ? d - 3 : 0, g = d - lo + 1;
+      long long acc = 0;  // in units of 2^(-rb d), d the group's highest diagonal
+      for (int sh = 0; d >= lo; --d, sh += rb) {
+        long long t = 0;
+        for (int u = parts.of_diag(d); u > 0; --u, ++plane) t += __ldcs(q + plane * stride);
+        acc += t * (1ll << sh);
+      }
+      v = v * pow2i(-4 * rb) + (double)acc;  // every group but the last holds four diagonals
+      if (d >= 0) continue;
+      int e = e0 + eb[j] - rb * (g - 1);
+      // two exact power-of-two steps (each factor normal); beyond |e| = 2044 the
+      // result is 0 or infinite either way
+      e = (e < -2044) ? -2044 : (e > 2044 ? 2044 : e);
+      const int e1 = e / 2;
+      v = alpha * ((v * pow2i(e1)) * pow2i(e - e1));
+    }
+    double* c = C + i + j * ldc;
+    *c = (beta == 0.0) ? v : v + beta * *c;
+  }
+}
+
 // 3-D map over the slices S[s][rows][Kp] (bf16), box 64 (K) x box_rows x 1.
 bool slice_map(CUtensorMap* map, const __nv_bfloat16* S, int64_t rows, int64_t Kp, int s, int box_rows) {
   EncodeTiledFn fn = encode_tiled();
@@ -671,12 +722,11 @@ bool slice_map(CUtensorMap* map, const __nv_bfloat16* S, int64_t rows, int64_t K
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 template <int TCN, int CS>
-int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB, const int* ea, const int* eb,
-              int64_t M, int64_t N, int64_t Kp, int sl, int bits, int64_t chunk, double alpha, double beta,
-              double* C, int64_t ldc, bool lower, cudaStream_t st) {
+int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB, int64_t M, int64_t N, int64_t Kp,
+              const OzParts& parts, int64_t chunk, int32_t* P, bool lower, cudaStream_t st) {
   CUtensorMap ma, mb;
-  FL_CHECK(ctx, slice_map(&ma, SA, M, Kp, sl, TC_M) && slice_map(&mb, SB, N, Kp, sl, TCN / CS), FRACLAP_ERR_CUDA,
-           "ozaki_gemm: tensor map encoding failed");
+  FL_CHECK(ctx, slice_map(&ma, SA, M, Kp, parts.D, TC_M) && slice_map(&mb, SB, N, Kp, parts.D, TCN / CS),
+           FRACLAP_ERR_CUDA, "ozaki_gemm: tensor map encoding failed");
   const size_t smem = (size_t)OzTile<TCN>::STAGES * OzTile<TCN>::STAGE_BYTES + 1024;
   auto kern = ozaki_tc_kernel<TCN, CS>;
   FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -684,16 +734,10 @@ int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB
   const int TM = (int)cdiv(cdiv(M, TC_M), CS), TN = (int)cdiv(N, TCN);
   const int G = std::max(1, std::min(ctx->oz_group > 0 ? ctx->oz_group : TM, TM));
   const int64_t tiles = ozaki_tile_count(TM, TN, G, lower, CS * TC_M, TCN);
-  FL_CHECK(ctx, tiles * CS <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: too many tiles");
-  int lw = lower ? 1 : 0;
-  if (CS == 1) {
-    kern<<<(unsigned)tiles, TC_THREADS, smem, st>>>(ma, mb, ea, eb, M, N, Kp, sl, bits, chunk, alpha, beta, C, ldc,
-                                                    lw, G, ctx->wait_cycles, ctx->d_status);
-    return 0;
-  }
+  FL_CHECK(ctx, tiles * parts.count() * CS <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: too many tiles");
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * CS));
-  cfg.blockDim = dim3(TC_THREADS);
+  cfg.gridDim = dim3((unsigned)(tiles * parts.count() * CS));
+  cfg.blockDim = dim3(OzTile<TCN>::THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -702,23 +746,35 @@ int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, ma, mb, ea, eb, M, N, Kp, sl, bits, chunk, alpha, beta, C, ldc, lw, G,
+  cfg.numAttrs = (CS > 1) ? 1 : 0;
+  FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, ma, mb, M, N, Kp, parts, chunk, (int)tiles, P, lower ? 1 : 0, G,
                                   ctx->wait_cycles, ctx->d_status));
   return 0;
 }
 
 }  // namespace
 
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s) {
+// The most digits that s slices are cut into (see ozaki_gemm), and the int32
+// entries of the tensor-core route's planes for up to that many, at either digit
+// width.
+static int max_digits(int s) { return (s <= 5 || s == 8) ? s + 1 : s; }
+static int64_t plane_entries(int64_t M, int64_t N, int64_t Kp, int D, bool lower) {
+  int64_t t = 0;
+  for (int d = 1; d <= D; ++d)
+    for (int w = 7; w <= 8; ++w) t = std::max<int64_t>(t, oz_parts(M, N, Kp, d, w, lower).count());
+  return t * plane_size(M, N, lower);
+}
+
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower) {
   const int64_t Kp = cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD;
-  s = (8 * s + 6) / 7;  // room for the largest digit count (s + 1 up to s = 5, s + 1 at 8)
+  const int D = max_digits(s);
   Arena ar;
-  ar.take<__nv_bfloat16>((int64_t)s * M * Kp);
-  ar.take<__nv_bfloat16>((int64_t)s * N * Kp);
+  ar.take<__nv_bfloat16>((int64_t)D * M * Kp);
+  ar.take<__nv_bfloat16>((int64_t)D * N * Kp);
   ar.take<int>(M);
   ar.take<int>(N);
   ar.take<unsigned long long>(std::max(M, N));
+  ar.take<int32_t>(plane_entries(M, N, Kp, D, lower));
   return ar.off;
 }
 
@@ -763,13 +819,15 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   FL_CHECK(ctx, s >= 1 && s <= 8, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: slices must be 1..8");
   FL_CHECK(ctx, cdiv(N, OZ_BN) <= 65535, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: N too large");
   const int64_t Kp = cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD;
-  const int smax = (8 * s + 6) / 7;
+  FL_CHECK(ctx, !lower || M >= N, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: a lower product needs M >= N");
+  const int smax = max_digits(s);
   __nv_bfloat16* SA = ar->take<__nv_bfloat16>((int64_t)smax * M * Kp);
   __nv_bfloat16* SB = ar->take<__nv_bfloat16>((int64_t)smax * N * Kp);
   int* ea = ar->take<int>(M);
   int* eb = ar->take<int>(N);
   unsigned long long* mx = ar->take<unsigned long long>(std::max(M, N));
-  FL_CHECK(ctx, mx != nullptr, FRACLAP_ERR_ALLOC, "ozaki_gemm: workspace too small");
+  int32_t* P = ar->take<int32_t>(plane_entries(M, N, Kp, smax, lower));
+  FL_CHECK(ctx, mx != nullptr && P != nullptr, FRACLAP_ERR_ALLOC, "ozaki_gemm: workspace too small");
   // op(A) rows: trans -> A stored K x M; op(B) columns = rows of op(B)^T
   // Digit magnitude w and count D for s slices of 8 bits: with w = 8 (short K,
   // one chunk; or the knob) s digits of 9 bits (7 for s = 8: 63 bits, within
@@ -778,8 +836,9 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   // ceil(8 s / 7) sign-magnitude digits of 7 bits (s = 6 and 7 reach that with
   // s).  Measured at 8810 x 8810 x 8810 on 128 x 192 tiles, those against
   // these: s = 7 52.3 ms and 3.3e-15 from FP64, now 39.6 ms and 3.2e-15; s = 6
-  // 41.0 ms and 1.0e-13, now 30.2 ms and 9.3e-14.  w = 8 at s = 7 takes 66 ms:
-  // its four times more chunk sums, each drained and converted by the epilogue.
+  // 41.0 ms and 1.0e-13, now 30.2 ms and 9.3e-14.  (On 128 x 256 tiles without
+  // the folds 28.8 and 21.4 ms; w = 8 at s = 7 32.0 ms: the same pairs and four
+  // times more chunk sums to drain and convert.)
   int bits = 8, sl = std::min(s, 7);
   if (K > 256 && ctx->oz_bits != 8) {
     bits = 7;
@@ -795,14 +854,17 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   if (ctx->tensor_route == 1) {
     const int tw = (N <= 128) ? 128 : ctx->oz_tile_n;  // a narrow output takes the 128-column tile
     const int cs = ctx->oz_cluster;
-#define FL_OZ_LAUNCH(W, K) \
-  launch_tc<W, K>(ctx, SA, SB, ea, eb, M, N, Kp, sl, bits, chunk, alpha, beta, C, ldc, lower, st)
+    const OzParts parts = oz_parts(M, N, Kp, sl, bits, lower);
+#define FL_OZ_LAUNCH(W, K) launch_tc<W, K>(ctx, SA, SB, M, N, Kp, parts, chunk, P, lower, st)
     if (cs == 2) {
       FL_TRY(tw == 256 ? FL_OZ_LAUNCH(256, 2) : tw == 192 ? FL_OZ_LAUNCH(192, 2) : FL_OZ_LAUNCH(128, 2));
     } else {
       FL_TRY(tw == 256 ? FL_OZ_LAUNCH(256, 1) : tw == 192 ? FL_OZ_LAUNCH(192, 1) : FL_OZ_LAUNCH(128, 1));
     }
 #undef FL_OZ_LAUNCH
+    count_launch(ctx);
+    combine_planes<<<dim3((unsigned)cdiv(M, 256), (unsigned)std::min<int64_t>(N, 16384)), 256, 0, st>>>(
+        P, ea, eb, M, N, parts, bits, alpha, beta, C, ldc, lower ? 1 : 0);
   } else {
     dim3 grid((unsigned)cdiv(M, OZ_BM), (unsigned)cdiv(N, OZ_BN));
     ozaki_kernel<<<grid, OZ_NT, 0, st>>>(SA, SB, ea, eb, M, N, Kp, sl, bits, chunk, alpha, beta, C, ldc, lower);

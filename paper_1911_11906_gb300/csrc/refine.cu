@@ -892,7 +892,7 @@ size_t refine_ws(const fraclap_ctx* ctx, int64_t n) {
   const int64_t cmax = std::min<int64_t>(n, kMaxBigCluster);
   ar.take<double>(4 * cmax * cmax + cmax);
   ar.take<double>(small_cluster_doubles(n));
-  return ar.off + std::max(cluster_eig_ws(ctx, cmax), ozaki_ws(n, n, n, kRefineSlices));
+  return ar.off + std::max(cluster_eig_ws(ctx, cmax), ozaki_ws(n, n, n, kRefineSlices, true));
 }
 
 int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t* col,
