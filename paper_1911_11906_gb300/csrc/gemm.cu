@@ -139,6 +139,7 @@ __device__ __forceinline__ void gemm_tile(const GemmDescT<T>& d, int64_t m0, int
 
 template <class T, bool TA, bool TB, int MODE, bool ATOMIC>
 __global__ void __launch_bounds__(NT) gemm_kernel(GemmDescT<T> d, int64_t kchunk) {
+  if (d.only_if && *d.only_if == 0) return;
   const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
   const int64_t kbeg = (int64_t)blockIdx.z * kchunk;
   const int64_t kend = (kbeg + kchunk < d.K) ? kbeg + kchunk : d.K;
@@ -341,6 +342,7 @@ __device__ __forceinline__ void dg_finish(const GemmDescT<double>& d, double v, 
 template <bool TB, int MODE>
 __global__ void __launch_bounds__(DG_NT) dgemm_rows_kernel(GemmDescT<double> d, int64_t kper, int ncol) {
   __shared__ double red[DG_NC][DG_NC][DG_ROWS];
+  if (d.only_if && *d.only_if == 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t m0 = (int64_t)(blockIdx.x / cg::this_cluster().num_blocks()) * DG_ROWS, n0 = (int64_t)blockIdx.y * ncol;
   const int nc = (int)((d.N - n0 < ncol) ? d.N - n0 : ncol);
@@ -392,6 +394,7 @@ __global__ void __launch_bounds__(DG_NT) dgemm_rows_kernel(GemmDescT<double> d, 
 // K, each warp holds four rows x eight columns, and a butterfly that halves
 // the 32 sums at every step leaves one output per lane.
 __global__ void __launch_bounds__(DG_NT) dgemm_dots_kernel(GemmDescT<double> d, int64_t kper, int ncol) {
+  if (d.only_if && *d.only_if == 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t m0 = (int64_t)(blockIdx.x / cg::this_cluster().num_blocks()) * DG_ROWS + 4 * warp;
   const int64_t n0 = (int64_t)blockIdx.y * ncol;

@@ -213,6 +213,7 @@ struct GemmDescT {
   const T* B2; int64_t ldb2;
   int64_t K2;
   double alpha, beta;
+  const int* only_if = nullptr;  // FP64: a device flag; 0 leaves C as it is
 };
 using GemmDesc = GemmDescT<double>;
 
@@ -311,10 +312,11 @@ int cluster_eig(fraclap_ctx* ctx, double* S, int64_t c, double* w, double* Q, Ar
                 cudaStream_t st);
 
 // FP64-accurate GEMM through BF16 tensor-core slices (ozaki.cu).
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false);
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false, int digits = 0);
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
-               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits = 0);
+               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits = 0,
+               int* nonfinite = nullptr);
 
 // Banded LDL^T (no pivoting) of the symmetric CSR matrix of half-bandwidth
 // b: Lb(t, j) = L(j + t, j), Lr(t, i) = L(i, i - t) (both ld b + 1, n

@@ -51,11 +51,12 @@ __device__ __forceinline__ int exponent_above(unsigned long long t) {
   return e;
 }
 
-// Exponent of the largest |entry| of each row of op(A) (rows = M, length K).
+// Exponent of the largest |entry| of each row of op(A) (rows = M, length K);
+// an infinity or NaN, which has no digits, sets *nonfinite.
 // One block per row.  The magnitudes are compared as the integers of their
 // IEEE bit patterns with the sign cleared (the same order as the values), so
 // the FP64 pipe is not used.
-__global__ void row_exponents(const double* A, int64_t lda, bool trans, int64_t K, int* ex) {
+__global__ void row_exponents(const double* A, int64_t lda, bool trans, int64_t K, int* ex, int* nonfinite) {
   const int64_t i = blockIdx.x;
   unsigned long long m = 0;
   for (int64_t k = threadIdx.x; k < K; k += blockDim.x) {
@@ -74,6 +75,7 @@ __global__ void row_exponents(const double* A, int64_t lda, bool trans, int64_t 
     unsigned long long t = 0;
     for (unsigned w = 0; w < blockDim.x / 32; ++w) t = red[w] > t ? red[w] : t;
     ex[i] = exponent_above(t);
+    if (nonfinite && (t >> 52) == 2047) *nonfinite = 1;
   }
 }
 
@@ -95,9 +97,11 @@ __global__ void row_absmax_strided(const double* A, int64_t lda, int64_t M, int6
   }
   if (m != 0) atomicMax(&mx[i], m);
 }
-__global__ void exponents_of_max(const unsigned long long* mx, int64_t M, int* ex) {
+__global__ void exponents_of_max(const unsigned long long* mx, int64_t M, int* ex, int* nonfinite) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < M) ex[i] = exponent_above(mx[i]);
+  if (i >= M) return;
+  ex[i] = exponent_above(mx[i]);
+  if (nonfinite && (mx[i] >> 52) == 2047) *nonfinite = 1;
 }
 
 // Fraction bits of D digits of radix 2^r: r D - 1 (the leading digit reaches
@@ -169,6 +173,19 @@ __global__ void make_slices(const double* A, int64_t lda, bool trans, int64_t M,
   }
 }
 
+// One digit (shift rs, field mask) of eight entries as a 16-byte store.
+__device__ __forceinline__ void put_eight(const unsigned long long (&v)[8], int rs, uint32_t mask, float off,
+                                          __nv_bfloat16* out) {
+  uint32_t o[4];
+#pragma unroll
+  for (int h = 0; h < 4; ++h) {
+    const __nv_bfloat162 two = __floats2bfloat162_rn(field_value((uint32_t)(v[2 * h] >> rs) & mask, off),
+                                                     field_value((uint32_t)(v[2 * h + 1] >> rs) & mask, off));
+    o[h] = *reinterpret_cast<const uint32_t*>(&two);
+  }
+  *reinterpret_cast<uint4*>(out) = make_uint4(o[0], o[1], o[2], o[3]);
+}
+
 // The slices of an operand whose rows are contiguous (trans), for r D <= 64:
 // a thread takes eight consecutive entries of a row and writes each digit's
 // eight BF16 values as one 16-byte store (Kp is a multiple of 64, so every
@@ -186,37 +203,39 @@ __global__ void make_slices_rows(const double* A, int64_t lda, int64_t M, int64_
     unsigned long long v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = biased_digits((k0 + q < K) ? A[k0 + q + i * lda] : 0.0, e, tb, bias);
-    for (int p = 0; p < D; ++p) {
-      const int rs = rb * (D - 1 - p);
-      const uint32_t mask = (p > 0) ? (1u << rb) - 1u : 0xFFFFFFFFu;
-      uint32_t o[4];
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const __nv_bfloat162 two = __floats2bfloat162_rn(field_value((uint32_t)(v[2 * h] >> rs) & mask, off),
-                                                         field_value((uint32_t)(v[2 * h + 1] >> rs) & mask, off));
-        o[h] = *reinterpret_cast<const uint32_t*>(&two);
-      }
-      *reinterpret_cast<uint4*>(S + ((int64_t)p * M + i) * Kp + k0) = make_uint4(o[0], o[1], o[2], o[3]);
-    }
+    for (int p = 0; p < D; ++p) put_eight(v, rb * (D - 1 - p), p > 0 ? (1u << rb) - 1u : 0xFFFFFFFFu, off,
+                                          S + ((int64_t)p * M + i) * Kp + k0);
   }
 }
 
-// The same slices of an untransposed column-major operand (rows strided):
-// 32 x 32 tiles of (i, k) staged in shared memory, read along i and written
-// along k, so that both the FP64 reads and the BF16 writes are contiguous
-// within a warp.  Block 32 x 8 threads; grid (ceil(M / 32), Kp / 32).
-__global__ void make_slices_strided(const double* A, int64_t lda, int64_t M, int64_t K, int64_t Kp,
-                                    const int* ex, int D, int w, __nv_bfloat16* S) {
-  __shared__ double tile[32][33];
-  const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int64_t i = i0 + threadIdx.x, k = k0 + r;
-    tile[r][threadIdx.x] = (i < M && k < K) ? A[i + k * lda] : 0.0;
+// The same slices of an untransposed column-major operand (rows strided), for
+// r D <= 64: 64 x 64 tiles of (i, k) staged in shared memory, read along i and
+// written along k, a digit's eight consecutive values of a row as one 16-byte
+// store, so that eight lanes fill a 128-byte line (a 2-byte store per lane and
+// digit before: exponents and slices of an 8835 x 8835 operand at 7 digits 0.77
+// -> 0.58 ms).  256 threads; grid (ceil(M / 64), Kp / 64).
+__global__ void __launch_bounds__(256) make_slices_strided(const double* A, int64_t lda, int64_t M, int64_t K,
+                                                           int64_t Kp, const int* ex, int D, int w, __nv_bfloat16* S) {
+  __shared__ double tile[64][65];
+  const int64_t i0 = (int64_t)blockIdx.x * 64, k0 = (int64_t)blockIdx.y * 64;
+  for (int t = threadIdx.x; t < 64 * 64; t += 256) {
+    const int64_t i = i0 + t % 64, k = k0 + t / 64;
+    tile[t / 64][t % 64] = (i < M && k < K) ? A[i + k * lda] : 0.0;
   }
   __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int64_t i = i0 + r, k = k0 + threadIdx.x;
-    if (i < M) write_digits(tile[threadIdx.x][r], ex[i], D, w, S + i * Kp + k, M * Kp);
+  const int rb = w + 1, tb = digit_frac_bits(w, D);
+  const unsigned long long bias = digit_bias(w, D);
+  const float off = 8388608.0f + (float)(1 << w);
+  const int kk = (threadIdx.x & 7) * 8;
+  for (int r = threadIdx.x >> 3; r < 64; r += 32) {
+    const int64_t i = i0 + r;
+    if (i >= M) break;
+    const int e = ex[i];
+    unsigned long long v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = biased_digits(tile[kk + q][r], e, tb, bias);
+    for (int p = 0; p < D; ++p) put_eight(v, rb * (D - 1 - p), p > 0 ? (1u << rb) - 1u : 0xFFFFFFFFu, off,
+                                          S + ((int64_t)p * M + i) * Kp + k0 + kk);
   }
 }
 
@@ -765,9 +784,9 @@ static int64_t plane_entries(int64_t M, int64_t N, int64_t Kp, int D, bool lower
   return t * plane_size(M, N, lower);
 }
 
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower) {
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits) {
   const int64_t Kp = cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD;
-  const int D = max_digits(s);
+  const int D = (digits > 0) ? digits : max_digits(s);
   Arena ar;
   ar.take<__nv_bfloat16>((int64_t)D * M * Kp);
   ar.take<__nv_bfloat16>((int64_t)D * N * Kp);
@@ -780,47 +799,51 @@ size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower) {
 
 // Exponents and digit slices of the rows of op(X) (R rows of length K):
 // contiguous rows (trans) one block per row; strided rows through the
-// column-parallel maximum and the tiled slicing.
+// column-parallel maximum and the tiled slicing.  More than 64 bits of digits
+// take the general kernel.
 int slice_operand(fraclap_ctx* ctx, const double* X, int64_t ldx, bool trans, int64_t R, int64_t K, int64_t Kp,
-                  int sl, int bits, int* ex, __nv_bfloat16* S, unsigned long long* mx, cudaStream_t st) {
-  if (trans || Kp / 32 > 65535 || cdiv(K, OZ_MAX_KCH) > 65535) {
-    row_exponents<<<(unsigned)R, 256, 0, st>>>(X, ldx, trans, K, ex);
-    count_launch(ctx);
-    if (trans && sl * (bits + 1) <= 64) {
-      const unsigned gs = (unsigned)std::min<int64_t>(cdiv(R * (Kp / 8), 256), 152 * 16);
-      make_slices_rows<<<gs, 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl, bits, S);
-    } else {
-      const unsigned gs = (unsigned)std::min<int64_t>(cdiv(R * Kp, 256), 152 * 32);
-      make_slices<<<gs, 256, 0, st>>>(X, ldx, trans, R, K, Kp, ex, sl, bits, S);
-    }
-    count_launch(ctx);
+                  int sl, int bits, int* ex, __nv_bfloat16* S, unsigned long long* mx, int* nonfinite, cudaStream_t st) {
+  const bool fits = sl * (bits + 1) <= 64;
+  const bool tiled = fits && Kp / 64 <= 65535;
+  if (trans || cdiv(K, OZ_MAX_KCH) > 65535) {
+    row_exponents<<<(unsigned)R, 256, 0, st>>>(X, ldx, trans, K, ex, nonfinite);
   } else {
     FL_CUDA(ctx, cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * (size_t)R, st));
     row_absmax_strided<<<dim3((unsigned)cdiv(R, 256), (unsigned)std::max<int64_t>(cdiv(K, OZ_MAX_KCH), 1)), 256, 0,
                          st>>>(X, ldx, R, K, mx);
     count_launch(ctx);
-    exponents_of_max<<<(unsigned)cdiv(R, 256), 256, 0, st>>>(mx, R, ex);
-    count_launch(ctx);
-    make_slices_strided<<<dim3((unsigned)cdiv(R, 32), (unsigned)(Kp / 32)), dim3(32, 8), 0, st>>>(
-        X, ldx, R, K, Kp, ex, sl, bits, S);
-    count_launch(ctx);
+    exponents_of_max<<<(unsigned)cdiv(R, 256), 256, 0, st>>>(mx, R, ex, nonfinite);
   }
+  count_launch(ctx);
+  if (trans && fits) {
+    const unsigned gs = (unsigned)std::min<int64_t>(cdiv(R * (Kp / 8), 256), 152 * 16);
+    make_slices_rows<<<gs, 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl, bits, S);
+  } else if (tiled) {
+    make_slices_strided<<<dim3((unsigned)cdiv(R, 64), (unsigned)(Kp / 64)), 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl,
+                                                                                         bits, S);
+  } else {
+    const unsigned gs = (unsigned)std::min<int64_t>(cdiv(R * Kp, 256), 152 * 32);
+    make_slices<<<gs, 256, 0, st>>>(X, ldx, trans, R, K, Kp, ex, sl, bits, S);
+  }
+  count_launch(ctx);
   FL_CUDA(ctx, cudaGetLastError());
   return 0;
 }
 
 // C = alpha op(A) op(B) + beta C, FP64-accurate through s BF16 slices
 // (s = 7 for full FP64 accuracy of the products).  lower: only C(i,j), i >= j.
-// digits > 0 sets the digits per operand itself (8 bits each at w = 7).
+// digits > 0 sets the digits per operand itself (8 bits each at w = 7);
+// nonfinite (device, may be null) is set to 1 when an operand holds an infinity
+// or NaN, which the digits do not represent: C is then meaningless.
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
-               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits) {
+               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits, int* nonfinite) {
   if (M <= 0 || N <= 0) return 0;
   FL_CHECK(ctx, s >= 1 && s <= 8, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: slices must be 1..8");
   FL_CHECK(ctx, cdiv(N, OZ_BN) <= 65535, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: N too large");
   const int64_t Kp = cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD;
   FL_CHECK(ctx, !lower || M >= N, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: a lower product needs M >= N");
-  const int smax = max_digits(s);
+  const int smax = (digits > 0) ? digits : max_digits(s);
   __nv_bfloat16* SA = ar->take<__nv_bfloat16>((int64_t)smax * M * Kp);
   __nv_bfloat16* SB = ar->take<__nv_bfloat16>((int64_t)smax * N * Kp);
   int* ea = ar->take<int>(M);
@@ -848,8 +871,8 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   FL_CHECK(ctx, sl <= smax, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: too many digits");
   const int64_t chunk = (int64_t)1 << (24 - 2 * bits);
   // rows of op(A) and columns of op(B): contiguous when trans, else strided
-  FL_TRY(slice_operand(ctx, A, lda, ta, M, K, Kp, sl, bits, ea, SA, mx, st));
-  FL_TRY(slice_operand(ctx, B, ldb, !tb, N, K, Kp, sl, bits, eb, SB, mx, st));
+  FL_TRY(slice_operand(ctx, A, lda, ta, M, K, Kp, sl, bits, ea, SA, mx, nonfinite, st));
+  FL_TRY(slice_operand(ctx, B, ldb, !tb, N, K, Kp, sl, bits, eb, SB, mx, nonfinite, st));
   StageTimer tm(ctx, kStageSliceProducts, st);
   if (ctx->tensor_route == 1) {
     const int tw = (N <= 128) ? 128 : ctx->oz_tile_n;  // a narrow output takes the 128-column tile
