@@ -154,7 +154,10 @@ int eig_full_mixed(fraclap_ctx* ctx, const double* A_dev, int64_t n, int64_t lda
 size_t fraclap_apply_workspace_bytes(int64_t n, int64_t m, int64_t k);
 /* The same for this context's setting of fraclap_set_apply_slices. */
 size_t fraclap_apply_workspace_bytes_ctx(const fraclap_ctx* ctx, int64_t n, int64_t m, int64_t k);
-/* Products of frac_apply: 0 (default) on the FP64 GEMM engine; s = 1..8 as
+/* Products of frac_apply: 0 (default) at FP64 accuracy, on the FP64 GEMM engine
+ * or, where that is faster and the workspace has room for it (the _ctx size),
+ * from 8 digits of 8 bits per operand (2^-63 relative to |row max| |column max|
+ * per term, exact sums; infinities and NaN take the FP64 engine); s = 1..8 as
  * products of s BF16 slices on the tensor cores (error about 2^-8s relative
  * to |row max| |column max| per term; s = 7 is FP64-level, s = 5 about 1e-12). */
 int fraclap_set_apply_slices(fraclap_ctx* ctx, int slices);

@@ -127,6 +127,7 @@ class Context:
     def __init__(self, band_width: int = 0, leaf_size: int = 0, wait_timeout_s: float = 0.0):
         self.lib = load_library()
         self.handle = ctypes.c_void_p()
+        self.apply_slices = 0
         opts = _Opts(band_width, leaf_size, wait_timeout_s)
         rc = self.lib.fraclap_create(ctypes.byref(self.handle), ctypes.byref(opts))
         if rc != 0:
@@ -178,8 +179,9 @@ class Context:
         self.check(self.lib.fraclap_set_refine_tau(self.handle, float(tau)))
 
     def set_apply_slices(self, slices: int):
-        """frac_apply products: 0 = FP64 engine; s = 1..8 BF16 slices on the tensor cores."""
+        """frac_apply products: 0 = FP64 accuracy (FP64 engine or 8 digits); s = 1..8 BF16 slices on the tensor cores."""
         self.check(self.lib.fraclap_set_apply_slices(self.handle, int(slices)))
+        self.apply_slices = int(slices)
 
     SCHEDULE_KNOBS = {"ozaki_group": 0, "ozaki_bits": 1, "fp32_stages_tc": 2, "ozaki_tile_n": 3, "q2_parts": 4,
                       "ozaki_cluster": 5}
@@ -309,6 +311,21 @@ def empty_colmajor(rows: int, cols: int, device=None) -> torch.Tensor:
     return torch.empty((cols, rows), dtype=torch.float64, device=device or "cuda").t()
 
 
+def _apply_workspace(ctx: Context, n: int, m: int, k: int, device, mass: bool = False) -> torch.Tensor:
+    """Scratch of an apply: the context's size, or, when that does not fit the
+    device, the smaller one of the FP64 engine (which the library then takes)."""
+    lib = ctx.lib
+    nbytes = (lib.fraclap_apply_mass_workspace_bytes if mass else lib.fraclap_apply_workspace_bytes_ctx)(
+        ctx.handle, n, m, k)
+    try:
+        return torch.empty(max(nbytes, 1), dtype=torch.uint8, device=device)
+    except torch.OutOfMemoryError:
+        spare = lib.fraclap_apply_workspace_bytes_ctx(ctx.handle, n, m, k) - lib.fraclap_apply_workspace_bytes(n, m, k)
+        if ctx.apply_slices or spare <= 0:
+            raise
+        return torch.empty(max(nbytes - spare, 1), dtype=torch.uint8, device=device)
+
+
 def fd_assemble(mask: torch.Tensor, h: float, dense: bool = True, ctx: Context | None = None,
                 stream=None):
     """Assembles the FD Laplacian of a uint8 mask ([y, x] or [z, y, x]) on the GPU.
@@ -402,8 +419,7 @@ def frac_apply(V: torch.Tensor, lam: torch.Tensor, F: torch.Tensor, pair_f, pair
     lam = _dev(lam, torch.float64, "lam", dev, n)
     U = _out(out, torch.float64, "out", dev, n, k) if out is not None else empty_colmajor(n, k, dev)
     if workspace is None:
-        nbytes = ctx.lib.fraclap_apply_workspace_bytes_ctx(ctx.handle, n, m, k)
-        workspace = torch.empty(max(nbytes, 1), dtype=torch.uint8, device=dev)
+        workspace = _apply_workspace(ctx, n, m, k, dev)
     else:
         workspace = _ws(workspace, dev)
     st = ctypes.c_void_p(_stream(stream))
@@ -433,8 +449,7 @@ def frac_diffusion(V: torch.Tensor, lam: torch.Tensor, U0: torch.Tensor, pair_f,
     lam = _dev(lam, torch.float64, "lam", dev, n)
     U = _out(out, torch.float64, "out", dev, n, k) if out is not None else empty_colmajor(n, k, dev)
     if workspace is None:
-        nbytes = ctx.lib.fraclap_apply_workspace_bytes_ctx(ctx.handle, n, m, k)
-        workspace = torch.empty(max(nbytes, 1), dtype=torch.uint8, device=dev)
+        workspace = _apply_workspace(ctx, n, m, k, dev)
     else:
         workspace = _ws(workspace, dev)
     st = ctypes.c_void_p(_stream(stream))
@@ -467,8 +482,7 @@ class ApplyGraph:
         if self.pair_alpha.numel() != k or (self.pair_t is not None and self.pair_t.numel() != k):
             raise ValueError("pair arrays differ in length")
         self.U = _out(out, torch.float64, "out", dev, n, k) if out is not None else empty_colmajor(n, k, dev)
-        nbytes = self.ctx.lib.fraclap_apply_workspace_bytes_ctx(self.ctx.handle, n, m, k)
-        self.workspace = torch.empty(max(nbytes, 1), dtype=torch.uint8, device=dev)
+        self.workspace = _apply_workspace(self.ctx, n, m, k, dev)
         self.handle = ctypes.c_void_p()
         torch.cuda.synchronize(dev)  # the buffers above are ready before the capture reads their addresses
         self.ctx.check(self.ctx.lib.fraclap_apply_graph_create(
@@ -750,8 +764,7 @@ def frac_apply_mass(Phi: torch.Tensor, theta: torch.Tensor, rowptr, col, valM, F
     if pa.numel() != k:
         raise ValueError("pair_f and pair_alpha differ in length")
     U = _out(out, torch.float64, "out", dev, n, k) if out is not None else empty_colmajor(n, k, dev)
-    nbytes = ctx.lib.fraclap_apply_mass_workspace_bytes(ctx.handle, n, m, k)
-    ws = torch.empty(max(nbytes, 1), dtype=torch.uint8, device=dev)
+    ws = _apply_workspace(ctx, n, m, k, dev, mass=True)
     ctx.check(ctx.lib.frac_apply_mass(ctx.handle, _ptr(Phi), _ld(Phi), _ptr(theta), n, _ptr(rowptr), _ptr(col),
                                       _ptr(valM), _ptr(F), _ld(F), m, _ptr(pf), _ptr(pa), k, _ptr(U), _ld(U), _ptr(ws),
                                       ws.numel(), ctypes.c_void_p(_stream(stream))))

@@ -9,7 +9,8 @@
 // powers are exp(e log lambda) with CUDA's double-precision log() and exp().  The GEMMs run on
 // the FP64 engine, or (context setting apply_slices = s > 0) as products of
 // s BF16 slices on the tensor cores, accurate to about 2^-8s relative to
-// |row max| |column max| per term (s = 7: FP64 level).  A zero or negative
+// |row max| |column max| per term (s = 7: FP64 level).  With s = 0 large
+// products are formed from 8 digits (63 bits) too, see digits_pay.  A zero or negative
 // eigenvalue met with alpha != 0 raises FRACLAP_ERR_NOT_SPD in the device
 // status.
 #include <cmath>
@@ -54,6 +55,30 @@ __global__ void spectral_scale(const double* lambda, int64_t n, const double* W,
   }
 }
 
+// FP64 products (apply_slices = 0) of large operands: the FP64 pipe takes
+// 2 n^2 (m + k) / 1.2 TFLOP/s whatever the memory does, while cutting V twice
+// into kFp64Digits digits of 8 bits and multiplying those takes little more
+// than the bytes.  8 digits hold every entry to 2^-63 of its row's or column's
+// largest, and the sums are exact, so the result is at least as accurate as the
+// FP64 sums: GB300, n = 8835, 16 forcings, 128 pairs 19.7 -> 2.9 ms and 3.1e-15
+// -> 2.7e-15 from exact.  The line (a factor of 1.5 in the estimate) keeps small
+// applies, which the launches bound, on the FP64 pipe: n = 2304, 25 columns 0.36 ms.
+// An infinity or NaN has no digits: the slicing raises a flag, and the FP64
+// product behind each sliced one runs only then.
+constexpr int kFp64Digits = 8;
+bool digits_pay(const fraclap_ctx* ctx, int64_t n, int64_t m, int64_t k) {
+  if (ctx->apply_slices != 0 || ctx->tensor_route != 1) return false;
+  const double nn = (double)n * (double)n;
+  // microseconds: FP64 pipe; slices, pairs of 128-column tiles, launches
+  const double fp64 = 2.0 * nn * (double)(m + k) / 1.2e6;
+  const double cols = 128.0 * (double)(cdiv(m, 128) + cdiv(k, 128));
+  const double digits = 1.5e-5 * nn + 72.0 * nn * cols / 0.9e9 + 150.0;
+  return fp64 > 1.5 * digits;
+}
+size_t digits_ws(int64_t n, int64_t m, int64_t k) {
+  return std::max(ozaki_ws(n, m, n, 7, false, kFp64Digits), ozaki_ws(n, k, n, 7, false, kFp64Digits)) + 1024;
+}
+
 // The body shared by frac_apply and frac_diffusion.
 int spectral_apply(fraclap_ctx* ctx, const char* name, const double* V_dev, int64_t ldv,
                    const double* lambda_dev, int64_t n, const double* F_dev, int64_t ldf, int64_t m,
@@ -69,17 +94,32 @@ int spectral_apply(fraclap_ctx* ctx, const char* name, const double* V_dev, int6
   FL_CHECK(ctx, k <= 65535 && m <= 65535 * 64, FRACLAP_ERR_UNSUPPORTED, "%s: at most 65535 pairs per call", name);
   StageTimer timer(ctx, kStageApply, st);
   Arena ar;
-  FL_TRY(get_workspace(ctx, work_dev, work_bytes, fraclap_apply_workspace_bytes_ctx(ctx, n, m, k), &ar));
+  const size_t full = fraclap_apply_workspace_bytes_ctx(ctx, n, m, k), base = fraclap_apply_workspace_bytes(n, m, k);
+  // a workspace without room for the digits is served by the FP64 engine
+  bool by_digits = digits_pay(ctx, n, m, k) && (!work_dev || work_bytes >= align256(full));
+  int rc = get_workspace(ctx, work_dev, work_bytes, (ctx->apply_slices > 0 || by_digits) ? full : base, &ar);
+  if (rc == FRACLAP_ERR_ALLOC && by_digits) {
+    by_digits = false;
+    rc = get_workspace(ctx, work_dev, work_bytes, base, &ar);
+  }
+  if (rc != 0) return rc;
   double* W = ar.take<double>(n * m);
   double* C = ar.take<double>(n * k);
   FL_CHECK(ctx, W && C, FRACLAP_ERR_ALLOC, "%s: workspace too small", name);
-  const int ozs = ctx->apply_slices;
+  int* nonfinite = nullptr;
+  if (by_digits) {
+    nonfinite = ar.take<int>(1);
+    FL_CUDA(ctx, cudaMemsetAsync(nonfinite, 0, sizeof(int), st));
+  }
+  const int ozs = by_digits ? 7 : ctx->apply_slices, dig = by_digits ? kFp64Digits : 0;
   // W = V^T F
   if (ozs > 0) {
     Arena oz = ar;
-    FL_TRY(ozaki_gemm(ctx, true, false, n, m, n, 1.0, V_dev, ldv, F_dev, ldf, 0.0, W, n, ozs, false, &oz, st));
-  } else {
-    GemmDesc d{n, m, n, V_dev, ldv, F_dev, ldf, W, n, nullptr, 0, nullptr, 0, 0, 1.0, 0.0};
+    FL_TRY(ozaki_gemm(ctx, true, false, n, m, n, 1.0, V_dev, ldv, F_dev, ldf, 0.0, W, n, ozs, false, &oz, st, dig,
+                      nonfinite));
+  }
+  if (ozs == 0 || by_digits) {
+    GemmDesc d{n, m, n, V_dev, ldv, F_dev, ldf, W, n, nullptr, 0, nullptr, 0, 0, 1.0, 0.0, nonfinite};
     FL_TRY(gemm(ctx, true, false, kGemmPlain, d, 1, st));
   }
   spectral_scale<<<dim3((unsigned)cdiv(n, 256), (unsigned)cdiv(k, kScalePairs)), 256, 0, st>>>(
@@ -89,9 +129,11 @@ int spectral_apply(fraclap_ctx* ctx, const char* name, const double* V_dev, int6
   // U = V C
   if (ozs > 0) {
     Arena oz = ar;
-    FL_TRY(ozaki_gemm(ctx, false, false, n, k, n, 1.0, V_dev, ldv, C, n, 0.0, U_dev, ldu, ozs, false, &oz, st));
-  } else {
-    GemmDesc d{n, k, n, V_dev, ldv, C, n, U_dev, ldu, nullptr, 0, nullptr, 0, 0, 1.0, 0.0};
+    FL_TRY(ozaki_gemm(ctx, false, false, n, k, n, 1.0, V_dev, ldv, C, n, 0.0, U_dev, ldu, ozs, false, &oz, st, dig,
+                      nonfinite));
+  }
+  if (ozs == 0 || by_digits) {
+    GemmDesc d{n, k, n, V_dev, ldv, C, n, U_dev, ldu, nullptr, 0, nullptr, 0, 0, 1.0, 0.0, nonfinite};
     FL_TRY(gemm(ctx, false, false, kGemmPlain, d, 1, st));
   }
   return 0;
@@ -110,7 +152,9 @@ extern "C" size_t fraclap_apply_workspace_bytes(int64_t n, int64_t m, int64_t k)
 
 extern "C" size_t fraclap_apply_workspace_bytes_ctx(const fraclap_ctx* ctx, int64_t n, int64_t m, int64_t k) {
   const size_t base = fraclap_apply_workspace_bytes(n, m, k);
-  if (!ctx || ctx->apply_slices <= 0 || base == 0) return base;
+  if (!ctx || base == 0) return base;
+  if (n > 0 && m > 0 && k > 0 && digits_pay(ctx, n, m, k)) return base + align256(sizeof(int)) + digits_ws(n, m, k);
+  if (ctx->apply_slices <= 0) return base;
   const int64_t nn = n > 0 ? n : 1;
   return base + std::max(ozaki_ws(nn, m > 0 ? m : 1, nn, ctx->apply_slices),
                          ozaki_ws(nn, k > 0 ? k : 1, nn, ctx->apply_slices)) + 1024;

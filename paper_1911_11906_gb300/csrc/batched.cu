@@ -109,7 +109,7 @@ extern "C" int fraclap_solve_batched(fraclap_ctx* ctx, const fraclap_problem* pr
       if (p.n == 0) continue;
       need = std::max(need, p.rowptr_dev ? fraclap_eig_mixed_workspace_bytes(ctx->workers[w], p.n)
                                          : fraclap_eig_workspace_bytes(ctx->workers[w], p.n));
-      if (p.k > 0) need = std::max(need, fraclap_apply_workspace_bytes(p.n, p.m, p.k));
+      if (p.k > 0) need = std::max(need, fraclap_apply_workspace_bytes_ctx(ctx->workers[w], p.n, p.m, p.k));
     }
     if (need == 0) continue;
     Arena ar;

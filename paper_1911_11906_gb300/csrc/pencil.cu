@@ -231,7 +231,11 @@ extern "C" int frac_apply_mass(fraclap_ctx* ctx, const double* Phi_dev, int64_t 
   FL_CHECK(ctx, rowptr_dev && col_dev && valM_dev && F_dev, FRACLAP_ERR_INVALID_ARG, "frac_apply_mass: null pointer");
   FL_CHECK(ctx, ldf >= n, FRACLAP_ERR_INVALID_ARG, "frac_apply_mass: ldf < n");
   Arena ar;
-  FL_TRY(get_workspace(ctx, work_dev, work_bytes, fraclap_apply_mass_workspace_bytes(ctx, n, m, k), &ar));
+  size_t need = fraclap_apply_mass_workspace_bytes(ctx, n, m, k);
+  // FP64 products: the sizes without the digits' scratch do too (see frac_apply)
+  if (work_dev && ctx->apply_slices == 0)
+    need = std::min(need, need - fraclap_apply_workspace_bytes_ctx(ctx, n, m, k) + fraclap_apply_workspace_bytes(n, m, k));
+  FL_TRY(get_workspace(ctx, work_dev, work_bytes, need, &ar));
   double* B = ar.take<double>(n * m);
   FL_CHECK(ctx, B != nullptr, FRACLAP_ERR_ALLOC, "frac_apply_mass: workspace too small");
   csr_spmm<<<dim3((unsigned)cdiv(n, 256), (unsigned)m), 256, 0, st>>>(n, rowptr_dev, col_dev, valM_dev, F_dev, ldf,
