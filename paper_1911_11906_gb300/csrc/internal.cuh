@@ -277,7 +277,8 @@ template <class T>
 struct Stage2T {
   T* refl;        // (n-1) * kmax * b
   double* rtau;   // (n-1) * kmax
-  int* progress;  // 2 (n + 1): completed steps per sweep, then published subdiagonal values
+  int* progress;  // n + 1: completed steps per sweep
+  T* beta;        // (n-1) * kmax: subdiagonal values as the steps publish them
   T* ut;          // block factors of the back-transformation (b = 32, 64)
   int64_t kmax;
 };

@@ -13,11 +13,10 @@
 // the two are disjoint once k' >= k+3; at k' = k+2 they share only the
 // entry (s+(k+2)b, s+(k+1)b), which step k+2 of sweep s-1 sets to the new
 // subdiagonal value beta of its reflector before anything else.  Sweep s may
-// therefore run step k as soon as sweep s-1 has finished its step k+1 and
-// published the beta of its step k+2 (written to the band right after it is
-// computed, with a second counter): sweeps run in a pipeline, one CTA per
-// sweep in flight, each CTA waiting (bounded in time) on the counters of its
-// predecessor.
+// therefore start step k as soon as sweep s-1 has finished its step k+1, and
+// takes that one entry from the word in which sweep s-1 publishes the beta of
+// its step k+2 as soon as it is computed: sweeps run in a pipeline, one CTA per
+// sweep in flight, each CTA waiting (bounded in time) for its predecessor.
 //
 // The reflectors H(s,k) of one sweep act on disjoint rows; H(s,k) and
 // H(s',k') with k > k', s > s' or k < k', s < s' act on disjoint rows as
@@ -44,7 +43,7 @@ struct SbArgs {
   T* refl;        // (n-1) * kmax * b
   double* rtau;   // (n-1) * kmax
   int* progress;  // n, completed steps per sweep
-  int* beta_progress;  // n, steps per sweep whose subdiagonal value is in the band
+  T* beta;        // (n-1) * kmax, subdiagonal values as they are computed (all bits set until then)
   int32_t* status;
   long long limit;
 };
@@ -95,10 +94,113 @@ struct SbShape {
   static constexpr int NW = NT / 32;
 };
 
+// Named barrier `id` over `count` threads (a multiple of 32).
+__device__ __forceinline__ void bar_sync(int id, int count) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int count) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// Householder scalars of (x0, tail = sum of the other squares > 0): beta = -+
+// sqrt(x0^2 + tail), tau = (beta - x0) / beta and 1 / (x0 - beta).
+__device__ __forceinline__ void sb_scalars(double x0, double tail, int lane, double* beta, double* tu, double* inv) {
+  const double alpha = sqrt(x0 * x0 + tail);
+  const double b = (x0 >= 0.0) ? -alpha : alpha;
+  // one division, on two lanes
+  const double q = ((lane & 1) ? 1.0 : b - x0) / ((lane & 1) ? x0 - b : b);
+  *beta = b;
+  *tu = __shfl_sync(0xffffffffu, q, 0);
+  *inv = __shfl_sync(0xffffffffu, q, 1);
+}
+// The same for FP32 entries, to within a few units of 2^-52 and in a third of
+// the dependent FP64 operations: with r = 1 / sqrt(sigma), |beta| = sigma r, tau
+// = 1 + |x0| r and 1 / |x0 - beta| = r / tau.  r and 1 / tau come from an FP32
+// start by one step of Halley's (third-order) iteration, which takes 2^-22 to
+// below 2^-60.  sigma is scaled to [1, 4) by its exponent: squares of FP32
+// entries are normal doubles; anything else (an infinity, a NaN) takes the
+// general form.
+__device__ __forceinline__ void sb_scalars_f32(double x0, double tail, int lane, double* beta, double* tu, double* inv) {
+  const double sigma = fma(x0, x0, tail);
+  const int hi = __double2hiint(sigma), E = (hi >> 20) - 1023;  // sigma > 0
+  if (E < -1000 || E > 1000) {
+    sb_scalars(x0, tail, lane, beta, tu, inv);
+    return;
+  }
+  const int k = E >> 1;
+  const double ss = __hiloint2double(hi - 2 * k * (1 << 20), __double2loint(sigma));
+  const double r0 = (double)rsqrtf((float)ss);
+  const double e = fma(-(ss * r0), r0, 1.0);
+  const double rs = fma(r0, e * fma(0.375, e, 0.5), r0);
+  const double r = __hiloint2double(__double2hiint(rs) - k * (1 << 20), __double2loint(rs));  // rs 2^-k
+  const double alpha = sigma * r, t = fma(fabs(x0), r, 1.0);
+  const double y0 = (double)(1.0f / (float)t);
+  const double f = fma(-t, y0, 1.0);
+  const double y = fma(y0, fma(f, f, f), y0);
+  *beta = (x0 >= 0.0) ? -alpha : alpha;
+  *tu = t;
+  *inv = (x0 >= 0.0) ? r * y : -(r * y);
+}
+
+// One published word: a NaN is made the canonical one, so that no value is the
+// "not yet" pattern of all bits set.
+__device__ __forceinline__ void sb_publish(float* p, float v) {
+  const unsigned b = (v != v) ? 0x7FC00000u : __float_as_uint(v);
+  asm volatile("st.relaxed.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(b) : "memory");
+}
+__device__ __forceinline__ void sb_publish(double* p, double v) {
+  const long long b = (v != v) ? 0x7FF8000000000000ll : __double_as_longlong(v);
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(b) : "memory");
+}
+__device__ __forceinline__ bool sb_published(const float* p, float* v) {
+  unsigned b;
+  asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(b) : "l"(p) : "memory");
+  *v = __uint_as_float(b);
+  return b != 0xFFFFFFFFu;
+}
+__device__ __forceinline__ bool sb_published(const double* p, double* v) {
+  long long b;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(b) : "l"(p) : "memory");
+  *v = __longlong_as_double(b);
+  return b != -1ll;
+}
+
+// The step is a chain, so what it need not wait for is taken off it by two
+// extra warps.  The Householder warp forms the next reflector's scalars from
+// the column x, the first that a step's update finishes, and publishes beta,
+// while the NT working threads finish and store the step, wait for the
+// predecessor and load the next D and E; the
+// release warp orders the step's stores and advances the progress counter
+// while the working threads are already in the next step.  Barriers of a step:
+// X (x is in shared memory: the working threads arrive, the Householder warp
+// waits), ready (everybody), work (twice, the working threads), done (the
+// working threads arrive, the release warp waits); an arrival cannot overtake
+// the wait of the step before, which the ready barrier follows.  The abort flag
+// alternates with the step, so that a warp that is late to read it at one ready
+// barrier does not see what is raised on the way to the next.
+//
+// Bound: the lag between sweeps, two steps and a hand-over.  GB300, FP32 b = 64,
+// n = 8810: 117 ms with the scalars (a chain of some 4000 cycles of FP64
+// latency), the release fences and the beta counter on the step's chain, 83 with
+// the two warps, 77 with x published before the rest of the update and the
+// shorter scalars, 62 with beta as a self-validating word (7.0 us a sweep);
+// n = 3001 38 -> 18.5 ms; FP64 b = 32, n = 2304 43.7 -> 29.1 ms, there bound by
+// the FP64 pipe (some 8000 of a step's 11000 cycles).
+// In a waiting loop that began at t0: true when another CTA has failed or the
+// wait has reached its limit (which is then reported).
+template <class T>
+__device__ __forceinline__ bool sb_give_up(const SbArgs<T>& a, long long t0) {
+  if (*(volatile int32_t*)a.status != 0) return true;
+  if (clock64() - t0 <= a.limit) return false;
+  raise_status(a.status, FRACLAP_ERR_TIMEOUT);
+  return true;
+}
+
 template <class T, int B, int NG>
-__global__ void __launch_bounds__(SbShape<B, NG>::NT) sb2st_kernel(SbArgs<T> a) {
+__global__ void __launch_bounds__(SbShape<B, NG>::NT + 64) sb2st_kernel(SbArgs<T> a) {
   using Sh = SbShape<B, NG>;
-  constexpr int C = Sh::C, W = Sh::W, H = Sh::H, NW = Sh::NW, LDS = B + 1;
+  constexpr int C = Sh::C, W = Sh::W, H = Sh::H, NW = Sh::NW, LDS = B + 1, NT = Sh::NT;
+  constexpr int kBarX = 1, kBarReady = 2, kBarWork = 3, kBarDone = 4;
   __shared__ T Ds[B * LDS];     // transpose of D's lower triangle
   __shared__ T xs[B];           // the column x
   __shared__ T red_p[NG][B], red_e[NG][B];
@@ -106,55 +208,93 @@ __global__ void __launch_bounds__(SbShape<B, NG>::NT) sb2st_kernel(SbArgs<T> a) 
   __shared__ T kpart[NW];
   __shared__ T wfull[B], eyfull[B], wqfull[B];  // w = p - K v, tau E v, tau F^T v
   __shared__ double s_hh[3];    // beta, tau, 1 / v0
-  __shared__ int s_abort;
+  __shared__ int s_abort[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool active = tid < B * NG;
-  const int t = tid % B, g = active ? tid / B : 0;
   const int64_t n = a.n;
   constexpr int ldb = 2 * B;
   T* band = a.band;
 #define BAND(i, j) band[((i) - (j)) + (int64_t)(j) * ldb]
+  if (tid < 2) s_abort[tid] = 0;
+  __syncthreads();
+  int step = 0;  // over all sweeps of this CTA, the same in every warp
 
+  if (warp == NW) {  // ---- Householder warp (norms in FP64) ----
+    for (int64_t s = blockIdx.x; s < n - 1; s += gridDim.x) {
+      const int64_t ns = sb_nsteps(s, n, B);
+      for (int64_t k = 0; k < ns; ++k, ++step) {
+        bar_sync(kBarX, NT + 32);  // xs is complete
+        double tail = 0.0;
+        for (int j = 1 + lane; j < B; j += 32) tail += (double)xs[j] * (double)xs[j];
+        tail = warp_sum(tail);
+        const double x0 = (double)xs[0];
+        double beta = x0, tu = 0.0, inv = 0.0;
+        if (tail > 0.0) {
+          if (sizeof(T) == 4) sb_scalars_f32(x0, tail, lane, &beta, &tu, &inv);
+          else sb_scalars(x0, tail, lane, &beta, &tu, &inv);
+          if (tu == 0.0) inv = 0.0;
+        }
+        if (lane == 0) {
+          s_hh[0] = beta;
+          s_hh[1] = tu;
+          s_hh[2] = inv;
+          a.rtau[s * a.kmax + k] = tu;
+          // the entry sweep s+1 reads at step k-2: one word, so nothing to order
+          sb_publish(a.beta + s * a.kmax + k, (T)beta);
+        }
+        bar_sync(kBarReady, NT + 64);
+        if (s_abort[step & 1]) return;
+      }
+    }
+    return;
+  }
+  if (warp == NW + 1) {  // ---- release warp ----
+    for (int64_t s = blockIdx.x; s < n - 1; s += gridDim.x) {
+      const int64_t ns = sb_nsteps(s, n, B);
+      for (int64_t k = 0; k < ns; ++k, ++step) {
+        bar_sync(kBarReady, NT + 64);
+        if (s_abort[step & 1]) return;
+        bar_sync(kBarDone, NT + 32);  // the step's stores are issued
+        if (lane == 0) st_release_gpu(a.progress + s, (int)(k + 1));  // orders the CTA's stores (after the barrier)
+      }
+    }
+    return;
+  }
+
+  const bool active = tid < B * NG;
+  const int t = tid % B, g = active ? tid / B : 0;
   T XF[C];
   for (int64_t s = blockIdx.x; s < n - 1; s += gridDim.x) {
     const int64_t ns = sb_nsteps(s, n, B);
     const int64_t ns_prev = (s > 0) ? sb_nsteps(s - 1, n, B) : 0;
-    for (int64_t k = 0; k < ns; ++k) {
-      // ---- wait for sweep s-1 to have completed step k+1 and published
-      // the beta of step k+2 ----
-      if (tid == 0) {
-        int ok = 1;
-        if (s > 0) {
-          const int64_t need = (k + 2 < ns_prev) ? k + 2 : ns_prev;
-          const int64_t need_b = (k + 3 < ns_prev) ? k + 3 : ns_prev;
-          const long long t0 = clock64();
-          while (ld_acquire_gpu(a.progress + (s - 1)) < need || ld_acquire_gpu(a.beta_progress + (s - 1)) < need_b) {
-            if (*(volatile int32_t*)a.status != 0) { ok = 0; break; }
-            if (clock64() - t0 > a.limit) {
-              raise_status(a.status, FRACLAP_ERR_TIMEOUT);
-              ok = 0;
-              break;
-            }
-            __nanosleep(32);
-          }
-        }
-        s_abort = !ok;
-      }
-      __syncthreads();
-      if (s_abort) return;
-
+    for (int64_t k = 0; k < ns; ++k, ++step) {
       const int64_t r0 = s + 1 + k * B;
       const int L = (int)((n - r0 < B) ? n - r0 : B);
       const int64_t r1 = r0 + L - 1;
       const int64_t c = (k == 0) ? s : r0 - B;
       const int nf = (int)(r0 - 1 - c);  // 0 at step 0, b - 1 after
       const int Lb = (int)((n - 1 - r1 < B) ? n - 1 - r1 : B);
-
+      // ---- wait for sweep s-1 to have completed step k+1: every warp by itself ----
+      if (s > 0) {
+        const int need = (int)(k + 2 < ns_prev ? k + 2 : ns_prev);
+        if (lane == 0) {
+          const long long t0 = clock64();
+          while (ld_acquire_gpu(a.progress + (s - 1)) < need)
+            if (sb_give_up(a, t0)) {
+              s_abort[step & 1] = 1;
+              break;
+            }
+        }
+        __syncwarp();
+      }
       // ---- load (all of a thread's loads in flight together) ----
       if (k == 0) {
 #pragma unroll
         for (int i = 0; i < C; ++i) XF[i] = T(0);
-        if (active && g == 0 && t < L) XF[0] = __ldcg(&BAND(r0 + t, c));
+        if (active && g == 0) {
+          if (t < L) XF[0] = __ldcg(&BAND(r0 + t, c));
+          xs[t] = XF[0];
+        }
+        bar_arrive(kBarX, NT + 32);
       }
       T Dr[C], Er[C];
 #pragma unroll
@@ -168,37 +308,23 @@ __global__ void __launch_bounds__(SbShape<B, NG>::NT) sb2st_kernel(SbArgs<T> a) 
         const int u = g + NG * i;
         if (active && u <= t) Ds[u + t * LDS] = Dr[i];
       }
-      if (active && g == 0) xs[t] = XF[0];
-      __syncthreads();
-      // ---- Householder scalars (warp 0; norms in FP64) ----
-      if (warp == 0) {
-        double tail = 0.0;
-        for (int j = 1 + lane; j < B; j += 32) tail += (double)xs[j] * (double)xs[j];
-        tail = warp_sum(tail);
-        if (lane == 0) {
-          const double x0 = (double)xs[0];
-          double beta = x0, v0 = 1.0, tu = 0.0;
-          if (tail > 0.0) {
-            const double alpha = sqrt(x0 * x0 + tail);
-            beta = (x0 >= 0.0) ? -alpha : alpha;
-            v0 = x0 - beta;
-            tu = (beta - x0) / beta;
+      // the last entry of E is the subdiagonal value of sweep s-1's step k+2
+      if (s > 0 && k + 2 < ns_prev && t == B - 1 && g == (B - 1) % NG && active && Lb == B && L == B) {
+        const T* word = a.beta + (s - 1) * a.kmax + k + 2;
+        const long long t0 = clock64();
+        while (!sb_published(word, &Er[C - 1]))
+          if (sb_give_up(a, t0)) {
+            s_abort[step & 1] = 1;
+            break;
           }
-          s_hh[0] = beta;
-          s_hh[1] = tu;
-          s_hh[2] = (tu == 0.0) ? 0.0 : 1.0 / v0;
-          // the entry sweep s+1 reads at step k-2: published now, not at the
-          // end of the step (the store below writes the same value again)
-          __stcg(&BAND(r0, c), (T)beta);
-          st_release_gpu(a.beta_progress + s, (int)(k + 1));
-        }
       }
+      bar_sync(kBarReady, NT + 64);  // the scalars, D's lower triangle and the abort flag
+      if (s_abort[step & 1]) return;
 #pragma unroll
       for (int i = 0; i < C; ++i) {
         const int u = g + NG * i;
         if (active && u > t) Dr[i] = Ds[t + u * LDS];  // upper triangle from the transpose
       }
-      __syncthreads();
       const double tu = s_hh[1];
       const T inv = (T)s_hh[2];
       const T vt = (t == 0) ? T(1) : xs[t] * inv;  // v, with v(0) = 1
@@ -209,7 +335,6 @@ __global__ void __launch_bounds__(SbShape<B, NG>::NT) sb2st_kernel(SbArgs<T> a) 
         vu[i] = (u == 0) ? T(1) : xs[u] * inv;
       }
       if (active && g == 0) a.refl[((int64_t)s * a.kmax + k) * B + t] = vt;
-      if (tid == 0) a.rtau[s * a.kmax + k] = tu;
       // ---- partial sums: F^T v (over rows), D v and E v (over columns), v^T D v ----
       {
         T pv[C];
@@ -235,7 +360,7 @@ __global__ void __launch_bounds__(SbShape<B, NG>::NT) sb2st_kernel(SbArgs<T> a) 
         for (int o = 16; o >= 1; o /= 2) kk += __shfl_xor_sync(0xffffffffu, kk, o);
         if (lane == 0) kpart[warp] = kk;
       }
-      __syncthreads();
+      bar_sync(kBarWork, NT);
       // ---- full sums, once per row / column ----
       if (tid < B) {
         const T tuT = (T)tu;
@@ -256,19 +381,24 @@ __global__ void __launch_bounds__(SbShape<B, NG>::NT) sb2st_kernel(SbArgs<T> a) 
         eyfull[tid] = tuT * es;
         wqfull[tid] = tuT * cs;
       }
-      __syncthreads();
+      bar_sync(kBarWork, NT);
       // ---- rank-one and rank-two updates in registers ----
       const T wt = wfull[t], eyt = eyfull[t];
+      const T beta = (T)s_hh[0];  // before x: the Householder warp then overwrites the scalars
+      Er[0] -= eyt * vu[0];
+      if (k + 1 < ns) {  // the first column of E is the next step's x
+        if (active && g == 0) xs[t] = Er[0];
+        bar_arrive(kBarX, NT + 32);
+      }
 #pragma unroll
       for (int i = 0; i < C; ++i) {
         const int u = g + NG * i;
         XF[i] -= vt * wqfull[u];
         if (u <= t) Dr[i] -= vt * wfull[u] + wt * vu[i];  // only the stored triangle
-        Er[i] -= eyt * vu[i];
+        if (i > 0) Er[i] -= eyt * vu[i];
       }
       // ---- store x (annihilated), F and D's lower triangle; E moves on ----
       if (active && t < L) {
-        const T beta = (T)s_hh[0];
 #pragma unroll
         for (int i = 0; i < C; ++i) {
           const int u = g + NG * i;
@@ -279,8 +409,7 @@ __global__ void __launch_bounds__(SbShape<B, NG>::NT) sb2st_kernel(SbArgs<T> a) 
       }
 #pragma unroll
       for (int i = 0; i < C; ++i) XF[i] = Er[i];
-      __syncthreads();
-      if (tid == 0) st_release_gpu(a.progress + s, (int)(k + 1));  // orders the CTA's stores (after the barrier)
+      bar_arrive(kBarDone, NT + 32);
     }
   }
 #undef BAND
@@ -796,15 +925,16 @@ int stage2_take(Arena* ar, int64_t n, int b, Stage2T<T>* s) {
   const int64_t nsw = (n >= 2) ? n - 1 : 0;
   s->refl = ar->take<T>(nsw * s->kmax * b);
   s->rtau = ar->take<double>(nsw * s->kmax);
-  s->progress = ar->take<int>(2 * (n + 1));  // completed steps, then published betas
+  s->beta = ar->take<T>(nsw * s->kmax);
   // -U of every block of b reflectors (one step, b consecutive sweeps): 2b x b each
   s->ut = (b == 32 || b == 64) ? ar->take<T>(s->kmax * (s->kmax + 1) / 2 * 2 * b * b) : nullptr;
+  s->progress = ar->take<int>(n + 1);
   return 0;
 }
 
 template <class T, int B, int NG>
 int sb2st_launch(fraclap_ctx* ctx, SbArgs<T> a, cudaStream_t st) {
-  constexpr int NT = SbShape<B, NG>::NT;
+  constexpr int NT = SbShape<B, NG>::NT + 64;  // and the Householder and release warps
   int per_sm = 0;
   FL_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sb2st_kernel<T, B, NG>, NT, 0));
   FL_CHECK(ctx, per_sm >= 1, FRACLAP_ERR_UNSUPPORTED, "sb2st: kernel does not fit on an SM");
@@ -820,9 +950,10 @@ template <class T>
 int sb2st_run(fraclap_ctx* ctx, T* band, int64_t n, int b, double* d, double* e, Stage2T<T>* s,
               cudaStream_t st) {
   if (n >= 2) {
-    FL_CUDA(ctx, cudaMemsetAsync(s->progress, 0, sizeof(int) * 2 * (n + 1), st));
+    FL_CUDA(ctx, cudaMemsetAsync(s->progress, 0, sizeof(int) * (n + 1), st));
+    FL_CUDA(ctx, cudaMemsetAsync(s->beta, 0xFF, sizeof(T) * (n - 1) * s->kmax, st));
     FL_CUDA(ctx, cudaMemsetAsync(s->rtau, 0, sizeof(double) * (n - 1) * s->kmax, st));
-    SbArgs<T> a{band, n, b, s->kmax, s->refl, s->rtau, s->progress, s->progress + (n + 1), ctx->d_status,
+    SbArgs<T> a{band, n, b, s->kmax, s->refl, s->rtau, s->progress, s->beta, ctx->d_status,
                 ctx->wait_cycles};
     int rc = 0;
     switch (b) {
