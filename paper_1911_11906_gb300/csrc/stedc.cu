@@ -21,12 +21,15 @@
 //   vectors: U(j, i) = zhat_j / (d_j - lambda_i), normalised;
 //   GEMM: Q_new = Q_sorted(:, kept) U  (batched, device-side descriptors);
 //   finalise: deflated and new eigenvalues merged into ascending order.
+// Every step but the preparation's chain of rotations spreads over all rows,
+// columns or values of a level.
 #include "internal.cuh"
 
 namespace fraclap {
 namespace {
 
 constexpr double kEps = 2.220446049250313e-16;
+constexpr int kQuotMax = 200 * 1024;  // shared memory for the quotients of one vector
 
 __host__ __device__ __forceinline__ int64_t leaf_bound(int64_t i, int64_t n, int L) {
   return (i * n) >> L;
@@ -58,8 +61,8 @@ struct DcBuf {
   int* rot_j;
   double* rot_c;
   double* rot_s;
-  int* outsrc;    // n: final column -> source (>= 0: new column i; < 0: -1 - deflated sorted pos)
-  double* outval; // n: final eigenvalues
+  int* outsrc;    // n: deflated values placed before each survivor
+  double* outval; // n: scratch (unsorted D of the merge)
   MergeInfo* info;  // per merge
   GemmDescT<T>* desc;  // per merge
   T* Wq;          // gathered Q, n_m x n_m per merge
@@ -393,10 +396,11 @@ __global__ void dc_merge_prep(DcBuf<T> B, const double* e, const double* lambda,
   B.desc[j] = d;
 }
 
-// Gather Q columns into sorted order and apply the deflation rotations.
-// grid: (ceil(nmax/128), nmerge); thread = row of the merge block.
+// Gather Q columns into sorted order.  grid: (ceil(nmax / 128), nmerge, column
+// groups); thread = row of the merge block, kGatherCols columns.
+constexpr int kGatherCols = 32;
 template <class T>
-__global__ void dc_gather(DcBuf<T> B, const T* Z, int64_t ldz, int64_t nmax) {
+__global__ void __launch_bounds__(128) dc_gather(DcBuf<T> B, const T* Z, int64_t ldz, int64_t nmax) {
   const MergeInfo inf = B.info[blockIdx.y];
   const int64_t nm = inf.hi - inf.lo;
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -404,18 +408,52 @@ __global__ void dc_gather(DcBuf<T> B, const T* Z, int64_t ldz, int64_t nmax) {
   const int64_t lo = inf.lo, n1 = inf.mid - inf.lo;
   T* Wq = B.Wq + lo * nmax;
   const int* perm = B.perm + lo;
-  for (int64_t i = 0; i < nm; ++i) {
+  const int64_t i0 = (int64_t)blockIdx.z * kGatherCols;
+  const int64_t i1 = (i0 + kGatherCols < nm) ? i0 + kGatherCols : nm;
+#pragma unroll 4
+  for (int64_t i = i0; i < i1; ++i) {
     const int64_t c = perm[i];
     // block-diagonal: row r of block 1 pairs with columns of block 1 only
     const bool same = (r < n1) == (c < n1);
     Wq[r + i * nm] = same ? Z[(lo + r) + (lo + c) * ldz] : T(0);
   }
-  for (int64_t q = 0; q < inf.nrot; ++q) {
-    const int64_t a = B.rot_i[lo + q], b = B.rot_j[lo + q];
-    const double c = B.rot_c[lo + q], s = B.rot_s[lo + q];
-    const double xa = Wq[r + a * nm], xb = Wq[r + b * nm];
-    Wq[r + a * nm] = (T)(c * xa + s * xb);
-    Wq[r + b * nm] = (T)(-s * xa + c * xb);
+}
+
+// The deflation rotations, in order, on the gathered columns; thread = row.  A
+// column is shared by consecutive rotations only (the second column of one is
+// the first of the next, and stays in a register), so the columns of eight
+// rotations are read at once.
+template <class T>
+__global__ void __launch_bounds__(64) dc_rotate(DcBuf<T> B, int64_t nmax) {
+  const MergeInfo inf = B.info[blockIdx.y];
+  const int64_t nm = inf.hi - inf.lo;
+  const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= nm || inf.nrot == 0) return;
+  const int64_t lo = inf.lo;
+  T* W = B.Wq + lo * nmax + r;
+  constexpr int RB = 8;
+  int last = -1;      // the column held in `carry`
+  T carry = T(0);
+  for (int64_t q0 = 0; q0 < inf.nrot; q0 += RB) {
+    const int m = (int)((inf.nrot - q0 < RB) ? inf.nrot - q0 : RB);
+    T xa[RB], xb[RB];
+#pragma unroll
+    for (int q = 0; q < RB; ++q)
+      if (q < m) {
+        xa[q] = W[(int64_t)B.rot_i[lo + q0 + q] * nm];
+        xb[q] = W[(int64_t)B.rot_j[lo + q0 + q] * nm];
+      }
+#pragma unroll
+    for (int q = 0; q < RB; ++q)
+      if (q < m) {
+        const int a = B.rot_i[lo + q0 + q], b = B.rot_j[lo + q0 + q];
+        const double c = B.rot_c[lo + q0 + q], s = B.rot_s[lo + q0 + q];
+        const double va = (a == last) ? carry : xa[q], vb = xb[q];
+        W[(int64_t)a * nm] = (T)(c * va + s * vb);
+        carry = (T)(-s * va + c * vb);
+        last = b;
+        W[(int64_t)b * nm] = carry;
+      }
   }
 }
 
@@ -533,28 +571,39 @@ __global__ void __launch_bounds__(32 * kSecWarps) dc_secular(DcBuf<T> B, int32_t
 }
 
 // Gu-Eisenstat: zhat_i^2 = (lam_{K-1} - d_i)/rho * prod_{j<K-1} (lam_j - d_i)/(d_j' - d_i).
+// A warp per entry, the lanes' products of every 32nd factor multiplied by a
+// butterfly (the factors pair off around 1, so no partial product drifts).
 template <class T>
-__global__ void dc_zhat(DcBuf<T> B) {
+__global__ void __launch_bounds__(32 * kSecWarps) dc_zhat(DcBuf<T> B) {
   const MergeInfo inf = B.info[blockIdx.y];
   const int64_t K = inf.K;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= K) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t i = (int64_t)blockIdx.x * kSecWarps + (threadIdx.x >> 5);
+  if (i >= K) return;  // warp-uniform
   const double* dd = B.dd + inf.lo;
   const double* tau = B.tau + inf.lo;
   const int* org = B.org + inf.lo;
-  double prod = ((dd[org[K - 1]] - dd[i]) + tau[K - 1]) / inf.rho;
-  for (int64_t j = 0; j + 1 < K; ++j) {
-    const double num = (dd[org[j]] - dd[i]) + tau[j];
-    const double den = (j < i) ? dd[j] - dd[i] : dd[j + 1] - dd[i];
+  const double di = dd[i];
+  double prod = 1.0;
+  for (int64_t j = lane; j + 1 < K; j += 32) {
+    const double num = (dd[org[j]] - di) + tau[j];
+    const double den = (j < i) ? dd[j] - di : dd[j + 1] - di;
     prod *= num / den;
   }
-  const double zi = B.zz[inf.lo + i];
-  B.zhat[inf.lo + i] = copysign(sqrt(fmax(prod, 0.0)), zi);
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) prod *= __shfl_xor_sync(0xffffffffu, prod, o);
+  if (lane == 0) {
+    prod *= ((dd[org[K - 1]] - di) + tau[K - 1]) / inf.rho;
+    B.zhat[inf.lo + i] = copysign(sqrt(fmax(prod, 0.0)), B.zz[inf.lo + i]);
+  }
 }
 
-// U(:, i) = zhat ./ (d - lambda_i), normalised; one CTA per (column, merge).
+// U(:, i) = zhat ./ (d - lambda_i), normalised; one CTA per (column, merge).  The
+// quotients (the FP64 pipe's work) are kept in shared memory between the norm
+// and the scaling when the launch gave room for them (cached).
 template <class T>
-__global__ void dc_vectors(DcBuf<T> B, int64_t nmax) {
+__global__ void dc_vectors(DcBuf<T> B, int64_t nmax, int cached) {
+  extern __shared__ __align__(16) double dc_quot[];
   const MergeInfo inf = B.info[blockIdx.y];
   const int64_t K = inf.K, i = blockIdx.x;
   if (i >= K) return;
@@ -567,6 +616,7 @@ __global__ void dc_vectors(DcBuf<T> B, int64_t nmax) {
   double s = 0.0;
   for (int64_t j = threadIdx.x; j < K; j += blockDim.x) {
     const double v = zh[j] / ((dd[j] - dorg) - t);
+    if (cached) dc_quot[j] = v;  // read back by this thread
     s += v * v;
   }
   __shared__ double red[32];
@@ -581,12 +631,12 @@ __global__ void dc_vectors(DcBuf<T> B, int64_t nmax) {
   __syncthreads();
   const double inv = 1.0 / sqrt(red[0]);
   for (int64_t j = threadIdx.x; j < K; j += blockDim.x)
-    u[j] = (T)(zh[j] / ((dd[j] - dorg) - t) * inv);
+    u[j] = (T)((cached ? dc_quot[j] : zh[j] / ((dd[j] - dorg) - t)) * inv);
 }
 
-// Qnd(:, q) = Wq(:, kept[q]) for survivors; grid (ceil(nmax/128), nmerge).
+// Qnd(:, q) = Wq(:, kept[q]) for survivors; grid (ceil(nmax/128), nmerge, column groups).
 template <class T>
-__global__ void dc_gather_kept(DcBuf<T> B, int64_t nmax) {
+__global__ void __launch_bounds__(128) dc_gather_kept(DcBuf<T> B, int64_t nmax) {
   const MergeInfo inf = B.info[blockIdx.y];
   const int64_t nm = inf.hi - inf.lo;
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -594,40 +644,80 @@ __global__ void dc_gather_kept(DcBuf<T> B, int64_t nmax) {
   const T* Wq = B.Wq + inf.lo * nmax;
   T* Q = B.Qnd + inf.lo * nmax;
   const int* kept = B.kept + inf.lo;
-  for (int64_t q = 0; q < inf.K; ++q) Q[r + q * nm] = Wq[r + (int64_t)kept[q] * nm];
+  const int64_t q0 = (int64_t)blockIdx.z * kGatherCols;
+  const int64_t q1 = (q0 + kGatherCols < inf.K) ? q0 + kGatherCols : inf.K;
+#pragma unroll 4
+  for (int64_t q = q0; q < q1; ++q) Q[r + q * nm] = Wq[r + (int64_t)kept[q] * nm];
 }
 
-// Final ascending order of the merged spectrum (thread 0 per merge).
+// An integer in the order of the doubles (both zeros alike).
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v + 0.0);
+  return b < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)b) : b;
+}
+
+// Ranks of the merged spectrum, as a sequential merge of the survivors (in
+// their order) with the deflated values (sorted, equal ones in their order)
+// would place them: survivor a goes after the deflated values below the
+// largest of the survivors up to a (outsrc[a]: their number), deflated value b
+// has rank[b] deflated values before it (perm[rank] = b).  A thread per value;
+// the deflated values pass through shared memory as integer keys.  grid
+// (ceil(nmax / 256), nmerge).
 template <class T>
-__global__ void dc_order(DcBuf<T> B) {
-  if (threadIdx.x != 0) return;
-  const MergeInfo inf = B.info[blockIdx.x];
+__global__ void __launch_bounds__(256) dc_order(DcBuf<T> B) {
+  const MergeInfo inf = B.info[blockIdx.y];
   const int64_t lo = inf.lo, nm = inf.hi - inf.lo, K = inf.K, nd = nm - K;
+  const int64_t i0 = (int64_t)blockIdx.x * 256;
+  if (i0 >= nm) return;
   const int* kept = B.kept + lo;
   const double* Dp = B.Dp + lo;
-  int* defl = B.perm + lo;  // perm no longer needed: sorted deflated positions
-  for (int64_t q = 0; q < nd; ++q) defl[q] = kept[K + q];
-  for (int64_t q = 1; q < nd; ++q) {  // insertion sort by value (nearly sorted)
-    const int v = defl[q];
-    int64_t p = q - 1;
-    while (p >= 0 && Dp[defl[p]] > Dp[v]) { defl[p + 1] = defl[p]; --p; }
-    defl[p + 1] = v;
-  }
   const double* dd = B.dd + lo;
   const double* tau = B.tau + lo;
   const int* org = B.org + lo;
-  int* out = B.outsrc + lo;
-  double* val = B.outval + lo;
-  int64_t a = 0, b = 0;
-  for (int64_t o = 0; o < nm; ++o) {
-    const double va = (a < K) ? dd[org[a]] + tau[a] : 0.0;
-    const double vb = (b < nd) ? Dp[defl[b]] : 0.0;
-    bool take_a = (b >= nd) || (a < K && va <= vb);
-    // ascending in signed space; reversed when the merge was flipped
-    const int64_t pos = (inf.sign > 0) ? o : nm - 1 - o;
-    if (take_a) { out[pos] = (int)a; val[pos] = inf.sign * va; ++a; }
-    else { out[pos] = -1 - defl[b]; val[pos] = inf.sign * vb; ++b; }
+  __shared__ long long key[256], red[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t i = i0 + tid;
+  constexpr long long kLow = (long long)0x8000000000000000ull;
+  const bool surv = i < K, defl = i >= K && i < nm;
+  // largest survivor up to i: this block's prefix, and all survivors before it
+  long long mine = surv ? order_key(dd[org[i]] + tau[i]) : kLow, before = kLow;
+  for (int64_t a = tid; a < i0 && a < K; a += 256) {
+    const long long v = order_key(dd[org[a]] + tau[a]);
+    before = v > before ? v : before;
   }
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long v = __shfl_up_sync(0xffffffffu, mine, o);
+    if (lane >= o && v > mine) mine = v;
+  }
+  for (int o = 16; o >= 1; o >>= 1) {
+    const long long v = __shfl_xor_sync(0xffffffffu, before, o);
+    before = v > before ? v : before;
+  }
+  key[tid] = mine;
+  if (lane == 0) red[warp] = before;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) {
+    before = red[w] > before ? red[w] : before;
+    if (w < warp) mine = key[32 * w + 31] > mine ? key[32 * w + 31] : mine;
+  }
+  mine = before > mine ? before : mine;
+  const long long self = defl ? order_key(Dp[kept[i]]) : mine;
+  int cnt = 0;
+  for (int64_t b0 = 0; b0 < nd; b0 += 256) {
+    __syncthreads();
+    if (b0 + tid < nd) key[tid] = order_key(Dp[kept[K + b0 + tid]]);
+    __syncthreads();
+    const int m = (int)((nd - b0 < 256) ? nd - b0 : 256);
+    const int eq = (int)((i - K - b0 < 0) ? 0 : (i - K - b0 < m ? i - K - b0 : m));  // equal keys before i come first
+    if (defl) {
+      for (int q = 0; q < eq; ++q) cnt += key[q] <= self;
+      for (int q = eq; q < m; ++q) cnt += key[q] < self;
+    } else {
+      for (int q = 0; q < m; ++q) cnt += key[q] < self;
+    }
+  }
+  if (surv) B.outsrc[lo + i] = cnt;
+  if (defl) B.perm[lo + cnt] = (int)(i - K);
 }
 
 // Z(lo:hi, lo + p) = chosen column; lambda(lo + p) = value.  grid (nmax, nmerge).
@@ -636,12 +726,25 @@ __global__ void dc_scatter(DcBuf<T> B, double* lambda, T* Z, int64_t ldz, int64_
   const MergeInfo inf = B.info[blockIdx.y];
   const int64_t nm = inf.hi - inf.lo, p = blockIdx.x;
   if (p >= nm) return;
-  const int src = B.outsrc[inf.lo + p];
-  const T* col = (src >= 0) ? B.G + inf.lo * nmax + (int64_t)src * nm
-                            : B.Wq + inf.lo * nmax + (int64_t)(-1 - src) * nm;
+  // ascending in signed space; reversed when the merge was flipped
+  const int64_t o = (inf.sign > 0) ? p : nm - 1 - p;
+  // the first survivor at or after place o (survivor a is at a + outsrc[a])
+  const int* c = B.outsrc + inf.lo;
+  int64_t l = 0, h = inf.K;
+  while (l < h) {
+    const int64_t m = (l + h) >> 1;
+    if (m + c[m] < o) l = m + 1;
+    else h = m;
+  }
+  const bool surv = l < inf.K && l + c[l] == o;
+  const int64_t src = surv ? l : (int64_t)B.kept[inf.lo + inf.K + B.perm[inf.lo + o - l]];
+  const T* col = surv ? B.G + inf.lo * nmax + src * nm : B.Wq + inf.lo * nmax + src * nm;
   T* dst = Z + inf.lo + (inf.lo + p) * ldz;
   for (int64_t r = threadIdx.x; r < nm; r += blockDim.x) dst[r] = col[r];
-  if (threadIdx.x == 0) lambda[inf.lo + p] = B.outval[inf.lo + p];
+  if (threadIdx.x == 0) {
+    const double v = surv ? B.dd[inf.lo + B.org[inf.lo + src]] + B.tau[inf.lo + src] : B.Dp[inf.lo + src];
+    lambda[inf.lo + p] = inf.sign * v;
+  }
 }
 
 int tree_levels(int64_t n, int leaf) {
@@ -723,21 +826,27 @@ int stedc_run(fraclap_ctx* ctx, const double* d, const double* e, int64_t n, dou
     FL_CHECK(ctx, nmerge <= 65535 && nmax < (1LL << 31), FRACLAP_ERR_UNSUPPORTED, "stedc: too large");
     dc_merge_prep<T><<<(unsigned)nmerge, 128, 0, st>>>(B, e, lambda, Z, ldz, n, L, level, nmax);
     count_launch(ctx);
-    const dim3 rows((unsigned)cdiv(nmax, 128), (unsigned)nmerge);
-    dc_gather<T><<<rows, 128, 0, st>>>(B, Z, ldz, nmax);
+    const dim3 blocks((unsigned)cdiv(nmax, 128), (unsigned)nmerge, (unsigned)cdiv(nmax, kGatherCols));
+    FL_CHECK(ctx, blocks.z <= 65535, FRACLAP_ERR_UNSUPPORTED, "stedc: too large");
+    dc_gather<T><<<blocks, 128, 0, st>>>(B, Z, ldz, nmax);
+    count_launch(ctx);
+    dc_rotate<T><<<dim3((unsigned)cdiv(nmax, 64), (unsigned)nmerge), 64, 0, st>>>(B, nmax);
     count_launch(ctx);
     dc_secular<T><<<dim3((unsigned)cdiv(nmax, kSecWarps), (unsigned)nmerge), 32 * kSecWarps, 0, st>>>(
         B, ctx->d_status);
     count_launch(ctx);
-    dc_zhat<T><<<rows, 128, 0, st>>>(B);
+    dc_zhat<T><<<dim3((unsigned)cdiv(nmax, kSecWarps), (unsigned)nmerge), 32 * kSecWarps, 0, st>>>(B);
     count_launch(ctx);
-    dc_vectors<T><<<dim3((unsigned)nmax, (unsigned)nmerge), 128, 0, st>>>(B, nmax);
+    const size_t quot = sizeof(double) * (size_t)nmax;
+    const bool cached = quot <= kQuotMax;
+    FL_CUDA(ctx, cudaFuncSetAttribute(dc_vectors<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kQuotMax));
+    dc_vectors<T><<<dim3((unsigned)nmax, (unsigned)nmerge), 128, cached ? quot : 0, st>>>(B, nmax, cached ? 1 : 0);
     count_launch(ctx);
-    dc_gather_kept<T><<<rows, 128, 0, st>>>(B, nmax);
+    dc_gather_kept<T><<<blocks, 128, 0, st>>>(B, nmax);
     count_launch(ctx);
     FL_CUDA(ctx, cudaGetLastError());
     FL_TRY(gemm_batched<T>(ctx, false, false, B.desc, (int)nmerge, nmax, nmax, st));
-    dc_order<T><<<(unsigned)nmerge, 32, 0, st>>>(B);
+    dc_order<T><<<dim3((unsigned)cdiv(nmax, 256), (unsigned)nmerge), 256, 0, st>>>(B);
     count_launch(ctx);
     dc_scatter<T><<<dim3((unsigned)nmax, (unsigned)nmerge), 128, 0, st>>>(B, lambda, Z, ldz, nmax);
     count_launch(ctx);
