@@ -31,6 +31,7 @@ struct fraclap_ctx {
   size_t tc_scratch_bytes = 0;   // (set by the caller of the FP32 stages, null otherwise)
   long long wait_cycles = 0;     // wait_timeout_s in SM clock cycles (upper bound)
   int32_t* d_status = nullptr;   // device status word (0 = ok, else a FRACLAP_ERR_*)
+  int panel_cluster_fits[2] = {-1, -1};  // FP32, FP64 panels on one cluster: 1, 0, or -1 (not asked yet)
   unsigned* d_barrier = nullptr; // grid-barrier state for cooperative kernels
   void* ws = nullptr;            // context-owned workspace
   size_t ws_bytes = 0;
@@ -256,7 +257,6 @@ struct Stage1T {
   T* Y;              // b * b
   T* Mm;             // b * b
   double* gram;      // b * b
-  T* gramT;          // b * b (cluster panel route)
   double* partials;  // 2 * G * 2b
   int64_t npanel;
   int64_t vtotal;
@@ -342,6 +342,47 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// Householder scalars of (x0, tail = sum of the other squares > 0): beta = -+
+// sqrt(x0^2 + tail), tau = (beta - x0) / beta and 1 / (x0 - beta).  Every lane of
+// a warp calls it with the same arguments.
+__device__ __forceinline__ void householder_scalars(double x0, double tail, int lane, double* beta, double* tu, double* inv) {
+  const double alpha = sqrt(x0 * x0 + tail);
+  const double b = (x0 >= 0.0) ? -alpha : alpha;
+  // one division, on two lanes
+  const double q = ((lane & 1) ? 1.0 : b - x0) / ((lane & 1) ? x0 - b : b);
+  *beta = b;
+  *tu = __shfl_sync(0xffffffffu, q, 0);
+  *inv = __shfl_sync(0xffffffffu, q, 1);
+}
+// The same for FP32 entries, to within a few units of 2^-52 and in a third of
+// the dependent FP64 operations: with r = 1 / sqrt(sigma), |beta| = sigma r, tau
+// = 1 + |x0| r and 1 / |x0 - beta| = r / tau.  r and 1 / tau come from an FP32
+// start by one step of Halley's (third-order) iteration, which takes 2^-22 to
+// below 2^-60.  sigma is scaled to [1, 4) by its exponent: squares of FP32
+// entries are normal doubles; anything else (an infinity, a NaN) takes the
+// general form.
+__device__ __forceinline__ void householder_scalars_f32(double x0, double tail, int lane, double* beta, double* tu, double* inv) {
+  const double sigma = fma(x0, x0, tail);
+  const int hi = __double2hiint(sigma), E = (hi >> 20) - 1023;  // sigma > 0
+  if (E < -1000 || E > 1000) {
+    householder_scalars(x0, tail, lane, beta, tu, inv);
+    return;
+  }
+  const int k = E >> 1;
+  const double ss = __hiloint2double(hi - 2 * k * (1 << 20), __double2loint(sigma));
+  const double r0 = (double)rsqrtf((float)ss);
+  const double e = fma(-(ss * r0), r0, 1.0);
+  const double rs = fma(r0, e * fma(0.375, e, 0.5), r0);
+  const double r = __hiloint2double(__double2hiint(rs) - k * (1 << 20), __double2loint(rs));  // rs 2^-k
+  const double alpha = sigma * r, t = fma(fabs(x0), r, 1.0);
+  const double y0 = (double)(1.0f / (float)t);
+  const double f = fma(-t, y0, 1.0);
+  const double y = fma(y0, fma(f, f, f), y0);
+  *beta = (x0 >= 0.0) ? -alpha : alpha;
+  *tu = t;
+  *inv = (x0 >= 0.0) ? r * y : -(r * y);
 }
 
 __device__ __forceinline__ int ld_acquire_gpu(const int* p) {

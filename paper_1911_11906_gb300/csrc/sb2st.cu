@@ -102,46 +102,6 @@ __device__ __forceinline__ void bar_arrive(int id, int count) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// Householder scalars of (x0, tail = sum of the other squares > 0): beta = -+
-// sqrt(x0^2 + tail), tau = (beta - x0) / beta and 1 / (x0 - beta).
-__device__ __forceinline__ void sb_scalars(double x0, double tail, int lane, double* beta, double* tu, double* inv) {
-  const double alpha = sqrt(x0 * x0 + tail);
-  const double b = (x0 >= 0.0) ? -alpha : alpha;
-  // one division, on two lanes
-  const double q = ((lane & 1) ? 1.0 : b - x0) / ((lane & 1) ? x0 - b : b);
-  *beta = b;
-  *tu = __shfl_sync(0xffffffffu, q, 0);
-  *inv = __shfl_sync(0xffffffffu, q, 1);
-}
-// The same for FP32 entries, to within a few units of 2^-52 and in a third of
-// the dependent FP64 operations: with r = 1 / sqrt(sigma), |beta| = sigma r, tau
-// = 1 + |x0| r and 1 / |x0 - beta| = r / tau.  r and 1 / tau come from an FP32
-// start by one step of Halley's (third-order) iteration, which takes 2^-22 to
-// below 2^-60.  sigma is scaled to [1, 4) by its exponent: squares of FP32
-// entries are normal doubles; anything else (an infinity, a NaN) takes the
-// general form.
-__device__ __forceinline__ void sb_scalars_f32(double x0, double tail, int lane, double* beta, double* tu, double* inv) {
-  const double sigma = fma(x0, x0, tail);
-  const int hi = __double2hiint(sigma), E = (hi >> 20) - 1023;  // sigma > 0
-  if (E < -1000 || E > 1000) {
-    sb_scalars(x0, tail, lane, beta, tu, inv);
-    return;
-  }
-  const int k = E >> 1;
-  const double ss = __hiloint2double(hi - 2 * k * (1 << 20), __double2loint(sigma));
-  const double r0 = (double)rsqrtf((float)ss);
-  const double e = fma(-(ss * r0), r0, 1.0);
-  const double rs = fma(r0, e * fma(0.375, e, 0.5), r0);
-  const double r = __hiloint2double(__double2hiint(rs) - k * (1 << 20), __double2loint(rs));  // rs 2^-k
-  const double alpha = sigma * r, t = fma(fabs(x0), r, 1.0);
-  const double y0 = (double)(1.0f / (float)t);
-  const double f = fma(-t, y0, 1.0);
-  const double y = fma(y0, fma(f, f, f), y0);
-  *beta = (x0 >= 0.0) ? -alpha : alpha;
-  *tu = t;
-  *inv = (x0 >= 0.0) ? r * y : -(r * y);
-}
-
 // One published word: a NaN is made the canonical one, so that no value is the
 // "not yet" pattern of all bits set.
 __device__ __forceinline__ void sb_publish(float* p, float v) {
@@ -229,8 +189,8 @@ __global__ void __launch_bounds__(SbShape<B, NG>::NT + 64) sb2st_kernel(SbArgs<T
         const double x0 = (double)xs[0];
         double beta = x0, tu = 0.0, inv = 0.0;
         if (tail > 0.0) {
-          if (sizeof(T) == 4) sb_scalars_f32(x0, tail, lane, &beta, &tu, &inv);
-          else sb_scalars(x0, tail, lane, &beta, &tu, &inv);
+          if (sizeof(T) == 4) householder_scalars_f32(x0, tail, lane, &beta, &tu, &inv);
+          else householder_scalars(x0, tail, lane, &beta, &tu, &inv);
           if (tu == 0.0) inv = 0.0;
         }
         if (lane == 0) {

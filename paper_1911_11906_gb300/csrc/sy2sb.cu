@@ -21,7 +21,8 @@ namespace cg = cooperative_groups;
 
 constexpr int PQR_NT = 256;
 constexpr int kClusterMax = 16;                  // CTAs of the cluster panel kernel (non-portable above 8)
-constexpr int kPanelClusterSmemMax = 220 * 1024;  // panel rows one CTA of the cluster holds
+constexpr int kPanelClusterSmemMax = 217 * 1024;  // panel rows one CTA of the cluster holds
+constexpr int64_t kPanelFp64Rows = 1200;          // FP64 panels of the cluster kernel
 constexpr int kPanelSmemMax = 180 * 1024;  // largest panel slice one CTA holds
 
 // Cooperative panel QR.  P: m x bw panel (ld ldp) in the working matrix.
@@ -167,189 +168,216 @@ panel_qr_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t ldv,
 }
 
 // The same panel factorisation on one thread-block cluster (up to 16 CTAs)
-// when the panel fits in their shared memory: each column's partial sums are
-// read from the other CTAs' shared memory (distributed shared memory) after
-// one hardware cluster barrier, in the same rank order everywhere, instead of
-// a grid-wide barrier and global atomics.  Partial sums are double-buffered
-// by column parity, so one barrier per column suffices: a CTA writes the
-// next column's partials only after the barrier that ends everyone's reads
-// of the same buffer two columns back.  Writes R, the reflectors and the
-// explicit V; the Gram matrix and T follow in separate kernels.
+// when the panel fits in their shared memory, with T of the compact WY form.
+// Per column, every CTA's partial dot products and the pivot row are written
+// into all CTAs' shared memory (distributed shared memory) before one hardware
+// cluster barrier and added there in rank order; the buffers alternate by
+// column parity, so one barrier a column suffices.  One warp forms the
+// reflector's scalars while the others add the columns' sums.  Then G = V^T V
+// (each CTA's rows in 4 x 4 register tiles, the partial sums added over the
+// cluster), and T, the inverse of diag(1/tau) + strictly-upper(G) (Schreiber
+// and Van Loan's form of H_1 ... H_bw = I - V T V^T), column by column, dealt to
+// the CTAs, a warp each: T(k, j) = -tau_k sum_{k < q <= j} G(k, q) T(q, j) from
+// k = j down, in FP64, which holds for tau_k = 0 as well.
+// Bound: the chain of a column (dots, barrier, FP64 scalars, update).  GB300,
+// with the Gram product and T's kernel it replaces, a panel of FP32 b = 64: m up
+// to 7735 some 520 -> 418 us, up to 2753 400 -> 257 us; the band reduction at n =
+// 2753 24.8 -> 19.0 ms; FP64 b = 32, n = 779 10.9 -> 7.6 ms (165 us a panel).
+// G, a CTA's part and the FP64 sum, in the place of V
+template <class T>
+constexpr size_t panel_gram_smem() {
+  return 64 * 64 * sizeof(T) + 64 * 65 * sizeof(double);
+}
 template <class T>
 __global__ void __launch_bounds__(PQR_NT)
-panel_qr_cluster_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t ldv, double* tau,
-                        int64_t rows_per_cta) {
+panel_qr_cluster_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t ldv, double* tau, T* Tf,
+                        int rows_per_cta, int ld) {
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* S = reinterpret_cast<T*>(smem_raw);  // rows_per_cta x bw, column-major (ld rows_per_cta)
-  __shared__ double part[2][2 * 64];
-  __shared__ double red[2 * 64 + 4];
-  __shared__ double sw[64];
-  __shared__ T swt[64];  // sw in the working precision (converted once per column, not once per row)
-  __shared__ double s_coef[4];
-  const unsigned rank = cluster.block_rank(), CS = cluster.num_blocks();
+  T* S = reinterpret_cast<T*>(smem_raw);  // rows_per_cta x bw, column-major (ld)
+  __shared__ T recv[2][kClusterMax][64];  // every CTA's partial dot products
+  __shared__ T piv[2][64];                // the pivot row
+  __shared__ double g[64];                // their sums
+  __shared__ T swt[64];
+  __shared__ double s_tau[64];
+  __shared__ double s_coef[3];            // beta, tau, 1 / (x0 - beta)
+  const int rank = (int)cluster.block_rank(), CS = (int)cluster.num_blocks();
   const int64_t rb = (int64_t)rank * rows_per_cta;
-  const int64_t re = (rb + rows_per_cta < m) ? rb + rows_per_cta : m;
-  const int64_t nr = (re > rb) ? re - rb : 0;
-  const int64_t ld = rows_per_cta;
+  const int nr = (int)((rb + rows_per_cta < m) ? rows_per_cta : (m > rb ? m - rb : 0));
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = PQR_NT / 32;
 
   for (int c = 0; c < bw; ++c)
-    for (int64_t r = tid; r < nr; r += PQR_NT) S[r + c * ld] = P[(rb + r) + c * ldp];
-  __syncthreads();
+    for (int r = tid; r < nr; r += PQR_NT) S[r + c * ld] = P[(rb + r) + c * ldp];
+  cluster.sync();  // every CTA of the cluster runs before its shared memory is written
 
   const int nref = (m < bw) ? (int)m : bw;
   for (int c = 0; c < nref; ++c) {
-    double* mine = part[c & 1];
-    const int64_t r0 = (c > rb) ? c - rb : 0;  // first local row with global row >= c
+    const int buf = c & 1;
+    const int r0 = (c > rb) ? (int)((c - rb < nr) ? c - rb : nr) : 0;  // first local row with global row >= c
     {
-      // per-CTA partial dots in the working precision (FP64 work on ~m/16 rows
-      // would occupy GB300's narrow FP64 pipe); the cluster sum is FP64.  A
-      // warp takes columns j = c + warp + 8 q, all in one pass over its rows
-      // (the pivot column read once, eight independent sums).
+      // partial dots in the working precision (the cluster sum is FP64); a warp
+      // takes columns j = c + warp + 8 q in one pass over its rows
       constexpr int QMAX = 64 / 8;
       T sum[QMAX];
 #pragma unroll
       for (int q = 0; q < QMAX; ++q) sum[q] = T(0);
-      for (int64_t r = r0 + lane; r < nr; r += 32) {
-        const int64_t gr = rb + r;
+      for (int r = r0 + lane; r < nr; r += 32) {
         const T pc = S[r + c * ld];
+        const bool pivot = rb + r == c;  // g_c: rows > c only
 #pragma unroll
         for (int q = 0; q < QMAX; ++q) {
           const int j = c + warp + nwarp * q;
-          if (j < bw && !(j == c && gr == c)) sum[q] += pc * S[r + j * ld];  // g_c: rows > c only
+          if (j < bw && !(j == c && pivot)) sum[q] += pc * S[r + j * ld];
         }
       }
+      // eight sums over 32 lanes: three halving exchanges leave one per lane,
+      // two butterflies finish it; four lanes then hold column idx
+      int idx = 0;
 #pragma unroll
-      for (int q = 0; q < QMAX; ++q) {
-        T v = sum[q];
+      for (int s = 0; s < 3; ++s) {
+        const int half = QMAX >> (s + 1), o = 16 >> s;
+        const bool up = (lane & o) != 0;
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const int j = c + warp + nwarp * q;
-        if (lane == 0 && j < bw) mine[j] = (double)v;
+        for (int q = 0; q < QMAX / 2; ++q)
+          if (q < half) {
+            const T send = up ? sum[q] : sum[q + half];
+            const T keep = up ? sum[q + half] : sum[q];
+            sum[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        if (up) idx += half;
+      }
+      T v = sum[0];
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      const int j = c + warp + nwarp * idx;
+      if (j < bw)
+        for (int q = lane & 3; q < CS; q += 4) *cluster.map_shared_rank(&recv[buf][rank][j], q) = v;
+    }
+    if (c >= rb && c < rb + nr) {
+      const int j = tid & 63;
+      if (j >= c && j < bw) {
+        const T v = S[(int)(c - rb) + j * ld];
+        for (int q = tid >> 6; q < CS; q += PQR_NT / 64) *cluster.map_shared_rank(&piv[buf][j], q) = v;
       }
     }
-    for (int j = c + tid; j < bw; j += PQR_NT) mine[bw + j] = (c >= rb && c < re) ? (double)S[(c - rb) + j * ld] : 0.0;
     cluster.sync();
-    for (int t = tid; t < 2 * (bw - c); t += PQR_NT) {
-      const int slot = (t < bw - c) ? c + t : bw + c + (t - (bw - c));
-      double v[kClusterMax];  // all remote loads in flight, then the sum in rank order
+    if (warp == 0) {
+      double tail = (lane < CS) ? (double)recv[buf][lane][c] : 0.0;
 #pragma unroll
-      for (int q = 0; q < kClusterMax; ++q)
-        v[q] = (q < (int)CS) ? cluster.map_shared_rank(&part[c & 1][0], q)[slot] : 0.0;
-      double sum = 0.0;
-#pragma unroll
-      for (int q = 0; q < kClusterMax; ++q) sum += v[q];
-      red[(t < bw - c) ? t : 64 + (t - (bw - c))] = sum;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      const double tail = red[0], x0 = red[64];
-      double beta = x0, v0 = 1.0, tu = 0.0;
+      for (int o = 8; o >= 1; o >>= 1) tail += __shfl_xor_sync(0xffffffffu, tail, o);
+      tail = __shfl_sync(0xffffffffu, tail, 0);
+      const double x0 = (double)piv[buf][c];
+      double beta = x0, tu = 0.0, inv = 0.0;
       if (tail > 0.0 && m - c > 1) {
-        const double alpha = sqrt(x0 * x0 + tail);
-        beta = (x0 >= 0.0) ? -alpha : alpha;
-        v0 = x0 - beta;
-        tu = (beta - x0) / beta;
+        if (sizeof(T) == 4) householder_scalars_f32(x0, tail, lane, &beta, &tu, &inv);
+        else householder_scalars(x0, tail, lane, &beta, &tu, &inv);
       }
-      s_coef[0] = beta;
-      s_coef[1] = 1.0 / v0;
-      s_coef[2] = tu;
-      if (rank == 0) tau[c] = tu;
+      if (lane == 0) {
+        s_coef[0] = beta;
+        s_coef[1] = tu;
+        s_coef[2] = inv;
+        s_tau[c] = tu;
+        if (rank == 0) tau[c] = tu;
+      }
+    } else {
+      // the other columns' sums: two lanes a column, rank order halves
+      const int t = tid - 32, j = c + 1 + (t >> 1), q0 = (t & 1) * (kClusterMax / 2);
+      double s = 0.0;
+      if (j < bw)
+        for (int q = q0; q < q0 + kClusterMax / 2 && q < CS; ++q) s += (double)recv[buf][q][j];
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      if (j < bw && (t & 1) == 0) g[j] = s;
     }
     __syncthreads();
-    const double beta = s_coef[0], inv_v0 = s_coef[1], tu = s_coef[2];
-    for (int j = c + 1 + tid; j < bw; j += PQR_NT) {
-      const double g = red[j - c], pc = red[64 + (j - c)];
-      sw[j] = (tu == 0.0) ? 0.0 : tu * (g - beta * pc) * inv_v0;
-      swt[j] = (T)sw[j];
-    }
+    const double beta = s_coef[0], tu = s_coef[1], inv = s_coef[2];
+    // w_j = tau v^T p_j, v^T p_j = (g_j - beta p_j(c)) / v0
+    if (tid < 64 && tid > c && tid < bw) swt[tid] = (T)(tu * (g[tid] - beta * (double)piv[buf][tid]) * inv);
     __syncthreads();
-    for (int64_t r = r0 + tid; r < nr; r += PQR_NT) {
-      const int64_t gr = rb + r;
-      double vr;
-      if (gr == c) {
-        vr = 1.0;
+    const T ih = (T)inv, il = (T)(inv - (double)ih);  // the product with inv rounded once
+    for (int r = r0 + tid; r < nr; r += PQR_NT) {
+      T vt;
+      if (rb + r == c) {
+        vt = T(1);
         S[r + c * ld] = (T)beta;
       } else {
-        vr = (tu == 0.0) ? 0.0 : (double)S[r + c * ld] * inv_v0;
-        S[r + c * ld] = (T)vr;
+        const T x = S[r + c * ld];
+        vt = (sizeof(T) == 8) ? x * ih : fma(x, ih, x * il);  // 0 when tau = 0 (inv = 0)
+        S[r + c * ld] = vt;
       }
-      if (tu != 0.0) {
-        const T vt = (T)vr;
+      if (tu != 0.0)
         for (int j = c + 1; j < bw; ++j) S[r + j * ld] -= vt * swt[j];
-      }
     }
     __syncthreads();
   }
-  for (int c = nref; c < bw && rank == 0 && tid == 0; ++c) tau[c] = 0.0;
+  for (int c = nref + tid; c < bw; c += PQR_NT) {
+    s_tau[c] = 0.0;
+    if (rank == 0) tau[c] = 0.0;
+  }
+  // R and the reflectors to P, V to Vout; S becomes V (rows past nr are zero)
   for (int c = 0; c < bw; ++c)
-    for (int64_t r = tid; r < nr; r += PQR_NT) {
-      const int64_t gr = rb + r;
-      const T sv = S[r + c * ld];
-      P[gr + c * ldp] = sv;
+    for (int r = tid; r < rows_per_cta; r += PQR_NT) {
       T v = T(0);
-      if (c < nref) v = (gr < c) ? T(0) : (gr == c ? T(1) : sv);
-      Vout[gr + c * ldv] = v;
-    }
-  cluster.sync();  // no CTA leaves while another may still read its partial sums
-}
-
-// T of the compact WY form from tau and the Gram matrix G = V^T V (bw x bw).
-// When every tau is nonzero, T^-1 = diag(1/tau) + strictly-upper(G)
-// (Schreiber and Van Loan's form of H_1 ... H_bw = I - V T V^T): T is that
-// triangle's inverse, formed row by row from the bottom, X(i, j) =
-// -(1 / U(i, i)) sum_{i < k <= j} U(i, k) X(k, j), all columns of a row at
-// once and each sum split over four lanes (one barrier per row).  Otherwise
-// the column recurrence T(i, i) = tau_i, T(0:i, i) = -tau_i T(0:i, 0:i) G(0:i, i).
-// One CTA of 256 threads.
-template <class T>
-__global__ void __launch_bounds__(PQR_NT) panel_t_kernel(const T* gram, const double* tau, int bw, T* Tf) {
-  __shared__ double U[64][65];  // U(i, k), i <= k
-  __shared__ double Ts[64 * 64];
-  __shared__ double y[64];
-  __shared__ int s_zero;
-  const int tid = threadIdx.x;
-  if (tid == 0) s_zero = 0;
-  __syncthreads();
-  for (int p = tid; p < bw * bw; p += PQR_NT) {
-    const int i = p % bw, k = p / bw;
-    if (i < k) U[i][k] = (double)gram[i + k * bw];
-    else if (i == k) {
-      const double t = tau[i];
-      if (t == 0.0) s_zero = 1;
-      U[i][i] = (t == 0.0) ? 1.0 : 1.0 / t;
-    }
-    Ts[p] = 0.0;
-  }
-  __syncthreads();
-  if (!s_zero) {
-    static_assert(PQR_NT == 256, "four lanes per column of a 64-wide panel");
-    const int j = tid >> 2, part = tid & 3;  // column j, lanes 4j .. 4j + 3 of one warp
-    for (int i = bw - 1; i >= 0; --i) {
-      double sum = 0.0;
-      if (j > i && j < bw)
-        for (int k = i + 1 + part; k <= j; k += 4) sum += U[i][k] * Ts[k + j * bw];
-      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-      if (part == 0 && j < bw && j >= i) Ts[i + j * bw] = (j == i) ? 1.0 / U[i][i] : -sum / U[i][i];
-      __syncthreads();
-    }
-  } else {
-    for (int i = 0; i < bw; ++i) {
-      const double ti = tau[i];
-      if (tid < i) y[tid] = (double)gram[tid + i * bw];
-      __syncthreads();
-      if (tid < i) {
-        double sum = 0.0;
-        for (int q = tid; q < i; ++q) sum += Ts[tid + q * bw] * y[q];
-        Ts[tid + i * bw] = -ti * sum;
+      if (r < nr) {
+        const int64_t gr = rb + r;
+        const T sv = S[r + c * ld];
+        P[gr + c * ldp] = sv;
+        if (c < nref) v = (gr < c) ? T(0) : (gr == c ? T(1) : sv);
+        Vout[gr + c * ldv] = v;
       }
-      if (tid == 0) Ts[i + i * bw] = ti;
-      __syncthreads();
+      S[r + c * ld] = v;
     }
+  __syncthreads();
+  // this CTA's part of G: entries (ti + 16 a, tj + 16 b) of the upper triangle
+  const int ti = tid & 15, tj = tid >> 4;
+  T acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+  const int nb = (bw + 15) / 16;
+  for (int r = 0; r < nr; ++r) {
+    T x[4], y[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      x[a] = (a < nb && ti + 16 * a < bw) ? S[r + (ti + 16 * a) * ld] : T(0);
+      y[a] = (a < nb && tj + 16 * a < bw) ? S[r + (tj + 16 * a) * ld] : T(0);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = a; b < 4; ++b) acc[a][b] += x[a] * y[b];
   }
-  for (int p = tid; p < bw * bw; p += PQR_NT) Tf[p] = (T)Ts[p];
+  __syncthreads();
+  T* Gp = S;                                       // 64 x 64: this CTA's part
+  double* Gd = reinterpret_cast<double*>(smem_raw + 64 * 64 * sizeof(T));  // [column][row], 64 x 65: the sum
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = a; b < 4; ++b) Gp[(ti + 16 * a) + (tj + 16 * b) * 64] = acc[a][b];
+  cluster.sync();
+  for (int e = rank * PQR_NT + tid; e < 64 * 64; e += CS * PQR_NT) {
+    const int i = e & 63, k = e >> 6;
+    if (i >= k || k >= bw) continue;
+    T s = T(0);
+    for (int q = 0; q < CS; ++q) s += cluster.map_shared_rank(Gp, q)[e];
+    for (int q = 0; q < CS; ++q) cluster.map_shared_rank(Gd, q)[k * 65 + i] = (double)s;
+  }
+  cluster.sync();
+  for (int j = rank + CS * warp; j < bw; j += CS * nwarp) {
+    double a0 = 0.0, a1 = 0.0, t0 = 0.0, t1 = 0.0;  // rows lane and lane + 32: sum so far, T(., j)
+    for (int k = j; k >= 0; --k) {
+      const double sum = __shfl_sync(0xffffffffu, (k < 32) ? a0 : a1, k & 31);
+      const double x = (k == j) ? s_tau[j] : -s_tau[k] * sum;
+      if (lane == (k & 31)) {
+        if (k < 32) t0 = x;
+        else t1 = x;
+      }
+      if (lane < k) a0 = fma(Gd[k * 65 + lane], x, a0);
+      if (lane + 32 < k) a1 = fma(Gd[k * 65 + lane + 32], x, a1);
+    }
+    if (lane < bw) Tf[lane + j * bw] = (T)t0;
+    if (lane + 32 < bw) Tf[lane + 32 + j * bw] = (T)t1;
+  }
 }
 
 // Band extraction: band(off, j) = A(j + off, j) for off <= b, 0 for b < off < ldb.
@@ -380,7 +408,6 @@ int stage1_take(Arena* ar, int64_t n, int b, int G, Stage1T<T>* s) {
   s->Y = ar->take<T>((int64_t)b * b);
   s->Mm = ar->take<T>((int64_t)b * b);
   s->gram = ar->take<double>((int64_t)b * b);
-  s->gramT = ar->take<T>((int64_t)b * b);
   s->partials = ar->take<double>(3 * 2 * (int64_t)b);
   return 0;
 }
@@ -396,25 +423,24 @@ static int panel_grid(fraclap_ctx* ctx, int64_t m, int bw, size_t elem, int64_t*
   return G;
 }
 
-// Panel on one cluster, then G = V^T V (split over the rows) and T.  Returns
-// 1 (nothing launched) when the panel does not fit in a cluster's shared
-// memory or no cluster of that size can be resident; < 0 on a CUDA error.
+// Panel on one cluster.  Returns 1 (nothing launched) when the panel does not
+// fit in a cluster's shared memory or no cluster of that size can be resident;
+// < 0 on a CUDA error.
 template <class T>
-int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, double* tau, T* gramT, T* Tf,
-                  cudaStream_t st) {
-  // FP64 panels keep the grid kernel: spread over all SMs, their FP64 dot
-  // products are not bound by one SM's narrow FP64 pipe
-  if (sizeof(T) == 8) return 1;
-  const int64_t cap = kPanelClusterSmemMax / ((int64_t)b * (int64_t)sizeof(T));
+int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, double* tau, T* Tf, cudaStream_t st) {
+  // FP64: past some 1200 rows sixteen SMs' FP64 pipes lose to the grid kernel's
+  // dot products on all SMs
+  if (sizeof(T) == 8 && m > kPanelFp64Rows) return 1;
+  const int64_t most = sizeof(T) == 8 ? kPanelClusterSmemMax - 10 * 1024 : kPanelClusterSmemMax;
+  const int64_t cap = most / ((int64_t)b * (int64_t)sizeof(T)) - 1;
   const int limit = std::max(1, std::min(kClusterMax, ctx->sm_count));
-  int CS = (int)std::max<int64_t>(cdiv(m, cap), std::min<int64_t>(limit, cdiv(m, 128)));
+  int CS = (int)std::max<int64_t>(cdiv(m, cap), std::min<int64_t>(limit, cdiv(m, sizeof(T) == 8 ? 48 : 128)));
   if (CS > limit) return 1;
-  const int64_t rows = cdiv(m, CS);
+  const int rows = (int)cdiv(m, CS);
   CS = (int)cdiv(m, rows);
-  const size_t smem = (size_t)rows * b * sizeof(T);
-  FL_CUDA(ctx, cudaFuncSetAttribute(panel_qr_cluster_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  FL_CUDA(ctx, cudaFuncSetAttribute(panel_qr_cluster_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    kPanelClusterSmemMax));
+  const int ld = rows | 1;  // odd: the Gram tiles read 16 columns of a row at once
+  const size_t smem = std::max<size_t>((size_t)ld * b * sizeof(T), panel_gram_smem<T>());
+  auto kern = panel_qr_cluster_kernel<T>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)CS);
   cfg.blockDim = dim3(PQR_NT);
@@ -427,21 +453,24 @@ int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, d
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, panel_qr_cluster_kernel<T>, &cfg) != cudaSuccess || clusters < 1) {
-    cudaGetLastError();
-    return 1;
+  // asked once per context: the largest cluster with the largest panel is resident
+  int& fits = ctx->panel_cluster_fits[sizeof(T) == 8 ? 1 : 0];
+  if (fits < 0) {
+    FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+    cudaLaunchConfig_t full = cfg;
+    cudaLaunchAttribute big = attr[0];
+    big.val.clusterDim.x = (unsigned)limit;
+    full.gridDim = dim3((unsigned)limit);
+    full.dynamicSmemBytes = (size_t)most;
+    full.attrs = &big;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &full) != cudaSuccess) cudaGetLastError();
+    fits = clusters >= 1 ? 1 : 0;
   }
-  int bw = b;
+  if (!fits) return 1;
   count_launch(ctx);
-  FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, panel_qr_cluster_kernel<T>, P, ldp, m, bw, V, m, tau, rows));
-  using D = GemmDescT<T>;
-  FL_CUDA(ctx, cudaMemsetAsync(gramT, 0, sizeof(T) * b * b, st));
-  FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{b, b, m, V, m, V, m, gramT, b, nullptr, 0, nullptr, 0, 0, 1.0, 1.0},
-                 (int)std::min<int64_t>(cdiv(m, 512), 16), st));
-  panel_t_kernel<T><<<1, PQR_NT, 0, st>>>(gramT, tau, b, Tf);
-  count_launch(ctx);
-  FL_CUDA(ctx, cudaGetLastError());
+  FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, P, ldp, m, b, V, m, tau, Tf, rows, ld));
   return 0;
 }
 
@@ -457,7 +486,7 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
     T* P = Aw + (j0 + b) + j0 * lda;
     T* V = s->Vstore + voff;
     T* Tf = s->Tstore + p * b * b;
-    const int crc = panel_cluster(ctx, P, lda, m, b, V, s->tau + p * b, s->gramT, Tf, st);
+    const int crc = panel_cluster(ctx, P, lda, m, b, V, s->tau + p * b, Tf, st);
     if (crc < 0) return crc;
     if (crc == 0) {
       // done on one cluster
