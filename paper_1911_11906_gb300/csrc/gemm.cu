@@ -168,135 +168,252 @@ __global__ void __launch_bounds__(NT) gemm_batched_kernel(const GemmDescT<T>* de
 }
 
 // ---------------------------------------------------------------------------
-// FP32: 128 x 128 output tile, 8-deep k steps, 256 threads with 8 x 8 outputs
-// each (rows 4 tx.. and 64 + 4 tx.., columns 4 ty.. and 64 + 4 ty..), read
-// from shared memory as float4 (16 loads per 64 FMAs, against 8 per 16 on
-// the 64 x 64 tile); the next k step is fetched into registers while the
-// current one is multiplied (double-buffered shared memory, one barrier per
-// step).  Plain and lower-C forms, fused second product, split-K, batched.
-constexpr int SG_M = 128, SG_N = 128, SG_K = 8, SG_NT = 256, SG_LD = SG_M + 4;
+// FP32 products: 128 threads per output tile, each TM x TN outputs in registers,
+// k steps of 16 (8 on the large tile) double-buffered in shared memory (the next step is fetched
+// into registers while the current one is multiplied).  The multiplications are
+// packed pairs (fma.rn.f32x2) along the rows: half the issue slots, so that the
+// shared-memory reads -- (TM + TN) / (TM TN) words an FMA, what bounds a SIMT
+// product on this chip -- fit beside them.  128 x 128 tiles at 16 x 8 outputs a
+// thread for outputs of at least 256 x 256; 128 x 64 and 64 x 128 at 8 x 8 for
+// narrow outputs, whose long sums a cluster of CTAs along K shares (partial
+// tiles added over distributed shared memory in rank order: no atomics, no
+// zeroing).  Forms: plain, lower-C, symmetric A (its lower triangle read:
+// blocks above the diagonal from their mirror, in either case coalesced), a
+// second product into the same C, batched.  GB300, before and now: 8192^3 45.1
+// -> 53.0 TFLOP/s; symmetric 4405 x 64 some 230 -> 93 us, 1114 x 32 98 -> 15 us;
+// the merges' products at n = 7735 21.5 -> 15.0 ms, the first back-transformation
+// there 39.7 -> 35.4 ms, the band reduction 90 -> 79 ms.
+constexpr int SG_NT = 128, SG_K = 16, SG_K_BIG = 8;
 
-template <bool TA, bool TB>
-__device__ __forceinline__ void sg_fetch(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t M,
-                                         int64_t N, int64_t kend, int64_t m0, int64_t n0, int64_t k0,
-                                         float (&ra)[4], float (&rb)[4]) {
-  const int tid = threadIdx.x;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (!TA) {
-      const int64_t gm = m0 + tid % SG_M, gk = k0 + tid / SG_M + 2 * q;
-      ra[q] = (gm < M && gk < kend) ? A[gm + gk * lda] : 0.0f;
-    } else {
-      const int64_t gk = k0 + tid % SG_K, gm = m0 + tid / SG_K + 32 * q;
-      ra[q] = (gm < M && gk < kend) ? A[gk + gm * lda] : 0.0f;
-    }
-    if (!TB) {
-      const int64_t gk = k0 + tid % SG_K, gn = n0 + tid / SG_K + 32 * q;
-      rb[q] = (gn < N && gk < kend) ? B[gk + gn * ldb] : 0.0f;
-    } else {
-      const int64_t gn = n0 + tid % SG_N, gk = k0 + tid / SG_N + 2 * q;
-      rb[q] = (gn < N && gk < kend) ? B[gn + gk * ldb] : 0.0f;
-    }
-  }
+__device__ __forceinline__ unsigned long long sg_pair(float a, float b) {
+  unsigned long long v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+  return v;
+}
+__device__ __forceinline__ void sg_fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 
-template <bool TA, bool TB>
-__device__ __forceinline__ void sg_stash(float (*As)[SG_LD], float (*Bs)[SG_LD], const float (&ra)[4],
-                                         const float (&rb)[4]) {
-  const int tid = threadIdx.x;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (!TA) As[tid / SG_M + 2 * q][tid % SG_M] = ra[q];
-    else As[tid % SG_K][tid / SG_K + 32 * q] = ra[q];
-    if (!TB) Bs[tid % SG_K][tid / SG_K + 32 * q] = rb[q];
-    else Bs[tid / SG_N + 2 * q][tid % SG_N] = rb[q];
+// One operand's k step in registers: BX entries along x (rows of op(A) or
+// columns of op(B)) by SG_K along k.  XC: x is the contiguous direction of the
+// storage; entry (x, k) at p[x + k ld], else at p[k + x ld].
+template <int BX, bool XC, int SG_K>
+struct SgStep {
+  static constexpr int PER = BX * SG_K / SG_NT;
+  static __device__ __forceinline__ int x_of(int q) {
+    return XC ? ((BX == 128) ? (int)threadIdx.x : (int)(threadIdx.x % BX)) : (int)(threadIdx.x / SG_K) + (SG_NT / SG_K) * q;
   }
-}
+  static __device__ __forceinline__ int k_of(int q) {
+    return XC ? ((BX == 128) ? q : (int)(threadIdx.x / BX) + (SG_NT / BX) * q) : (int)(threadIdx.x % SG_K);
+  }
+  static __device__ __forceinline__ void fetch(float (&r)[PER], const float* p, int64_t ld, int64_t X, int64_t kend,
+                                               int64_t x0, int64_t k0) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int64_t x = x0 + x_of(q), k = k0 + k_of(q);
+      r[q] = (x < X && k < kend) ? (XC ? p[x + k * ld] : p[k + x * ld]) : 0.0f;
+    }
+  }
+  // symmetric storage, lower triangle: entry (x, k) at p[x + k ld] if x >= k, else its mirror
+  static __device__ __forceinline__ void fetch_sym(float (&r)[PER], const float* p, int64_t ld, int64_t X, int64_t kend,
+                                                   int64_t x0, int64_t k0) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int64_t x = x0 + x_of(q), k = k0 + k_of(q);
+      r[q] = (x < X && k < kend) ? (x >= k ? p[x + k * ld] : p[k + x * ld]) : 0.0f;
+    }
+  }
+  static __device__ __forceinline__ void stash(float* s, const float (&r)[PER]) {  // s: SG_K x (BX + 4)
+#pragma unroll
+    for (int q = 0; q < PER; ++q) s[k_of(q) * (BX + 4) + x_of(q)] = r[q];
+  }
+};
 
-template <bool TA, bool TB>
-__device__ __forceinline__ void sg_accumulate(float (&acc)[8][8], float (*As)[SG_K][SG_LD],
-                                              float (*Bs)[SG_K][SG_LD], const float* A, int64_t lda,
-                                              const float* B, int64_t ldb, int64_t M, int64_t N, int64_t m0,
-                                              int64_t n0, int64_t kbeg, int64_t kend) {
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float ra[4], rb[4];
-  sg_fetch<TA, TB>(A, lda, B, ldb, M, N, kend, m0, n0, kbeg, ra, rb);
+template <int BM, int BN, int TM, int TN, int SG_K>
+struct SgTile {
+  static_assert((BM / TM) * (BN / TN) == SG_NT, "128 threads");
+  static constexpr int GX = BM / TM, GY = BN / TN;  // threads along the rows and columns
+  static constexpr int STEP = SG_K * (BM + 4 + BN + 4);  // words of one buffered k step
+  // thread (tx, ty): rows 4 (tx + GX i) + e, columns 4 (ty + GY j) + e
+  static __device__ __forceinline__ int row(int i) { return 4 * ((int)threadIdx.x % GX + GX * (i / 4)) + i % 4; }
+  static __device__ __forceinline__ int col(int j) { return 4 * ((int)threadIdx.x / GX + GY * (j / 4)) + j % 4; }
+};
+
+template <int BM, int BN, int TM, int TN, int SG_K, bool TA, bool TB, int MODE>
+__device__ __forceinline__ void sg_accumulate(unsigned long long (&acc)[TM / 2][TN], float* smem, const float* A,
+                                              int64_t lda, const float* B, int64_t ldb, int64_t M, int64_t N,
+                                              int64_t m0, int64_t n0, int64_t kbeg, int64_t kend) {
+  using Tile = SgTile<BM, BN, TM, TN, SG_K>;
+  using SA = SgStep<BM, !TA, SG_K>;
+  using SM = SgStep<BM, false, SG_K>;  // the mirrored half of a symmetric A
+  using SB = SgStep<BN, TB, SG_K>;
+  float ra[SA::PER], rb[SB::PER];
+  // symmetric A: 0 below the diagonal, 1 above it, 2 across it
+  auto side = [&](int64_t k0) { return k0 + SG_K - 1 <= m0 ? 0 : (k0 >= m0 + BM - 1 ? 1 : 2); };
+  auto fetch = [&](int64_t k0) {
+    if (MODE == kGemmSymA) {
+      const int sd = side(k0);
+      if (sd == 0) SA::fetch(ra, A, lda, M, kend, m0, k0);
+      else if (sd == 1) SM::fetch(ra, A, lda, M, kend, m0, k0);
+      else SA::fetch_sym(ra, A, lda, M, kend, m0, k0);
+    } else {
+      SA::fetch(ra, A, lda, M, kend, m0, k0);
+    }
+    SB::fetch(rb, B, ldb, N, kend, n0, k0);
+  };
+  auto stash = [&](float* buf, int64_t k0) {
+    if (MODE == kGemmSymA && side(k0) == 1) SM::stash(buf, ra);
+    else SA::stash(buf, ra);
+    SB::stash(buf + SG_K * (BM + 4), rb);
+  };
+  fetch(kbeg);
   __syncthreads();  // the buffers may still be read by a previous product
-  sg_stash<TA, TB>(As[0], Bs[0], ra, rb);
+  stash(smem, kbeg);
   __syncthreads();
   int buf = 0;
   for (int64_t k0 = kbeg; k0 < kend; k0 += SG_K) {
     const bool more = k0 + SG_K < kend;
-    if (more) sg_fetch<TA, TB>(A, lda, B, ldb, M, N, kend, m0, n0, k0 + SG_K, ra, rb);
+    if (more) fetch(k0 + SG_K);
+    const float* as = smem + buf * Tile::STEP;
+    const float* bs = as + SG_K * (BM + 4);
 #pragma unroll
     for (int k = 0; k < SG_K; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][4 * tx]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][64 + 4 * tx]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][4 * ty]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][64 + 4 * ty]);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      unsigned long long a[TM / 2];
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < TM; i += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(as + k * (BM + 4) + Tile::row(i));
+        a[i / 2] = sg_pair(v.x, v.y);
+        a[i / 2 + 1] = sg_pair(v.z, v.w);
+      }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      for (int j = 0; j < TN; j += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(bs + k * (BN + 4) + Tile::col(j));
+        const float b[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const unsigned long long bb = sg_pair(b[e], b[e]);
+#pragma unroll
+          for (int i = 0; i < TM / 2; ++i) sg_fma2(acc[i][j + e], a[i], bb);
+        }
+      }
     }
-    if (more) sg_stash<TA, TB>(As[buf ^ 1], Bs[buf ^ 1], ra, rb);
+    if (more) stash(smem + (buf ^ 1) * Tile::STEP, k0 + SG_K);
     __syncthreads();
     buf ^= 1;
   }
 }
 
-template <bool TA, bool TB, int MODE, bool ATOMIC>
-__device__ __forceinline__ void sg_tile(const GemmDescT<float>& d, int64_t m0, int64_t n0, int64_t kbeg,
-                                        int64_t kend) {
-  __shared__ __align__(16) float As[2][SG_K][SG_LD];
-  __shared__ __align__(16) float Bs[2][SG_K][SG_LD];
-  if (MODE == kGemmLowerC && m0 + SG_M - 1 < n0) return;  // tile entirely above the diagonal
-  float acc[8][8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-  if (kend > kbeg) sg_accumulate<TA, TB>(acc, As, Bs, d.A, d.lda, d.B, d.ldb, d.M, d.N, m0, n0, kbeg, kend);
-  if (d.K2 > 0 && kbeg == 0)
-    sg_accumulate<TA, TB>(acc, As, Bs, d.A2, d.lda2, d.B2, d.ldb2, d.M, d.N, m0, n0, 0, d.K2);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int64_t gn = n0 + (j < 4 ? 4 * ty + j : 64 + 4 * ty + j - 4);
-    if (gn >= d.N) continue;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int64_t gm = m0 + (i < 4 ? 4 * tx + i : 64 + 4 * tx + i - 4);
-      if (gm >= d.M) continue;
-      if (MODE == kGemmLowerC && gm < gn) continue;
-      float* c = d.C + gm + gn * d.ldc;
-      const float v = (float)d.alpha * acc[i][j];
-      if (ATOMIC) atomicAdd(c, v);
-      else *c = (d.beta == 0.0) ? v : v + (float)d.beta * *c;
-    }
-  }
+template <int MODE>
+__device__ __forceinline__ void sg_write(const GemmDescT<float>& d, int64_t gm, int64_t gn, float v) {
+  if (gm >= d.M || gn >= d.N || (MODE == kGemmLowerC && gm < gn)) return;
+  float* c = d.C + gm + gn * d.ldc;
+  v *= (float)d.alpha;
+  *c = (d.beta == 0.0) ? v : v + (float)d.beta * *c;
 }
 
-template <bool TA, bool TB, int MODE, bool ATOMIC>
-__global__ void __launch_bounds__(SG_NT, 2) sgemm_big_kernel(GemmDescT<float> d, int64_t kchunk) {
-  const int64_t m0 = (int64_t)blockIdx.x * SG_M, n0 = (int64_t)blockIdx.y * SG_N;
-  const int64_t kbeg = (int64_t)blockIdx.z * kchunk;
-  const int64_t kend = (kbeg + kchunk < d.K) ? kbeg + kchunk : d.K;
-  sg_tile<TA, TB, MODE, ATOMIC>(d, m0, n0, kbeg, kend);
+// One tile over k in [kbeg, kend) (and the whole second product), shared by the
+// CTAs of a cluster along K when CLUSTER.
+template <int BM, int BN, int TM, int TN, int SG_K, bool TA, bool TB, int MODE, bool CLUSTER>
+__device__ __forceinline__ void sg_tile(const GemmDescT<float>& d, int64_t m0, int64_t n0, int64_t kbeg, int64_t kend) {
+  using Tile = SgTile<BM, BN, TM, TN, SG_K>;
+  constexpr int WORDS = CLUSTER ? (2 * Tile::STEP > BM * BN ? 2 * Tile::STEP : BM * BN) : 2 * Tile::STEP;
+  __shared__ __align__(16) float smem[WORDS];
+  unsigned long long acc[TM / 2][TN];
+#pragma unroll
+  for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0ull;
+  if (kend > kbeg)
+    sg_accumulate<BM, BN, TM, TN, SG_K, TA, TB, MODE>(acc, smem, d.A, d.lda, d.B, d.ldb, d.M, d.N, m0, n0, kbeg, kend);
+  if (d.K2 > 0)  // (a product with a second one is not shared along K)
+    sg_accumulate<BM, BN, TM, TN, SG_K, TA, TB, MODE>(acc, smem, d.A2, d.lda2, d.B2, d.ldb2, d.M, d.N, m0, n0, 0, d.K2);
+  if (CLUSTER) {
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    if (S > 1) {
+      // (the last k step ended with a barrier; a CTA without steps has read nothing)
+#pragma unroll
+      for (int j = 0; j < TN; ++j)
+#pragma unroll
+        for (int i = 0; i < TM; i += 4) {
+          float4 v;
+          asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(acc[i / 2][j]));
+          asm("mov.b64 {%0, %1}, %2;" : "=f"(v.z), "=f"(v.w) : "l"(acc[i / 2 + 1][j]));
+          *reinterpret_cast<float4*>(&smem[Tile::col(j) * BM + Tile::row(i)]) = v;
+        }
+      cluster.sync();
+      for (int e = rank * SG_NT + (int)threadIdx.x; e < BM * BN; e += S * SG_NT) {
+        float v = 0.0f;
+        for (int q = 0; q < S; ++q) v += cluster.map_shared_rank(smem, q)[e];
+        sg_write<MODE>(d, m0 + e % BM, n0 + e / BM, v);
+      }
+      cluster.sync();  // a peer's tile stays until it is read
+      return;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < TN; ++j)
+#pragma unroll
+    for (int i = 0; i < TM; i += 2) {
+      float x, y;
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(acc[i / 2][j]));
+      sg_write<MODE>(d, m0 + Tile::row(i), n0 + Tile::col(j), x);
+      sg_write<MODE>(d, m0 + Tile::row(i) + 1, n0 + Tile::col(j), y);
+    }
+}
+
+template <bool TA, bool TB, int MODE>
+__global__ void __launch_bounds__(SG_NT, 2) sgemm_big_kernel(GemmDescT<float> d) {
+  const int64_t m0 = (int64_t)blockIdx.x * 128, n0 = (int64_t)blockIdx.y * 128;
+  if (MODE == kGemmLowerC && m0 + 127 < n0) return;  // tile entirely above the diagonal
+  sg_tile<128, 128, 16, 8, SG_K_BIG, TA, TB, MODE, false>(d, m0, n0, 0, d.K);
 }
 
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(SG_NT, 2) sgemm_big_batched_kernel(const GemmDescT<float>* descs) {
   const GemmDescT<float> d = descs[blockIdx.z];
-  const int64_t m0 = (int64_t)blockIdx.x * SG_M, n0 = (int64_t)blockIdx.y * SG_N;
+  const int64_t m0 = (int64_t)blockIdx.x * 128, n0 = (int64_t)blockIdx.y * 128;
   if (d.M <= 0 || d.N <= 0 || m0 >= d.M || n0 >= d.N) return;
-  sg_tile<TA, TB, kGemmPlain, false>(d, m0, n0, 0, d.K > 0 ? d.K : 0);
+  sg_tile<128, 128, 16, 8, SG_K_BIG, TA, TB, kGemmPlain, false>(d, m0, n0, 0, d.K > 0 ? d.K : 0);
 }
 
-// The large-tile FP32 kernel pays off once both output dimensions fill it.
+template <int BM, int BN, bool TA, bool TB, int MODE>
+__global__ void __launch_bounds__(SG_NT, 4) sgemm_narrow_kernel(GemmDescT<float> d, int64_t kper) {
+  const int S = (int)cg::this_cluster().num_blocks();
+  const int64_t m0 = (int64_t)(blockIdx.x / S) * BM, n0 = (int64_t)blockIdx.y * BN;
+  const int64_t kbeg = (int64_t)cg::this_cluster().block_rank() * kper;
+  if (MODE == kGemmLowerC && m0 + BM - 1 < n0) return;  // tile entirely above the diagonal (S = 1)
+  sg_tile<BM, BN, 8, 8, SG_K, TA, TB, MODE, true>(d, m0, n0, kbeg, (kbeg + kper < d.K) ? kbeg + kper : d.K);
+}
+
+// The 128 x 128 tiles pay off once both output dimensions fill them.
 inline bool sg_big(int64_t M, int64_t N) { return M >= 256 && N >= 256; }
+// Narrow outputs: one dimension of at most 128, the other of at least as much.
+inline bool sg_narrow(int64_t M, int64_t N) { return std::min(M, N) <= 128 && std::max(M, N) >= 128; }
+
+template <int BM, int BN, bool TA, bool TB, int MODE>
+int launch_sg_narrow(fraclap_ctx* ctx, const GemmDescT<float>& d, cudaStream_t st) {
+  const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
+  const int64_t gx = cdiv(d.M, BM), gy = cdiv(d.N, BN);
+  FL_CHECK(ctx, gy <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm: N = %lld too large", (long long)d.N);
+  int S = 1;  // CTAs per tile along K: until three CTAs an SM, at least 64 of K each
+  while (MODE != kGemmLowerC && S < 8 && gx * gy * S < 3 * sms && d.K2 == 0 && d.K >= 128 * (int64_t)S) S *= 2;
+  const int64_t kper = std::max<int64_t>(cdiv(cdiv(d.K, S), SG_K) * SG_K, SG_K);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(gx * S), (unsigned)gy, 1);
+  cfg.blockDim = dim3(SG_NT);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)S;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, sgemm_narrow_kernel<BM, BN, TA, TB, MODE>, d, kper));
+  count_launch(ctx);
+  return 0;
+}
 
 // ---------------------------------------------------------------------------
 // FP64 products without padding.  The FP64 pipe retires about 1.7 FMAs per
@@ -476,23 +593,22 @@ int launch_narrow(fraclap_ctx* ctx, const GemmDescT<double>& d, cudaStream_t st)
 
 template <class T, bool TA, bool TB, int MODE>
 int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st) {
-  if constexpr (std::is_same<T, float>::value && MODE != kGemmSymA) {
-    if (sg_big(d.M, d.N)) {
-      const int64_t gx = cdiv(d.M, SG_M), gy = cdiv(d.N, SG_N);
+  if constexpr (std::is_same<T, float>::value) {
+    // short sums into large outputs are bound by C's traffic and latency: the
+    // smaller tile has four CTAs an SM to overlap them
+    const bool shallow = d.K + d.K2 <= 160;
+    if (MODE != kGemmSymA && sg_big(d.M, d.N) && shallow) return launch_sg_narrow<128, 64, TA, TB, MODE>(ctx, d, st);
+    if (MODE != kGemmSymA && sg_big(d.M, d.N)) {
+      const int64_t gx = cdiv(d.M, 128), gy = cdiv(d.N, 128);
       FL_CHECK(ctx, gy <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm: N = %lld too large", (long long)d.N);
-      if (split_k <= 1 || d.K2 > 0) {
-        sgemm_big_kernel<TA, TB, MODE, false><<<dim3((unsigned)gx, (unsigned)gy, 1), SG_NT, 0, st>>>(
-            d, d.K > 0 ? d.K : 1);
-      } else {
-        const int64_t kchunk = cdiv(cdiv(d.K, split_k), SG_K) * SG_K;
-        const int64_t gz = cdiv(d.K, kchunk);
-        sgemm_big_kernel<TA, TB, MODE, true><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), SG_NT, 0, st>>>(
-            d, kchunk);
-      }
+      sgemm_big_kernel<TA, TB, MODE><<<dim3((unsigned)gx, (unsigned)gy, 1), SG_NT, 0, st>>>(d);
       count_launch(ctx);
       FL_CUDA(ctx, cudaGetLastError());
       return 0;
     }
+    if (MODE != kGemmLowerC && d.K2 == 0 && sg_narrow(d.M, d.N))
+      return d.M >= d.N ? launch_sg_narrow<128, 64, TA, TB, MODE>(ctx, d, st)
+                        : launch_sg_narrow<64, 128, TA, TB, MODE>(ctx, d, st);
   }
   if constexpr (std::is_same<T, double>::value && MODE != kGemmLowerC && !(TA && TB)) {
     if (d.K2 == 0 && dg_narrow(ctx, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
@@ -557,7 +673,7 @@ int gemm_batched(fraclap_ctx* ctx, bool ta, bool tb, const GemmDescT<T>* d_descs
   if (count <= 0 || max_m <= 0 || max_n <= 0) return 0;
   if constexpr (std::is_same<T, float>::value) {
     if (sg_big(max_m, max_n)) {
-      const int64_t gx = cdiv(max_m, SG_M), gy = cdiv(max_n, SG_N);
+      const int64_t gx = cdiv(max_m, 128), gy = cdiv(max_n, 128);
       FL_CHECK(ctx, gy <= 65535 && count <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm_batched: too large");
       dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)count);
       if (!ta && !tb) sgemm_big_batched_kernel<false, false><<<grid, SG_NT, 0, st>>>(d_descs);
