@@ -356,26 +356,34 @@ __device__ __forceinline__ void householder_scalars(double x0, double tail, int 
   *tu = __shfl_sync(0xffffffffu, q, 0);
   *inv = __shfl_sync(0xffffffffu, q, 1);
 }
-// The same for FP32 entries, to within a few units of 2^-52 and in a third of
-// the dependent FP64 operations: with r = 1 / sqrt(sigma), |beta| = sigma r, tau
-// = 1 + |x0| r and 1 / |x0 - beta| = r / tau.  r and 1 / tau come from an FP32
-// start by one step of Halley's (third-order) iteration, which takes 2^-22 to
-// below 2^-60.  sigma is scaled to [1, 4) by its exponent: squares of FP32
-// entries are normal doubles; anything else (an infinity, a NaN) takes the
-// general form.
+// 1 / sqrt(s) of a normal s > 0 with an exponent within +-1000, to within a few
+// units of 2^-53: s is scaled to [1, 4) by its exponent and an FP32 start taken
+// through one step of Halley's (third-order) iteration, which takes 2^-22 to
+// below 2^-60 -- a third of the dependent FP64 operations of a square root and a
+// division, each of them some 100 cycles on this chip.
+__device__ __forceinline__ bool rsqrt_in_range(double s) {
+  const int E = (__double2hiint(s) >> 20) - 1023;  // s >= 0
+  return E >= -1000 && E <= 1000;
+}
+__device__ __forceinline__ double rsqrt_halley(double s) {
+  const int hi = __double2hiint(s), k = ((hi >> 20) - 1023) >> 1;
+  const double m = __hiloint2double(hi - 2 * k * (1 << 20), __double2loint(s));
+  const double r0 = (double)rsqrtf((float)m);
+  const double e = fma(-(m * r0), r0, 1.0);
+  const double r = fma(r0, e * fma(0.375, e, 0.5), r0);
+  return __hiloint2double(__double2hiint(r) - k * (1 << 20), __double2loint(r));  // r 2^-k
+}
+// The scalars for FP32 entries, to within a few units of 2^-52: with r = 1 /
+// sqrt(sigma), |beta| = sigma r, tau = 1 + |x0| r and 1 / |x0 - beta| = r / tau,
+// 1 / tau by one third-order step too.  Squares of FP32 entries are in range;
+// anything else (an infinity, a NaN) takes the general form.
 __device__ __forceinline__ void householder_scalars_f32(double x0, double tail, int lane, double* beta, double* tu, double* inv) {
-  const double sigma = fma(x0, x0, tail);
-  const int hi = __double2hiint(sigma), E = (hi >> 20) - 1023;  // sigma > 0
-  if (E < -1000 || E > 1000) {
+  const double sigma = fma(x0, x0, tail);  // > 0
+  if (!rsqrt_in_range(sigma)) {
     householder_scalars(x0, tail, lane, beta, tu, inv);
     return;
   }
-  const int k = E >> 1;
-  const double ss = __hiloint2double(hi - 2 * k * (1 << 20), __double2loint(sigma));
-  const double r0 = (double)rsqrtf((float)ss);
-  const double e = fma(-(ss * r0), r0, 1.0);
-  const double rs = fma(r0, e * fma(0.375, e, 0.5), r0);
-  const double r = __hiloint2double(__double2hiint(rs) - k * (1 << 20), __double2loint(rs));  // rs 2^-k
+  const double r = rsqrt_halley(sigma);
   const double alpha = sigma * r, t = fma(fabs(x0), r, 1.0);
   const double y0 = (double)(1.0f / (float)t);
   const double f = fma(-t, y0, 1.0);
@@ -383,6 +391,13 @@ __device__ __forceinline__ void householder_scalars_f32(double x0, double tail, 
   *beta = (x0 >= 0.0) ? -alpha : alpha;
   *tu = t;
   *inv = (x0 >= 0.0) ? r * y : -(r * y);
+}
+
+// An integer in the order of the doubles (both zeros alike): comparisons of
+// doubles take the FP64 pipe.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v + 0.0);
+  return b < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)b) : b;
 }
 
 __device__ __forceinline__ int ld_acquire_gpu(const int* p) {

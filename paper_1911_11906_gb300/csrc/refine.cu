@@ -110,10 +110,26 @@ __global__ void frob_norms(const double* S, int64_t lds, const double* R, int64_
 // without tiles write zeros, and reduce_segments adds the segments of each
 // entry in a fixed order.  Thread (row lane, column group w) reads coalesced
 // 256-byte column segments.  Block 256 = 32 x 8, grid 2 nt S.
+// Two matrices at once (blockIdx.y), each with its vector y, taken as x = y inv.
+struct PowerVecs {
+  double* y;      // 2 x n: y, then normalised as it is read
+  double* inv;    // 2: 1 / |y|
+  double* P;      // 2 x S x n, 2 x S x n: the segments' partial sums
+  double* Q;
+  double* part;   // 2 x ceil(n / 256): CTA sums of y^2
+  double* est;    // 2: |y|
+  unsigned* done; // 2: CTAs that have finished (0 between launches)
+};
 constexpr int kSymvSeg = 16;
-__global__ void __launch_bounds__(256) symv_segments(const double* M, int64_t ldm, int64_t n, const double* x,
-                                                     double* P, double* Q, int S) {
+__global__ void __launch_bounds__(256) symv_segments(const double* M0, const double* M1, int64_t ldm, int64_t n,
+                                                     PowerVecs v, int S) {
   __shared__ double red[8][33];
+  const int which = blockIdx.y;
+  const double* M = which ? M1 : M0;
+  const double* x = v.y + which * n;
+  const double inv = v.inv[which];
+  double* P = v.P + (int64_t)which * S * n;
+  double* Q = v.Q + (int64_t)which * S * n;
   const int64_t nt = (n + 31) / 32;
   const int tx = threadIdx.x & 31, w = threadIdx.x >> 5;
   int64_t b = blockIdx.x;
@@ -138,7 +154,7 @@ __global__ void __launch_bounds__(256) symv_segments(const double* M, int64_t ld
       double t = 0.0;
 #pragma unroll
       for (int q = 0; q < 8; ++q) t += red[q][tx];
-      P[(int64_t)seg * n + gi] = t;
+      P[(int64_t)seg * n + gi] = t * inv;
     }
   } else {
     const int64_t J = strip;
@@ -156,58 +172,62 @@ __global__ void __launch_bounds__(256) symv_segments(const double* M, int64_t ld
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const double v = warp_sum(acc[q]);
+      const double cs = warp_sum(acc[q]);
       const int64_t gj = J * 32 + w * 4 + q;
-      if (tx == 0 && gj < n) Q[(int64_t)seg * n + gj] = v;
+      if (tx == 0 && gj < n) Q[(int64_t)seg * n + gj] = cs * inv;
     }
   }
 }
-// y_i = sum_s P[s n + i] + sum_s Q[s n + i] - shift_i x_i (into P's first
-// segment), and each CTA's sum of y_i^2 into part[blockIdx.x].  Block 256.
-__global__ void reduce_segments(double* P, const double* Q, int S, const double* shift, const double* x,
-                                int64_t n, double* part) {
+// y_i = sum_s P[s n + i] + sum_s Q[s n + i] - shift_i x_i and each CTA's sum of
+// y_i^2; the CTA that finishes last adds those in order: |y| into est, 1 / |y|
+// into inv.  (One launch for both matrices and no third kernel: an iteration
+// was six launches, which bound small problems.)  Block 256, grid (nb, 2).
+__global__ void __launch_bounds__(256) reduce_segments(PowerVecs v, int S, const double* shift0, int64_t n) {
   __shared__ double red[8];
+  __shared__ int s_last;
+  const int which = blockIdx.y;
+  const double* P = v.P + (int64_t)which * S * n;
+  const double* Q = v.Q + (int64_t)which * S * n;
+  double* yv = v.y + which * n;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double y2 = 0.0;
   if (i < n) {
     double y = 0.0;
     for (int q = 0; q < S; ++q) y += P[(int64_t)q * n + i];
     for (int q = 0; q < S; ++q) y += Q[(int64_t)q * n + i];
-    y -= shift ? shift[i] * x[i] : 0.0;
-    P[i] = y;
+    if (which == 0) y -= shift0[i] * (yv[i] * v.inv[0]);
+    yv[i] = y;
     y2 = y * y;
   }
   y2 = warp_sum(y2);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = y2;
   __syncthreads();
+  double* part = v.part + (int64_t)which * gridDim.x;
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < 8; ++w) t += red[w];
-    part[blockIdx.x] = t;
-  }
-}
-// |y| from the CTAs' partial sums (added in order), x = y / |y|, *est = |y|.
-__global__ void normalize_parts(const double* y, const double* part, int nparts, int64_t n, double* x, double* est) {
-  __shared__ double nrm_sh;
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int q = 0; q < nparts; ++q) t += part[q];
-    nrm_sh = sqrt(t);
+    __stcg(part + blockIdx.x, t);
+    __threadfence();
+    s_last = atomicAdd(v.done + which, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  const double nrm = nrm_sh;
-  const double inv = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) x[i] = y[i] * inv;
-  if (threadIdx.x == 0) *est = nrm;
+  if (!s_last || threadIdx.x != 0) return;
+  __threadfence();
+  double t = 0.0;
+  for (unsigned q = 0; q < gridDim.x; ++q) t += __ldcg(part + q);
+  const double nrm = sqrt(t);
+  v.est[which] = nrm;
+  v.inv[which] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+  v.done[which] = 0;
 }
 
-
-__global__ void start_vec(double* x, int64_t n) {
+__global__ void start_vec(double* x, int64_t n, double* inv) {  // both vectors
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < 2) inv[i] = 1.0;
   if (i < n) {
     // deterministic, sign-varying start with components in every direction
     const uint64_t h = (uint64_t)(i + 1) * 0x9E3779B97F4A7C15ull;
-    x[i] = ((double)(h >> 11) * (1.0 / 9007199254740992.0) - 0.5) / sqrt((double)n);
+    x[i] = x[n + i] = ((double)(h >> 11) * (1.0 / 9007199254740992.0) - 0.5) / sqrt((double)n);
   }
 }
 
@@ -439,21 +459,22 @@ __global__ void add_correction(double* X, int64_t ldx, const float* P, int64_t n
 // memory, the chunk counts added into rank (zeroed before; integer sums, so
 // the order of the additions does not matter).  Block 256, grid
 // (ceil(n / 256), ceil(n / kRankChunk)).
-constexpr int kRankChunk = 1024;
+// The comparisons are of integer keys (256 chunks of 1024 FP64 comparisons took
+// 154 us whatever n, all of it the FP64 pipe's).
+constexpr int kRankChunk = 256;
 __global__ void __launch_bounds__(256) ranks(const double* lt, int64_t n, int* rank) {
-  __shared__ double sl[kRankChunk];
+  __shared__ long long sl[kRankChunk];
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t j0 = (int64_t)blockIdx.y * kRankChunk;
   const int64_t j1 = (j0 + kRankChunk < n) ? j0 + kRankChunk : n;
-  for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) sl[j - j0] = lt[j];
+  for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) sl[j - j0] = order_key(lt[j]);
   __syncthreads();
   if (i >= n) return;
-  const double v = lt[i];
+  const long long v = order_key(lt[i]);
   int r = 0;
-  for (int64_t j = j0; j < j1; ++j) {
-    const double u = sl[j - j0];
-    r += (u < v) || (u == v && j < i);
-  }
+  const int m = (int)(j1 - j0), eq = (int)((i - j0 < 0) ? 0 : (i - j0 < m ? i - j0 : m));  // j < i count when equal
+  for (int j = 0; j < eq; ++j) r += sl[j] <= v;
+  for (int j = eq; j < m; ++j) r += sl[j] < v;
   if (r) atomicAdd(rank + i, r);
 }
 
@@ -888,7 +909,8 @@ size_t refine_ws(const fraclap_ctx* ctx, int64_t n) {
   ar.take<int>(n);             // cluster id per sorted position
   ar.take<int>(n + 1);         // big-cluster marks + flag
   ar.take<int>(2 * n + 2);     // cluster list + count
-  ar.take<double>(8);          // norms, delta
+  ar.take<double>(8);          // norms, delta, 1 / |y|
+  ar.take<unsigned>(2);        // finished CTAs of the norm reductions
   const int64_t cmax = std::min<int64_t>(n, kMaxBigCluster);
   ar.take<double>(4 * cmax * cmax + cmax);
   ar.take<double>(small_cluster_doubles(n));
@@ -912,6 +934,7 @@ int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t
   int* bigm = ar->take<int>(n + 1);
   int* clist = ar->take<int>(2 * n + 2);
   double* scal = ar->take<double>(8);
+  unsigned* done = ar->take<unsigned>(2);
   ctx->refine_stats.clear();
   const int64_t cmax = std::min<int64_t>(n, kMaxBigCluster);
   double* cbuf = ar->take<double>(4 * cmax * cmax + cmax);
@@ -926,6 +949,7 @@ int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t
   using D32 = GemmDescT<float>;
   bool converged = false;
   StageSpan span(ctx, st);
+  FL_CUDA(ctx, cudaMemsetAsync(done, 0, 2 * sizeof(unsigned), st));
   for (int it = 0; it < iters && !converged; ++it) {
     // AX = A X
     span.start(kStageRefineNorms);
@@ -960,25 +984,25 @@ int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t
     count_launch(ctx);
     gershgorin<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(n, rowptr, val, nA);
     count_launch(ctx);
-    {  // 2-norm estimates of S - diag(l) and R (power iteration)
-      double* xv = ls;              // reuse: n doubles
-      double* yv = AX;              // reuse: first n doubles
-      for (int which = 0; which < 2; ++which) {
-        const double* M = which == 0 ? S : R;
-        const double* shift = which == 0 ? lt : nullptr;
-        start_vec<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(xv, n);
-        count_launch(ctx);
-        const int64_t nt = cdiv(n, 32);
-        const int S = (int)cdiv(nt, kSymvSeg);
-        const unsigned nb = (unsigned)cdiv(n, 256);
-        double* yc = AX + (int64_t)S * n;     // the segments' partial sums: 2 S n doubles of the n x n scratch
-        double* part = yc + (int64_t)S * n;  // nb CTA sums of y^2
-        for (int pit = 0; pit < 12; ++pit) {
-          symv_segments<<<(unsigned)(2 * nt * S), 256, 0, st>>>(M, n, n, xv, yv, yc, S);
-          reduce_segments<<<nb, 256, 0, st>>>(yv, yc, S, shift, xv, n, part);
-          normalize_parts<<<1, 1024, 0, st>>>(yv, part, (int)nb, n, xv, scal + 4 + which);
-          for (int q = 0; q < 3; ++q) count_launch(ctx);
-        }
+    {  // 2-norm estimates of S - diag(l) and R (power iteration), both at once
+      const int64_t nt = cdiv(n, 32);
+      const int Sg = (int)cdiv(nt, kSymvSeg);
+      const unsigned nb = (unsigned)cdiv(n, 256);
+      // in the n x n scratch of A X: 2 n + 4 Sg n + 2 nb doubles
+      PowerVecs pv;
+      pv.y = AX;
+      pv.P = pv.y + 2 * n;
+      pv.Q = pv.P + 2 * (int64_t)Sg * n;
+      pv.part = pv.Q + 2 * (int64_t)Sg * n;
+      pv.est = scal + 4;
+      pv.inv = scal + 6;
+      pv.done = done;
+      start_vec<<<nb, 256, 0, st>>>(pv.y, n, pv.inv);
+      count_launch(ctx);
+      for (int pit = 0; pit < 12; ++pit) {
+        symv_segments<<<dim3((unsigned)(2 * nt * Sg), 2), 256, 0, st>>>(S, R, n, n, pv, Sg);
+        reduce_segments<<<dim3(nb, 2), 256, 0, st>>>(pv, Sg, lt, n);
+        for (int q = 0; q < 2; ++q) count_launch(ctx);
       }
     }
     cluster_threshold<<<1, 1, 0, st>>>(scal, scal + 4, nA, delta);

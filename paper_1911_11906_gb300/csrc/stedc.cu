@@ -141,14 +141,25 @@ __global__ void dc_leaf(const double* D, const double* e, int64_t n, int L, doub
           const double mu = c - bb * bb / (delta + (delta >= 0.0 ? rr : -rr));
           double x = d[l] - mu, z = ee[l];
           for (int k = l; k < hi_i; ++k) {
-            const double r = hypot(x, z);
-            double cc = 1.0, sn = 0.0;
-            if (r != 0.0) { cc = x / r; sn = z / r; }
+            // the rotation's chain bounds a leaf: one reciprocal root instead of
+            // a hypot and two divisions, unless x^2 + z^2 leaves the range
+            const double r2 = fma(x, x, z * z);
+            double r, cc = 1.0, sn = 0.0;
+            if (rsqrt_in_range(r2)) {
+              const double ri = rsqrt_halley(r2);
+              r = r2 * ri;
+              cc = x * ri;
+              sn = z * ri;
+            } else {
+              r = hypot(x, z);
+              if (r != 0.0) { cc = x / r; sn = z / r; }
+            }
             if (k > l) ee[k - 1] = r;
             const double dk = d[k], dk1 = d[k + 1], ek = ee[k];
-            d[k] = cc * cc * dk + 2.0 * cc * sn * ek + sn * sn * dk1;
-            d[k + 1] = sn * sn * dk - 2.0 * cc * sn * ek + cc * cc * dk1;
-            ee[k] = cc * sn * (dk1 - dk) + (cc * cc - sn * sn) * ek;
+            const double c2 = cc * cc, s2 = sn * sn, cs = cc * sn, t = 2.0 * cs * ek;
+            d[k] = c2 * dk + t + s2 * dk1;
+            d[k + 1] = s2 * dk - t + c2 * dk1;
+            ee[k] = cs * (dk1 - dk) + (c2 - s2) * ek;
             sc[w][k] = cc;
             ss[w][k] = sn;
             if (k + 1 < hi_i) {
@@ -648,12 +659,6 @@ __global__ void __launch_bounds__(128) dc_gather_kept(DcBuf<T> B, int64_t nmax) 
   const int64_t q1 = (q0 + kGatherCols < inf.K) ? q0 + kGatherCols : inf.K;
 #pragma unroll 4
   for (int64_t q = q0; q < q1; ++q) Q[r + q * nm] = Wq[r + (int64_t)kept[q] * nm];
-}
-
-// An integer in the order of the doubles (both zeros alike).
-__device__ __forceinline__ long long order_key(double v) {
-  const long long b = __double_as_longlong(v + 0.0);
-  return b < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)b) : b;
 }
 
 // Ranks of the merged spectrum, as a sequential merge of the survivors (in
