@@ -340,7 +340,8 @@ int fraclap_sgemm(fraclap_ctx* ctx, int trans_a, int trans_b, int form, int64_t 
  * carries its CSR; band width 32) of its dense A into
  * lambda_dev / V_dev and, when k > 0, the spectral apply of its k pairs into
  * U_dev (as frac_apply; Sec. II eq. poisson_solution).  The problems are
- * spread over `workers` concurrent streams (0: 16), each with its own share
+ * spread over `workers` concurrent streams (0: 16; never more than the device
+ * has hardware queues: 8, or CUDA_DEVICE_MAX_CONNECTIONS), each with its own share
  * of the SMs and a context-owned workspace sized for its largest problem;
  * the caller's stream waits for all of them.  probs is a host array; every
  * pointer in it is a device pointer owned by the caller, and distinct
@@ -584,9 +585,10 @@ int fraclap_partition_spectrum(fraclap_ctx* ctx, int64_t n, const int64_t* rowpt
  *    tile, 128, 192 or 256 (rows are 128; outputs of at most 128 columns
  *    always take 128) [256].
  *  FRACLAP_SCHED_Q2_PARTS: at half-bandwidth 64, the lanes that share one
- *    column's window of the stage-2 back-transformation: 4, 8 or 16 (16, 8 or
- *    4 rows per lane; more parts give more warps over the same columns; FP64
- *    takes 8 when asked for 4), or 0 for the default 8 [0].
+ *    column's window of the stage-2 back-transformation, one reflector after
+ *    the other: 4, 8 or 16 (16, 8 or 4 rows per lane; more parts give more
+ *    warps over the same columns; FP64 takes 8 when asked for 4), or 0 for
+ *    blocks of reflectors, which is faster at every size [0].
  *  FRACLAP_SCHED_OZAKI_CLUSTER: CTAs of the slice-product kernel per thread-
  *    block cluster, 1 or 2: the two CTAs of a cluster take consecutive tile
  *    rows of one tile column and share its B tile through TMA multicast,
