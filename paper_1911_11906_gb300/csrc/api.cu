@@ -88,7 +88,6 @@ struct EigWork {
   double* d;      // n
   double* e;      // n
   T* W1;          // b x n
-  T* W2;          // b x n
   Stage1T<T> s1;
   Stage2T<T> s2;
 };
@@ -101,7 +100,6 @@ int eig_take(Arena* ar, const fraclap_ctx* ctx, int64_t n, EigWork<T>* w) {
   w->d = ar->take<double>(n);
   w->e = ar->take<double>(n);
   w->W1 = ar->take<T>((int64_t)b * n);
-  w->W2 = ar->take<T>((int64_t)b * n);
   stage1_take<T>(ar, n, b, ctx->sm_count, &w->s1);
   stage2_take<T>(ar, n, b, &w->s2);
   return 0;
@@ -172,7 +170,7 @@ int back_transform(fraclap_ctx* ctx, int64_t n, EigWork<T>* w, T* Z, int64_t ldz
   }
   {
     StageTimer t(ctx, kStageBackQ1, st);
-    FL_TRY(q1_apply_run<T>(ctx, &w->s1, n, b, Z, ldz, n, w->W1, w->W2, st));
+    FL_TRY(q1_apply_run<T>(ctx, &w->s1, n, b, Z, ldz, n, w->W1, st));
   }
   return 0;
 }

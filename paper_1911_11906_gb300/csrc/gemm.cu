@@ -606,7 +606,9 @@ int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st
       FL_CUDA(ctx, cudaGetLastError());
       return 0;
     }
-    if (MODE != kGemmLowerC && d.K2 == 0 && sg_narrow(d.M, d.N))
+    // (and small ones with a long sum, unless the caller splits it)
+    const bool deep = split_k <= 1 && d.K >= 512 && std::max(d.M, d.N) <= 128;
+    if (MODE != kGemmLowerC && d.K2 == 0 && (sg_narrow(d.M, d.N) || deep))
       return d.M >= d.N ? launch_sg_narrow<128, 64, TA, TB, MODE>(ctx, d, st)
                         : launch_sg_narrow<64, 128, TA, TB, MODE>(ctx, d, st);
   }

@@ -250,11 +250,10 @@ int gemm_batched(fraclap_ctx* ctx, bool ta, bool tb, const GemmDescT<T>* d_descs
 template <class T>
 struct Stage1T {
   T* Vstore;         // sum_j m_j * b: explicit V of every panel
-  T* Tstore;         // npanel * b * b
+  T* Tf;             // b * b, the panel in work
   double* tau;       // npanel * b
-  T* XT;             // n * b
+  T* XTstore;        // the same of V T
   T* X;              // n * b
-  T* Y;              // b * b
   T* Mm;             // b * b
   double* gram;      // b * b
   double* partials;  // 2 * G * 2b
@@ -270,7 +269,7 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
               cudaStream_t st);
 template <class T>
 int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, int64_t ldz,
-                 int64_t ncols, T* W1, T* W2, cudaStream_t st);
+                 int64_t ncols, T* W1, cudaStream_t st);
 
 // Stage 2 (band -> tridiagonal) workspace: the bulge-chasing reflectors.
 template <class T>

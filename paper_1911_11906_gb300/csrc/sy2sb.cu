@@ -7,7 +7,7 @@
 // column, added by FP64 atomics, from which the reflector and its effect on
 // the panel follow).  The
 // trailing matrix is then updated as A22 <- Q^T A22 Q = A22 - W V^T - V W^T
-// with X = A22 (V T), W = X - 1/2 V (T^T V^T X), through the GEMM engine
+// with X = A22 (V T), W = X - 1/2 V ((V T)^T X), through the GEMM engine
 // (symmetric A22 read from its lower triangle; lower-triangular rank-2b
 // update).  FP64 throughout; the Householder norms and scalings stay FP64.
 #include <cooperative_groups.h>
@@ -401,11 +401,10 @@ int stage1_take(Arena* ar, int64_t n, int b, int G, Stage1T<T>* s) {
   s->vtotal = 0;
   for (int64_t j = 0; j < s->npanel; ++j) s->vtotal += (n - j * b - b) * b;
   s->Vstore = ar->take<T>(s->vtotal);
-  s->Tstore = ar->take<T>(s->npanel * b * b);
+  s->Tf = ar->take<T>((int64_t)b * b);
   s->tau = ar->take<double>(s->npanel * b);
-  s->XT = ar->take<T>(n * b);
+  s->XTstore = ar->take<T>(s->vtotal);
   s->X = ar->take<T>(n * b);
-  s->Y = ar->take<T>((int64_t)b * b);
   s->Mm = ar->take<T>((int64_t)b * b);
   s->gram = ar->take<double>((int64_t)b * b);
   s->partials = ar->take<double>(3 * 2 * (int64_t)b);
@@ -485,7 +484,7 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
     const int64_t j0 = p * b, m = n - j0 - b;
     T* P = Aw + (j0 + b) + j0 * lda;
     T* V = s->Vstore + voff;
-    T* Tf = s->Tstore + p * b * b;
+    T* Tf = s->Tf;
     const int crc = panel_cluster(ctx, P, lda, m, b, V, s->tau + p * b, Tf, st);
     if (crc < 0) return crc;
     if (crc == 0) {
@@ -517,19 +516,19 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
     }
     T* A22 = Aw + (j0 + b) + (j0 + b) * lda;
     using D = GemmDescT<T>;
-    // XT = V T  (m x b)
-    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, Tf, b, s->XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
+    // XT = V T  (m x b), kept for the back-transformation
+    T* XT = s->XTstore + voff;
+    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, Tf, b, XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
     // X = A22 XT (A22 symmetric, lower triangle); narrow products share their
     // long sums by themselves, the TF32 route splits them into a zeroed X
     const bool tf32 = sizeof(T) == 4 && ctx->tc_scratch;
     if (tf32) FL_CUDA(ctx, cudaMemsetAsync(s->X, 0, sizeof(T) * m * b, st));
-    FL_TRY(gemm<T>(ctx, false, false, kGemmSymA, D{m, b, m, A22, lda, s->XT, m, s->X, m, nullptr, 0, nullptr, 0, 0, 1.0, tf32 ? 1.0 : 0.0}, tf32 ? (int)std::min<int64_t>(cdiv(m, 1024), 16) : 1, st));
-    // Y = V^T X  (b x b), split over the long dimension (FP64: by itself)
-    const bool split = sizeof(T) == 4;
-    if (split) FL_CUDA(ctx, cudaMemsetAsync(s->Y, 0, sizeof(T) * b * b, st));
-    FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{b, b, m, V, m, s->X, m, s->Y, b, nullptr, 0, nullptr, 0, 0, 1.0, split ? 1.0 : 0.0}, split ? (int)cdiv(m, 256) : 1, st));
-    // Mm = T^T Y
-    FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{b, b, b, Tf, b, s->Y, b, s->Mm, b, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
+    FL_TRY(gemm<T>(ctx, false, false, kGemmSymA, D{m, b, m, A22, lda, XT, m, s->X, m, nullptr, 0, nullptr, 0, 0, 1.0, tf32 ? 1.0 : 0.0}, tf32 ? (int)std::min<int64_t>(cdiv(m, 1024), 16) : 1, st));
+    // Mm = XT^T X  (b x b): narrow products share the long sum over a cluster's
+    // eight CTAs; past 4096 rows more CTAs with atomics are faster in FP32
+    const bool split = sizeof(T) == 4 && m > 4096;
+    if (split) FL_CUDA(ctx, cudaMemsetAsync(s->Mm, 0, sizeof(T) * b * b, st));
+    FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{b, b, m, XT, m, s->X, m, s->Mm, b, nullptr, 0, nullptr, 0, 0, 1.0, split ? 1.0 : 0.0}, split ? (int)cdiv(m, 256) : 1, st));
     // W = X - 1/2 V Mm  (in X)
     FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, s->Mm, b, s->X, m, nullptr, 0, nullptr, 0, 0, -0.5, 1.0}, 1, st));
     // A22 -= W V^T + V W^T  (lower triangle)
@@ -543,25 +542,24 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
 }
 
 // Back-transformation by Q1 = Q_0 Q_1 ... Q_{p-1}: Z <- Q1 Z (n x ncols).
-// Applied from the last panel to the first: Z(rows_j, :) -= V_j (T_j (V_j^T Z(rows_j, :))).
+// Applied from the last panel to the first: Z(rows_j, :) -= (V_j T_j) (V_j^T Z(rows_j, :)),
+// V_j T_j as the reduction formed it: two products a panel.
 template <class T>
 int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, int64_t ldz,
-                 int64_t ncols, T* W1, T* W2, cudaStream_t st) {
+                 int64_t ncols, T* W1, cudaStream_t st) {
   int64_t voff = s->vtotal;
   using D = GemmDescT<T>;
   if (sizeof(T) == 4 && ctx->tc_scratch) {
-    // tensor-core shapes (tall and wide products): W1^T = Z_r^T V (n x b),
-    // W2^T = W1^T T^T, Z_r -= V W2 -- the same three products, transposed
+    // tensor-core shapes (tall and wide products): W1^T = Z_r^T V (n x b), Z_r -=
+    // (V T) W1 -- the same products, transposed
     for (int64_t p = s->npanel - 1; p >= 0; --p) {
       const int64_t j0 = p * b, m = n - j0 - b;
       voff -= m * b;
       const T* V = s->Vstore + voff;
-      const T* Tf = s->Tstore + p * b * b;
       T* Zr = Z + (j0 + b);
       FL_CUDA(ctx, cudaMemsetAsync(W1, 0, sizeof(T) * b * ncols, st));
       FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{ncols, b, m, Zr, ldz, V, m, W1, ncols, nullptr, 0, nullptr, 0, 0, 1.0, 1.0}, (int)std::min<int64_t>(cdiv(m, 1024), 16), st));
-      FL_TRY(gemm<T>(ctx, false, true, kGemmPlain, D{ncols, b, b, W1, ncols, Tf, b, W2, ncols, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
-      FL_TRY(gemm<T>(ctx, false, true, kGemmPlain, D{m, ncols, b, V, m, W2, ncols, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
+      FL_TRY(gemm<T>(ctx, false, true, kGemmPlain, D{m, ncols, b, s->XTstore + voff, m, W1, ncols, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
     }
     return 0;
   }
@@ -569,14 +567,11 @@ int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, 
     const int64_t j0 = p * b, m = n - j0 - b;
     voff -= m * b;
     const T* V = s->Vstore + voff;
-    const T* Tf = s->Tstore + p * b * b;
     T* Zr = Z + (j0 + b);
     // W1 = V^T Zr  (b x ncols)
     FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{b, ncols, m, V, m, Zr, ldz, W1, b, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
-    // W2 = T W1
-    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{b, ncols, b, Tf, b, W1, b, W2, b, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
-    // Zr -= V W2
-    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, ncols, b, V, m, W2, b, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
+    // Zr -= (V T) W1
+    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, ncols, b, s->XTstore + voff, m, W1, b, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
   }
   return 0;
 }
@@ -585,7 +580,7 @@ template int stage1_take<double>(Arena*, int64_t, int, int, Stage1T<double>*);
 template int stage1_take<float>(Arena*, int64_t, int, int, Stage1T<float>*);
 template int sy2sb_run<double>(fraclap_ctx*, double*, int64_t, int64_t, int, double*, Stage1T<double>*, cudaStream_t);
 template int sy2sb_run<float>(fraclap_ctx*, float*, int64_t, int64_t, int, float*, Stage1T<float>*, cudaStream_t);
-template int q1_apply_run<double>(fraclap_ctx*, const Stage1T<double>*, int64_t, int, double*, int64_t, int64_t, double*, double*, cudaStream_t);
-template int q1_apply_run<float>(fraclap_ctx*, const Stage1T<float>*, int64_t, int, float*, int64_t, int64_t, float*, float*, cudaStream_t);
+template int q1_apply_run<double>(fraclap_ctx*, const Stage1T<double>*, int64_t, int, double*, int64_t, int64_t, double*, cudaStream_t);
+template int q1_apply_run<float>(fraclap_ctx*, const Stage1T<float>*, int64_t, int, float*, int64_t, int64_t, float*, cudaStream_t);
 
 }  // namespace fraclap

@@ -10,7 +10,8 @@ import torch
 pytestmark = pytest.mark.gpu
 
 SHAPES = [(1, 1, 1), (127, 129, 15), (128, 64, 16), (129, 65, 17), (64, 128, 400), (63, 1000, 513), (1000, 33, 2049),
-          (256, 256, 161), (257, 300, 8), (300, 259, 160), (700, 513, 333), (130, 127, 1300)]
+          (256, 256, 161), (257, 300, 8), (300, 259, 160), (700, 513, 333), (130, 127, 1300),
+          (32, 32, 511), (64, 64, 512), (33, 100, 2051), (1, 5, 4000)]
 
 
 def _mat(rows, cols, pad, g):
