@@ -22,7 +22,7 @@ namespace cg = cooperative_groups;
 constexpr int PQR_NT = 256;
 constexpr int kClusterMax = 16;                  // CTAs of the cluster panel kernel (non-portable above 8)
 constexpr int kPanelClusterSmemMax = 217 * 1024;  // panel rows one CTA of the cluster holds
-constexpr int64_t kPanelFp64Rows = 1200;          // FP64 panels of the cluster kernel
+constexpr int64_t kPanelFp64Rows = 4096;          // FP64 panels of the cluster kernels
 constexpr int kPanelSmemMax = 180 * 1024;  // largest panel slice one CTA holds
 
 // Cooperative panel QR.  P: m x bw panel (ld ldp) in the working matrix.
@@ -167,6 +167,28 @@ panel_qr_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t ldv,
   for (int p = tid; p < bw * bw; p += PQR_NT) Tf[p] = (T)Ts[p];
 }
 
+// Columns j, j + step, ... of T (a warp): the inverse of diag(1/tau) +
+// strictly-upper(G), T(k, j) = -tau_k sum_{k < q <= j} G(k, q) T(q, j) from k = j
+// down, in FP64; G(i, k) at 65 k + i.
+template <class TG, class T>
+__device__ __forceinline__ void panel_t_columns(const TG* G, const double* s_tau, int bw, int j, int step, int lane, T* Tf) {
+  for (; j < bw; j += step) {
+    double a0 = 0.0, a1 = 0.0, t0 = 0.0, t1 = 0.0;  // rows lane and lane + 32: sum so far, T(., j)
+    for (int k = j; k >= 0; --k) {
+      const double sum = __shfl_sync(0xffffffffu, (k < 32) ? a0 : a1, k & 31);
+      const double x = (k == j) ? s_tau[j] : -s_tau[k] * sum;
+      if (lane == (k & 31)) {
+        if (k < 32) t0 = x;
+        else t1 = x;
+      }
+      if (lane < k) a0 = fma((double)G[k * 65 + lane], x, a0);
+      if (lane + 32 < k) a1 = fma((double)G[k * 65 + lane + 32], x, a1);
+    }
+    if (lane < bw) Tf[lane + j * bw] = (T)t0;
+    if (lane + 32 < bw) Tf[lane + 32 + j * bw] = (T)t1;
+  }
+}
+
 // The same panel factorisation on one thread-block cluster (up to 16 CTAs)
 // when the panel fits in their shared memory, with T of the compact WY form.
 // Per column, every CTA's partial dot products and the pivot row are written
@@ -179,10 +201,8 @@ panel_qr_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t ldv,
 // and Van Loan's form of H_1 ... H_bw = I - V T V^T), column by column, dealt to
 // the CTAs, a warp each: T(k, j) = -tau_k sum_{k < q <= j} G(k, q) T(q, j) from
 // k = j down, in FP64, which holds for tau_k = 0 as well.
-// Bound: the chain of a column (dots, barrier, FP64 scalars, update).  GB300,
-// with the Gram product and T's kernel it replaces, a panel of FP32 b = 64: m up
-// to 7735 some 520 -> 418 us, up to 2753 400 -> 257 us; the band reduction at n =
-// 2753 24.8 -> 19.0 ms; FP64 b = 32, n = 779 10.9 -> 7.6 ms (165 us a panel).
+// Bound: the chain of a column (dots, barrier, FP64 scalars, update), some 6 us
+// at 480 rows a CTA.  It takes the panels past the register kernel's rows.
 // G, a CTA's part and the FP64 sum, in the place of V
 template <class T>
 constexpr size_t panel_gram_smem() {
@@ -363,21 +383,267 @@ panel_qr_cluster_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t l
     for (int q = 0; q < CS; ++q) cluster.map_shared_rank(Gd, q)[k * 65 + i] = (double)s;
   }
   cluster.sync();
-  for (int j = rank + CS * warp; j < bw; j += CS * nwarp) {
-    double a0 = 0.0, a1 = 0.0, t0 = 0.0, t1 = 0.0;  // rows lane and lane + 32: sum so far, T(., j)
-    for (int k = j; k >= 0; --k) {
-      const double sum = __shfl_sync(0xffffffffu, (k < 32) ? a0 : a1, k & 31);
-      const double x = (k == j) ? s_tau[j] : -s_tau[k] * sum;
-      if (lane == (k & 31)) {
-        if (k < 32) t0 = x;
-        else t1 = x;
-      }
-      if (lane < k) a0 = fma(Gd[k * 65 + lane], x, a0);
-      if (lane + 32 < k) a1 = fma(Gd[k * 65 + lane + 32], x, a1);
+  panel_t_columns<double>(Gd, s_tau, bw, rank + CS * warp, CS * nwarp, lane, Tf);
+}
+
+// The same factorisation with the panel in registers, for panels of at most 32 R
+// rows a CTA: warp w of a CTA holds its rows of columns w, w + NW, ..., lane l
+// rows l + 32 i, so that a column's step reads only the reflector from shared
+// memory.  A step: every column's dot product with the rows of p_c below the
+// pivot goes to all CTAs with the pivot row (gathered first: one row of 16-byte
+// stores for each CTA; single values cost some 2 clocks each), one cluster
+// barrier, then
+//   j = c: sum of squares, the reflector's scalars (FP64, one warp);
+//   j > c: w_j = tau (p_j(c) + (p_c^T p_j) / (x0 - beta)), p_j -= w_j v;
+//   j < c: G(j, c) = V_j(c) + (p_c^T V_j) / (x0 - beta), the Gram matrix of T.
+// Bound: the chain of that step.  GB300, FP32, b = 64, clocks a column at m = 2551
+// (5111): dots 680 (820), exchange and barrier 1340 (1350), scalars 2230 (2280), w
+// 430 (760), update 1050 (1000), in all some 190 (209) us a panel with T and the
+// loads; the kernel on shared memory took 257 and 418.  The band reduction at n =
+// 1114 7.0 -> 5.1 ms, 2753 15.6 -> 11.1, 7735 78.2 -> 53.9, FP64 779 7.2 -> 5.8.
+// A warp's FP64 operation holds the SM's FP64 pipe for some 16 clocks, so only
+// the scalars and w are FP64 there; FP32 panels' sums over the CTAs are carried
+// exactly in pairs of FP32 values.
+template <class T>
+constexpr int kPanelRegsWarps = sizeof(T) == 8 ? 8 : 16;
+// s + v = s' + e exactly (Knuth)
+__device__ __forceinline__ void two_sum(float& s, float v, float& e) {
+  const float t = __fadd_rn(s, v), z = __fadd_rn(t, -s);
+  e = __fadd_rn(e, __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(v, -z)));
+  s = t;
+}
+__device__ __forceinline__ void two_sum(double& s, double v, double&) { s += v; }
+
+// The sum of the first 16 lanes' values >= 0 (the others hold 0), in every lane.  FP32 values are
+// added as integers in units of 2^-59 of the largest one's exponent and rounded
+// once: no FP64 operation, each of which costs a lone warp some 100 clocks.
+__device__ __forceinline__ double warp_sum_nonneg(double v) {
+#pragma unroll
+  for (int o = 8; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return __shfl_sync(0xffffffffu, v, 0);
+}
+__device__ __forceinline__ double warp_sum_nonneg(float v) {
+  const unsigned bits = __float_as_uint(v) & 0x7fffffffu;
+  const unsigned top = __reduce_max_sync(0xffffffffu, bits);
+  if (top >= 0x7f800000u) return warp_sum_nonneg((double)v);  // an infinity or a NaN
+  const int ex = (int)(bits >> 23), em = (int)(top >> 23);
+  const unsigned man = (bits & 0x7fffffu) | (ex > 0 ? 0x800000u : 0u);
+  const int drop = max(em, 1) - max(ex, 1);  // man 2^(max(ex, 1) - 150)
+  const unsigned long long u = drop < 59 ? ((unsigned long long)man << 35) >> drop : 0ull;
+  // values below 2^59, in pieces whose sums fit 32 bits
+  const unsigned long long a = __reduce_add_sync(0xffffffffu, (unsigned)(u & 0x7ffffffu));
+  const unsigned long long b = __reduce_add_sync(0xffffffffu, (unsigned)((u >> 27) & 0x7ffffffu));
+  const unsigned long long c = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 54));
+  const unsigned long long total = a + (b << 27) + (c << 54);  // < 2^64
+  if (total == 0) return 0.0;
+  // total 2^(max(em, 1) - 185) to 53 bits, nearest even, without the FP64 pipe
+  const int z = __clzll((long long)total);
+  const unsigned long long norm = total << z, rem = norm & 0x7ff;
+  unsigned long long d = (norm >> 11) + ((unsigned long long)(1022 + 63 - z + max(em, 1) - 185) << 52);
+  if (rem > 0x400 || (rem == 0x400 && (d & 1))) ++d;  // a carry moves to the next exponent
+  return __longlong_as_double((long long)d);
+}
+
+template <class T, int Q, int R>
+__global__ void __launch_bounds__(32 * kPanelRegsWarps<T>, 1)
+panel_qr_regs_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t ldv, double* tau, T* Tf,
+                     int rows_per_cta) {
+  constexpr int NW = kPanelRegsWarps<T>, NT = 32 * NW;
+  constexpr int GL = NW / 4;              // lanes that share a later column's sum, on warps 1 .. 2 GL
+  constexpr int EW = 2 * GL + 1;          // the earlier columns' sums, on warps EW and EW + 1
+  static_assert(NW * Q <= 64 && (Q & (Q - 1)) == 0 && EW + 2 <= NW, "columns and warps");
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* G = reinterpret_cast<T*>(smem_raw);  // 64 x 65: G(j, c) at 65 c + j
+  __shared__ T col[2][32 * R];            // this CTA's rows of the column in work
+  __shared__ __align__(16) T part[2][64];               // this CTA's dot products, the pivot row
+  __shared__ __align__(16) T recv[2][kClusterMax][64];  // every CTA's
+  __shared__ __align__(16) T piv[2][64];
+  __shared__ T g[2][64];                  // their sums
+  __shared__ T sw[64];
+  __shared__ double s_tau[64];
+  __shared__ double s_coef[3];            // beta, tau, 1 / (x0 - beta)
+  __shared__ T s_work[3];                 // the last in two parts, beta
+  __shared__ int s_any;                   // tau != 0
+  const int rank = (int)cluster.block_rank(), CS = (int)cluster.num_blocks();
+  const int64_t rb = (int64_t)rank * rows_per_cta;
+  const int nr = (int)((rb + rows_per_cta < m) ? rows_per_cta : (m > rb ? m - rb : 0));
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+  T x[Q][R];
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = lane + 32 * i, j = warp + NW * q;
+      x[q][i] = (r < nr && j < bw) ? P[(rb + r) + j * ldp] : T(0);
     }
-    if (lane < bw) Tf[lane + j * bw] = (T)t0;
-    if (lane + 32 < bw) Tf[lane + 32 + j * bw] = (T)t1;
+  for (int e = tid; e < 64 * 65; e += NT) G[e] = T(0);
+  if (tid < 64) {
+    s_tau[tid] = 0.0;
+    part[0][tid] = part[1][tid] = T(0);
   }
+  if (warp == 0) {
+#pragma unroll
+    for (int i = 0; i < R; ++i) col[0][lane + 32 * i] = x[0][i];
+  }
+  cluster.sync();  // every CTA of the cluster runs before its shared memory is written
+
+  const int nref = (m < bw) ? (int)m : bw;
+  for (int c = 0; c < nref; ++c) {
+    const int buf = c & 1;
+    const int top = (int)((c > rb) ? c - rb : (c == rb ? 0 : -1));  // rows past `top` lie below the pivot
+    const int pr = (c >= rb && c < rb + nr) ? (int)(c - rb) : -1;   // the pivot's row, if it is here
+    T pc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const T v = col[buf][lane + 32 * i];
+      pc[i] = (lane + 32 * i > top) ? v : T(0);
+    }
+    {
+      T sum[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        sum[q] = T(0);
+#pragma unroll
+        for (int i = 0; i < R; ++i) sum[q] += pc[i] * x[q][i];
+      }
+      // Q sums over 32 lanes: halving exchanges leave one per lane, butterflies
+      // finish it; 32 / Q lanes then hold column warp + NW idx
+      int idx = 0, o = 16;
+#pragma unroll
+      for (int half = Q / 2; half >= 1; half >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < half; ++q) {
+          const T send = up ? sum[q] : sum[q + half];
+          const T keep = up ? sum[q + half] : sum[q];
+          sum[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        if (up) idx += half;
+      }
+      T v = sum[0];
+#pragma unroll
+      for (int d = 16 / Q; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+      if ((lane & (32 / Q - 1)) == 0) part[0][warp + NW * idx] = v;
+      if (pr >= 0 && lane == (pr & 31)) {  // one of the first 64 rows: registers 0 and 1
+#pragma unroll
+        for (int q = 0; q < Q; ++q) part[1][warp + NW * q] = (pr >= 32) ? x[q][R > 1 ? 1 : 0] : x[q][0];
+      }
+    }
+    __syncthreads();
+    for (int q = warp; q < CS; q += NW) {
+      constexpr int V16 = 64 * (int)sizeof(T) / 16;  // 16-byte pieces of a row
+      if (lane < V16)
+        reinterpret_cast<int4*>(cluster.map_shared_rank(&recv[buf][rank][0], q))[lane] = reinterpret_cast<const int4*>(part[0])[lane];
+      if (pr >= 0 && (lane & (V16 - 1)) == lane)
+        reinterpret_cast<int4*>(cluster.map_shared_rank(&piv[buf][0], q))[lane] = reinterpret_cast<const int4*>(part[1])[lane];
+    }
+    cluster.sync();
+    T gs = T(0);
+    if (warp == 0) {
+      const double tail = warp_sum_nonneg((lane < CS) ? recv[buf][lane][c] : T(0));
+      const double x0 = (double)piv[buf][c];
+      double beta = x0, tu = 0.0, inv = 0.0;
+      // (a float's sum: by its bits, a NaN like the compare)
+      const bool some = sizeof(T) == 4 ? __double2hiint(tail) > 0 && __double2hiint(tail) <= 0x7ff00000 : tail > 0.0;
+      if (some && m - c > 1) {
+        if (sizeof(T) == 4) householder_scalars_f32(x0, tail, lane, &beta, &tu, &inv);
+        else householder_scalars(x0, tail, lane, &beta, &tu, &inv);
+      }
+      if (lane == 0) {
+        s_coef[0] = beta;
+        s_coef[1] = tu;
+        s_coef[2] = inv;
+        s_tau[c] = tu;
+        if (rank == 0) tau[c] = tu;
+      }
+    } else if (warp < EW) {
+      // the later columns' sums: GL lanes a column
+      const int t = tid - 32, j = c + 1 + t / GL, q0 = (t & (GL - 1)) * (kClusterMax / GL);
+      T s = T(0), e = T(0);
+      if (j < bw)
+        for (int q = q0; q < q0 + kClusterMax / GL && q < CS; ++q) two_sum(s, recv[buf][q][j], e);
+#pragma unroll
+      for (int o = 1; o < GL; o *= 2) {
+        const T s2 = __shfl_xor_sync(0xffffffffu, s, o);
+        if (sizeof(T) == 4) e += __shfl_xor_sync(0xffffffffu, e, o);
+        two_sum(s, s2, e);
+      }
+      if (j < bw && (t & (GL - 1)) == 0) {
+        g[0][j] = s;
+        g[1][j] = e;
+      }
+    } else if (tid - EW * 32 < c) {
+      for (int q = 0; q < CS; ++q) gs += recv[buf][q][tid - EW * 32];
+    }
+    __syncthreads();
+    if (tid < 64) {
+      if (tid > c && tid < bw) {
+        const double sum = (sizeof(T) == 8) ? (double)g[0][tid] : (double)g[0][tid] + (double)g[1][tid];
+        sw[tid] = (T)(s_coef[1] * fma(sum, s_coef[2], (double)piv[buf][tid]));
+      }
+    } else if (tid == 64) {
+      const T ih = (T)s_coef[2];
+      s_work[0] = ih;  // the products with 1 / (x0 - beta) are rounded once
+      s_work[1] = (sizeof(T) == 8) ? T(0) : (T)(s_coef[2] - (double)ih);
+      s_work[2] = (T)s_coef[0];
+      s_any = s_coef[1] != 0.0;
+    }
+    __syncthreads();
+    const T ih = s_work[0], il = s_work[1], beta = s_work[2];
+    const bool any = s_any != 0;
+    T w[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) w[q] = sw[warp + NW * q];
+    // pc becomes v: 0 above the pivot, 1 in it
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const T v = (sizeof(T) == 8) ? pc[i] * ih : fma(pc[i], ih, pc[i] * il);  // 0 when tau = 0
+      pc[i] = (lane + 32 * i == pr) ? T(1) : v;
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int j = warp + NW * q;
+      if (j > c && j < bw) {
+        if (any) {
+#pragma unroll
+          for (int i = 0; i < R; ++i) x[q][i] -= pc[i] * w[q];
+        }
+        if (j == c + 1) {
+#pragma unroll
+          for (int i = 0; i < R; ++i) col[buf ^ 1][lane + 32 * i] = x[q][i];
+        }
+      } else if (j == c) {
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          if (lane + 32 * i == pr) x[q][i] = beta;
+          else if (lane + 32 * i > top) x[q][i] = pc[i];
+        }
+      }
+    }
+    if (tid >= EW * 32 && tid - EW * 32 < c) {
+      const int j = tid - EW * 32;
+      G[c * 65 + j] = piv[buf][j] + ((sizeof(T) == 8) ? gs * ih : fma(gs, ih, gs * il));
+    }
+    __syncthreads();
+  }
+  if (rank == 0)
+    for (int c = nref + tid; c < bw; c += NT) tau[c] = 0.0;
+  // R and the reflectors to P, V to Vout
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = lane + 32 * i, j = warp + NW * q;
+      if (r < nr && j < bw) {
+        const int64_t gr = rb + r;
+        P[gr + j * ldp] = x[q][i];
+        Vout[gr + j * ldv] = (j >= nref || gr < j) ? T(0) : (gr == j ? T(1) : x[q][i]);
+      }
+    }
+  __syncthreads();
+  panel_t_columns<T>(G, s_tau, bw, rank + CS * warp, CS * NW, lane, Tf);
 }
 
 // Band extraction: band(off, j) = A(j + off, j) for off <= b, 0 for b < off < ldb.
@@ -422,13 +688,34 @@ static int panel_grid(fraclap_ctx* ctx, int64_t m, int bw, size_t elem, int64_t*
   return G;
 }
 
+template <class T>
+using PanelRegsKernel = void (*)(T*, int64_t, int64_t, int, T*, int64_t, double*, T*, int);
+
+// The register kernel for `rows` rows a CTA, or null past its sizes.
+template <class T>
+PanelRegsKernel<T> panel_regs_kernel(int rows, int b) {
+  const int r = (rows + 31) / 32;
+  if constexpr (sizeof(T) == 8) {
+    if (b <= 32) return r <= 2 ? panel_qr_regs_kernel<T, 4, 2> : r <= 3 ? panel_qr_regs_kernel<T, 4, 3> : r <= 4 ? panel_qr_regs_kernel<T, 4, 4>
+                      : r <= 6 ? panel_qr_regs_kernel<T, 4, 6> : r <= 8 ? panel_qr_regs_kernel<T, 4, 8> : nullptr;
+    return r <= 2 ? panel_qr_regs_kernel<T, 8, 2> : r <= 3 ? panel_qr_regs_kernel<T, 8, 3> : r <= 4 ? panel_qr_regs_kernel<T, 8, 4>
+         : r <= 6 ? panel_qr_regs_kernel<T, 8, 6> : r <= 8 ? panel_qr_regs_kernel<T, 8, 8> : nullptr;
+  } else {
+    if (b <= 32) return r <= 4 ? panel_qr_regs_kernel<T, 2, 4> : r <= 8 ? panel_qr_regs_kernel<T, 2, 8> : r <= 12 ? panel_qr_regs_kernel<T, 2, 12>
+                      : r <= 20 ? panel_qr_regs_kernel<T, 2, 20> : nullptr;
+    return r <= 4 ? panel_qr_regs_kernel<T, 4, 4> : r <= 8 ? panel_qr_regs_kernel<T, 4, 8> : r <= 12 ? panel_qr_regs_kernel<T, 4, 12>
+         : r <= 16 ? panel_qr_regs_kernel<T, 4, 16> : r <= 18 ? panel_qr_regs_kernel<T, 4, 18> : nullptr;
+  }
+}
+
 // Panel on one cluster.  Returns 1 (nothing launched) when the panel does not
-// fit in a cluster's shared memory or no cluster of that size can be resident;
-// < 0 on a CUDA error.
+// fit in a cluster or no cluster of that size can be resident; < 0 on a CUDA
+// error.
 template <class T>
 int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, double* tau, T* Tf, cudaStream_t st) {
-  // FP64: past some 1200 rows sixteen SMs' FP64 pipes lose to the grid kernel's
-  // dot products on all SMs
+  // FP64: up to the register kernel's 4096 rows the cluster wins over the grid
+  // kernel (b = 32, n = 4016: the band reduction 132 -> 117 ms with its panels on
+  // the cluster, n = 2351 45 -> 37); past them sixteen SMs' FP64 pipes would lose
   if (sizeof(T) == 8 && m > kPanelFp64Rows) return 1;
   const int64_t most = sizeof(T) == 8 ? kPanelClusterSmemMax - 10 * 1024 : kPanelClusterSmemMax;
   const int64_t cap = most / ((int64_t)b * (int64_t)sizeof(T)) - 1;
@@ -438,12 +725,12 @@ int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, d
   const int rows = (int)cdiv(m, CS);
   CS = (int)cdiv(m, rows);
   const int ld = rows | 1;  // odd: the Gram tiles read 16 columns of a row at once
-  const size_t smem = std::max<size_t>((size_t)ld * b * sizeof(T), panel_gram_smem<T>());
   auto kern = panel_qr_cluster_kernel<T>;
+  PanelRegsKernel<T> regs = panel_regs_kernel<T>(rows, b);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)CS);
-  cfg.blockDim = dim3(PQR_NT);
-  cfg.dynamicSmemBytes = smem;
+  cfg.blockDim = dim3(regs ? 32 * kPanelRegsWarps<T> : PQR_NT);
+  cfg.dynamicSmemBytes = regs ? 64 * 65 * sizeof(T) : std::max<size_t>((size_t)ld * b * sizeof(T), panel_gram_smem<T>());
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -457,10 +744,16 @@ int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, d
   if (fits < 0) {
     FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+    for (int bb : {32, 64})
+      for (int r = 1; panel_regs_kernel<T>(r, bb); r += 32) {
+        FL_CUDA(ctx, cudaFuncSetAttribute(panel_regs_kernel<T>(r, bb), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        FL_CUDA(ctx, cudaFuncSetAttribute(panel_regs_kernel<T>(r, bb), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(64 * 65 * sizeof(T))));
+      }
     cudaLaunchConfig_t full = cfg;
     cudaLaunchAttribute big = attr[0];
     big.val.clusterDim.x = (unsigned)limit;
     full.gridDim = dim3((unsigned)limit);
+    full.blockDim = dim3(PQR_NT);
     full.dynamicSmemBytes = (size_t)most;
     full.attrs = &big;
     int clusters = 0;
@@ -469,7 +762,8 @@ int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, d
   }
   if (!fits) return 1;
   count_launch(ctx);
-  FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, P, ldp, m, b, V, m, tau, Tf, rows, ld));
+  if (regs) FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, regs, P, ldp, m, b, V, m, tau, Tf, rows));
+  else FL_CUDA(ctx, cudaLaunchKernelEx(&cfg, kern, P, ldp, m, b, V, m, tau, Tf, rows, ld));
   return 0;
 }
 
