@@ -11,9 +11,9 @@
 //   C = Z diag(theta) Z^T by eig_full,
 //   Phi = L^-T D^-1/2 Z (a scaling, then one banded backward solve),
 // so that Phi^T M Phi = I and K Phi = M Phi diag(theta).  The banded solves
-// give each right-hand side column to one thread and keep its last b + 1
-// values in a shared-memory ring; the factor is read row-wise (forward) or
-// column-wise (backward), the same addresses for the whole warp.
+// give each right-hand side column to one warp, its window of b + 1 values in
+// registers; past b = 256 to one thread, its last b + 1 values in a
+// shared-memory ring.
 #include "internal.cuh"
 
 namespace fraclap {
@@ -71,6 +71,77 @@ band_bwd_solve(const double* __restrict__ Lb, int64_t ld, int64_t n, double* X, 
     R[ipos * nt] = t;
     if (active) x[i] = t;
     ipos = (ipos == 0) ? ld - 1 : ipos - 1;
+  }
+}
+
+// X <- L^-1 X (FWD, Lc = the column-wise band Lc(t, i) = L(i + t, i)) or L^-T X
+// (Lc = the row-wise copy Lc(t, i) = L(i, i - t), rows taken from the last one
+// up).  A warp per column: register r of lane l holds the value at position
+// p0 + 32 r + l, 32 R >= b; each position in turn is broadcast and its multiples
+// taken off the b after it, then 32 finished values leave and 32 enter, in
+// contiguous accesses.  Every forward value sees the operations of the ring
+// kernel in their order.
+// Bound: the chain of a position (broadcast, FMA) and the FP64 pipe, (R + 1)
+// operations a position, column and warp; the ring kernel waits for b dependent
+// FMAs and an uncoalesced load at every position, which costs more at every b it
+// was tried at.  GB300, the pencil's work outside the dense eigensolver (three
+// solves, the factorisation): n = 751, b = 41 7.8 -> 3.4 ms; n = 2000, b = 41
+// 21.0 -> 9.3; n = 4000, b = 65 64 -> 29, b = 129 126 -> 55, b = 250 341 -> 231.
+template <int R, bool FWD>
+__global__ void __launch_bounds__(128)
+band_solve_window(const double* __restrict__ Lc, int64_t ld, int64_t n, double* X, int64_t ldx, int64_t ncols) {
+  const int lane = threadIdx.x & 31;
+  const int64_t j = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (j >= ncols) return;
+  double* x = X + j * ldx;
+  auto at = [&](int64_t p) { return FWD ? p : n - 1 - p; };
+  double w[R + 1];
+#pragma unroll
+  for (int r = 0; r <= R; ++r) {
+    const int64_t p = 32 * r + lane;
+    w[r] = p < n ? x[at(p)] : 0.0;
+  }
+  for (int64_t p0 = 0; p0 < n; p0 += 32) {
+    const int64_t pn = p0 + 32 * (R + 1) + lane;
+    const double next = pn < n ? x[at(pn)] : 0.0;
+    const int len = (int)(n - p0 < 32 ? n - p0 : 32);
+#pragma unroll 8
+    for (int u = 0; u < len; ++u) {
+      const double* L = Lc + at(p0 + u) * ld;
+      double l[R + 1];
+      bool in[R + 1];
+#pragma unroll
+      for (int r = 0; r <= R; ++r) {
+        const int t = 32 * r + lane - u;
+        in[r] = t > 0 && t < ld && p0 + 32 * r + lane < n;
+        l[r] = in[r] ? L[t] : 0.0;
+      }
+      const double xi = __shfl_sync(0xffffffffu, w[0], u);
+#pragma unroll
+      for (int r = 0; r <= R; ++r)
+        if (in[r]) w[r] = fma(-l[r], xi, w[r]);
+    }
+    if (p0 + lane < n) x[at(p0 + lane)] = w[0];
+#pragma unroll
+    for (int r = 0; r < R; ++r) w[r] = w[r + 1];
+    w[R] = next;
+  }
+}
+
+using BandSolveKernel = void (*)(const double*, int64_t, int64_t, double*, int64_t, int64_t);
+template <bool FWD>
+BandSolveKernel band_window_kernel(int64_t b) {
+  switch ((b + 31) / 32) {
+    case 0:
+    case 1: return band_solve_window<1, FWD>;
+    case 2: return band_solve_window<2, FWD>;
+    case 3: return band_solve_window<3, FWD>;
+    case 4: return band_solve_window<4, FWD>;
+    case 5: return band_solve_window<5, FWD>;
+    case 6: return band_solve_window<6, FWD>;
+    case 7: return band_solve_window<7, FWD>;
+    case 8: return band_solve_window<8, FWD>;
+    default: return nullptr;
   }
 }
 
@@ -139,8 +210,16 @@ void pencil_take(Arena* ar, int64_t n, int64_t b, PencilWork* w) {
 
 size_t eig_ws_for(const fraclap_ctx* ctx, int64_t n) { return fraclap_eig_workspace_bytes(ctx, n); }
 
-int band_solve_launch(fraclap_ctx* ctx, bool forward, const double* L, int64_t ld, int64_t n, double* X,
-                      int64_t ldx, int64_t ncols, cudaStream_t st) {
+int band_solve_launch(fraclap_ctx* ctx, bool forward, const double* Lb, const double* Lr, int64_t ld, int64_t n,
+                      double* X, int64_t ldx, int64_t ncols, cudaStream_t st) {
+  if (auto window = forward ? band_window_kernel<true>(ld - 1) : band_window_kernel<false>(ld - 1)) {
+    FL_CHECK(ctx, cdiv(ncols, 4) <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "eig_pencil: too many columns");
+    window<<<(unsigned)cdiv(ncols, 4), 128, 0, st>>>(forward ? Lb : Lr, ld, n, X, ldx, ncols);
+    count_launch(ctx);
+    FL_CUDA(ctx, cudaGetLastError());
+    return 0;
+  }
+  const double* L = forward ? Lr : Lb;
   int nt = PS_NT_MAX;  // columns per CTA: as many as the ring of ld values each leaves room for
   while (nt > 4 && (size_t)ld * nt * sizeof(double) > kRingSmemMax) nt /= 2;
   const size_t smem = (size_t)ld * nt * sizeof(double);
@@ -195,10 +274,10 @@ extern "C" int eig_pencil(fraclap_ctx* ctx, const double* K_dev, int64_t ldk, in
   // Y = L^-1 K in the output buffer, then C = L^-1 Y^T = L^-1 K L^-T, scaled
   sym_from_lower<<<g, 256, 0, st>>>(K_dev, ldk, n, Phi_dev, ldp);
   count_launch(ctx);
-  FL_TRY(band_solve_launch(ctx, true, w.Lr, ld, n, Phi_dev, ldp, n, st));
+  FL_TRY(band_solve_launch(ctx, true, w.Lb, w.Lr, ld, n, Phi_dev, ldp, n, st));
   transpose_sq<<<dim3((unsigned)cdiv(n, 32), (unsigned)cdiv(n, 32)), dim3(32, 8), 0, st>>>(Phi_dev, ldp, n, w.C, n);
   count_launch(ctx);
-  FL_TRY(band_solve_launch(ctx, true, w.Lr, ld, n, w.C, n, n, st));
+  FL_TRY(band_solve_launch(ctx, true, w.Lb, w.Lr, ld, n, w.C, n, n, st));
   scale_rows_cols<<<g, 256, 0, st>>>(w.C, n, n, n, w.r, 1);
   count_launch(ctx);
   FL_CUDA(ctx, cudaGetLastError());
@@ -208,7 +287,7 @@ extern "C" int eig_pencil(fraclap_ctx* ctx, const double* K_dev, int64_t ldk, in
   // Phi = L^-T D^-1/2 Z
   scale_rows_cols<<<g, 256, 0, st>>>(Phi_dev, ldp, n, n, w.r, 0);
   count_launch(ctx);
-  FL_TRY(band_solve_launch(ctx, false, w.Lb, ld, n, Phi_dev, ldp, n, st));
+  FL_TRY(band_solve_launch(ctx, false, w.Lb, w.Lr, ld, n, Phi_dev, ldp, n, st));
   return 0;
 }
 
