@@ -553,6 +553,41 @@ __global__ void __launch_bounds__(DG_NT) dgemm_dots_kernel(GemmDescT<double> d, 
   dg_finish<kGemmPlain>(d, acc[0], m0 + idx / DG_NC, (j < nc) ? n0 + j : d.N);
 }
 
+// Lower C = alpha (A B^T + A2 B2^T) + beta C of short sums (the reduction's
+// rank-2b updates): 32 x 32 tiles, a lane per row, eight warps of four columns, the
+// operands straight from L1, every entry's sum in the order of the 64 x 64 tile.
+// Four times the tiles even out the SMs' shares of the FP64 pipe, which bounds
+// both: GB300, b = 32, the band reduction at n = 779 5.8 -> 5.0 ms, 2351 36.6 ->
+// 32.7, 4016 116.6 -> 110.7.
+__global__ void __launch_bounds__(DG_NT) dgemm_lower_kernel(GemmDescT<double> d) {
+  const int64_t m0 = (int64_t)blockIdx.x * 32, n0 = (int64_t)blockIdx.y * 32;
+  if (m0 + 31 < n0) return;  // tile entirely above the diagonal
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t gm = m0 + lane, am = gm < d.M ? gm : d.M - 1;
+  const int64_t gn = n0 + 4 * warp;
+  int64_t bn[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) bn[j] = gn + j < d.N ? gn + j : d.N - 1;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  auto sum = [&](const double* A, int64_t lda, const double* B, int64_t ldb, int64_t K) {
+#pragma unroll 4
+    for (int64_t k = 0; k < K; ++k) {
+      const double a = A[am + k * lda];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[j] = fma(a, B[bn[j] + k * ldb], acc[j]);
+    }
+  };
+  sum(d.A, d.lda, d.B, d.ldb, d.K);
+  if (d.K2 > 0) sum(d.A2, d.lda2, d.B2, d.ldb2, d.K2);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (gm >= d.M || gn + j >= d.N || gm < gn + j) continue;
+    double* c = d.C + gm + (gn + j) * d.ldc;
+    const double v = d.alpha * acc[j];
+    *c = (d.beta == 0.0) ? v : v + d.beta * *c;
+  }
+}
+
 // True when the FP64 product takes the kernels above: fewer than four 64 x 64
 // tiles per SM (a last wave of idle SMs costs more than a tile's reuse of its
 // operands saves; at 9 tiles per SM, 2304 x 2304 x 32, both take 357 us), or
@@ -614,6 +649,15 @@ int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st
   }
   if constexpr (std::is_same<T, double>::value && MODE != kGemmLowerC && !(TA && TB)) {
     if (d.K2 == 0 && dg_narrow(ctx, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
+  }
+  if constexpr (std::is_same<T, double>::value && MODE == kGemmLowerC && !TA && TB) {
+    // short sums; long ones take the 64 x 64 tile's shared memory
+    if ((split_k <= 1 || d.K2 > 0) && d.K + d.K2 <= 160 && cdiv(d.N, 32) <= 65535 && d.M > 0 && d.N > 0) {
+      dgemm_lower_kernel<<<dim3((unsigned)cdiv(d.M, 32), (unsigned)cdiv(d.N, 32)), DG_NT, 0, st>>>(d);
+      count_launch(ctx);
+      FL_CUDA(ctx, cudaGetLastError());
+      return 0;
+    }
   }
   const int64_t gx = cdiv(d.M, BM), gy = cdiv(d.N, BN);
   FL_CHECK(ctx, gy <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm: N = %lld too large", (long long)d.N);
