@@ -36,8 +36,9 @@ __global__ void merge_status(int32_t* parent, int32_t* child) {
 
 // Streams beyond the device's hardware queues (8 unless the process asked for
 // more before its first CUDA call) share one and wait for each other's kernels:
-// 32 problems of n = 180 to 1843 on a GB300 took 170 ms on 8 streams, 245 on 16
-// (103 on 16 with 32 queues), so no more streams than queues run at one time.
+// 32 problems of n = 180 to 1843 on a GB300 took 171 ms on 8 streams, 244 on 16
+// (103 on 16 with 32 queues), so no more streams than queues run at one time
+// (153 ms since the panels stay in registers).
 int hardware_queues() {
   const char* e = getenv("CUDA_DEVICE_MAX_CONNECTIONS");
   const int q = e ? atoi(e) : 0;

@@ -8,7 +8,8 @@
 // recurrence, and bisection on it gives any index range of eigenvalues
 // without the divide and conquer.
 //
-// Banded LDL^T on the GPU: one CTA per shift.  In the natural dof order the
+// Banded LDL^T on the GPU: one CTA per shift, or a cluster of CTAs where few
+// shifts would leave SMs idle.  In the natural dof order the
 // Laplacian (and the finite-element pencil) is banded with half-width b (the
 // grid row length in 2-D, the plane size in 3-D), and the factorisation
 // fills exactly that band.  Step j needs only columns j .. j + b: a window of

@@ -14,7 +14,7 @@
 //     merge of the two sorted spectra, deflation of small |z_i| and of close
 //     pairs (Givens rotations), compaction of the K surviving entries;
 //   gather: Q columns in sorted order, rotations applied per row;
-//   secular: one thread per root of 1 + rho sum z_j^2/(d_j - x) = 0, solved
+//   secular: one warp per root of 1 + rho sum z_j^2/(d_j - x) = 0, solved
 //     in shifted coordinates x = d_org + tau (org = nearer pole) by a
 //     two-pole rational model with bisection safeguard;
 //   Gu-Eisenstat: z recomputed from the roots (orthogonal vectors);

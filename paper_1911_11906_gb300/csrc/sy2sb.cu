@@ -1,15 +1,16 @@
 // Stage 1 of the two-stage reduction: dense symmetric -> band of half-width b.
 //
 // Panel j (columns j0..j0+b-1) is factorised P = Q_j R with Q_j = I - V T V^T
-// (compact WY) by a cooperative kernel: the panel's rows are split over the
-// CTAs and stay in shared memory, and each Householder column costs one
-// grid-wide reduction (the dot products of the pivot column with every later
-// column, added by FP64 atomics, from which the reflector and its effect on
-// the panel follow).  The
-// trailing matrix is then updated as A22 <- Q^T A22 Q = A22 - W V^T - V W^T
-// with X = A22 (V T), W = X - 1/2 V ((V T)^T X), through the GEMM engine
-// (symmetric A22 read from its lower triangle; lower-triangular rank-2b
-// update).  FP64 throughout; the Householder norms and scalings stay FP64.
+// (compact WY) on one thread-block cluster, its rows split over the CTAs'
+// registers or, for taller panels, shared memory; each Householder column costs
+// one cluster barrier (the dot products of the pivot column with every other
+// column, from which the reflector and its effect on the panel follow).  Panels
+// past a cluster's room take a cooperative kernel over all SMs, with FP64 atomics
+// and a grid barrier per column.  The trailing matrix is then updated as
+// A22 <- Q^T A22 Q = A22 - W V^T - V W^T with X = A22 (V T), W = X - 1/2 V ((V T)^T X),
+// through the GEMM engine (symmetric A22 read from its lower triangle;
+// lower-triangular rank-2b update).  In FP64 or FP32; the Householder scalars are
+// FP64 in both, and FP32 norms are added over the CTAs exactly.
 #include <cooperative_groups.h>
 
 #include "internal.cuh"
