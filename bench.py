@@ -228,7 +228,7 @@ def refine_slice_counts(iterations: int, cap: int, digit_bits: int = 7) -> list:
 
 # DRAM bytes per BF16 flop of ozaki_tc_kernel from an ncu capture of the 4096^3
 # product; None whenever the kernel changes until it is captured again.
-OZAKI_DRAM_BYTES_PER_FLOP = None
+OZAKI_DRAM_BYTES_PER_FLOP = 1.36e-3
 
 
 def run_path(F, ctx, p, path, args, mask, Fd, pf, pa, U, app_ws, barrier, steps=None, warmup=None):
@@ -377,7 +377,7 @@ def run_gpu(args, rank, world, local_rank):
         dur = q2_ms / max(q2_cnt, 1)
         work = q2_flops(n, b)
         traffic = None
-        roof = {"kernel": "q2t_apply_kernel (back-transformation by the bulge-chasing reflectors, FP64)",
+        roof = {"kernel": "q2_block_kernel and its factors (back-transformation by the bulge-chasing reflectors, FP64)",
                 "bound": "alu", "peak": round(fp64_peak, 4),
                 "peak_source": "measured FP64 FMA throughput (fraclap_fma_throughput); no FP64 figure in "
                                "MEASURED_PEAKS.json"}
@@ -395,7 +395,7 @@ def run_gpu(args, rank, world, local_rank):
             launches_per_step += 2
         work = total / max(launches_per_step, 1)
         # the captured figure holds for the captured tile width and no cluster
-        captured = R["ctx"].get_schedule("ozaki_tile_n") == 192 and R["ctx"].get_schedule("ozaki_cluster") == 1
+        captured = R["ctx"].get_schedule("ozaki_tile_n") == 256 and R["ctx"].get_schedule("ozaki_cluster") == 1
         traffic = OZAKI_DRAM_BYTES_PER_FLOP * work if (OZAKI_DRAM_BYTES_PER_FLOP and captured) else None
         # the kernel runs inside a seconds-long step: the sustained BF16 figure is its peak
         peak = _measured_peak("bf16_tflops_sustained") or _measured_peak("bf16_tflops") or 1700.0
