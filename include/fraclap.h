@@ -588,7 +588,8 @@ int fraclap_partition_spectrum(fraclap_ctx* ctx, int64_t n, const int64_t* rowpt
  *    column's window of the stage-2 back-transformation, one reflector after
  *    the other: 4, 8 or 16 (16, 8 or 4 rows per lane; more parts give more
  *    warps over the same columns; FP64 takes 8 when asked for 4), or 0 for
- *    blocks of reflectors, which is faster at every size [0].
+ *    the library's choice: blocks of reflectors, and in FP64 past some 4256
+ *    columns the reflectors one by one in 8 lanes [0].
  *  FRACLAP_SCHED_OZAKI_CLUSTER: CTAs of the slice-product kernel per thread-
  *    block cluster, 1 or 2: the two CTAs of a cluster take consecutive tile
  *    rows of one tile column and share its B tile through TMA multicast,

@@ -972,13 +972,17 @@ int q2_apply_run(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int b, T* Z, 
                  int64_t ncols, T* Yt, int64_t ldy, cudaStream_t st) {
   if (n < 2 || ncols <= 0) return 0;
   FL_TRY(transpose_run<T>(ctx, Z, ldz, Yt, ldy, n, ncols, st));
-  if ((b == 64 && ctx->q2_parts == 0) || b == 32) {
+  const int64_t sm = ctx->sm_count > 0 ? ctx->sm_count : 152;
+  // FP64 at b = 64: with seven warps an SM the reflectors one by one keep the FP64
+  // pipe busy too, for fewer operations (n = 7735 1333 ms against 1363, 4016 185
+  // against 187; 2351 64 against 33)
+  const bool single = sizeof(T) == 8 && b == 64 && cdiv(ncols, 4) >= 7 * sm;
+  if ((b == 64 && ctx->q2_parts == 0 && !single) || b == 32) {
     // Columns per CTA: the fewest columns on the busiest SM, the wider CTA at a
     // tie (it reuses the factors more).  FP32, b = 64, 64 / 32 / 16 columns: n =
     // 7735 52.6 / 58.1 / 76.5 ms, 4741 20.3 / 15.1 / 16.3, 2740 6.8 / 5.1 / 5.5,
     // 1200 1.47 / 1.14 / 0.91.
-    const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
-    const auto cost = [&](int ncb) { return cdiv(cdiv(ncols, ncb), sms) * ncb; };
+    const auto cost = [&](int ncb) { return cdiv(cdiv(ncols, ncb), sm) * ncb; };
     int rc = 0;
     if constexpr (sizeof(T) == 8) {
       if (b == 64) rc = q2_blocks_launch<T, 64, 16>(ctx, s, n, ncols, Yt, ldy, st);
