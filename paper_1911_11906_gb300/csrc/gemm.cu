@@ -554,47 +554,60 @@ __global__ void __launch_bounds__(DG_NT) dgemm_dots_kernel(GemmDescT<double> d, 
 }
 
 // Lower C = alpha (A B^T + A2 B2^T) + beta C of short sums (the reduction's
-// rank-2b updates): 32 x 32 tiles, a lane per row, eight warps of four columns, the
+// rank-2b updates), and the batched C = alpha A B + beta C (the merges of divide
+// and conquer): 32 x 32 tiles, a lane per row, eight warps of four columns, the
 // operands straight from L1, every entry's sum in the order of the 64 x 64 tile.
 // Four times the tiles even out the SMs' shares of the FP64 pipe, which bounds
 // both: GB300, b = 32, the band reduction at n = 779 5.8 -> 5.0 ms, 2351 36.6 ->
-// 32.7, 4016 116.6 -> 110.7.
-__global__ void __launch_bounds__(DG_NT) dgemm_lower_kernel(GemmDescT<double> d) {
-  const int64_t m0 = (int64_t)blockIdx.x * 32, n0 = (int64_t)blockIdx.y * 32;
-  if (m0 + 31 < n0) return;  // tile entirely above the diagonal
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t gm = m0 + lane, am = gm < d.M ? gm : d.M - 1;
-  const int64_t gn = n0 + 4 * warp;
-  int64_t bn[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) bn[j] = gn + j < d.N ? gn + j : d.N - 1;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  auto sum = [&](const double* A, int64_t lda, const double* B, int64_t ldb, int64_t K) {
+// 32.7, 4016 116.6 -> 110.7; the merges: divide and conquer at n = 779 4.1 -> 3.8,
+// 2351 29.2 -> 26.5, 4016 115 -> 111, 7735 725 -> 709.
+template <bool TB>
+__device__ __forceinline__ void dgemm_small_sum(double (&acc)[4], const double* A, int64_t lda, const double* B, int64_t ldb, int64_t K,
+                                                int64_t row, const int64_t (&col)[4]) {
 #pragma unroll 4
-    for (int64_t k = 0; k < K; ++k) {
-      const double a = A[am + k * lda];
+  for (int64_t k = 0; k < K; ++k) {
+    const double a = A[row + k * lda];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[j] = fma(a, B[bn[j] + k * ldb], acc[j]);
-    }
-  };
-  sum(d.A, d.lda, d.B, d.ldb, d.K);
-  if (d.K2 > 0) sum(d.A2, d.lda2, d.B2, d.ldb2, d.K2);
+    for (int j = 0; j < 4; ++j) acc[j] = fma(a, TB ? B[col[j] + k * ldb] : B[k + col[j] * ldb], acc[j]);
+  }
+}
+template <bool TB, bool LOWER>
+__device__ __forceinline__ void dgemm_small_tile(const GemmDescT<double>& d) {
+  const int64_t m0 = (int64_t)blockIdx.x * 32, n0 = (int64_t)blockIdx.y * 32;
+  if (m0 >= d.M || n0 >= d.N || (LOWER && m0 + 31 < n0)) return;  // past C, or entirely above its diagonal
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t gm = m0 + lane, gn = n0 + 4 * warp;
+  int64_t col[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) col[j] = gn + j < d.N ? gn + j : d.N - 1;
+  const int64_t row = gm < d.M ? gm : d.M - 1;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  dgemm_small_sum<TB>(acc, d.A, d.lda, d.B, d.ldb, d.K, row, col);
+  if (LOWER && d.K2 > 0) dgemm_small_sum<TB>(acc, d.A2, d.lda2, d.B2, d.ldb2, d.K2, row, col);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    if (gm >= d.M || gn + j >= d.N || gm < gn + j) continue;
+    if (gm >= d.M || gn + j >= d.N || (LOWER && gm < gn + j)) continue;
     double* c = d.C + gm + (gn + j) * d.ldc;
     const double v = d.alpha * acc[j];
     *c = (d.beta == 0.0) ? v : v + d.beta * *c;
   }
 }
+__global__ void __launch_bounds__(DG_NT) dgemm_lower_kernel(GemmDescT<double> d) { dgemm_small_tile<true, true>(d); }
+__global__ void __launch_bounds__(DG_NT) dgemm_small_batched_kernel(const GemmDescT<double>* descs) {
+  const GemmDescT<double> d = descs[blockIdx.z];
+  dgemm_small_tile<false, false>(d);
+}
 
-// True when the FP64 product takes the kernels above: fewer than four 64 x 64
-// tiles per SM (a last wave of idle SMs costs more than a tile's reuse of its
+// True when the FP64 product takes the kernels above.  A B: fewer than four 64 x
+// 64 tiles per SM (a last wave of idle SMs costs more than a tile's reuse of its
 // operands saves; at 9 tiles per SM, 2304 x 2304 x 32, both take 357 us), or
-// more than a tenth of the tiles is padding.
-inline bool dg_narrow(const fraclap_ctx* ctx, int64_t M, int64_t N) {
+// more than a tenth of the tiles is padding.  A^T B, whose dot products reach
+// 0.78 of the tile's rate (64 x 8810 x 4405 6.1 against 4.7 ms): when the tiles'
+// waves cost more than that (64 x 4000 x 2000 1.1 against 2.1 ms).
+inline bool dg_narrow(const fraclap_ctx* ctx, bool ta, int64_t M, int64_t N) {
   const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
   const int64_t tiles = cdiv(M, BM) * cdiv(N, BN);
+  if (ta) return (double)(cdiv(tiles, sms) * sms * BM * BN) > 1.28 * (double)M * (double)N;
   return tiles < 4 * sms || (double)(tiles * BM * BN) > 1.1 * (double)M * (double)N;
 }
 
@@ -648,7 +661,7 @@ int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st
                         : launch_sg_narrow<64, 128, TA, TB, MODE>(ctx, d, st);
   }
   if constexpr (std::is_same<T, double>::value && MODE != kGemmLowerC && !(TA && TB)) {
-    if (d.K2 == 0 && dg_narrow(ctx, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
+    if (d.K2 == 0 && dg_narrow(ctx, TA, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
   }
   if constexpr (std::is_same<T, double>::value && MODE == kGemmLowerC && !TA && TB) {
     // short sums; long ones take the 64 x 64 tile's shared memory
@@ -732,9 +745,14 @@ int gemm_batched(fraclap_ctx* ctx, bool ta, bool tb, const GemmDescT<T>* d_descs
     }
   }
   const int64_t gx = cdiv(max_m, BM), gy = cdiv(max_n, BN);
-  FL_CHECK(ctx, gy <= 65535 && count <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm_batched: too large");
+  FL_CHECK(ctx, 2 * gy <= 65535 && count <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm_batched: too large");
   dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)count);
-  if (!ta && !tb) gemm_batched_kernel<T, false, false><<<grid, NT, 0, st>>>(d_descs);
+  if (!ta && !tb) {
+    if constexpr (std::is_same<T, double>::value)
+      dgemm_small_batched_kernel<<<dim3((unsigned)cdiv(max_m, 32), (unsigned)cdiv(max_n, 32), (unsigned)count), DG_NT, 0, st>>>(d_descs);
+    else
+      gemm_batched_kernel<T, false, false><<<grid, NT, 0, st>>>(d_descs);
+  }
   else if (!ta && tb) gemm_batched_kernel<T, false, true><<<grid, NT, 0, st>>>(d_descs);
   else if (ta && !tb) gemm_batched_kernel<T, true, false><<<grid, NT, 0, st>>>(d_descs);
   else gemm_batched_kernel<T, true, true><<<grid, NT, 0, st>>>(d_descs);
