@@ -661,7 +661,9 @@ int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st
                         : launch_sg_narrow<64, 128, TA, TB, MODE>(ctx, d, st);
   }
   if constexpr (std::is_same<T, double>::value && MODE != kGemmLowerC && !(TA && TB)) {
-    if (d.K2 == 0 && dg_narrow(ctx, TA, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
+    // (a caller that splits the sums of 64 tiles or more fills the SMs by itself)
+    const bool own = TA && split_k > 1 && cdiv(d.M, BM) * cdiv(d.N, BN) >= 64;
+    if (d.K2 == 0 && !own && dg_narrow(ctx, TA, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
   }
   if constexpr (std::is_same<T, double>::value && MODE == kGemmLowerC && !TA && TB) {
     // short sums; long ones take the 64 x 64 tile's shared memory
