@@ -51,17 +51,16 @@ __device__ __forceinline__ int exponent_above(unsigned long long t) {
   return e;
 }
 
-// Exponent of the largest |entry| of each row of op(A) (rows = M, length K);
+// Exponent of the largest |entry| of each row of op(A), rows contiguous (length K);
 // an infinity or NaN, which has no digits, sets *nonfinite.
 // One block per row.  The magnitudes are compared as the integers of their
 // IEEE bit patterns with the sign cleared (the same order as the values), so
 // the FP64 pipe is not used.
-__global__ void row_exponents(const double* A, int64_t lda, bool trans, int64_t K, int* ex, int* nonfinite) {
+__global__ void row_exponents(const double* A, int64_t lda, int64_t K, int* ex, int* nonfinite) {
   const int64_t i = blockIdx.x;
   unsigned long long m = 0;
   for (int64_t k = threadIdx.x; k < K; k += blockDim.x) {
-    const double v = trans ? A[k + i * lda] : A[i + k * lda];
-    const unsigned long long u = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+    const unsigned long long u = (unsigned long long)__double_as_longlong(A[k + i * lda]) & 0x7FFFFFFFFFFFFFFFull;
     m = u > m ? u : m;
   }
   __shared__ unsigned long long red[32];
@@ -385,26 +384,26 @@ struct OzTile {
 // 2^e for e in [-1022, 1023], from its bit pattern.
 __device__ __forceinline__ double pow2i(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// The digit pairs (p, q = dg - p) and the K-chunks of one item, for D digits,
-// nchunk chunks and at most U pairs per item: diagonals from the longest
-// (dg = D - 1) down, so that the longest items start first.  An item adds at
-// most 127 chunk sums (127 2^24 < 2^31): a K of more chunks is cut too.
+// The digit pairs (p, q = dg - p) of one item, for D digits, nchunk K-chunks and
+// at most U pairs per item: diagonals from the longest (dg = D - 1) down, so that
+// the longest items start first.  An item adds at most kMaxChunks chunk sums,
+// which fit 31 bits (127 2^24 < 2^31); K beyond that many chunks is multiplied
+// in ranges (see ozaki_gemm).
+constexpr int kMaxChunks = 127;
 struct OzParts {
-  int D, U, nchunk, cper, kparts;
-  __host__ __device__ int of_diag(int dg) const { return (dg + U) / U * kparts; }
+  int D, U, nchunk;
+  __host__ __device__ int of_diag(int dg) const { return (dg + U) / U; }
   __host__ __device__ int count() const {
     int t = 0;
     for (int dg = 0; dg < D; ++dg) t += of_diag(dg);
     return t;
   }
-  __device__ void get(int part, int* dg, int* p0, int* p1, int* c0, int* c1) const {
+  __device__ void get(int part, int* dg, int* p0, int* p1) const {
     int d = D - 1;
     while (part >= of_diag(d)) part -= of_diag(d--);
     *dg = d;
-    *p0 = part / kparts * U;
+    *p0 = part * U;
     *p1 = (*p0 + U < d + 1) ? *p0 + U : d + 1;
-    *c0 = part % kparts * cper;
-    *c1 = (*c0 + cper < nchunk) ? *c0 + cper : nchunk;
   }
 };
 // A plane: M x N column-major, or (lower, M >= N) its columns from the diagonal
@@ -425,9 +424,7 @@ inline OzParts oz_parts(int64_t M, int64_t N, int64_t Kp, int D, int w, bool low
   o.nchunk = (int)cdiv(Kp, chunk);
   const int64_t tiles = cdiv(M, TC_M) * cdiv(N, TC_M) / (lower ? 2 : 1);
   const int64_t even = cdiv(std::max<int64_t>(tiles, 1) * (D * (D + 1) / 2), 152);
-  o.U = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(D, even), 127 / std::min(o.nchunk, 127)));
-  o.cper = std::min(o.nchunk, 127);
-  o.kparts = (int)cdiv(o.nchunk, o.cper);
+  o.U = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(D, even), kMaxChunks / o.nchunk));
   return o;
 }
 
@@ -507,8 +504,9 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
   const int rank = (CS > 1) ? (int)cluster_ctarank() : 0;
   // items: all tiles (or clusters of tiles) of the first group of pairs, then of the next
   const int unit = (int)(blockIdx.x / CS), part = unit / tiles, tile = unit - part * tiles;
-  int dg, pbeg, pend, cbeg, cend;
-  parts.get(part, &dg, &pbeg, &pend, &cbeg, &cend);
+  int dg, pbeg, pend;
+  parts.get(part, &dg, &pbeg, &pend);
+  const int nchunk = parts.nchunk;
   int tm, tn;
   if (CS == 1) {
     ozaki_tile_of(tile, TM, TN, group, lower != 0, TC_M, TC_N, &tm, &tn);
@@ -555,7 +553,7 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
       int it = 0;
       bool ok = true;
       for (int p = pbeg; p < pend && ok; ++p)
-          for (int c = cbeg; c < cend && ok; ++c) {
+          for (int c = 0; c < nchunk && ok; ++c) {
             const int q = dg - p;
             const int64_t c0 = (int64_t)c * chunk;
             const int nkb = (int)(((Kp - c0) < chunk ? (Kp - c0) : chunk) / TC_KB);
@@ -597,7 +595,7 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
       int it = 0, chunk_i = 0;
       bool ok = true;
       for (int p = pbeg; p < pend && ok; ++p)
-          for (int c = cbeg; c < cend && ok; ++c, ++chunk_i) {
+          for (int c = 0; c < nchunk && ok; ++c, ++chunk_i) {
             const int buf = chunk_i % NBUF;
             if (!mbar_wait(&acc_empty[buf], ((chunk_i / NBUF) & 1) ^ 1, limit) || *(volatile int*)&abort_sh) {
               ok = false;
@@ -637,14 +635,14 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
   } else {
     // ---------------- epilogue: exact integer sums ----------------
     // A chunk sum is an integer of at most 2^24 (exact in FP32), so it converts
-    // exactly to int32, and an item's at most 127 of them add exactly.
+    // exactly to int32, and an item's at most kMaxChunks of them add exactly.
     const int lg = warp & 3;                          // TMEM lane quarter of this warp
     const int cbase = ((warp - 2) >> 2) * TC_EPI_COLS;  // this warp's columns of the tile
     const int64_t row = m0 + lg * 32 + lane;          // output row of this thread
     int acc[TC_EPI_COLS];
 #pragma unroll
     for (int j = 0; j < TC_EPI_COLS; ++j) acc[j] = 0;
-    const int nacc = (pend - pbeg) * (cend - cbeg);
+    const int nacc = (pend - pbeg) * nchunk;
     bool ok = true;
     for (int chunk_i = 0; chunk_i < nacc; ++chunk_i) {
       const int buf = chunk_i % NBUF;
@@ -690,10 +688,11 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
 }
 
 // C = alpha 2^(e_i + f_j - 2t + r (2D - 2)) sum_dg 2^(-r dg) P_dg + beta C from the
-// items' planes.  Up to four diagonals at a time are one exact 64-bit integer
-// (a diagonal's sum is below 2^31 times its items, and three shifts of at most
-// 9 bits follow), so an element costs a conversion and an FMA per four
-// diagonals; the lowest diagonals are added first.
+// items' planes.  Up to four diagonals at a time are one exact 64-bit integer: a
+// diagonal is at most D kMaxChunks chunk sums of 2^24, below 2^34.2, and three
+// shifts of at most 9 bits follow, so that a group stays below 2^61.3.  An
+// element costs a conversion and an FMA per four diagonals; the lowest diagonals
+// are added first.
 __global__ void combine_planes(const int32_t* __restrict__ P, const int* __restrict__ ea, const int* __restrict__ eb,
                                int64_t M, int64_t N, OzParts parts, int w, double alpha, double beta, double* C,
                                int64_t ldc, int lower) {
@@ -773,6 +772,8 @@ int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB
 
 }  // namespace
 
+// The longest K of one pass: kMaxChunks chunks of digits of magnitude w.
+static int64_t oz_range(int w) { return (int64_t)kMaxChunks << (24 - 2 * w); }
 // The most digits that s slices are cut into (see ozaki_gemm), and the int32
 // entries of the tensor-core route's planes for up to that many, at either digit
 // width.
@@ -780,12 +781,12 @@ static int max_digits(int s) { return (s <= 5 || s == 8) ? s + 1 : s; }
 static int64_t plane_entries(int64_t M, int64_t N, int64_t Kp, int D, bool lower) {
   int64_t t = 0;
   for (int d = 1; d <= D; ++d)
-    for (int w = 7; w <= 8; ++w) t = std::max<int64_t>(t, oz_parts(M, N, Kp, d, w, lower).count());
+    for (int w = 7; w <= 8; ++w) t = std::max<int64_t>(t, oz_parts(M, N, std::min(Kp, oz_range(w)), d, w, lower).count());
   return t * plane_size(M, N, lower);
 }
 
 size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits) {
-  const int64_t Kp = cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD;
+  const int64_t Kp = cdiv(std::max<int64_t>(std::min(K, oz_range(7)), 1), OZ_KPAD) * OZ_KPAD;
   const int D = (digits > 0) ? digits : max_digits(s);
   Arena ar;
   ar.take<__nv_bfloat16>((int64_t)D * M * Kp);
@@ -804,9 +805,8 @@ size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits) 
 int slice_operand(fraclap_ctx* ctx, const double* X, int64_t ldx, bool trans, int64_t R, int64_t K, int64_t Kp,
                   int sl, int bits, int* ex, __nv_bfloat16* S, unsigned long long* mx, int* nonfinite, cudaStream_t st) {
   const bool fits = sl * (bits + 1) <= 64;
-  const bool tiled = fits && Kp / 64 <= 65535;
-  if (trans || cdiv(K, OZ_MAX_KCH) > 65535) {
-    row_exponents<<<(unsigned)R, 256, 0, st>>>(X, ldx, trans, K, ex, nonfinite);
+  if (trans) {
+    row_exponents<<<(unsigned)R, 256, 0, st>>>(X, ldx, K, ex, nonfinite);
   } else {
     FL_CUDA(ctx, cudaMemsetAsync(mx, 0, sizeof(unsigned long long) * (size_t)R, st));
     row_absmax_strided<<<dim3((unsigned)cdiv(R, 256), (unsigned)std::max<int64_t>(cdiv(K, OZ_MAX_KCH), 1)), 256, 0,
@@ -818,7 +818,7 @@ int slice_operand(fraclap_ctx* ctx, const double* X, int64_t ldx, bool trans, in
   if (trans && fits) {
     const unsigned gs = (unsigned)std::min<int64_t>(cdiv(R * (Kp / 8), 256), 152 * 16);
     make_slices_rows<<<gs, 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl, bits, S);
-  } else if (tiled) {
+  } else if (fits) {  // (K of a range: both grids' second dimension is below 2100)
     make_slices_strided<<<dim3((unsigned)cdiv(R, 64), (unsigned)(Kp / 64)), 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl,
                                                                                          bits, S);
   } else {
@@ -830,20 +830,11 @@ int slice_operand(fraclap_ctx* ctx, const double* X, int64_t ldx, bool trans, in
   return 0;
 }
 
-// C = alpha op(A) op(B) + beta C, FP64-accurate through s BF16 slices
-// (s = 7 for full FP64 accuracy of the products).  lower: only C(i,j), i >= j.
-// digits > 0 sets the digits per operand itself (8 bits each at w = 7);
-// nonfinite (device, may be null) is set to 1 when an operand holds an infinity
-// or NaN, which the digits do not represent: C is then meaningless.
-int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
-               const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
-               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits, int* nonfinite) {
-  if (M <= 0 || N <= 0) return 0;
-  FL_CHECK(ctx, s >= 1 && s <= 8, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: slices must be 1..8");
-  FL_CHECK(ctx, cdiv(N, OZ_BN) <= 65535, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: N too large");
+// One range of K (see ozaki_gemm): sl digits of magnitude `bits` per operand, room for smax.
+static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double* A,
+                       int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc, int sl, int smax,
+                       int bits, bool lower, Arena* ar, cudaStream_t st, int* nonfinite) {
   const int64_t Kp = cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD;
-  FL_CHECK(ctx, !lower || M >= N, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: a lower product needs M >= N");
-  const int smax = (digits > 0) ? digits : max_digits(s);
   __nv_bfloat16* SA = ar->take<__nv_bfloat16>((int64_t)smax * M * Kp);
   __nv_bfloat16* SB = ar->take<__nv_bfloat16>((int64_t)smax * N * Kp);
   int* ea = ar->take<int>(M);
@@ -852,23 +843,6 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   int32_t* P = ar->take<int32_t>(plane_entries(M, N, Kp, smax, lower));
   FL_CHECK(ctx, mx != nullptr && P != nullptr, FRACLAP_ERR_ALLOC, "ozaki_gemm: workspace too small");
   // op(A) rows: trans -> A stored K x M; op(B) columns = rows of op(B)^T
-  // Digit magnitude w and count D for s slices of 8 bits: with w = 8 (short K,
-  // one chunk; or the knob) s digits of 9 bits (7 for s = 8: 63 bits, within
-  // the FP64 rounding of the result); with w = 7 digits of 8 bits, one more
-  // than s up to s = 5 and at s = 8, so that no s is less accurate than
-  // ceil(8 s / 7) sign-magnitude digits of 7 bits (s = 6 and 7 reach that with
-  // s).  Measured at 8810 x 8810 x 8810 on 128 x 192 tiles, those against
-  // these: s = 7 52.3 ms and 3.3e-15 from FP64, now 39.6 ms and 3.2e-15; s = 6
-  // 41.0 ms and 1.0e-13, now 30.2 ms and 9.3e-14.  (On 128 x 256 tiles without
-  // the folds 28.8 and 21.4 ms; w = 8 at s = 7 32.0 ms: the same pairs and four
-  // times more chunk sums to drain and convert.)
-  int bits = 8, sl = std::min(s, 7);
-  if (K > 256 && ctx->oz_bits != 8) {
-    bits = 7;
-    sl = (s <= 5 || s == 8) ? s + 1 : s;  // s = 8: 72 bits
-  }
-  if (digits > 0) sl = digits;
-  FL_CHECK(ctx, sl <= smax, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: too many digits");
   const int64_t chunk = (int64_t)1 << (24 - 2 * bits);
   // rows of op(A) and columns of op(B): contiguous when trans, else strided
   FL_TRY(slice_operand(ctx, A, lda, ta, M, K, Kp, sl, bits, ea, SA, mx, nonfinite, st));
@@ -894,6 +868,50 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   }
   count_launch(ctx);
   FL_CUDA(ctx, cudaGetLastError());
+  return 0;
+}
+
+// C = alpha op(A) op(B) + beta C, FP64-accurate through s BF16 slices
+// (s = 7 for full FP64 accuracy of the products).  lower: only C(i,j), i >= j.
+// digits > 0 sets the digits per operand itself (8 bits each at w = 7);
+// nonfinite (device, may be null) is set to 1 when an operand holds an infinity
+// or NaN, which the digits do not represent: C is then meaningless.
+int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
+               const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
+               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits, int* nonfinite) {
+  if (M <= 0 || N <= 0) return 0;
+  FL_CHECK(ctx, s >= 1 && s <= 8, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: slices must be 1..8");
+  FL_CHECK(ctx, cdiv(N, OZ_BN) <= 65535, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: N too large");
+  FL_CHECK(ctx, !lower || M >= N, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: a lower product needs M >= N");
+  // Digit magnitude w and count D for s slices of 8 bits: with w = 8 (short K,
+  // one chunk; or the knob) s digits of 9 bits (7 for s = 8: 63 bits, within
+  // the FP64 rounding of the result); with w = 7 digits of 8 bits, one more
+  // than s up to s = 5 and at s = 8, so that no s is less accurate than
+  // ceil(8 s / 7) sign-magnitude digits of 7 bits (s = 6 and 7 reach that with
+  // s).  Measured at 8810 x 8810 x 8810 on 128 x 192 tiles, those against
+  // these: s = 7 52.3 ms and 3.3e-15 from FP64, now 39.6 ms and 3.2e-15; s = 6
+  // 41.0 ms and 1.0e-13, now 30.2 ms and 9.3e-14.  (On 128 x 256 tiles without
+  // the folds 28.8 and 21.4 ms; w = 8 at s = 7 32.0 ms: the same pairs and four
+  // times more chunk sums to drain and convert.)
+  int bits = 8, sl = std::min(s, 7);
+  if (K > 256 && ctx->oz_bits != 8) {
+    bits = 7;
+    sl = (s <= 5 || s == 8) ? s + 1 : s;  // s = 8: 72 bits
+  }
+  if (digits > 0) sl = digits;
+  const int smax = (digits > 0) ? digits : max_digits(s);
+  FL_CHECK(ctx, sl <= smax, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: too many digits");
+  // K in ranges, each added into C in FP64: 130048 (w = 7) or 32512 (w = 8), so
+  // that the integer sums of a range cannot overflow whatever the operands
+  const Arena scratch = *ar;
+  int64_t k0 = 0;
+  do {
+    const int64_t kr = std::min(K - k0, oz_range(bits));
+    *ar = scratch;
+    FL_TRY(ozaki_range(ctx, ta, tb, M, N, kr, alpha, A + (ta ? k0 : k0 * lda), lda, B + (tb ? k0 * ldb : k0), ldb,
+                       k0 == 0 ? beta : 1.0, C, ldc, sl, smax, bits, lower, ar, st, nonfinite));
+    k0 += kr;
+  } while (k0 < K);
   return 0;
 }
 
