@@ -445,7 +445,10 @@ int fraclap_fma_throughput(fraclap_ctx* ctx, int precision, int64_t iters, doubl
  * BF16 tensor cores by Ozaki's error-free splitting into `slices` 8-bit slices
  * per row/column (7 slices: full FP64 accuracy; fewer: about 8*slices bits
  * relative to the row and column maxima).  The engine behind the
- * refinement's residual products.  work: fraclap_dgemm_ozaki_workspace_bytes. */
+ * refinement's residual products.  work: fraclap_dgemm_ozaki_workspace_bytes, the
+ * digits and, in one block of C or several, the planes of exact sums: at most
+ * 4 GiB or 2 ceil(8 slices / 7) (m + n) k bytes, whichever is more (and, null,
+ * the context's own, which also does with the latter). */
 size_t fraclap_dgemm_ozaki_workspace_bytes(int64_t m, int64_t n, int64_t k, int slices);
 int fraclap_dgemm_ozaki(fraclap_ctx* ctx, int trans_a, int trans_b, int64_t m, int64_t n,
                         int64_t k, double alpha, const double* A_dev, int64_t lda,

@@ -677,11 +677,14 @@ def dgemm_ozaki(A: torch.Tensor, B: torch.Tensor, trans_a=False, trans_b=False, 
     else:
         C = _out(C, torch.float64, "C", A.device, m, n)
     nbytes = ctx.lib.fraclap_dgemm_ozaki_workspace_bytes(m, n, k, slices)
-    ws = torch.empty(max(nbytes, 1), dtype=torch.uint8, device=A.device)
+    try:
+        ws = torch.empty(max(nbytes, 1), dtype=torch.uint8, device=A.device)
+    except torch.OutOfMemoryError:
+        ws = None  # the library's own, in the smallest size that it can do with
     st = ctypes.c_void_p(_stream(stream))
     ctx.check(ctx.lib.fraclap_dgemm_ozaki(ctx.handle, int(trans_a), int(trans_b), m, n, k, float(alpha), _ptr(A),
                                           _ld(A), _ptr(B), _ld(B), float(beta), _ptr(C), _ld(C), int(slices),
-                                          _ptr(ws), ws.numel(), st))
+                                          _ptr(ws), 0 if ws is None else ws.numel(), st))
     ctx.sync(stream)
     return C
 

@@ -312,7 +312,7 @@ int cluster_eig(fraclap_ctx* ctx, double* S, int64_t c, double* w, double* Q, Ar
                 cudaStream_t st);
 
 // FP64-accurate GEMM through BF16 tensor-core slices (ozaki.cu).
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false, int digits = 0);
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false, int digits = 0, bool tight = false);
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
                int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits = 0,

@@ -250,8 +250,8 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
 __global__ void __launch_bounds__(OZ_NT)
 ozaki_kernel(const __nv_bfloat16* __restrict__ SA, const __nv_bfloat16* __restrict__ SB,
              const int* __restrict__ ea, const int* __restrict__ eb, int64_t M, int64_t N,
-             int64_t Kp, int s, int bits, int64_t chunk, double alpha, double beta, double* C,
-             int64_t ldc, bool lower) {
+             int64_t arows, int64_t Kp, int s, int bits, int64_t chunk, double alpha, double beta, double* C,
+             int64_t ldc, bool lower) {  // arows: rows of A's slices, of which M are multiplied
   __shared__ uint32_t As[OZ_BM][OZ_LDS];
   __shared__ uint32_t Bs[OZ_BN][OZ_LDS];
   const int64_t m0 = (int64_t)blockIdx.x * OZ_BM, n0 = (int64_t)blockIdx.y * OZ_BN;
@@ -270,7 +270,7 @@ ozaki_kernel(const __nv_bfloat16* __restrict__ SA, const __nv_bfloat16* __restri
 
   for (int p = 0; p < s; ++p) {
     for (int q = 0; p + q < s; ++q) {  // slices p, q (0-based): p + q <= s - 1
-      const __nv_bfloat16* Ap = SA + (int64_t)p * M * Kp;
+      const __nv_bfloat16* Ap = SA + (int64_t)p * arows * Kp;
       const __nv_bfloat16* Bq = SB + (int64_t)q * N * Kp;
       const double scale = ldexp(1.0, (bits + 1) * (2 * s - 2 - p - q) - 2 * digit_frac_bits(bits, s));
       for (int64_t c0 = 0; c0 < Kp; c0 += chunk) {
@@ -727,12 +727,12 @@ __global__ void combine_planes(const int32_t* __restrict__ P, const int* __restr
   }
 }
 
-// 3-D map over the slices S[s][rows][Kp] (bf16), box 64 (K) x box_rows x 1.
-bool slice_map(CUtensorMap* map, const __nv_bfloat16* S, int64_t rows, int64_t Kp, int s, int box_rows) {
+// 3-D map over `rows` rows of the slices S[s][of][Kp] (bf16), box 64 (K) x box_rows x 1.
+bool slice_map(CUtensorMap* map, const __nv_bfloat16* S, int64_t rows, int64_t of, int64_t Kp, int s, int box_rows) {
   EncodeTiledFn fn = encode_tiled();
   if (!fn) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)rows, (cuuint64_t)s};
-  const cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)rows * Kp * 2};
+  const cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)of * Kp * 2};
   const cuuint32_t box[3] = {TC_KB, (cuuint32_t)box_rows, 1};
   const cuuint32_t estr[3] = {1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)S, dims, strides, box, estr,
@@ -740,10 +740,10 @@ bool slice_map(CUtensorMap* map, const __nv_bfloat16* S, int64_t rows, int64_t K
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 template <int TCN, int CS>
-int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB, int64_t M, int64_t N, int64_t Kp,
-              const OzParts& parts, int64_t chunk, int32_t* P, bool lower, cudaStream_t st) {
+int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB, int64_t M, int64_t N, int64_t arows,
+              int64_t Kp, const OzParts& parts, int64_t chunk, int32_t* P, bool lower, cudaStream_t st) {
   CUtensorMap ma, mb;
-  FL_CHECK(ctx, slice_map(&ma, SA, M, Kp, parts.D, TC_M) && slice_map(&mb, SB, N, Kp, parts.D, TCN / CS),
+  FL_CHECK(ctx, slice_map(&ma, SA, M, arows, Kp, parts.D, TC_M) && slice_map(&mb, SB, N, N, Kp, parts.D, TCN / CS),
            FRACLAP_ERR_CUDA, "ozaki_gemm: tensor map encoding failed");
   const size_t smem = (size_t)OzTile<TCN>::STAGES * OzTile<TCN>::STAGE_BYTES + 1024;
   auto kern = ozaki_tc_kernel<TCN, CS>;
@@ -774,28 +774,80 @@ int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB
 
 // The longest K of one pass: kMaxChunks chunks of digits of magnitude w.
 static int64_t oz_range(int w) { return (int64_t)kMaxChunks << (24 - 2 * w); }
-// The most digits that s slices are cut into (see ozaki_gemm), and the int32
-// entries of the tensor-core route's planes for up to that many, at either digit
-// width.
+// The most digits that s slices are cut into (see ozaki_gemm), and the most
+// planes of the tensor-core route for up to that many, at either digit width.
 static int max_digits(int s) { return (s <= 5 || s == 8) ? s + 1 : s; }
-static int64_t plane_entries(int64_t M, int64_t N, int64_t Kp, int D, bool lower) {
-  int64_t t = 0;
+static int max_planes(int64_t M, int64_t N, int64_t Kp, int D, bool lower) {
+  int t = 0;
   for (int d = 1; d <= D; ++d)
-    for (int w = 7; w <= 8; ++w) t = std::max<int64_t>(t, oz_parts(M, N, std::min(Kp, oz_range(w)), d, w, lower).count());
-  return t * plane_size(M, N, lower);
+    for (int w = 7; w <= 8; ++w) t = std::max(t, oz_parts(M, N, std::min(Kp, oz_range(w)), d, w, lower).count());
+  return t;
+}
+static int64_t padded(int64_t K) { return cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD; }
+
+// The scratch of one range: A's digits, and for a block of C (mb rows of nb
+// columns) B's digits and the planes.  The planes are four bytes an entry of C
+// and item of the diagonals (7 to 28 of them for 7 slices), so C is formed block
+// by block where they do not fit beside the digits: strips of columns, each with
+// its own digits of B, and rows of a strip where even one tile column of all
+// rows does not fit.
+struct OzBlocks {
+  int64_t mb, nb;
+};
+struct OzScratch {
+  __nv_bfloat16 *SA, *SB;
+  int *ea, *eb;
+  unsigned long long* mx;
+  int32_t* P;
+};
+static OzScratch oz_take(Arena* ar, int64_t M, OzBlocks c, int64_t Kp, int D, int planes, bool lower) {
+  OzScratch w;
+  w.SA = ar->take<__nv_bfloat16>((int64_t)D * M * Kp);
+  w.SB = ar->take<__nv_bfloat16>((int64_t)D * c.nb * Kp);
+  w.ea = ar->take<int>(M);
+  w.eb = ar->take<int>(c.nb);
+  w.mx = ar->take<unsigned long long>(std::max(M, c.nb));
+  w.P = ar->take<int32_t>(planes * plane_size(c.mb, c.nb, lower));
+  return w;
+}
+static size_t oz_bytes(int64_t M, OzBlocks c, int64_t Kp, int D, int planes, bool lower) {
+  Arena ar;
+  oz_take(&ar, M, c, Kp, D, planes, lower);
+  return ar.off;
+}
+// The largest blocks that fit `room` bytes (mb = 0: none does): all of C, else
+// even strips of a multiple of 256 columns, else even blocks of a multiple of 128
+// rows of one such strip.
+static OzBlocks oz_blocks(int64_t M, int64_t N, int64_t Kp, int D, int planes, bool lower, size_t room) {
+  const auto fits = [&](int64_t mb, int64_t nb) { return oz_bytes(M, {mb, nb}, Kp, D, planes, lower) <= room; };
+  const auto part = [](int64_t total, int64_t unit, int64_t count) { return std::min(total, cdiv(cdiv(total, count), unit) * unit); };
+  if (fits(M, N)) return {M, N};
+  const auto most = [&](int64_t total, int64_t unit, auto ok) {  // fewest even parts that fit, 0: none
+    int64_t lo = 1, hi = cdiv(total, unit) + 1;
+    while (lo < hi) {
+      const int64_t c = (lo + hi) / 2;
+      if (ok(part(total, unit, c))) hi = c;
+      else lo = c + 1;
+    }
+    return lo > cdiv(total, unit) ? (int64_t)0 : part(total, unit, lo);
+  };
+  if (const int64_t nb = most(N, 256, [&](int64_t v) { return fits(M, v); })) return {M, nb};
+  if (lower) return {0, 0};
+  const int64_t nb = std::min<int64_t>(N, 256);
+  return {most(M, 128, [&](int64_t v) { return fits(v, nb); }), nb};
 }
 
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits) {
-  const int64_t Kp = cdiv(std::max<int64_t>(std::min(K, oz_range(7)), 1), OZ_KPAD) * OZ_KPAD;
-  const int D = (digits > 0) ? digits : max_digits(s);
-  Arena ar;
-  ar.take<__nv_bfloat16>((int64_t)D * M * Kp);
-  ar.take<__nv_bfloat16>((int64_t)D * N * Kp);
-  ar.take<int>(M);
-  ar.take<int>(N);
-  ar.take<unsigned long long>(std::max(M, N));
-  ar.take<int32_t>(plane_entries(M, N, Kp, D, lower));
-  return ar.off;
+// All of C in one block up to 4 GiB, or up to what the digits of s slices took
+// without planes where that is more (16 (M + N) K bytes for 7 slices; `tight`:
+// only that): no product needs more than it did when every diagonal was folded
+// into C on the fly, but for small ones.
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits, bool tight) {
+  const int64_t Kp = padded(std::min(K, oz_range(7)));
+  const int D = (digits > 0) ? digits : max_digits(s), planes = max_planes(M, N, Kp, D, lower);
+  const size_t whole = oz_bytes(M, {M, N}, Kp, D, planes, lower);
+  const size_t least = oz_bytes(M, {lower ? M : std::min<int64_t>(M, 1024), std::min<int64_t>(N, 256)}, Kp, D, planes, lower);
+  const size_t fold = align256((size_t)((8 * s + 6) / 7) * 2 * (size_t)(M + N) * (size_t)padded(K));
+  return std::min(whole, std::max({least, fold, tight ? (size_t)0 : (size_t)4 << 30}));
 }
 
 // Exponents and digit slices of the rows of op(X) (R rows of length K):
@@ -830,29 +882,15 @@ int slice_operand(fraclap_ctx* ctx, const double* X, int64_t ldx, bool trans, in
   return 0;
 }
 
-// One range of K (see ozaki_gemm): sl digits of magnitude `bits` per operand, room for smax.
-static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double* A,
-                       int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc, int sl, int smax,
-                       int bits, bool lower, Arena* ar, cudaStream_t st, int* nonfinite) {
-  const int64_t Kp = cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD;
-  __nv_bfloat16* SA = ar->take<__nv_bfloat16>((int64_t)smax * M * Kp);
-  __nv_bfloat16* SB = ar->take<__nv_bfloat16>((int64_t)smax * N * Kp);
-  int* ea = ar->take<int>(M);
-  int* eb = ar->take<int>(N);
-  unsigned long long* mx = ar->take<unsigned long long>(std::max(M, N));
-  int32_t* P = ar->take<int32_t>(plane_entries(M, N, Kp, smax, lower));
-  FL_CHECK(ctx, mx != nullptr && P != nullptr, FRACLAP_ERR_ALLOC, "ozaki_gemm: workspace too small");
-  // op(A) rows: trans -> A stored K x M; op(B) columns = rows of op(B)^T
+// One block of C: M rows of A's slices (of `arows`), N columns of B's.
+static int ozaki_block(fraclap_ctx* ctx, const OzScratch& z, const __nv_bfloat16* SA, const int* ea, int64_t M, int64_t N,
+                       int64_t arows, int64_t Kp, const OzParts& parts, int bits, double alpha, double beta, double* C,
+                       int64_t ldc, bool lower, cudaStream_t st) {
   const int64_t chunk = (int64_t)1 << (24 - 2 * bits);
-  // rows of op(A) and columns of op(B): contiguous when trans, else strided
-  FL_TRY(slice_operand(ctx, A, lda, ta, M, K, Kp, sl, bits, ea, SA, mx, nonfinite, st));
-  FL_TRY(slice_operand(ctx, B, ldb, !tb, N, K, Kp, sl, bits, eb, SB, mx, nonfinite, st));
-  StageTimer tm(ctx, kStageSliceProducts, st);
   if (ctx->tensor_route == 1) {
     const int tw = (N <= 128) ? 128 : ctx->oz_tile_n;  // a narrow output takes the 128-column tile
     const int cs = ctx->oz_cluster;
-    const OzParts parts = oz_parts(M, N, Kp, sl, bits, lower);
-#define FL_OZ_LAUNCH(W, K) launch_tc<W, K>(ctx, SA, SB, M, N, Kp, parts, chunk, P, lower, st)
+#define FL_OZ_LAUNCH(W, K) launch_tc<W, K>(ctx, SA, z.SB, M, N, arows, Kp, parts, chunk, z.P, lower, st)
     if (cs == 2) {
       FL_TRY(tw == 256 ? FL_OZ_LAUNCH(256, 2) : tw == 192 ? FL_OZ_LAUNCH(192, 2) : FL_OZ_LAUNCH(128, 2));
     } else {
@@ -861,13 +899,37 @@ static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N,
 #undef FL_OZ_LAUNCH
     count_launch(ctx);
     combine_planes<<<dim3((unsigned)cdiv(M, 256), (unsigned)std::min<int64_t>(N, 16384)), 256, 0, st>>>(
-        P, ea, eb, M, N, parts, bits, alpha, beta, C, ldc, lower ? 1 : 0);
+        z.P, ea, z.eb, M, N, parts, bits, alpha, beta, C, ldc, lower ? 1 : 0);
   } else {
     dim3 grid((unsigned)cdiv(M, OZ_BM), (unsigned)cdiv(N, OZ_BN));
-    ozaki_kernel<<<grid, OZ_NT, 0, st>>>(SA, SB, ea, eb, M, N, Kp, sl, bits, chunk, alpha, beta, C, ldc, lower);
+    ozaki_kernel<<<grid, OZ_NT, 0, st>>>(SA, z.SB, ea, z.eb, M, N, arows, Kp, parts.D, bits, chunk, alpha, beta, C, ldc,
+                                         lower);
   }
   count_launch(ctx);
   FL_CUDA(ctx, cudaGetLastError());
+  return 0;
+}
+
+// One range of K (see ozaki_gemm): D digits of magnitude `bits` per operand.
+static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double* A,
+                       int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc, int D, int bits,
+                       bool lower, Arena ar, cudaStream_t st, int* nonfinite) {
+  const int64_t Kp = padded(K);
+  const OzParts parts = oz_parts(M, N, Kp, D, bits, lower);
+  const OzBlocks c = oz_blocks(M, N, Kp, D, parts.count(), lower, ar.cap - ar.off);
+  FL_CHECK(ctx, c.mb > 0, FRACLAP_ERR_ALLOC, "ozaki_gemm: workspace too small");
+  const OzScratch z = oz_take(&ar, M, c, Kp, D, parts.count(), lower);
+  // rows of op(A) and columns of op(B): contiguous when trans, else strided
+  FL_TRY(slice_operand(ctx, A, lda, ta, M, K, Kp, D, bits, z.ea, z.SA, z.mx, nonfinite, st));
+  for (int64_t j = 0; j < N; j += c.nb) {
+    const int64_t nb = std::min(c.nb, N - j);
+    FL_TRY(slice_operand(ctx, B + (tb ? j : j * ldb), ldb, !tb, nb, K, Kp, D, bits, z.eb, z.SB, z.mx, nonfinite, st));
+    StageTimer tm(ctx, kStageSliceProducts, st);
+    for (int64_t i = lower ? j : 0; i < M; i += lower ? M : c.mb) {
+      const int64_t mb = lower ? M - j : std::min(c.mb, M - i);
+      FL_TRY(ozaki_block(ctx, z, z.SA + i * Kp, z.ea + i, mb, nb, M, Kp, parts, bits, alpha, beta, C + i + j * ldc, ldc, lower, st));
+    }
+  }
   return 0;
 }
 
@@ -899,17 +961,13 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
     sl = (s <= 5 || s == 8) ? s + 1 : s;  // s = 8: 72 bits
   }
   if (digits > 0) sl = digits;
-  const int smax = (digits > 0) ? digits : max_digits(s);
-  FL_CHECK(ctx, sl <= smax, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: too many digits");
   // K in ranges, each added into C in FP64: 130048 (w = 7) or 32512 (w = 8), so
   // that the integer sums of a range cannot overflow whatever the operands
-  const Arena scratch = *ar;
   int64_t k0 = 0;
   do {
     const int64_t kr = std::min(K - k0, oz_range(bits));
-    *ar = scratch;
     FL_TRY(ozaki_range(ctx, ta, tb, M, N, kr, alpha, A + (ta ? k0 : k0 * lda), lda, B + (tb ? k0 * ldb : k0), ldb,
-                       k0 == 0 ? beta : 1.0, C, ldc, sl, smax, bits, lower, ar, st, nonfinite));
+                       k0 == 0 ? beta : 1.0, C, ldc, sl, bits, lower, *ar, st, nonfinite));
     k0 += kr;
   } while (k0 < K);
   return 0;
@@ -936,7 +994,9 @@ extern "C" int fraclap_dgemm_ozaki(fraclap_ctx* ctx, int trans_a, int trans_b, i
   FL_CHECK(ctx, ldc >= m && lda >= (trans_a ? k : m) && ldb >= (trans_b ? n : k),
            FRACLAP_ERR_INVALID_ARG, "dgemm_ozaki: leading dimension too small");
   Arena ar;
-  FL_TRY(get_workspace(ctx, work_dev, work_bytes, ozaki_ws(m, n, k, slices) + 1024, &ar));
+  int rc = get_workspace(ctx, work_dev, work_bytes, ozaki_ws(m, n, k, slices) + 1024, &ar);
+  if (rc == FRACLAP_ERR_ALLOC) rc = get_workspace(ctx, work_dev, work_bytes, ozaki_ws(m, n, k, slices, false, 0, true) + 1024, &ar);
+  if (rc != 0) return rc;
   return ozaki_gemm(ctx, trans_a != 0, trans_b != 0, m, n, k, alpha, A_dev, lda, B_dev, ldb, beta,
                     C_dev, ldc, slices, false, &ar, (cudaStream_t)stream);
 }
