@@ -614,9 +614,19 @@ inline bool dg_narrow(const fraclap_ctx* ctx, bool ta, int64_t M, int64_t N) {
 template <bool TA, bool TB, int MODE>
 int launch_narrow(fraclap_ctx* ctx, const GemmDescT<double>& d, cudaStream_t st) {
   const int64_t sms = ctx->sm_count > 0 ? ctx->sm_count : 152;
+  constexpr int64_t kMostCols = 65535 * (int64_t)DG_NC;  // a grid's second dimension; more columns in turn
+  if (d.N > kMostCols) {
+    for (int64_t j = 0; j < d.N; j += kMostCols) {
+      GemmDescT<double> part = d;
+      part.N = (d.N - j < kMostCols) ? d.N - j : kMostCols;
+      part.B += TB ? j : j * d.ldb;
+      part.C += j * d.ldc;
+      FL_TRY((launch_narrow<TA, TB, MODE>(ctx, part, st)));
+    }
+    return 0;
+  }
   const int64_t gx = cdiv(d.M, DG_ROWS), gy = cdiv(d.N, DG_NC);
   const int ncol = (int)cdiv(d.N, gy);  // the columns dealt evenly
-  FL_CHECK(ctx, gy <= 65535, FRACLAP_ERR_UNSUPPORTED, "gemm: N = %lld too large", (long long)d.N);
   int S = 1;
   while (S < 8 && gx * gy * S < 4 * sms && d.K >= 256 * (int64_t)S) S *= 2;
   const int64_t kper = cdiv(cdiv(d.K > 0 ? d.K : 1, S), 32) * 32;
@@ -644,7 +654,7 @@ int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st
   if constexpr (std::is_same<T, float>::value) {
     // short sums into large outputs are bound by C's traffic and latency: the
     // smaller tile has four CTAs an SM to overlap them
-    const bool shallow = d.K + d.K2 <= 160;
+    const bool shallow = d.K + d.K2 <= 160 && cdiv(d.N, 64) <= 65535;
     if (MODE != kGemmSymA && sg_big(d.M, d.N) && shallow) return launch_sg_narrow<128, 64, TA, TB, MODE>(ctx, d, st);
     if (MODE != kGemmSymA && sg_big(d.M, d.N)) {
       const int64_t gx = cdiv(d.M, 128), gy = cdiv(d.N, 128);
