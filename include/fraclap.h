@@ -156,10 +156,13 @@ size_t fraclap_apply_workspace_bytes(int64_t n, int64_t m, int64_t k);
 size_t fraclap_apply_workspace_bytes_ctx(const fraclap_ctx* ctx, int64_t n, int64_t m, int64_t k);
 /* Products of frac_apply: 0 (default) at FP64 accuracy, on the FP64 GEMM engine
  * or, where that is faster and the workspace has room for it (the _ctx size),
- * from 8 digits of 8 bits per operand (2^-63 relative to |row max| |column max|
- * per term, exact sums; infinities and NaN take the FP64 engine); s = 1..8 as
- * products of s BF16 slices on the tensor cores (error about 2^-8s relative
- * to |row max| |column max| per term; s = 7 is FP64-level, s = 5 about 1e-12). */
+ * from 8 digits of 8 bits per operand.  Those are off by at most n 2^-61.9 |row
+ * max'| |column max'| (the powers of two above the maxima); an entry that this
+ * does not bound by n 2^-53 times the sum of its terms' magnitudes, as an FP64 sum
+ * is bounded, and everything with infinities or NaN is formed by the FP64 engine.
+ * s = 1..8 as products of s BF16 slices on the tensor cores (error about 2^-8s
+ * relative to |row max| |column max| per term; s = 7 is FP64-level, s = 5 about
+ * 1e-12). */
 int fraclap_set_apply_slices(fraclap_ctx* ctx, int slices);
 int frac_apply(fraclap_ctx* ctx, const double* V_dev, int64_t ldv, const double* lambda_dev,
                int64_t n, const double* F_dev, int64_t ldf, int64_t m,

@@ -10,7 +10,8 @@
 // the FP64 engine, or (context setting apply_slices = s > 0) as products of
 // s BF16 slices on the tensor cores, accurate to about 2^-8s relative to
 // |row max| |column max| per term (s = 7: FP64 level).  With s = 0 large
-// products are formed from 8 digits (63 bits) too, see digits_pay.  A zero or negative
+// products are formed from 8 digits too, where those hold an FP64 sum's
+// accuracy entry by entry, see digits_pay.  A zero or negative
 // eigenvalue met with alpha != 0 raises FRACLAP_ERR_NOT_SPD in the device
 // status.
 #include <cmath>
@@ -58,13 +59,16 @@ __global__ void spectral_scale(const double* lambda, int64_t n, const double* W,
 // FP64 products (apply_slices = 0) of large operands: the FP64 pipe takes
 // 2 n^2 (m + k) / 1.2 TFLOP/s whatever the memory does, while cutting V twice
 // into kFp64Digits digits of 8 bits and multiplying those takes little more
-// than the bytes.  8 digits hold every entry to 2^-63 of its row's or column's
-// largest, and the sums are exact, so the result is at least as accurate as the
-// FP64 sums: GB300, n = 8835, 16 forcings, 128 pairs 19.7 -> 2.9 ms and 3.1e-15
-// -> 2.7e-15 from exact.  The line (a factor of 1.5 in the estimate) keeps small
-// applies, which the launches bound, on the FP64 pipe: n = 2304, 25 columns 0.36 ms.
-// An infinity or NaN has no digits: the slicing raises a flag, and the FP64
-// product behind each sliced one runs only then.
+// than the bytes.  The digits are relative to the largest entry of a row or
+// column, so the products are guarded (see ozaki_gemm): an entry keeps its digits'
+// sum where that is within n 2^-53.9 of the sum of its terms' magnitudes, half of
+// what an FP64 sum guarantees, and all others are formed again by FP64 products
+// that skip the rest (graded columns against modes that vanish where the column
+// is large).  GB300, n = 8835, 16 forcings, 128 pairs: 19.7 -> 3.6 ms (2.9 without
+// the guard) and 3.1e-15 -> 2.8e-15 from exact.  The line (a factor of 1.5 in the
+// estimate) keeps small applies, which the launches bound, on the FP64 pipe: n =
+// 2304, 25 columns 0.36 ms.  An infinity or NaN has no digits: the slicing raises
+// a flag, and the whole FP64 product behind each sliced one runs only then.
 constexpr int kFp64Digits = 8;
 bool digits_pay(const fraclap_ctx* ctx, int64_t n, int64_t m, int64_t k) {
   if (ctx->apply_slices != 0 || ctx->tensor_route != 1) return false;
@@ -72,11 +76,27 @@ bool digits_pay(const fraclap_ctx* ctx, int64_t n, int64_t m, int64_t k) {
   // microseconds: FP64 pipe; slices, pairs of 128-column tiles, launches
   const double fp64 = 2.0 * nn * (double)(m + k) / 1.2e6;
   const double cols = 128.0 * (double)(cdiv(m, 128) + cdiv(k, 128));
-  const double digits = 1.5e-5 * nn + 72.0 * nn * cols / 0.9e9 + 150.0;
+  const double digits = 1.5e-5 * nn + 88.0 * nn * cols / 0.9e9 + 160.0;
   return fp64 > 1.5 * digits;
 }
+size_t guard_marks(int64_t n, int64_t cols) { return sizeof(unsigned) * (size_t)cdiv(n, kGuardRows) * (size_t)cdiv(cols, kGuardCols); }
 size_t digits_ws(int64_t n, int64_t m, int64_t k) {
-  return std::max(ozaki_ws(n, m, n, 7, false, kFp64Digits), ozaki_ws(n, k, n, 7, false, kFp64Digits)) + 1024;
+  const auto one = [&](int64_t cols) { return ozaki_ws(n, cols, n, 7, false, kFp64Digits, false, true); };
+  return align256(sizeof(int)) + align256(guard_marks(n, std::max(m, k))) + std::max(one(m), one(k)) + 1024;
+}
+// C (n x cols) = op(V) B by digits, the marked tiles again in FP64, or everything
+// when an operand holds an infinity or NaN.
+int digits_product(fraclap_ctx* ctx, bool ta, int64_t n, int64_t cols, const double* V, int64_t ldv, const double* B,
+                   int64_t ldb, double* C, int64_t ldc, const OzGuard& guard, Arena oz, cudaStream_t st) {
+  FL_CUDA(ctx, cudaMemsetAsync(guard.nonfinite, 0, sizeof(int), st));
+  FL_CUDA(ctx, cudaMemsetAsync(guard.marks, 0, guard_marks(n, cols), st));
+  FL_TRY(ozaki_gemm(ctx, ta, false, n, cols, n, 1.0, V, ldv, B, ldb, 0.0, C, ldc, 7, false, &oz, st, kFp64Digits, &guard));
+  GemmDesc d{n, cols, n, V, ldv, B, ldb, C, ldc, nullptr, 0, nullptr, 0, 0, 1.0, 0.0};
+  d.only_marked = guard.marks;
+  FL_TRY(gemm(ctx, ta, false, kGemmPlain, d, 1, st));
+  d.only_marked = nullptr;
+  d.only_if = guard.nonfinite;
+  return gemm(ctx, ta, false, kGemmPlain, d, 1, st);
 }
 
 // The body shared by frac_apply and frac_diffusion.
@@ -106,20 +126,20 @@ int spectral_apply(fraclap_ctx* ctx, const char* name, const double* V_dev, int6
   double* W = ar.take<double>(n * m);
   double* C = ar.take<double>(n * k);
   FL_CHECK(ctx, W && C, FRACLAP_ERR_ALLOC, "%s: workspace too small", name);
-  int* nonfinite = nullptr;
+  OzGuard guard{};
   if (by_digits) {
-    nonfinite = ar.take<int>(1);
-    FL_CUDA(ctx, cudaMemsetAsync(nonfinite, 0, sizeof(int), st));
+    guard.nonfinite = ar.take<int>(1);
+    guard.marks = ar.take<unsigned>((int64_t)(guard_marks(n, std::max(m, k)) / sizeof(unsigned)));
   }
-  const int ozs = by_digits ? 7 : ctx->apply_slices, dig = by_digits ? kFp64Digits : 0;
+  const int ozs = ctx->apply_slices;
   // W = V^T F
-  if (ozs > 0) {
+  if (by_digits) {
+    FL_TRY(digits_product(ctx, true, n, m, V_dev, ldv, F_dev, ldf, W, n, guard, ar, st));
+  } else if (ozs > 0) {
     Arena oz = ar;
-    FL_TRY(ozaki_gemm(ctx, true, false, n, m, n, 1.0, V_dev, ldv, F_dev, ldf, 0.0, W, n, ozs, false, &oz, st, dig,
-                      nonfinite));
-  }
-  if (ozs == 0 || by_digits) {
-    GemmDesc d{n, m, n, V_dev, ldv, F_dev, ldf, W, n, nullptr, 0, nullptr, 0, 0, 1.0, 0.0, nonfinite};
+    FL_TRY(ozaki_gemm(ctx, true, false, n, m, n, 1.0, V_dev, ldv, F_dev, ldf, 0.0, W, n, ozs, false, &oz, st));
+  } else {
+    GemmDesc d{n, m, n, V_dev, ldv, F_dev, ldf, W, n, nullptr, 0, nullptr, 0, 0, 1.0, 0.0};
     FL_TRY(gemm(ctx, true, false, kGemmPlain, d, 1, st));
   }
   spectral_scale<<<dim3((unsigned)cdiv(n, 256), (unsigned)cdiv(k, kScalePairs)), 256, 0, st>>>(
@@ -127,13 +147,13 @@ int spectral_apply(fraclap_ctx* ctx, const char* name, const double* V_dev, int6
   count_launch(ctx);
   FL_CUDA(ctx, cudaGetLastError());
   // U = V C
-  if (ozs > 0) {
+  if (by_digits) {
+    FL_TRY(digits_product(ctx, false, n, k, V_dev, ldv, C, n, U_dev, ldu, guard, ar, st));
+  } else if (ozs > 0) {
     Arena oz = ar;
-    FL_TRY(ozaki_gemm(ctx, false, false, n, k, n, 1.0, V_dev, ldv, C, n, 0.0, U_dev, ldu, ozs, false, &oz, st, dig,
-                      nonfinite));
-  }
-  if (ozs == 0 || by_digits) {
-    GemmDesc d{n, k, n, V_dev, ldv, C, n, U_dev, ldu, nullptr, 0, nullptr, 0, 0, 1.0, 0.0, nonfinite};
+    FL_TRY(ozaki_gemm(ctx, false, false, n, k, n, 1.0, V_dev, ldv, C, n, 0.0, U_dev, ldu, ozs, false, &oz, st));
+  } else {
+    GemmDesc d{n, k, n, V_dev, ldv, C, n, U_dev, ldu, nullptr, 0, nullptr, 0, 0, 1.0, 0.0};
     FL_TRY(gemm(ctx, false, false, kGemmPlain, d, 1, st));
   }
   return 0;
@@ -153,7 +173,7 @@ extern "C" size_t fraclap_apply_workspace_bytes(int64_t n, int64_t m, int64_t k)
 extern "C" size_t fraclap_apply_workspace_bytes_ctx(const fraclap_ctx* ctx, int64_t n, int64_t m, int64_t k) {
   const size_t base = fraclap_apply_workspace_bytes(n, m, k);
   if (!ctx || base == 0) return base;
-  if (n > 0 && m > 0 && k > 0 && digits_pay(ctx, n, m, k)) return base + align256(sizeof(int)) + digits_ws(n, m, k);
+  if (n > 0 && m > 0 && k > 0 && digits_pay(ctx, n, m, k)) return base + digits_ws(n, m, k);
   if (ctx->apply_slices <= 0) return base;
   const int64_t nn = n > 0 ? n : 1;
   return base + std::max(ozaki_ws(nn, m > 0 ? m : 1, nn, ctx->apply_slices),

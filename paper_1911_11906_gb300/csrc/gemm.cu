@@ -452,6 +452,16 @@ __device__ __forceinline__ void dg_finish(const GemmDescT<double>& d, double v, 
   *c = (d.beta == 0.0) ? v : v + d.beta * *c;
 }
 
+// The columns of its tile, one bit each, that this cluster forms: all nc of them,
+// the marked ones, or none.  (The same in every CTA of the cluster.)
+__device__ __forceinline__ unsigned dg_columns(const GemmDescT<double>& d, int nc) {
+  const unsigned all = (1u << nc) - 1u;
+  if (d.only_if && *d.only_if == 0) return 0u;
+  if (!d.only_marked) return all;
+  const int64_t S = cg::this_cluster().num_blocks();
+  return d.only_marked[(int64_t)blockIdx.y * (gridDim.x / S) + blockIdx.x / S] & all;
+}
+
 // op(A) = A (or symmetric, lower triangle read): a lane per row, eight warps
 // interleaved over K, up to eight columns in registers; the reads of A are
 // coalesced along the rows (in the mirrored half of a symmetric A a lane walks
@@ -459,10 +469,10 @@ __device__ __forceinline__ void dg_finish(const GemmDescT<double>& d, double v, 
 template <bool TB, int MODE>
 __global__ void __launch_bounds__(DG_NT) dgemm_rows_kernel(GemmDescT<double> d, int64_t kper, int ncol) {
   __shared__ double red[DG_NC][DG_NC][DG_ROWS];
-  if (d.only_if && *d.only_if == 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t m0 = (int64_t)(blockIdx.x / cg::this_cluster().num_blocks()) * DG_ROWS, n0 = (int64_t)blockIdx.y * ncol;
-  const int nc = (int)((d.N - n0 < ncol) ? d.N - n0 : ncol);
+  const unsigned cols = dg_columns(d, (int)((d.N - n0 < ncol) ? d.N - n0 : ncol));
+  if (cols == 0) return;
   const int64_t kbeg = (int64_t)cg::this_cluster().block_rank() * kper;
   const int64_t kend = (kbeg + kper < d.K) ? kbeg + kper : d.K;
   const int64_t row = m0 + lane;
@@ -484,7 +494,7 @@ __global__ void __launch_bounds__(DG_NT) dgemm_rows_kernel(GemmDescT<double> d, 
       for (int u = 0; u < KU; ++u) a[u] = a_at(k0 + u);
 #pragma unroll
       for (int j = 0; j < DG_NC; ++j)
-        if (j < nc) {
+        if (cols >> j & 1) {
           const double* b = Bp + j * bj + k0 * bk;
 #pragma unroll
           for (int u = 0; u < KU; ++u) acc[j] = fma(a[u], b[u * bk], acc[j]);
@@ -494,7 +504,7 @@ __global__ void __launch_bounds__(DG_NT) dgemm_rows_kernel(GemmDescT<double> d, 
         const double a = a_at(k);
 #pragma unroll
         for (int j = 0; j < DG_NC; ++j)
-          if (j < nc) acc[j] = fma(a, Bp[j * bj + k * bk], acc[j]);
+          if (cols >> j & 1) acc[j] = fma(a, Bp[j * bj + k * bk], acc[j]);
       }
     }
   }
@@ -504,18 +514,18 @@ __global__ void __launch_bounds__(DG_NT) dgemm_rows_kernel(GemmDescT<double> d, 
   double v = 0.0;  // thread (warp, lane): column warp, row lane, the warps' sums in order
 #pragma unroll
   for (int w = 0; w < DG_NT / 32; ++w) v += red[w][warp][lane];
-  dg_finish<MODE>(d, v, row, (warp < nc) ? n0 + warp : d.N);
+  dg_finish<MODE>(d, v, row, (cols >> warp & 1) ? n0 + warp : d.N);
 }
 
 // op(A) = A^T, op(B) = B (both contiguous along K): the lanes of a warp share
 // K, each warp holds four rows x eight columns, and a butterfly that halves
 // the 32 sums at every step leaves one output per lane.
 __global__ void __launch_bounds__(DG_NT) dgemm_dots_kernel(GemmDescT<double> d, int64_t kper, int ncol) {
-  if (d.only_if && *d.only_if == 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t m0 = (int64_t)(blockIdx.x / cg::this_cluster().num_blocks()) * DG_ROWS + 4 * warp;
   const int64_t n0 = (int64_t)blockIdx.y * ncol;
-  const int nc = (int)((d.N - n0 < ncol) ? d.N - n0 : ncol);
+  const unsigned cols = dg_columns(d, (int)((d.N - n0 < ncol) ? d.N - n0 : ncol));
+  if (cols == 0) return;
   const int64_t kbeg = (int64_t)cg::this_cluster().block_rank() * kper;
   const int64_t kend = (kbeg + kper < d.K) ? kbeg + kper : d.K;
   const double* Ap[4];
@@ -531,7 +541,7 @@ __global__ void __launch_bounds__(DG_NT) dgemm_dots_kernel(GemmDescT<double> d, 
     for (int r = 0; r < 4; ++r) a[r] = Ap[r][k];
 #pragma unroll
     for (int j = 0; j < DG_NC; ++j)
-      if (j < nc) {
+      if (cols >> j & 1) {
         const double b = Bp[j * d.ldb + k];
 #pragma unroll
         for (int r = 0; r < 4; ++r) acc[r * DG_NC + j] = fma(a[r], b, acc[r * DG_NC + j]);
@@ -550,7 +560,7 @@ __global__ void __launch_bounds__(DG_NT) dgemm_dots_kernel(GemmDescT<double> d, 
     if (up) idx += half;
   }
   const int j = idx % DG_NC;
-  dg_finish<kGemmPlain>(d, acc[0], m0 + idx / DG_NC, (j < nc) ? n0 + j : d.N);
+  dg_finish<kGemmPlain>(d, acc[0], m0 + idx / DG_NC, (cols >> j & 1) ? n0 + j : d.N);
 }
 
 // Lower C = alpha (A B^T + A2 B2^T) + beta C of short sums (the reduction's
@@ -621,14 +631,17 @@ int launch_narrow(fraclap_ctx* ctx, const GemmDescT<double>& d, cudaStream_t st)
       part.N = (d.N - j < kMostCols) ? d.N - j : kMostCols;
       part.B += TB ? j : j * d.ldb;
       part.C += j * d.ldc;
+      if (d.only_marked) part.only_marked += j / DG_NC * cdiv(d.M, DG_ROWS);
       FL_TRY((launch_narrow<TA, TB, MODE>(ctx, part, st)));
     }
     return 0;
   }
   const int64_t gx = cdiv(d.M, DG_ROWS), gy = cdiv(d.N, DG_NC);
-  const int ncol = (int)cdiv(d.N, gy);  // the columns dealt evenly
+  static_assert(DG_ROWS == kGuardRows && DG_NC == kGuardCols, "the marks' tiles");
+  const int ncol = d.only_marked ? DG_NC : (int)cdiv(d.N, gy);  // the columns dealt evenly
   int S = 1;
-  while (S < 8 && gx * gy * S < 4 * sms && d.K >= 256 * (int64_t)S) S *= 2;
+  // (few tiles of a grid are marked: four CTAs a tile whatever the grid)
+  while (S < 8 && (gx * gy * S < 4 * sms || (d.only_marked && S < 4)) && d.K >= 256 * (int64_t)S) S *= 2;
   const int64_t kper = cdiv(cdiv(d.K > 0 ? d.K : 1, S), 32) * 32;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(gx * S), (unsigned)gy, 1);
@@ -673,7 +686,7 @@ int launch(fraclap_ctx* ctx, const GemmDescT<T>& d, int split_k, cudaStream_t st
   if constexpr (std::is_same<T, double>::value && MODE != kGemmLowerC && !(TA && TB)) {
     // (a caller that splits the sums of 64 tiles or more fills the SMs by itself)
     const bool own = TA && split_k > 1 && cdiv(d.M, BM) * cdiv(d.N, BN) >= 64;
-    if (d.K2 == 0 && !own && dg_narrow(ctx, TA, d.M, d.N)) return launch_narrow<TA, TB, MODE>(ctx, d, st);
+    if (d.only_marked || (d.K2 == 0 && !own && dg_narrow(ctx, TA, d.M, d.N))) return launch_narrow<TA, TB, MODE>(ctx, d, st);
   }
   if constexpr (std::is_same<T, double>::value && MODE == kGemmLowerC && !TA && TB) {
     // short sums; long ones take the 64 x 64 tile's shared memory

@@ -20,7 +20,7 @@ struct fraclap_ctx {
   double wait_timeout_s = 10.0;
   int tensor_route = 1;          // slice products: 1 = tcgen05 + TMA, 0 = mma.sync
   double refine_tau = 1e-3;      // first-order coefficient above which a pair is clustered
-  int apply_slices = 0;          // frac_apply products: 0 = FP64 engine, s = s BF16 slices (tensor cores)
+  int apply_slices = 0;          // frac_apply products: 0 = at FP64 accuracy, s = s BF16 slices (tensor cores)
   int oz_group = 8;              // slice-product kernel: tile rows per raster group (0 = all rows)
   int oz_bits = 7;               // slice-product kernel: digit width for K > 256 (7 or 8)
   int oz_tile_n = 256;           // slice-product kernel: tile columns (128, 192 or 256)
@@ -215,6 +215,7 @@ struct GemmDescT {
   int64_t K2;
   double alpha, beta;
   const int* only_if = nullptr;  // FP64: a device flag; 0 leaves C as it is
+  const unsigned* only_marked = nullptr;  // FP64 (plain, K2 = 0): an OzGuard's marks; the rest of C stays as it is
 };
 using GemmDesc = GemmDescT<double>;
 
@@ -312,11 +313,22 @@ int cluster_eig(fraclap_ctx* ctx, double* S, int64_t c, double* w, double* Q, Ar
                 cudaStream_t st);
 
 // FP64-accurate GEMM through BF16 tensor-core slices (ozaki.cu).
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false, int digits = 0, bool tight = false);
+// OzGuard: marks (device, a word per tile of kGuardRows x kGuardCols of C with a
+// bit per column, tiles of a tile column consecutive; zeroed by the caller) where
+// the digits may hold less than an FP64 sum; *nonfinite (device) an infinity or
+// NaN in an operand.
+struct OzGuard {
+  int* nonfinite;
+  unsigned* marks;
+};
+constexpr int kGuardRows = 32, kGuardCols = 8;
+constexpr float kGuardSum = 0.00390625f;
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false, int digits = 0, bool tight = false,
+                bool guard = false);
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
                int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits = 0,
-               int* nonfinite = nullptr);
+               const OzGuard* guard = nullptr);
 
 // Banded LDL^T (no pivoting) of the symmetric CSR matrix of half-bandwidth
 // b: Lb(t, j) = L(j + t, j), Lr(t, i) = L(i, i - t) (both ld b + 1, n

@@ -14,8 +14,9 @@
 // carry one bit more than the magnitude w that bounds the chunk (the sign),
 // so 7 digits (28 pairs) hold the 56 bits that sign-magnitude digits of w
 // bits need 8 (36 pairs) for, at the same chunk length.  Pairs with p + q < D
-// are kept; the dropped tail and the rounding of the last digit are below
-// about 2^-rD relative to |row max| |column max| per term, with either sign.
+// are kept; the D - 1 dropped pairs of the next diagonal and the rounding of the
+// last digit are below about (D + 1) 2^-rD (r D = 64: 2 (D + 1) 2^-rD) relative to
+// |row max| |column max| per term, with either sign.
 // The result C = alpha 2^(e_i + f_j) sum + beta C is formed in FP64.
 //
 // Two tensor-core kernels compute the slice products: the sm_103a one uses
@@ -138,6 +139,15 @@ __host__ __device__ inline unsigned long long digit_bias(int w, int D) {
 // conversion instruction).
 __device__ __forceinline__ float field_value(uint32_t f, float off) { return __uint_as_float(0x4B000000u | f) - off; }
 
+// The bits of |a| 2^-e (a of a row of exponent e, so below 1) as BF16, rounded
+// towards zero; a nonzero entry below 2^-60 (or subnormal) counts as 2^-60.
+__device__ __forceinline__ uint32_t magnitude_bits(double a, int e) {
+  const unsigned long long t = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFull;
+  if (t == 0) return 0u;
+  const int E = (int)(t >> 52), f = E - 1023 - e + 127;
+  return (E == 0 || f < 67) ? 67u << 7 : ((uint32_t)f << 7) | (uint32_t)((t >> 45) & 127u);
+}
+
 // The D digits of one entry a of row i (exponent e = ex[i]) into S[p * pstride].
 __device__ __forceinline__ void write_digits(double a, int e, int D, int w, __nv_bfloat16* S, int64_t pstride) {
   const int rb = w + 1;
@@ -161,7 +171,7 @@ __device__ __forceinline__ void write_digits(double a, int e, int D, int w, __nv
 }
 
 __global__ void make_slices(const double* A, int64_t lda, bool trans, int64_t M, int64_t K,
-                            int64_t Kp, const int* ex, int D, int w, __nv_bfloat16* S) {
+                            int64_t Kp, const int* ex, int D, int w, int mag, __nv_bfloat16* S) {
   const int64_t total = M * Kp;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -169,6 +179,7 @@ __global__ void make_slices(const double* A, int64_t lda, bool trans, int64_t M,
     if (trans) { k = t % Kp; i = t / Kp; } else { i = t % M; k = t / M; }
     const double a = (k < K) ? (trans ? A[k + i * lda] : A[i + k * lda]) : 0.0;
     write_digits(a, ex[i], D, w, S + i * Kp + k, M * Kp);
+    if (mag) S[D * M * Kp + i * Kp + k] = __ushort_as_bfloat16((unsigned short)magnitude_bits(a, ex[i]));
   }
 }
 
@@ -185,10 +196,18 @@ __device__ __forceinline__ void put_eight(const unsigned long long (&v)[8], int 
   *reinterpret_cast<uint4*>(out) = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
+// Eight magnitudes as a 16-byte store.
+__device__ __forceinline__ void put_eight(const uint32_t (&m)[8], __nv_bfloat16* out) {
+  *reinterpret_cast<uint4*>(out) =
+      make_uint4(m[0] | m[1] << 16, m[2] | m[3] << 16, m[4] | m[5] << 16, m[6] | m[7] << 16);
+}
+
 // The slices of an operand whose rows are contiguous (trans), for r D <= 64:
 // a thread takes eight consecutive entries of a row and writes each digit's
 // eight BF16 values as one 16-byte store (Kp is a multiple of 64, so every
-// store is aligned); the digits are those of write_digits.
+// store is aligned); the digits are those of write_digits.  MAG: the magnitudes
+// are one plane more.
+template <bool MAG>
 __global__ void make_slices_rows(const double* A, int64_t lda, int64_t M, int64_t K, int64_t Kp,
                                  const int* ex, int D, int w, __nv_bfloat16* S) {
   const int64_t per_row = Kp / 8, total = M * per_row;
@@ -200,8 +219,14 @@ __global__ void make_slices_rows(const double* A, int64_t lda, int64_t M, int64_
     const int64_t i = t / per_row, k0 = (t % per_row) * 8;
     const int e = ex[i];
     unsigned long long v[8];
+    uint32_t m[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = biased_digits((k0 + q < K) ? A[k0 + q + i * lda] : 0.0, e, tb, bias);
+    for (int q = 0; q < 8; ++q) {
+      const double a = (k0 + q < K) ? A[k0 + q + i * lda] : 0.0;
+      v[q] = biased_digits(a, e, tb, bias);
+      if (MAG) m[q] = magnitude_bits(a, e);
+    }
+    if (MAG) put_eight(m, S + ((int64_t)D * M + i) * Kp + k0);
     for (int p = 0; p < D; ++p) put_eight(v, rb * (D - 1 - p), p > 0 ? (1u << rb) - 1u : 0xFFFFFFFFu, off,
                                           S + ((int64_t)p * M + i) * Kp + k0);
   }
@@ -213,6 +238,7 @@ __global__ void make_slices_rows(const double* A, int64_t lda, int64_t M, int64_
 // store, so that eight lanes fill a 128-byte line (a 2-byte store per lane and
 // digit before: exponents and slices of an 8835 x 8835 operand at 7 digits 0.77
 // -> 0.58 ms).  256 threads; grid (ceil(M / 64), Kp / 64).
+template <bool MAG>
 __global__ void __launch_bounds__(256) make_slices_strided(const double* A, int64_t lda, int64_t M, int64_t K,
                                                            int64_t Kp, const int* ex, int D, int w, __nv_bfloat16* S) {
   __shared__ double tile[64][65];
@@ -233,6 +259,12 @@ __global__ void __launch_bounds__(256) make_slices_strided(const double* A, int6
     unsigned long long v[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) v[q] = biased_digits(tile[kk + q][r], e, tb, bias);
+    if (MAG) {
+      uint32_t m[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) m[q] = magnitude_bits(tile[kk + q][r], e);
+      put_eight(m, S + D * M * Kp + i * Kp + k0 + kk);
+    }
     for (int p = 0; p < D; ++p) put_eight(v, rb * (D - 1 - p), p > 0 ? (1u << rb) - 1u : 0xFFFFFFFFu, off,
                                           S + ((int64_t)p * M + i) * Kp + k0 + kk);
   }
@@ -389,21 +421,33 @@ __device__ __forceinline__ double pow2i(int e) { return __longlong_as_double((lo
 // the longest items start first.  An item adds at most kMaxChunks chunk sums,
 // which fit 31 bits (127 2^24 < 2^31); K beyond that many chunks is multiplied
 // in ranges (see ozaki_gemm).
+// Guarded products (see ozaki_gemm) keep one diagonal more, dg = D, and have a
+// last item that multiplies the magnitudes (plane D of both operands).
 constexpr int kMaxChunks = 127;
 struct OzParts {
-  int D, U, nchunk;
-  __host__ __device__ int of_diag(int dg) const { return (dg + U) / U; }
-  __host__ __device__ int count() const {
+  int D, U, nchunk, guard;
+  __host__ __device__ int top() const { return D - 1 + guard; }
+  __host__ __device__ int pairs(int dg) const { return dg < D ? dg + 1 : 2 * D - 1 - dg; }
+  __host__ __device__ int of_diag(int dg) const { return (pairs(dg) + U - 1) / U; }
+  __host__ __device__ int count() const {  // items of digits
     int t = 0;
-    for (int dg = 0; dg < D; ++dg) t += of_diag(dg);
+    for (int dg = 0; dg <= top(); ++dg) t += of_diag(dg);
     return t;
   }
+  __host__ __device__ int items() const { return count() + guard; }
   __device__ void get(int part, int* dg, int* p0, int* p1) const {
-    int d = D - 1;
-    while (part >= of_diag(d)) part -= of_diag(d--);
+    int d = top();
+    while (d >= 0 && part >= of_diag(d)) part -= of_diag(d--);
+    if (d < 0) {  // the magnitudes
+      *dg = 2 * D;
+      *p0 = D;
+      *p1 = D + 1;
+      return;
+    }
+    const int first = d < D ? 0 : d - D + 1, end = first + pairs(d);
     *dg = d;
-    *p0 = part * U;
-    *p1 = (*p0 + U < d + 1) ? *p0 + U : d + 1;
+    *p0 = first + part * U;
+    *p1 = (*p0 + U < end) ? *p0 + U : end;
   }
 };
 // A plane: M x N column-major, or (lower, M >= N) its columns from the diagonal
@@ -417,13 +461,14 @@ __host__ __device__ inline int64_t plane_column(int64_t j, int64_t M, bool lower
 // U: all pairs of a diagonal, fewer when the longest item would then exceed an
 // even share of all pairs over the SMs (a function of the sizes alone, so that
 // the workspace and the sums do not depend on the context).
-inline OzParts oz_parts(int64_t M, int64_t N, int64_t Kp, int D, int w, bool lower) {
+inline OzParts oz_parts(int64_t M, int64_t N, int64_t Kp, int D, int w, bool lower, bool guard) {
   OzParts o;
   const int64_t chunk = (int64_t)1 << (24 - 2 * w);
   o.D = D;
+  o.guard = (guard && D > 1) ? 1 : 0;
   o.nchunk = (int)cdiv(Kp, chunk);
   const int64_t tiles = cdiv(M, TC_M) * cdiv(N, TC_M) / (lower ? 2 : 1);
-  const int64_t even = cdiv(std::max<int64_t>(tiles, 1) * (D * (D + 1) / 2), 152);
+  const int64_t even = cdiv(std::max<int64_t>(tiles, 1) * (D * (D + 1) / 2 + o.guard * D), 152);
   o.U = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(D, even), kMaxChunks / o.nchunk));
   return o;
 }
@@ -481,7 +526,7 @@ __device__ __forceinline__ void ozaki_tile_of(int64_t idx, int TM, int TN, int G
 // the whole pipeline (its peers need its share of B), also when its tile
 // lies past the last row or above the diagonal; its epilogue then writes
 // nothing.
-template <int TCN, int CS>
+template <int TCN, int CS, bool GUARD>
 __global__ void __launch_bounds__(OzTile<TCN>::THREADS, 1)
 ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int64_t M, int64_t N,
                 int64_t Kp, OzParts parts, int64_t chunk, int tiles, int32_t* P, int lower, int group, long long limit,
@@ -643,6 +688,7 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
 #pragma unroll
     for (int j = 0; j < TC_EPI_COLS; ++j) acc[j] = 0;
     const int nacc = (pend - pbeg) * nchunk;
+    const bool magnitudes = GUARD && pbeg == parts.D;
     bool ok = true;
     for (int chunk_i = 0; chunk_i < nacc; ++chunk_i) {
       const int buf = chunk_i % NBUF;
@@ -657,8 +703,13 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
         uint32_t r[16];
         tmem_ld16(taddr + j0, r);
         tmem_wait_ld();
+        if (!magnitudes) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j0 + j] += __float2int_rz(__uint_as_float(r[j]));
+          for (int j = 0; j < 16; ++j) acc[j0 + j] += __float2int_rz(__uint_as_float(r[j]));
+        } else {  // a sum of FP32, in the same registers
+#pragma unroll
+          for (int j = 0; j < 16; ++j) acc[j0 + j] = __float_as_int(__int_as_float(acc[j0 + j]) + __uint_as_float(r[j]));
+        }
       }
       tc_fence_before();
       __syncwarp();
@@ -692,11 +743,14 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
 // diagonal is at most D kMaxChunks chunk sums of 2^24, below 2^34.2, and three
 // shifts of at most 9 bits follow, so that a group stays below 2^61.3.  An
 // element costs a conversion and an FMA per four diagonals; the lowest diagonals
-// are added first.
+// are added first.  Guarded (never lower): a column of 32 rows with an entry whose
+// sum of magnitudes is neither 0 nor at least kGuardSum is marked (i0, j0: the
+// block's place in C, rows32: tiles along the rows).
 __global__ void combine_planes(const int32_t* __restrict__ P, const int* __restrict__ ea, const int* __restrict__ eb,
                                int64_t M, int64_t N, OzParts parts, int w, double alpha, double beta, double* C,
-                               int64_t ldc, int lower) {
+                               int64_t ldc, int lower, unsigned* marks, int64_t i0, int64_t j0, int64_t rows32) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = plane_size(M, N, lower != 0);
+  const unsigned lanes = __ballot_sync(0xffffffffu, i < M);
   if (i >= M) return;
   const int rb = w + 1, D = parts.D;
   const int e0 = ea[i] - 2 * digit_frac_bits(w, D) + rb * (2 * D - 2);
@@ -705,7 +759,7 @@ __global__ void combine_planes(const int32_t* __restrict__ P, const int* __restr
     const int32_t* q = P + i + plane_column(j, M, lower != 0);
     double v = 0.0;
     int plane = 0;
-    for (int d = D - 1; d >= 0;) {  // planes from the highest dg (lowest weight) up
+    for (int d = parts.top(); d >= 0;) {  // planes from the highest dg (lowest weight) up
       const int lo = (d >= 4) ? d - 3 : 0, g = d - lo + 1;
       long long acc = 0;  // in units of 2^(-rb d), d the group's highest diagonal
       for (int sh = 0; d >= lo; --d, sh += rb) {
@@ -724,6 +778,12 @@ __global__ void combine_planes(const int32_t* __restrict__ P, const int* __restr
     }
     double* c = C + i + j * ldc;
     *c = (beta == 0.0) ? v : v + beta * *c;
+    if (parts.guard) {
+      const float sum = __int_as_float(__ldcs(q + plane * stride));
+      const bool mark = __any_sync(lanes, sum != 0.0f && !(sum >= kGuardSum));
+      if (mark && threadIdx.x % 32 == 0)
+        atomicOr(marks + ((j0 + j) / kGuardCols * rows32 + (i0 + i) / kGuardRows), 1u << ((j0 + j) % kGuardCols));
+    }
   }
 }
 
@@ -739,22 +799,23 @@ bool slice_map(CUtensorMap* map, const __nv_bfloat16* S, int64_t rows, int64_t o
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-template <int TCN, int CS>
+template <int TCN, int CS, bool GUARD>
 int launch_tc(fraclap_ctx* ctx, const __nv_bfloat16* SA, const __nv_bfloat16* SB, int64_t M, int64_t N, int64_t arows,
               int64_t Kp, const OzParts& parts, int64_t chunk, int32_t* P, bool lower, cudaStream_t st) {
   CUtensorMap ma, mb;
-  FL_CHECK(ctx, slice_map(&ma, SA, M, arows, Kp, parts.D, TC_M) && slice_map(&mb, SB, N, N, Kp, parts.D, TCN / CS),
+  const int planes = parts.D + parts.guard;
+  FL_CHECK(ctx, slice_map(&ma, SA, M, arows, Kp, planes, TC_M) && slice_map(&mb, SB, N, N, Kp, planes, TCN / CS),
            FRACLAP_ERR_CUDA, "ozaki_gemm: tensor map encoding failed");
   const size_t smem = (size_t)OzTile<TCN>::STAGES * OzTile<TCN>::STAGE_BYTES + 1024;
-  auto kern = ozaki_tc_kernel<TCN, CS>;
+  auto kern = ozaki_tc_kernel<TCN, CS, GUARD>;
   FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   // the raster counts clusters of CS tile rows (a tile of CS * 128 rows)
   const int TM = (int)cdiv(cdiv(M, TC_M), CS), TN = (int)cdiv(N, TCN);
   const int G = std::max(1, std::min(ctx->oz_group > 0 ? ctx->oz_group : TM, TM));
   const int64_t tiles = ozaki_tile_count(TM, TN, G, lower, CS * TC_M, TCN);
-  FL_CHECK(ctx, tiles * parts.count() * CS <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: too many tiles");
+  FL_CHECK(ctx, tiles * parts.items() * CS <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: too many tiles");
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * parts.count() * CS));
+  cfg.gridDim = dim3((unsigned)(tiles * parts.items() * CS));
   cfg.blockDim = dim3(OzTile<TCN>::THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -777,10 +838,10 @@ static int64_t oz_range(int w) { return (int64_t)kMaxChunks << (24 - 2 * w); }
 // The most digits that s slices are cut into (see ozaki_gemm), and the most
 // planes of the tensor-core route for up to that many, at either digit width.
 static int max_digits(int s) { return (s <= 5 || s == 8) ? s + 1 : s; }
-static int max_planes(int64_t M, int64_t N, int64_t Kp, int D, bool lower) {
+static int max_planes(int64_t M, int64_t N, int64_t Kp, int D, bool lower, bool guard) {
   int t = 0;
   for (int d = 1; d <= D; ++d)
-    for (int w = 7; w <= 8; ++w) t = std::max(t, oz_parts(M, N, std::min(Kp, oz_range(w)), d, w, lower).count());
+    for (int w = 7; w <= 8; ++w) t = std::max(t, oz_parts(M, N, std::min(Kp, oz_range(w)), d, w, lower, guard).items());
   return t;
 }
 static int64_t padded(int64_t K) { return cdiv(std::max<int64_t>(K, 1), OZ_KPAD) * OZ_KPAD; }
@@ -841,9 +902,10 @@ static OzBlocks oz_blocks(int64_t M, int64_t N, int64_t Kp, int D, int planes, b
 // without planes where that is more (16 (M + N) K bytes for 7 slices; `tight`:
 // only that): no product needs more than it did when every diagonal was folded
 // into C on the fly, but for small ones.
-size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits, bool tight) {
+size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits, bool tight, bool guard) {
   const int64_t Kp = padded(std::min(K, oz_range(7)));
-  const int D = (digits > 0) ? digits : max_digits(s), planes = max_planes(M, N, Kp, D, lower);
+  const int digs = (digits > 0) ? digits : max_digits(s), planes = max_planes(M, N, Kp, digs, lower, guard);
+  const int D = digs + (guard ? 1 : 0);  // and the magnitudes
   const size_t whole = oz_bytes(M, {M, N}, Kp, D, planes, lower);
   const size_t least = oz_bytes(M, {lower ? M : std::min<int64_t>(M, 1024), std::min<int64_t>(N, 256)}, Kp, D, planes, lower);
   const size_t fold = align256((size_t)((8 * s + 6) / 7) * 2 * (size_t)(M + N) * (size_t)padded(K));
@@ -855,7 +917,8 @@ size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower, int digits, 
 // column-parallel maximum and the tiled slicing.  More than 64 bits of digits
 // take the general kernel.
 int slice_operand(fraclap_ctx* ctx, const double* X, int64_t ldx, bool trans, int64_t R, int64_t K, int64_t Kp,
-                  int sl, int bits, int* ex, __nv_bfloat16* S, unsigned long long* mx, int* nonfinite, cudaStream_t st) {
+                  int sl, int bits, bool mag, int* ex, __nv_bfloat16* S, unsigned long long* mx, int* nonfinite,
+                  cudaStream_t st) {
   const bool fits = sl * (bits + 1) <= 64;
   if (trans) {
     row_exponents<<<(unsigned)R, 256, 0, st>>>(X, ldx, K, ex, nonfinite);
@@ -869,28 +932,30 @@ int slice_operand(fraclap_ctx* ctx, const double* X, int64_t ldx, bool trans, in
   count_launch(ctx);
   if (trans && fits) {
     const unsigned gs = (unsigned)std::min<int64_t>(cdiv(R * (Kp / 8), 256), 152 * 16);
-    make_slices_rows<<<gs, 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl, bits, S);
+    (mag ? make_slices_rows<true> : make_slices_rows<false>)<<<gs, 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl, bits, S);
   } else if (fits) {  // (K of a range: both grids' second dimension is below 2100)
-    make_slices_strided<<<dim3((unsigned)cdiv(R, 64), (unsigned)(Kp / 64)), 256, 0, st>>>(X, ldx, R, K, Kp, ex, sl,
-                                                                                         bits, S);
+    (mag ? make_slices_strided<true> : make_slices_strided<false>)<<<dim3((unsigned)cdiv(R, 64), (unsigned)(Kp / 64)),
+                                                                     256, 0, st>>>(X, ldx, R, K, Kp, ex, sl, bits, S);
   } else {
     const unsigned gs = (unsigned)std::min<int64_t>(cdiv(R * Kp, 256), 152 * 32);
-    make_slices<<<gs, 256, 0, st>>>(X, ldx, trans, R, K, Kp, ex, sl, bits, S);
+    make_slices<<<gs, 256, 0, st>>>(X, ldx, trans, R, K, Kp, ex, sl, bits, mag ? 1 : 0, S);
   }
   count_launch(ctx);
   FL_CUDA(ctx, cudaGetLastError());
   return 0;
 }
 
-// One block of C: M rows of A's slices (of `arows`), N columns of B's.
+// One block of C from (i0, j0): M rows of A's slices (of `arows`), N columns of B's.
 static int ozaki_block(fraclap_ctx* ctx, const OzScratch& z, const __nv_bfloat16* SA, const int* ea, int64_t M, int64_t N,
                        int64_t arows, int64_t Kp, const OzParts& parts, int bits, double alpha, double beta, double* C,
-                       int64_t ldc, bool lower, cudaStream_t st) {
+                       int64_t ldc, bool lower, const OzGuard* guard, int64_t i0, int64_t j0, cudaStream_t st) {
   const int64_t chunk = (int64_t)1 << (24 - 2 * bits);
   if (ctx->tensor_route == 1) {
     const int tw = (N <= 128) ? 128 : ctx->oz_tile_n;  // a narrow output takes the 128-column tile
     const int cs = ctx->oz_cluster;
-#define FL_OZ_LAUNCH(W, K) launch_tc<W, K>(ctx, SA, z.SB, M, N, arows, Kp, parts, chunk, z.P, lower, st)
+#define FL_OZ_LAUNCH(W, K)                                                                          \
+  (parts.guard ? launch_tc<W, K, true>(ctx, SA, z.SB, M, N, arows, Kp, parts, chunk, z.P, lower, st) \
+               : launch_tc<W, K, false>(ctx, SA, z.SB, M, N, arows, Kp, parts, chunk, z.P, lower, st))
     if (cs == 2) {
       FL_TRY(tw == 256 ? FL_OZ_LAUNCH(256, 2) : tw == 192 ? FL_OZ_LAUNCH(192, 2) : FL_OZ_LAUNCH(128, 2));
     } else {
@@ -899,7 +964,8 @@ static int ozaki_block(fraclap_ctx* ctx, const OzScratch& z, const __nv_bfloat16
 #undef FL_OZ_LAUNCH
     count_launch(ctx);
     combine_planes<<<dim3((unsigned)cdiv(M, 256), (unsigned)std::min<int64_t>(N, 16384)), 256, 0, st>>>(
-        z.P, ea, z.eb, M, N, parts, bits, alpha, beta, C, ldc, lower ? 1 : 0);
+        z.P, ea, z.eb, M, N, parts, bits, alpha, beta, C, ldc, lower ? 1 : 0, guard ? guard->marks : nullptr, i0, j0,
+        cdiv(arows, kGuardRows));
   } else {
     dim3 grid((unsigned)cdiv(M, OZ_BM), (unsigned)cdiv(N, OZ_BN));
     ozaki_kernel<<<grid, OZ_NT, 0, st>>>(SA, z.SB, ea, z.eb, M, N, arows, Kp, parts.D, bits, chunk, alpha, beta, C, ldc,
@@ -913,21 +979,24 @@ static int ozaki_block(fraclap_ctx* ctx, const OzScratch& z, const __nv_bfloat16
 // One range of K (see ozaki_gemm): D digits of magnitude `bits` per operand.
 static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double* A,
                        int64_t lda, const double* B, int64_t ldb, double beta, double* C, int64_t ldc, int D, int bits,
-                       bool lower, Arena ar, cudaStream_t st, int* nonfinite) {
+                       bool lower, Arena ar, cudaStream_t st, const OzGuard* guard) {
   const int64_t Kp = padded(K);
-  const OzParts parts = oz_parts(M, N, Kp, D, bits, lower);
-  const OzBlocks c = oz_blocks(M, N, Kp, D, parts.count(), lower, ar.cap - ar.off);
+  const OzParts parts = oz_parts(M, N, Kp, D, bits, lower, guard != nullptr);
+  const bool mag = parts.guard != 0;
+  int* nonfinite = guard ? guard->nonfinite : nullptr;
+  const OzBlocks c = oz_blocks(M, N, Kp, D + mag, parts.items(), lower, ar.cap - ar.off);
   FL_CHECK(ctx, c.mb > 0, FRACLAP_ERR_ALLOC, "ozaki_gemm: workspace too small");
-  const OzScratch z = oz_take(&ar, M, c, Kp, D, parts.count(), lower);
+  const OzScratch z = oz_take(&ar, M, c, Kp, D + mag, parts.items(), lower);
   // rows of op(A) and columns of op(B): contiguous when trans, else strided
-  FL_TRY(slice_operand(ctx, A, lda, ta, M, K, Kp, D, bits, z.ea, z.SA, z.mx, nonfinite, st));
+  FL_TRY(slice_operand(ctx, A, lda, ta, M, K, Kp, D, bits, mag, z.ea, z.SA, z.mx, nonfinite, st));
   for (int64_t j = 0; j < N; j += c.nb) {
     const int64_t nb = std::min(c.nb, N - j);
-    FL_TRY(slice_operand(ctx, B + (tb ? j : j * ldb), ldb, !tb, nb, K, Kp, D, bits, z.eb, z.SB, z.mx, nonfinite, st));
+    FL_TRY(slice_operand(ctx, B + (tb ? j : j * ldb), ldb, !tb, nb, K, Kp, D, bits, mag, z.eb, z.SB, z.mx, nonfinite, st));
     StageTimer tm(ctx, kStageSliceProducts, st);
     for (int64_t i = lower ? j : 0; i < M; i += lower ? M : c.mb) {
       const int64_t mb = lower ? M - j : std::min(c.mb, M - i);
-      FL_TRY(ozaki_block(ctx, z, z.SA + i * Kp, z.ea + i, mb, nb, M, Kp, parts, bits, alpha, beta, C + i + j * ldc, ldc, lower, st));
+      FL_TRY(ozaki_block(ctx, z, z.SA + i * Kp, z.ea + i, mb, nb, M, Kp, parts, bits, alpha, beta, C + i + j * ldc, ldc, lower,
+                         guard, i, j, st));
     }
   }
   return 0;
@@ -935,12 +1004,21 @@ static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N,
 
 // C = alpha op(A) op(B) + beta C, FP64-accurate through s BF16 slices
 // (s = 7 for full FP64 accuracy of the products).  lower: only C(i,j), i >= j.
-// digits > 0 sets the digits per operand itself (8 bits each at w = 7);
-// nonfinite (device, may be null) is set to 1 when an operand holds an infinity
-// or NaN, which the digits do not represent: C is then meaningless.
+// digits > 0 sets the digits per operand itself (8 bits each at w = 7).
+// guard (may be null) keeps the diagonal p + q = D too and tells which entries
+// the digits hold to the accuracy of an FP64 sum.  The digits are relative to
+// the largest entry of the row of op(A) and the column of op(B); in units of
+// 2^(e_i + f_j), an entry of C is off by at most K (2 2^-63 + 6 2^-70) < K 2^-61.9
+// for 8 digits, an FP64 sum by K 2^-53 times the sum of its terms' magnitudes.  A
+// product of the magnitudes (8 bits each, rounded down) gives that sum: where it
+// is at least kGuardSum = 2^-8 the digits' bound is K 2^-53.9 of it, and where it
+// is 0 every term is; columns of 32 rows with any other entry are marked for the
+// caller's FP64 product (2^-6 marked 2 % of the tiles of the n = 8835 apply, the
+// nodes beside the corners, for 0.4 ms more).  An infinity or NaN, which has no digits, sets *nonfinite: C is
+// then meaningless.
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
-               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits, int* nonfinite) {
+               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits, const OzGuard* guard) {
   if (M <= 0 || N <= 0) return 0;
   FL_CHECK(ctx, s >= 1 && s <= 8, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: slices must be 1..8");
   FL_CHECK(ctx, cdiv(N, OZ_BN) <= 65535, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: N too large");
@@ -967,7 +1045,7 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   do {
     const int64_t kr = std::min(K - k0, oz_range(bits));
     FL_TRY(ozaki_range(ctx, ta, tb, M, N, kr, alpha, A + (ta ? k0 : k0 * lda), lda, B + (tb ? k0 * ldb : k0), ldb,
-                       k0 == 0 ? beta : 1.0, C, ldc, sl, bits, lower, *ar, st, nonfinite));
+                       k0 == 0 ? beta : 1.0, C, ldc, sl, bits, lower, *ar, st, guard));
     k0 += kr;
   } while (k0 < K);
   return 0;
