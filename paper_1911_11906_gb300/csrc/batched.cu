@@ -113,20 +113,27 @@ extern "C" int fraclap_solve_batched(fraclap_ctx* ctx, const fraclap_problem* pr
     const double n = (double)probs[i].n;
     load[w] += n * n * n + 1.0;
   }
-  // size every worker's workspace before any launch (growing it later would synchronise)
+  // size every worker's workspace before any launch (growing it later would
+  // synchronise); applies that have no room for their digits take the FP64 engine
   for (int w = 0; w < W; ++w) {
-    size_t need = 0;
+    size_t need = 0, least = 0;
     for (int i : plan[w]) {
       const fraclap_problem& p = probs[i];
       if (p.n == 0) continue;
-      need = std::max(need, p.rowptr_dev ? fraclap_eig_mixed_workspace_bytes(ctx->workers[w], p.n)
-                                         : fraclap_eig_workspace_bytes(ctx->workers[w], p.n));
-      if (p.k > 0) need = std::max(need, fraclap_apply_workspace_bytes_ctx(ctx->workers[w], p.n, p.m, p.k));
+      least = std::max(least, p.rowptr_dev ? fraclap_eig_mixed_workspace_bytes(ctx->workers[w], p.n)
+                                           : fraclap_eig_workspace_bytes(ctx->workers[w], p.n));
+      if (p.k > 0) {
+        least = std::max(least, fraclap_apply_workspace_bytes(p.n, p.m, p.k));
+        need = std::max(need, fraclap_apply_workspace_bytes_ctx(ctx->workers[w], p.n, p.m, p.k));
+      }
+      need = std::max(need, least);
     }
     if (need == 0) continue;
     Arena ar;
     fraclap_ctx* wc = ctx->workers[w];
-    if (get_workspace(wc, nullptr, 0, need, &ar)) return set_error(ctx, FRACLAP_ERR_ALLOC, "solve_batched: %s", wc->last_error.c_str());
+    int rc = get_workspace(wc, nullptr, 0, need, &ar);
+    if (rc == FRACLAP_ERR_ALLOC && least < need) rc = get_workspace(wc, nullptr, 0, least, &ar);
+    if (rc) return set_error(ctx, FRACLAP_ERR_ALLOC, "solve_batched: %s", wc->last_error.c_str());
   }
   FL_CUDA(ctx, cudaEventRecord(ctx->batch_start, (cudaStream_t)stream));
   for (int w = 0; w < W; ++w) FL_CUDA(ctx, cudaStreamWaitEvent(ctx->worker_streams[w], ctx->batch_start, 0));
@@ -145,7 +152,7 @@ extern "C" int fraclap_solve_batched(fraclap_ctx* ctx, const fraclap_problem* pr
                    : eig_full(wc, p.A_dev, p.n, p.lda, p.lambda_dev, p.V_dev, p.ldv, nullptr, 0, nullptr, s);
       if (rc == 0 && p.k > 0)
         rc = frac_apply(wc, p.V_dev, p.ldv, p.lambda_dev, p.n, p.F_dev, p.ldf, p.m, p.pair_f_dev,
-                        p.pair_alpha_dev, p.k, p.U_dev, p.ldu, nullptr, 0, s);
+                        p.pair_alpha_dev, p.k, p.U_dev, p.ldu, wc->ws, wc->ws_bytes, s);
       if (rc) {
         rcs[w] = rc;
         failed[w] = i;

@@ -310,11 +310,13 @@ extern "C" int frac_apply_mass(fraclap_ctx* ctx, const double* Phi_dev, int64_t 
   FL_CHECK(ctx, rowptr_dev && col_dev && valM_dev && F_dev, FRACLAP_ERR_INVALID_ARG, "frac_apply_mass: null pointer");
   FL_CHECK(ctx, ldf >= n, FRACLAP_ERR_INVALID_ARG, "frac_apply_mass: ldf < n");
   Arena ar;
-  size_t need = fraclap_apply_mass_workspace_bytes(ctx, n, m, k);
-  // FP64 products: the sizes without the digits' scratch do too (see frac_apply)
-  if (work_dev && ctx->apply_slices == 0)
-    need = std::min(need, need - fraclap_apply_workspace_bytes_ctx(ctx, n, m, k) + fraclap_apply_workspace_bytes(n, m, k));
-  FL_TRY(get_workspace(ctx, work_dev, work_bytes, need, &ar));
+  // FP64 products: the size without the digits' scratch does too (see frac_apply)
+  const size_t need = fraclap_apply_mass_workspace_bytes(ctx, n, m, k);
+  const size_t least = ctx->apply_slices == 0 ? need - fraclap_apply_workspace_bytes_ctx(ctx, n, m, k) +
+                                                    fraclap_apply_workspace_bytes(n, m, k) : need;
+  int rc = get_workspace(ctx, work_dev, work_bytes, work_dev ? least : need, &ar);
+  if (rc == FRACLAP_ERR_ALLOC && least < need) rc = get_workspace(ctx, work_dev, work_bytes, least, &ar);
+  if (rc != 0) return rc;
   double* B = ar.take<double>(n * m);
   FL_CHECK(ctx, B != nullptr, FRACLAP_ERR_ALLOC, "frac_apply_mass: workspace too small");
   csr_spmm<<<dim3((unsigned)cdiv(n, 256), (unsigned)m), 256, 0, st>>>(n, rowptr_dev, col_dev, valM_dev, F_dev, ldf,
