@@ -83,7 +83,7 @@ __global__ void widen(const float* Z, int64_t n, double* V, int64_t ldv) {
 
 template <class T>
 struct EigWork {
-  T* Aw;          // n x n working copy (later the transposed eigenvectors)
+  T* Aw;          // n x n working copy (then the bulge chasing's betas, later the transposed eigenvectors)
   T* band;        // 2b x n
   double* d;      // n
   double* e;      // n
@@ -102,6 +102,7 @@ int eig_take(Arena* ar, const fraclap_ctx* ctx, int64_t n, EigWork<T>* w) {
   w->W1 = ar->take<T>((int64_t)b * n);
   stage1_take<T>(ar, n, b, ctx->sm_count, &w->s1);
   stage2_take<T>(ar, n, b, &w->s2);
+  w->s2.beta = w->Aw;  // free once the band is extracted; (n - 1) kmax <= n^2
   return 0;
 }
 
@@ -161,12 +162,22 @@ int reduce(fraclap_ctx* ctx, const double* A, int64_t n, int64_t lda, EigWork<T>
   return 0;
 }
 
+// `free`: the rest of the workspace (the tridiagonal solver's buffers among it),
+// for the block factors; without room there they take the panels' buffers, a step
+// or more at a time.
 template <class T>
-int back_transform(fraclap_ctx* ctx, int64_t n, EigWork<T>* w, T* Z, int64_t ldz, cudaStream_t st) {
+int back_transform(fraclap_ctx* ctx, int64_t n, EigWork<T>* w, T* Z, int64_t ldz, Arena free, cudaStream_t st) {
   const int b = ctx->band_width;
+  T* ut = w->s1.XX;
+  int64_t ut_len = w->s1.xx_len;
+  const int64_t room = (int64_t)((free.cap - std::min(free.cap, free.off)) / 256 * 256 / sizeof(T));
+  if (room > ut_len) {
+    ut = free.take<T>(room);
+    ut_len = room;
+  }
   {
     StageTimer t(ctx, kStageBackQ2, st);
-    FL_TRY(q2_apply_run<T>(ctx, &w->s2, n, b, Z, ldz, n, w->Aw, n, st));
+    FL_TRY(q2_apply_run<T>(ctx, &w->s2, n, b, Z, ldz, n, w->Aw, n, ut, ut_len, st));
   }
   {
     StageTimer t(ctx, kStageBackQ1, st);
@@ -186,8 +197,9 @@ int cluster_eig(fraclap_ctx* ctx, double* S, int64_t c, double* w, double* Q, Ar
   eig_take<double>(ar, ctx, c, &ew);
   FL_CHECK(ctx, ew.s2.progress != nullptr, FRACLAP_ERR_ALLOC, "cluster eig: workspace too small");
   FL_TRY(reduce<double>(ctx, S, c, c, &ew, st));
+  const Arena rest = *ar;
   FL_TRY(stedc_run<double>(ctx, ew.d, ew.e, c, w, Q, c, ar, st));
-  FL_TRY(back_transform<double>(ctx, c, &ew, Q, c, st));
+  FL_TRY(back_transform<double>(ctx, c, &ew, Q, c, rest, st));
   return 0;
 }
 
@@ -300,11 +312,12 @@ extern "C" int eig_full(fraclap_ctx* ctx, const double* A_dev, int64_t n, int64_
   eig_take<double>(&ar, ctx, n, &w);
   FL_CHECK(ctx, w.s2.progress != nullptr, FRACLAP_ERR_ALLOC, "eig_full: workspace too small");
   FL_TRY(reduce<double>(ctx, A_dev, n, lda, &w, st));
+  const Arena rest = ar;
   {
     StageTimer t(ctx, kStageTridiagDC, st);
     FL_TRY(stedc_run<double>(ctx, w.d, w.e, n, lambda_dev, V_dev, ldv, &ar, st));
   }
-  FL_TRY(back_transform<double>(ctx, n, &w, V_dev, ldv, st));
+  FL_TRY(back_transform<double>(ctx, n, &w, V_dev, ldv, rest, st));
   if (info_dev) FL_CUDA(ctx, cudaMemcpyAsync(info_dev, ctx->d_status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   return 0;
 }
@@ -331,7 +344,7 @@ extern "C" int fraclap_tridiagonalize(fraclap_ctx* ctx, const double* A_dev, int
     set_identity<<<(unsigned)cdiv(n * n, 256), 256, 0, st>>>(Q_dev, ldq, n);
     count_launch(ctx);
     FL_CUDA(ctx, cudaGetLastError());
-    FL_TRY(back_transform<double>(ctx, n, &w, Q_dev, ldq, st));
+    FL_TRY(back_transform<double>(ctx, n, &w, Q_dev, ldq, ar, st));
   }
   return 0;
 }
@@ -458,13 +471,14 @@ extern "C" int eig_full_mixed(fraclap_ctx* ctx, const double* A_dev, int64_t n, 
     TcScratch lend(ctx, ctx->fp32_stages_tc ? tcs : nullptr, tf32_scratch_bytes(n));
     FL_TRY(reduce<float>(ctx, A_dev, n, lda, &w, st));
   }
+  const Arena rest = ar;
   {
     StageTimer t(ctx, kStageTridiagDC, st);
     FL_TRY(stedc_run<float>(ctx, w.d, w.e, n, lambda_dev, Z, n, &ar, st));
   }
   {
     TcScratch lend(ctx, ctx->fp32_stages_tc ? tcs : nullptr, tf32_scratch_bytes(n));
-    FL_TRY(back_transform<float>(ctx, n, &w, Z, n, st));
+    FL_TRY(back_transform<float>(ctx, n, &w, Z, n, rest, st));
   }
   {
     StageTimer t(ctx, kStageRefine, st);

@@ -251,10 +251,12 @@ int gemm_batched(fraclap_ctx* ctx, bool ta, bool tb, const GemmDescT<T>* d_descs
 template <class T>
 struct Stage1T {
   T* Vstore;         // sum_j m_j * b: explicit V of every panel
-  T* Tf;             // b * b, the panel in work
+  T* Tstore;         // npanel * b * b
   double* tau;       // npanel * b
-  T* XTstore;        // the same of V T
   T* X;              // n * b
+  T* XT;             // n * b, V T of the panel in work
+  T* XX;             // X and XT as one buffer (xx_len entries, 2 b^2 ceil(n / b) or more)
+  int64_t xx_len;
   T* Mm;             // b * b
   double* gram;      // b * b
   double* partials;  // 2 * G * 2b
@@ -278,8 +280,7 @@ struct Stage2T {
   T* refl;        // (n-1) * kmax * b
   double* rtau;   // (n-1) * kmax
   int* progress;  // n + 1: completed steps per sweep
-  T* beta;        // (n-1) * kmax: subdiagonal values as the steps publish them
-  T* ut;          // block factors of the back-transformation (b = 32, 64)
+  T* beta;        // (n-1) * kmax: subdiagonal values as the steps publish them (set by the caller)
   int64_t kmax;
 };
 using Stage2 = Stage2T<double>;
@@ -289,10 +290,12 @@ int stage2_take(Arena* ar, int64_t n, int b, Stage2T<T>* s);
 template <class T>
 int sb2st_run(fraclap_ctx* ctx, T* band, int64_t n, int b, double* d, double* e, Stage2T<T>* s,
               cudaStream_t st);
-// Z <- Q2 Z through a transposed copy Yt (ncols x n, ld ldy >= ncols).
+// Z <- Q2 Z through a transposed copy Yt (ncols x n, ld ldy >= ncols).  ut: scratch
+// of ut_len entries for the block factors (b = 32, 64), at least 2 b^2 kmax; up to
+// b^2 kmax (kmax + 1) are used.
 template <class T>
 int q2_apply_run(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int b, T* Z, int64_t ldz,
-                 int64_t ncols, T* Yt, int64_t ldy, cudaStream_t st);
+                 int64_t ncols, T* Yt, int64_t ldy, T* ut, int64_t ut_len, cudaStream_t st);
 template <class T>
 int transpose_run(fraclap_ctx* ctx, const T* A, int64_t lda, T* Bm, int64_t ldb, int64_t rows,
                   int64_t cols, cudaStream_t st);

@@ -523,7 +523,7 @@ q2t_apply_kernel(const T* __restrict__ refl, const double* __restrict__ rtau, in
 // base = 1 + kB + qB; their product H(qB) ... H(qB + B - 1) is I - V T V^T with
 // V(i + t, i) = v_i(t), a parallelogram, and T upper triangular.  The factor
 // -U = -V T (stored by columns of 2B rows) is formed once per block by
-// q2_factor_kernel; q2_block_kernel then streams the blocks: a CTA owns NCB
+// q2_factor_kernel (as many steps at a time as the scratch holds); q2_block_kernel then streams the blocks: a CTA owns NCB
 // columns of Z, keeps the 2B rows of the window in shared memory, and for each
 // block forms W = V^T Z and Z += (-U) W as two small products in registers.
 // The next block's window is B rows higher: the upper half becomes the lower
@@ -583,7 +583,8 @@ constexpr size_t q2_factor_smem() {
 // factors; the FP64 work, some n^2 b / 8 FMAs, is a few per cent of the stage).
 template <class T, int B>
 __global__ void __launch_bounds__(256) q2_factor_kernel(const T* __restrict__ refl, const double* __restrict__ rtau,
-                                                        int64_t n, int64_t kmax, int64_t N0, T* __restrict__ ut) {
+                                                        int64_t n, int64_t kmax, int64_t N0, int64_t first,
+                                                        T* __restrict__ ut) {  // blocks from `first` on
   extern __shared__ __align__(128) unsigned char q2_smem[];
   constexpr int LD = B + 1;
   double* Ts = reinterpret_cast<double*>(q2_smem);
@@ -592,7 +593,7 @@ __global__ void __launch_bounds__(256) q2_factor_kernel(const T* __restrict__ re
   __shared__ double tau[B];
   const int tid = threadIdx.x;
   // block index -> (k, q): row k of the triangle has N0 - k blocks
-  const int64_t blk = blockIdx.x;
+  const int64_t blk = first + blockIdx.x;
   int64_t k = (int64_t)((2.0 * N0 + 1.0 - sqrt((2.0 * N0 + 1.0) * (2.0 * N0 + 1.0) - 8.0 * (double)blk)) * 0.5);
   if (k < 0) k = 0;
   while (k > 0 && q2_block_offset(k, N0) > blk) --k;
@@ -629,7 +630,7 @@ __global__ void __launch_bounds__(256) q2_factor_kernel(const T* __restrict__ re
   }
   __syncthreads();
   // -U(r, i) = -sum_{i' <= i, 0 <= r - i' < B} V(r, i') T(i', i), stored [i][r]
-  T* out = ut + blk * (2 * B * B);
+  T* out = ut + (int64_t)blockIdx.x * (2 * B * B);
   for (int e = tid; e < 2 * B * B; e += 256) {
     const int r = e % (2 * B), i = e / (2 * B);
     const int lo = (r >= B) ? r - B + 1 : 0, hi = (r < i) ? r : i;
@@ -657,8 +658,8 @@ struct alignas(sizeof(T) * N) Vec {
 
 template <class T, int B, int NCB>
 __global__ void __launch_bounds__(Q2Shape<T, B, NCB>::NT)
-q2_block_kernel(const T* __restrict__ refl, const T* __restrict__ ut, int64_t n, int64_t kmax, int64_t N0, T* Y,
-                int64_t ldy, int64_t ncols) {
+q2_block_kernel(const T* __restrict__ refl, const T* __restrict__ ut, int64_t n, int64_t kmax, int64_t N0, int64_t kbeg,
+                int64_t kend, T* Y, int64_t ldy, int64_t ncols) {  // steps kbeg .. kend - 1, whose factors ut holds
   using Sh = Q2Shape<T, B, NCB>;
   using P = Pair2<T>;
   constexpr int RT = Sh::RT, CT = Sh::CT, NT = Sh::NT, LC = Sh::LC, LDV = Sh::LDV;
@@ -726,7 +727,7 @@ q2_block_kernel(const T* __restrict__ refl, const T* __restrict__ ut, int64_t n,
     }
   };
   auto fetch_u = [&](int64_t blk) {
-    const T* src = ut + blk * (2 * B * B);
+    const T* src = ut + (blk - q2_block_offset(kbeg, N0)) * (2 * B * B);
     T* dst = Us;
     constexpr int E = 16 / sizeof(T);
     for (int p = tid * E; p < 2 * B * B; p += NT * E)
@@ -737,7 +738,7 @@ q2_block_kernel(const T* __restrict__ refl, const T* __restrict__ ut, int64_t n,
   };
 
   for (int p = tid; p < 2 * B * LDV; p += NT) Vs[p] = T(0);  // the corners outside the parallelogram stay zero
-  for (int64_t k = 0; k < kmax; ++k) {
+  for (int64_t k = kbeg; k < kend; ++k) {
     const int64_t N = N0 - k, row_k = 1 + k * B;  // blocks N - 1 .. 0, block q starts at row row_k + q B
     if (N <= 0) break;
     __syncthreads();  // the previous step's rows are in global memory, the buffers are free
@@ -885,9 +886,7 @@ int stage2_take(Arena* ar, int64_t n, int b, Stage2T<T>* s) {
   const int64_t nsw = (n >= 2) ? n - 1 : 0;
   s->refl = ar->take<T>(nsw * s->kmax * b);
   s->rtau = ar->take<double>(nsw * s->kmax);
-  s->beta = ar->take<T>(nsw * s->kmax);
-  // -U of every block of b reflectors (one step, b consecutive sweeps): 2b x b each
-  s->ut = (b == 32 || b == 64) ? ar->take<T>(s->kmax * (s->kmax + 1) / 2 * 2 * b * b) : nullptr;
+  s->beta = nullptr;
   s->progress = ar->take<int>(n + 1);
   return 0;
 }
@@ -948,20 +947,27 @@ int transpose_run(fraclap_ctx* ctx, const T* A, int64_t lda, T* Bm, int64_t ldb,
 
 // The block factors, then the blocks on CTAs of NCB columns each.
 template <class T, int B, int NCB>
-int q2_blocks_launch(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int64_t ncols, T* Yt, int64_t ldy,
-                     cudaStream_t st) {
+int q2_blocks_launch(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int64_t ncols, T* Yt, int64_t ldy, T* ut,
+                     int64_t ut_len, cudaStream_t st) {
   using Sh = Q2Shape<T, B, NCB>;
-  const int64_t N0 = s->kmax, blocks = N0 * (N0 + 1) / 2;  // N0 = ceil((n - 1) / B) = kmax
-  FL_CHECK(ctx, blocks <= INT32_MAX, FRACLAP_ERR_UNSUPPORTED, "q2 back-transformation: n too large");
+  const int64_t N0 = s->kmax, room = std::min<int64_t>(ut_len / (2 * B * B), INT32_MAX);  // N0 = ceil((n - 1) / B) = kmax
+  FL_CHECK(ctx, room >= N0, FRACLAP_ERR_ALLOC, "q2 back-transformation: workspace too small");
   constexpr size_t fsm = q2_factor_smem<B>();
   FL_CUDA(ctx, cudaFuncSetAttribute(q2_factor_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
-  q2_factor_kernel<T, B><<<(unsigned)blocks, 256, fsm, st>>>(s->refl, s->rtau, n, s->kmax, N0, s->ut);
-  count_launch(ctx);
   FL_CUDA(ctx, cudaFuncSetAttribute(q2_block_kernel<T, B, NCB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)Sh::SMEM));
-  q2_block_kernel<T, B, NCB><<<(unsigned)cdiv(ncols, NCB), Sh::NT, Sh::SMEM, st>>>(s->refl, s->ut, n, s->kmax, N0, Yt,
-                                                                                   ldy, ncols);
-  count_launch(ctx);
+  for (int64_t k = 0; k < N0;) {
+    const int64_t first = q2_block_offset(k, N0);
+    int64_t e = k + 1;
+    while (e < N0 && q2_block_offset(e + 1, N0) - first <= room) ++e;
+    q2_factor_kernel<T, B><<<(unsigned)(q2_block_offset(e, N0) - first), 256, fsm, st>>>(s->refl, s->rtau, n, s->kmax, N0,
+                                                                                        first, ut);
+    count_launch(ctx);
+    q2_block_kernel<T, B, NCB><<<(unsigned)cdiv(ncols, NCB), Sh::NT, Sh::SMEM, st>>>(s->refl, ut, n, s->kmax, N0, k, e,
+                                                                                     Yt, ldy, ncols);
+    count_launch(ctx);
+    k = e;
+  }
   FL_CUDA(ctx, cudaGetLastError());
   return 0;
 }
@@ -969,7 +975,7 @@ int q2_blocks_launch(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int64_t n
 // Z <- Q2 Z (n x ncols, ld ldz), through the transposed copy Yt (ld >= ncols).
 template <class T>
 int q2_apply_run(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int b, T* Z, int64_t ldz,
-                 int64_t ncols, T* Yt, int64_t ldy, cudaStream_t st) {
+                 int64_t ncols, T* Yt, int64_t ldy, T* ut, int64_t ut_len, cudaStream_t st) {
   if (n < 2 || ncols <= 0) return 0;
   FL_TRY(transpose_run<T>(ctx, Z, ldz, Yt, ldy, n, ncols, st));
   const int64_t sm = ctx->sm_count > 0 ? ctx->sm_count : 152;
@@ -985,16 +991,16 @@ int q2_apply_run(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int b, T* Z, 
     const auto cost = [&](int ncb) { return cdiv(cdiv(ncols, ncb), sm) * ncb; };
     int rc = 0;
     if constexpr (sizeof(T) == 8) {
-      if (b == 64) rc = q2_blocks_launch<T, 64, 16>(ctx, s, n, ncols, Yt, ldy, st);
-      else if (cost(16) <= cost(8)) rc = q2_blocks_launch<T, 32, 16>(ctx, s, n, ncols, Yt, ldy, st);
-      else rc = q2_blocks_launch<T, 32, 8>(ctx, s, n, ncols, Yt, ldy, st);
+      if (b == 64) rc = q2_blocks_launch<T, 64, 16>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
+      else if (cost(16) <= cost(8)) rc = q2_blocks_launch<T, 32, 16>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
+      else rc = q2_blocks_launch<T, 32, 8>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
     } else if (b == 64) {
-      if (cost(64) <= cost(32) && cost(64) <= cost(16)) rc = q2_blocks_launch<T, 64, 64>(ctx, s, n, ncols, Yt, ldy, st);
-      else if (cost(32) <= cost(16)) rc = q2_blocks_launch<T, 64, 32>(ctx, s, n, ncols, Yt, ldy, st);
-      else rc = q2_blocks_launch<T, 64, 16>(ctx, s, n, ncols, Yt, ldy, st);
+      if (cost(64) <= cost(32) && cost(64) <= cost(16)) rc = q2_blocks_launch<T, 64, 64>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
+      else if (cost(32) <= cost(16)) rc = q2_blocks_launch<T, 64, 32>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
+      else rc = q2_blocks_launch<T, 64, 16>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
     } else {
-      if (cost(32) <= cost(16)) rc = q2_blocks_launch<T, 32, 32>(ctx, s, n, ncols, Yt, ldy, st);
-      else rc = q2_blocks_launch<T, 32, 16>(ctx, s, n, ncols, Yt, ldy, st);
+      if (cost(32) <= cost(16)) rc = q2_blocks_launch<T, 32, 32>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
+      else rc = q2_blocks_launch<T, 32, 16>(ctx, s, n, ncols, Yt, ldy, ut, ut_len, st);
     }
     if (rc) return rc;
     return transpose_run<T>(ctx, Yt, ldy, Z, ldz, ncols, n, st);
@@ -1047,7 +1053,7 @@ template int sb2st_run<double>(fraclap_ctx*, double*, int64_t, int, double*, dou
 template int sb2st_run<float>(fraclap_ctx*, float*, int64_t, int, double*, double*, Stage2T<float>*, cudaStream_t);
 template int transpose_run<double>(fraclap_ctx*, const double*, int64_t, double*, int64_t, int64_t, int64_t, cudaStream_t);
 template int transpose_run<float>(fraclap_ctx*, const float*, int64_t, float*, int64_t, int64_t, int64_t, cudaStream_t);
-template int q2_apply_run<double>(fraclap_ctx*, const Stage2T<double>*, int64_t, int, double*, int64_t, int64_t, double*, int64_t, cudaStream_t);
-template int q2_apply_run<float>(fraclap_ctx*, const Stage2T<float>*, int64_t, int, float*, int64_t, int64_t, float*, int64_t, cudaStream_t);
+template int q2_apply_run<double>(fraclap_ctx*, const Stage2T<double>*, int64_t, int, double*, int64_t, int64_t, double*, int64_t, double*, int64_t, cudaStream_t);
+template int q2_apply_run<float>(fraclap_ctx*, const Stage2T<float>*, int64_t, int, float*, int64_t, int64_t, float*, int64_t, float*, int64_t, cudaStream_t);
 
 }  // namespace fraclap

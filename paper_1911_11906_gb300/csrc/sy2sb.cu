@@ -668,10 +668,14 @@ int stage1_take(Arena* ar, int64_t n, int b, int G, Stage1T<T>* s) {
   s->vtotal = 0;
   for (int64_t j = 0; j < s->npanel; ++j) s->vtotal += (n - j * b - b) * b;
   s->Vstore = ar->take<T>(s->vtotal);
-  s->Tf = ar->take<T>((int64_t)b * b);
+  s->Tstore = ar->take<T>(s->npanel * b * b);
   s->tau = ar->take<double>(s->npanel * b);
-  s->XTstore = ar->take<T>(s->vtotal);
-  s->X = ar->take<T>(n * b);
+  // X and XT are one buffer: the back-transformation's block factors of one step fit it
+  const int64_t x = cdiv(n * b, 64) * 64;
+  s->xx_len = x + n * b + 2 * (int64_t)b * b;
+  s->XX = ar->take<T>(s->xx_len);
+  s->X = s->XX;
+  s->XT = s->XX ? s->XX + x : nullptr;
   s->Mm = ar->take<T>((int64_t)b * b);
   s->gram = ar->take<double>((int64_t)b * b);
   s->partials = ar->take<double>(3 * 2 * (int64_t)b);
@@ -779,7 +783,7 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
     const int64_t j0 = p * b, m = n - j0 - b;
     T* P = Aw + (j0 + b) + j0 * lda;
     T* V = s->Vstore + voff;
-    T* Tf = s->Tf;
+    T* Tf = s->Tstore + p * b * b;
     const int crc = panel_cluster(ctx, P, lda, m, b, V, s->tau + p * b, Tf, st);
     if (crc < 0) return crc;
     if (crc == 0) {
@@ -811,8 +815,8 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
     }
     T* A22 = Aw + (j0 + b) + (j0 + b) * lda;
     using D = GemmDescT<T>;
-    // XT = V T  (m x b), kept for the back-transformation
-    T* XT = s->XTstore + voff;
+    // XT = V T  (m x b)
+    T* XT = s->XT;
     FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, Tf, b, XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
     // X = A22 XT (A22 symmetric, lower triangle); narrow products share their
     // long sums by themselves, the TF32 route splits them into a zeroed X
@@ -838,7 +842,8 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
 
 // Back-transformation by Q1 = Q_0 Q_1 ... Q_{p-1}: Z <- Q1 Z (n x ncols).
 // Applied from the last panel to the first: Z(rows_j, :) -= (V_j T_j) (V_j^T Z(rows_j, :)),
-// V_j T_j as the reduction formed it: two products a panel.
+// V_j T_j formed again (its n^2 / 2 entries would cost the memory of larger
+// problems; some 6 us a panel).
 template <class T>
 int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, int64_t ldz,
                  int64_t ncols, T* W1, cudaStream_t st) {
@@ -854,7 +859,8 @@ int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, 
       T* Zr = Z + (j0 + b);
       FL_CUDA(ctx, cudaMemsetAsync(W1, 0, sizeof(T) * b * ncols, st));
       FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{ncols, b, m, Zr, ldz, V, m, W1, ncols, nullptr, 0, nullptr, 0, 0, 1.0, 1.0}, (int)std::min<int64_t>(cdiv(m, 1024), 16), st));
-      FL_TRY(gemm<T>(ctx, false, true, kGemmPlain, D{m, ncols, b, s->XTstore + voff, m, W1, ncols, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
+      FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, s->Tstore + p * b * b, b, s->XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
+      FL_TRY(gemm<T>(ctx, false, true, kGemmPlain, D{m, ncols, b, s->XT, m, W1, ncols, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
     }
     return 0;
   }
@@ -869,7 +875,8 @@ int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, 
     if (split) FL_CUDA(ctx, cudaMemsetAsync(W1, 0, sizeof(T) * b * ncols, st));
     FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{b, ncols, m, V, m, Zr, ldz, W1, b, nullptr, 0, nullptr, 0, 0, 1.0, split ? 1.0 : 0.0}, split ? (int)std::min<int64_t>(cdiv(m, 1024), 16) : 1, st));
     // Zr -= (V T) W1
-    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, ncols, b, s->XTstore + voff, m, W1, b, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
+    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, s->Tstore + p * b * b, b, s->XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
+    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, ncols, b, s->XT, m, W1, b, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
   }
   return 0;
 }
