@@ -331,7 +331,7 @@ size_t ozaki_ws(int64_t M, int64_t N, int64_t K, int s, bool lower = false, int 
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
                int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits = 0,
-               const OzGuard* guard = nullptr);
+               const OzGuard* guard = nullptr, int width = 0);
 
 // Banded LDL^T (no pivoting) of the symmetric CSR matrix of half-bandwidth
 // b: Lb(t, j) = L(j + t, j), Lr(t, i) = L(i, i - t) (both ld b + 1, n

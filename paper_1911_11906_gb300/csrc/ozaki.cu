@@ -1004,7 +1004,8 @@ static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N,
 
 // C = alpha op(A) op(B) + beta C, FP64-accurate through s BF16 slices
 // (s = 7 for full FP64 accuracy of the products).  lower: only C(i,j), i >= j.
-// digits > 0 sets the digits per operand itself (8 bits each at w = 7).
+// digits > 0 sets the digits per operand itself (8 bits each at w = 7), width > 0
+// their magnitude bits w.
 // guard (may be null) keeps the diagonal p + q = D too and tells which entries
 // the digits hold to the accuracy of an FP64 sum.  The digits are relative to
 // the largest entry of the row of op(A) and the column of op(B); in units of
@@ -1018,7 +1019,7 @@ static int ozaki_range(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N,
 // then meaningless.
 int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha,
                const double* A, int64_t lda, const double* B, int64_t ldb, double beta, double* C,
-               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits, const OzGuard* guard) {
+               int64_t ldc, int s, bool lower, Arena* ar, cudaStream_t st, int digits, const OzGuard* guard, int width) {
   if (M <= 0 || N <= 0) return 0;
   FL_CHECK(ctx, s >= 1 && s <= 8, FRACLAP_ERR_INVALID_ARG, "ozaki_gemm: slices must be 1..8");
   FL_CHECK(ctx, cdiv(N, OZ_BN) <= 65535, FRACLAP_ERR_UNSUPPORTED, "ozaki_gemm: N too large");
@@ -1034,7 +1035,7 @@ int ozaki_gemm(fraclap_ctx* ctx, bool ta, bool tb, int64_t M, int64_t N, int64_t
   // the folds 28.8 and 21.4 ms; w = 8 at s = 7 32.0 ms: the same pairs and four
   // times more chunk sums to drain and convert.)
   int bits = 8, sl = std::min(s, 7);
-  if (K > 256 && ctx->oz_bits != 8) {
+  if (width == 7 || (width == 0 && K > 256 && ctx->oz_bits != 8)) {
     bits = 7;
     sl = (s <= 5 || s == 8) ? s + 1 : s;  // s = 8: 72 bits
   }

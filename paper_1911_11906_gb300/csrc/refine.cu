@@ -505,9 +505,14 @@ __global__ void copy_columns(const double* Xs, int64_t n, double* X, int64_t ldx
 constexpr double kConvergedR = 3e-9;
 // BF16 slices per operand in the refinement's residual products (7: FP64).
 constexpr int kRefineSlices = 7;
-constexpr int kRefineFirstSlices = 5;   // first iteration (40 bits)
+constexpr int kRefineFirstSlices = 5;   // first iteration (45 bits)
 constexpr int kRefineSecondSlices = 6;  // second iteration (48 bits)
-// each slice is one digit of 8 bits: 15, 21 and 28 digit pairs a product
+// One digit a slice: 15, 21 and 28 pairs a product, of 9, 8 and 8 bits.  Five
+// digits of 8 bits took 2 ms less at n = 8810 but held 40 bits, two fewer than six
+// sign-magnitude digits of 7, with up to 1.5 times their error (root mean square,
+// X^T X of orthonormal columns); six of 8 bits have 0.5 to 0.8 times the error of
+// seven of those.
+constexpr int kRefineFirstWidth = 8;
 
 __device__ void cluster_jacobi_body(const double* Sc, const double* Bc, int c, double* Q, double* w,
                                     int32_t* status) {
@@ -962,19 +967,22 @@ int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t
     // counts as the converged (last) one.
     const int slices_it = (it + 1 >= iters) ? kRefineSlices
                           : (it == 0 ? kRefineFirstSlices : (it == 1 ? kRefineSecondSlices : kRefineSlices));
+    const int width_it = slices_it == kRefineFirstSlices ? kRefineFirstWidth : 0;
     // R = I - X^T X, S = X^T (A X): lower triangles, FP64-accurate products
     // from BF16 tensor-core slices (the slices live in the scratch arena)
     {
       StageTimer tm(ctx, kStageResidualGemm, st);
       Arena oz = *ar;
-      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, -1.0, X, ldx, X, ldx, 0.0, R, n, slices_it, true, &oz, st, slices_it));
+      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, -1.0, X, ldx, X, ldx, 0.0, R, n, slices_it, true, &oz, st, slices_it,
+                        nullptr, width_it));
     }
     add_identity<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(R, n, n);
     count_launch(ctx);
     {
       StageTimer tm(ctx, kStageResidualGemm, st);
       Arena oz = *ar;
-      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, 1.0, X, ldx, AX, n, 0.0, S, n, slices_it, true, &oz, st, slices_it));
+      FL_TRY(ozaki_gemm(ctx, true, false, n, n, n, 1.0, X, ldx, AX, n, 0.0, S, n, slices_it, true, &oz, st, slices_it,
+                        nullptr, width_it));
     }
     span.start(kStageRefineNorms);
     ritz_values<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(S, n, R, n, n, lt);
