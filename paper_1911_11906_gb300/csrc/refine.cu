@@ -899,9 +899,15 @@ static int64_t small_cluster_doubles(int64_t n) {
   return 3 * ns * kMaxCluster * kMaxCluster + (n + 64) / 2 + (3 * ns + 64) / 2 + 64;
 }
 
+// The power iterations' segments of a strip, CTAs of a vector, and doubles in all
+// (see PowerVecs): more than n^2 up to n = 6.
+static int power_segments(int64_t n) { return (int)cdiv(cdiv(n, 32), kSymvSeg); }
+static int64_t power_ctas(int64_t n) { return cdiv(n, 256); }
+static int64_t ax_doubles(int64_t n) { return std::max(n * n, 2 * n + 4 * power_segments(n) * n + 2 * power_ctas(n)); }
+
 size_t refine_ws(const fraclap_ctx* ctx, int64_t n) {
   Arena ar;
-  ar.take<double>(n * n);      // AX, then sorted X
+  ar.take<double>(ax_doubles(n));  // AX, the power iterations' vectors, then sorted X
   ar.take<double>(n * n);      // R
   ar.take<double>(n * n);      // S
   ar.take<float>(n * n);       // E
@@ -925,7 +931,7 @@ size_t refine_ws(const fraclap_ctx* ctx, int64_t n) {
 int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t* col,
                const double* val, double* X, int64_t ldx, double* lambda, int iters, Arena* ar,
                cudaStream_t st) {
-  double* AX = ar->take<double>(n * n);
+  double* AX = ar->take<double>(ax_doubles(n));
   double* R = ar->take<double>(n * n);
   double* S = ar->take<double>(n * n);
   float* E = ar->take<float>(n * n);
@@ -994,10 +1000,9 @@ int refine_run(fraclap_ctx* ctx, int64_t n, const int64_t* rowptr, const int32_t
     count_launch(ctx);
     {  // 2-norm estimates of S - diag(l) and R (power iteration), both at once
       const int64_t nt = cdiv(n, 32);
-      const int Sg = (int)cdiv(nt, kSymvSeg);
-      const unsigned nb = (unsigned)cdiv(n, 256);
-      // in the n x n scratch of A X: 2 n + 4 Sg n + 2 nb doubles
-      PowerVecs pv;
+      const int Sg = power_segments(n);
+      const unsigned nb = (unsigned)power_ctas(n);
+      PowerVecs pv;  // in the scratch of A X
       pv.y = AX;
       pv.P = pv.y + 2 * n;
       pv.Q = pv.P + 2 * (int64_t)Sg * n;
