@@ -721,7 +721,7 @@ def run_batched_bench(args, steps=None, warmup=None):
                           "F": it["F"], "pair_f": it["pair_f"], "pair_alpha": it["pair_alpha"]})
         return batch
 
-    workers = 16 if args.no_autotune else autotune.best_workers(assemble_all())
+    workers = ctx.batched_workers(16, len(probs)) if args.no_autotune else autotune.best_workers(assemble_all())
 
     def step():
         state["out"] = F.solve_batched(assemble_all(), workers=workers, ctx=ctx)

@@ -344,7 +344,8 @@ int fraclap_sgemm(fraclap_ctx* ctx, int trans_a, int trans_b, int form, int64_t 
  * lambda_dev / V_dev and, when k > 0, the spectral apply of its k pairs into
  * U_dev (as frac_apply; Sec. II eq. poisson_solution).  The problems are
  * spread over `workers` concurrent streams (0: 16; never more than the device
- * has hardware queues: 8, or CUDA_DEVICE_MAX_CONNECTIONS), each with its own share
+ * has hardware queues: 8, or CUDA_DEVICE_MAX_CONNECTIONS when the context is
+ * made; fraclap_batched_workers says how many that gives), each with its own share
  * of the SMs and a context-owned workspace sized for its largest problem;
  * the caller's stream waits for all of them.  probs is a host array; every
  * pointer in it is a device pointer owned by the caller, and distinct
@@ -374,6 +375,7 @@ typedef struct fraclap_problem {
   const double* val_dev;
   int refine_iters;
 } fraclap_problem;
+int fraclap_batched_workers(const fraclap_ctx* ctx, int workers, int count);
 int fraclap_solve_batched(fraclap_ctx* ctx, const fraclap_problem* probs, int count, int workers,
                           fraclap_stream_t stream);
 

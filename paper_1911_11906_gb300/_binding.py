@@ -38,6 +38,7 @@ SIGNATURES = {
     "fraclap_set_profiling": (_i32, [_p, _i32]),
     "fraclap_stage_times": (_i32, [_p, _p, _p, _i32]),
     "fraclap_launch_count": (ctypes.c_longlong, [_p]),
+    "fraclap_batched_workers": (_i32, [_p, _i32, _i32]),
     "fraclap_refine_stats": (_i32, [_p, _p, _i32]),
     "fraclap_set_tensor_route": (_i32, [_p, _i32]),
     "fraclap_set_refine_tau": (_i32, [_p, _dbl]),
@@ -177,6 +178,13 @@ class Context:
     def set_refine_tau(self, tau: float):
         """Refinement safeguard: pairs with a first-order coefficient above tau are clustered."""
         self.check(self.lib.fraclap_set_refine_tau(self.handle, float(tau)))
+
+    def batched_workers(self, workers: int, count: int) -> int:
+        """The streams that solve_batched runs `count` problems on when asked for `workers`."""
+        n = self.lib.fraclap_batched_workers(self.handle, int(workers), int(count))
+        if n < 0:
+            self.check(n)
+        return n
 
     def set_apply_slices(self, slices: int):
         """frac_apply products: 0 = FP64 accuracy (FP64 engine or 8 digits); s = 1..8 BF16 slices on the tensor cores."""

@@ -145,11 +145,14 @@ def best_band_width(n: int, route: str = "mixed", candidates=(32, 64), tuner: Au
 
 def best_workers(problems: list, candidates=(4, 8, 16, 32), tuner: Autotuner | None = None,
                  reps: int = 1) -> int:
-    """Number of concurrent workers of the batched solver for a list of
-    problems in the form fraclap's solve_batched takes, measured on that list
+    """Number of concurrent workers of the batched solver (as many as run, see
+    Context.batched_workers) for a list of problems in the form fraclap's solve_batched takes, measured on that list
     and cached under its size profile (count, largest and total n, routes)."""
     from . import _binding as B
     tuner = tuner or Autotuner()
+    ctx = B.Context()
+    # counts that the library runs as the same number of streams are one candidate
+    candidates = tuple(dict.fromkeys(ctx.batched_workers(int(w), len(problems)) for w in candidates))
     ns = [int(p["A"].shape[0]) for p in problems]
     fields = {"device": _device_name(), "count": len(problems), "n_max_bucket": size_bucket(max(ns or [1])),
               "n_sum_bucket": size_bucket(sum(ns) or 1),
@@ -157,7 +160,6 @@ def best_workers(problems: list, candidates=(4, 8, 16, 32), tuner: Autotuner | N
     hit = tuner.lookup("batched_workers", fields, candidates)
     if hit is not None:
         return hit
-    ctx = B.Context()
     return tuner.choose("batched_workers", fields, candidates,
                         lambda w: _event_seconds(lambda: B.solve_batched(problems, workers=int(w), ctx=ctx)), reps)
 

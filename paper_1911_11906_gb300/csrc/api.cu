@@ -4,6 +4,7 @@
 #include <stdarg.h>
 
 #include <algorithm>
+#include <cstdlib>
 
 #include "internal.cuh"
 
@@ -243,6 +244,10 @@ extern "C" int fraclap_create(fraclap_ctx** out, const fraclap_opts* opts) {
   }
   // the wait limit is counted in SM clock cycles; 2.5 GHz bounds every clock
   ctx->wait_cycles = (long long)(ctx->wait_timeout_s * 2.5e9);
+  if (const char* env = getenv("CUDA_DEVICE_MAX_CONNECTIONS")) {
+    const int queues = atoi(env);
+    if (queues >= 1 && queues <= 32) ctx->hw_queues = queues;
+  }
   cudaError_t e = cudaGetDevice(&ctx->device);
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);

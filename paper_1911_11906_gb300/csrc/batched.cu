@@ -14,7 +14,6 @@
 // caller's stream waits for every worker; device errors of the workers are
 // merged into the context's status word.
 #include <algorithm>
-#include <cstdlib>
 #include <thread>
 #include <vector>
 
@@ -39,10 +38,8 @@ __global__ void merge_status(int32_t* parent, int32_t* child) {
 // 32 problems of n = 180 to 1843 on a GB300 took 171 ms on 8 streams, 244 on 16
 // (103 on 16 with 32 queues), so no more streams than queues run at one time
 // (153 ms since the panels stay in registers).
-int hardware_queues() {
-  const char* e = getenv("CUDA_DEVICE_MAX_CONNECTIONS");
-  const int q = e ? atoi(e) : 0;
-  return (q >= 1 && q <= 32) ? q : 8;
+int workers_for(const fraclap_ctx* ctx, int workers, int count) {
+  return std::max(1, std::min({workers > 0 ? workers : 16, count, 64, ctx->hw_queues}));
 }
 
 int ensure_workers(fraclap_ctx* ctx, int W) {
@@ -84,6 +81,10 @@ int ensure_workers(fraclap_ctx* ctx, int W) {
 
 }  // namespace
 
+extern "C" int fraclap_batched_workers(const fraclap_ctx* ctx, int workers, int count) {
+  return ctx && count >= 0 ? workers_for(ctx, workers, count) : FRACLAP_ERR_INVALID_ARG;
+}
+
 extern "C" int fraclap_solve_batched(fraclap_ctx* ctx, const fraclap_problem* probs, int count, int workers,
                                      fraclap_stream_t stream) {
   if (!ctx) return FRACLAP_ERR_INVALID_ARG;
@@ -99,7 +100,7 @@ extern "C" int fraclap_solve_batched(fraclap_ctx* ctx, const fraclap_problem* pr
     FL_CHECK(ctx, !p.rowptr_dev || (p.col_dev && p.val_dev && p.refine_iters >= 1 && p.refine_iters <= 8),
              FRACLAP_ERR_INVALID_ARG, "solve_batched: problem %d: incomplete CSR or refine_iters outside 1..8", i);
   }
-  const int W = std::max(1, std::min({workers > 0 ? workers : 16, count, 64, hardware_queues()}));
+  const int W = workers_for(ctx, workers, count);
   FL_TRY(ensure_workers(ctx, W));
   // deal the problems largest first to the least-loaded worker
   std::vector<int> order(count);

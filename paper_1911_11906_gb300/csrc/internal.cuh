@@ -31,6 +31,7 @@ struct fraclap_ctx {
   size_t tc_scratch_bytes = 0;   // (set by the caller of the FP32 stages, null otherwise)
   long long wait_cycles = 0;     // wait_timeout_s in SM clock cycles (upper bound)
   int32_t* d_status = nullptr;   // device status word (0 = ok, else a FRACLAP_ERR_*)
+  int hw_queues = 8;             // the device's hardware queues as the environment sets them when the context is made
   int panel_cluster_fits[2] = {-1, -1};  // FP32, FP64 panels on one cluster: 1, 0, or -1 (not asked yet)
   unsigned* d_barrier = nullptr; // grid-barrier state for cooperative kernels
   void* ws = nullptr;            // context-owned workspace
