@@ -203,7 +203,9 @@ __device__ __forceinline__ void panel_t_columns(const TG* G, const double* s_tau
 // the CTAs, a warp each: T(k, j) = -tau_k sum_{k < q <= j} G(k, q) T(q, j) from
 // k = j down, in FP64, which holds for tau_k = 0 as well.
 // Bound: the chain of a column (dots, barrier, FP64 scalars, update), some 6 us
-// at 480 rows a CTA.  It takes the panels past the register kernel's rows.
+// at 480 rows a CTA.  It takes the panels past the register kernel's rows: in FP32
+// those of more than some 9000 rows, in FP64 those of a batch's workers with fewer
+// than 16 SMs.
 // G, a CTA's part and the FP64 sum, in the place of V
 template <class T>
 constexpr size_t panel_gram_smem() {
@@ -744,26 +746,33 @@ int panel_cluster(fraclap_ctx* ctx, T* P, int64_t ldp, int64_t m, int b, T* V, d
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  // asked once per context: the largest cluster with the largest panel is resident
+  // asked once per context, for kClusterMax CTAs (a batch's workers have fewer SMs,
+  // and other numbers of them in another batch): every kernel of the panels is
+  // resident at its largest size
   int& fits = ctx->panel_cluster_fits[sizeof(T) == 8 ? 1 : 0];
   if (fits < 0) {
-    FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    FL_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+    bool all = true;
+    const auto resident = [&](const void* k, int threads, size_t smem) -> int {
+      FL_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      FL_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      cudaLaunchAttribute big = attr[0];
+      big.val.clusterDim.x = kClusterMax;
+      cudaLaunchConfig_t full = cfg;
+      full.gridDim = dim3(kClusterMax);
+      full.blockDim = dim3((unsigned)threads);
+      full.dynamicSmemBytes = smem;
+      full.attrs = &big;
+      full.numAttrs = 1;
+      int clusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&clusters, k, &full) != cudaSuccess) cudaGetLastError();
+      all = all && clusters >= 1;
+      return 0;
+    };
+    FL_TRY(resident((const void*)kern, PQR_NT, (size_t)most));
     for (int bb : {32, 64})
-      for (int r = 1; panel_regs_kernel<T>(r, bb); r += 32) {
-        FL_CUDA(ctx, cudaFuncSetAttribute(panel_regs_kernel<T>(r, bb), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        FL_CUDA(ctx, cudaFuncSetAttribute(panel_regs_kernel<T>(r, bb), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(64 * 65 * sizeof(T))));
-      }
-    cudaLaunchConfig_t full = cfg;
-    cudaLaunchAttribute big = attr[0];
-    big.val.clusterDim.x = (unsigned)limit;
-    full.gridDim = dim3((unsigned)limit);
-    full.blockDim = dim3(PQR_NT);
-    full.dynamicSmemBytes = (size_t)most;
-    full.attrs = &big;
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &full) != cudaSuccess) cudaGetLastError();
-    fits = clusters >= 1 ? 1 : 0;
+      for (int r = 1; panel_regs_kernel<T>(r, bb); r += 32)
+        FL_TRY(resident((const void*)panel_regs_kernel<T>(r, bb), 32 * kPanelRegsWarps<T>, 64 * 65 * sizeof(T)));
+    fits = all ? 1 : 0;
   }
   if (!fits) return 1;
   count_launch(ctx);

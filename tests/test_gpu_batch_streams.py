@@ -42,3 +42,27 @@ w = A.best_workers(probs, candidates=(4, 8, 16, 32), tuner=A.Autotuner(path))
 (val,) = [v for k, v in json.load(open(path))["entries"].items() if k.startswith("batched_workers:")]
 assert set(val["seconds"]) == {{"4", "8"}} and w in (4, 8)
 """, None)
+
+
+def test_fp64_panels_of_workers_with_few_sms():
+    """20 streams or more leave a worker 8 SMs or fewer: FP64 panels of more than 256
+    rows a CTA, in a batch after one whose workers had all 16 (tolerance 10 n eps)."""
+    _run("""
+import torch
+import paper_1911_11906_gb300 as F
+ctx = F.Context(wait_timeout_s=5.0)
+g = torch.Generator(device="cuda").manual_seed(1)
+def problem(n):
+    A = torch.randn(n, n, dtype=torch.float64, device="cuda", generator=g)
+    return {"A": A + A.t()}
+def check(p, out):
+    A, (lam, V, _) = p["A"], out
+    n, eps = A.shape[0], torch.finfo(torch.float64).eps
+    assert (V.t() @ V - torch.eye(n, dtype=torch.float64, device="cuda")).norm() <= 10 * n * eps
+    assert (A @ V - V * lam).norm() <= 10 * n * eps * A.norm()
+    assert ctx.batched_workers(32, 24) == 24
+for count, n in ((1, 300), (24, 2800), (24, 4200)):
+    probs = [problem(n)] + [problem(40 + i) for i in range(count - 1)]
+    for p, o in zip(probs, F.solve_batched(probs, workers=32, ctx=ctx)):
+        check(p, o)
+""", 32)
