@@ -216,9 +216,9 @@ def apply_slice_flops(n: int, m: int, k: int, slices: int, digit_bits: int = 7) 
 
 def refine_slice_counts(iterations: int, cap: int, digit_bits: int = 7) -> list:
     """Digits per operand of the refinement's two residual products in each
-    iteration: 40, 48 and then 56 bits (5, 6, 7 slices of 8 bits), the last
-    allowed iteration always full; as 7-bit digits (ceil(8 s / 7)) or, with
-    digit_bits = 8, the slices themselves."""
+    iteration: 5, 6 and then 7 slices, the last allowed iteration always full;
+    as 7-bit digits (ceil(8 s / 7)) or, with digit_bits = 8, the slices
+    themselves (the first iteration's digits have 9 bits)."""
     out = []
     for it in range(iterations):
         s8 = 7 if it + 1 >= cap else (5 if it == 0 else (6 if it == 1 else 7))
@@ -318,7 +318,7 @@ def run_gpu(args, rank, world, local_rank):
         ctx.set_apply_slices(APPLY_SLICES[path])
         app_ws = torch.empty(ctx.lib.fraclap_apply_workspace_bytes_ctx(ctx.handle, n, Fd.shape[1], k),
                              dtype=torch.uint8, device=dev)
-        # the FP64 route is the comparison when both run: fewer timed steps (it is 6x slower)
+        # the FP64 route is the comparison when both run: fewer timed steps (it is 13x slower)
         short = path == "fp64" and len(paths) > 1
         r = run_path(F, ctx, p, path, args, mask, Fd, pf, pa, U, app_ws, barrier,
                      steps=min(args.steps, 2) if short else None, warmup=min(args.warmup, 3) if short else None)
@@ -782,7 +782,9 @@ def run_apply_bench(args, diffusion=False, steps=None, warmup=None):
     lines = {}
     for slices in (0, 6):
         ctx.set_apply_slices(slices)
-        ws = torch.empty(ctx.lib.fraclap_apply_workspace_bytes_ctx(ctx.handle, p.n, Fd.shape[1], k),
+        # (0: the FP64 engine, which the smaller workspace asks for)
+        ws = torch.empty(ctx.lib.fraclap_apply_workspace_bytes_ctx(ctx.handle, p.n, Fd.shape[1], k) if slices else
+                         ctx.lib.fraclap_apply_workspace_bytes(p.n, Fd.shape[1], k),
                          dtype=torch.uint8, device=mask.device)
 
         def step():

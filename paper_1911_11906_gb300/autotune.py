@@ -173,12 +173,15 @@ def best_ozaki_schedule(n: int, slices: int = 7, groups=(0, 4, 8, 16), bits=(7,)
     `slices` BF16 slices (or, with cols, the apply's product V^T F of an
     n x n V and an n x cols F), measured on seeded matrices of that size
     through fraclap_dgemm_ozaki.  Returns {"ozaki_group": G, "ozaki_bits": w,
-    "ozaki_tile_n": t, "ozaki_cluster": c}; apply it with
+    "ozaki_tile_n": t, "ozaki_cluster": c} (c = 1 without a trial in a process
+    group of several ranks: multicast is for a process with the only GPU); apply it with
     apply_schedule(ctx, ...).  The digit widths tried default to 7 alone:
     the wider digits' four times more chunk sums cost more than their fewer
-    pairs save (66 against 40 ms at n = 8810 on a GB300 for 7 slices)."""
+    pairs save (32.0 against 28.8 ms at n = 8810 on a GB300 for 7 slices)."""
     import torch
     from . import _binding as B
+    if torch.distributed.is_available() and torch.distributed.is_initialized() and torch.distributed.get_world_size() > 1:
+        clusters = (1,)
     tuner = tuner or Autotuner()
     cands = [f"{g}/{w}/{t}/{c}" for c in clusters for t in tiles for w in bits for g in groups]
     fields = {"device": _device_name(), "n_bucket": size_bucket(n), "slices": int(slices)}
