@@ -25,7 +25,7 @@ struct fraclap_ctx {
   int oz_bits = 7;               // slice-product kernel: digit width for K > 256 (7 or 8)
   int oz_tile_n = 256;           // slice-product kernel: tile columns (128, 192 or 256)
   int oz_cluster = 1;            // slice-product kernel: CTAs per cluster sharing a B tile (1 or 2)
-  int q2_parts = 0;              // stage-2 back-transformation at b = 64: lane parts per window (0: default 8)
+  int q2_parts = 0;              // stage-2 back-transformation at b = 64: lane parts per window (0: blocks of reflectors, or 8)
   int fp32_stages_tc = 0;        // mixed route: FP32 band reduction and Q1 products on the tensor cores (TF32 x 3)
   void* tc_scratch = nullptr;    // split operands of the TF32 tensor-core route of FP32 GEMMs
   size_t tc_scratch_bytes = 0;   // (set by the caller of the FP32 stages, null otherwise)

@@ -583,7 +583,8 @@ __global__ void __launch_bounds__(32 * kSecWarps) dc_secular(DcBuf<T> B, int32_t
 
 // Gu-Eisenstat: zhat_i^2 = (lam_{K-1} - d_i)/rho * prod_{j<K-1} (lam_j - d_i)/(d_j' - d_i).
 // A warp per entry, the lanes' products of every 32nd factor multiplied by a
-// butterfly (the factors pair off around 1, so no partial product drifts).
+// butterfly (by interlacing every factor lies in (0, 1], so no partial product is
+// below the whole).
 template <class T>
 __global__ void __launch_bounds__(32 * kSecWarps) dc_zhat(DcBuf<T> B) {
   const MergeInfo inf = B.info[blockIdx.y];

@@ -10,7 +10,7 @@
 // A22 <- Q^T A22 Q = A22 - W V^T - V W^T with X = A22 (V T), W = X - 1/2 V ((V T)^T X),
 // through the GEMM engine (symmetric A22 read from its lower triangle;
 // lower-triangular rank-2b update).  In FP64 or FP32; the Householder scalars are
-// FP64 in both, and FP32 norms are added over the CTAs exactly.
+// FP64 in both, and FP32 norms are added over the CTAs to 2^-59 of the largest.
 #include <cooperative_groups.h>
 
 #include "internal.cuh"
@@ -405,8 +405,9 @@ panel_qr_cluster_kernel(T* P, int64_t ldp, int64_t m, int bw, T* Vout, int64_t l
 // loads; the kernel on shared memory took 257 and 418.  The band reduction at n =
 // 1114 7.0 -> 5.1 ms, 2753 15.6 -> 11.1, 7735 78.2 -> 53.9, FP64 779 7.2 -> 5.8.
 // A warp's FP64 operation holds the SM's FP64 pipe for some 16 clocks, so only
-// the scalars and w are FP64 there; FP32 panels' sums over the CTAs are carried
-// exactly in pairs of FP32 values.
+// the scalars and w are FP64 there; FP32 panels' sums over the CTAs are carried in
+// pairs of FP32 values, some 48 bits.  (The FP32 kernels of 16 and 18 rows a lane
+// spill some 50 and 320 bytes a thread.)
 template <class T>
 constexpr int kPanelRegsWarps = sizeof(T) == 8 ? 8 : 16;
 // s + v = s' + e exactly (Knuth)
