@@ -163,6 +163,19 @@ int reduce(fraclap_ctx* ctx, const double* A, int64_t n, int64_t lda, EigWork<T>
   return 0;
 }
 
+// Lends the panels' V T a piece of the workspace behind the next `front` bytes, if
+// there is one: the refinement's buffers, which are free until then.  Returns what
+// is left in front of it.
+template <class T>
+Arena lend_vt(Arena ar, size_t front, EigWork<T>* w) {
+  const size_t bytes = align256(sizeof(T) * (size_t)std::max<int64_t>(w->s1.vtotal, 1)), end = ar.cap / 256 * 256;
+  if (end >= ar.off + front + bytes) {
+    ar.cap = end - bytes;
+    w->s1.XTstore = reinterpret_cast<T*>(ar.base + ar.cap);
+  }
+  return ar;
+}
+
 // `free`: the rest of the workspace (the tridiagonal solver's buffers among it),
 // for the block factors; without room there they take the panels' buffers, a step
 // or more at a time.
@@ -470,13 +483,13 @@ extern "C" int eig_full_mixed(fraclap_ctx* ctx, const double* A_dev, int64_t n, 
   float* Z = ar.take<float>(n * n);
   char* tcs = ar.take<char>(tf32_scratch_bytes(n));
   FL_CHECK(ctx, Z != nullptr && tcs != nullptr, FRACLAP_ERR_ALLOC, "eig_full_mixed: workspace too small");
+  const Arena rest = lend_vt(ar, stedc_ws<float>(ctx, n), &w);
   {
     // FP32 products of the band reduction on the tensor cores (three TF32
     // products) when the context's schedule asks for it, else the FMA kernel
     TcScratch lend(ctx, ctx->fp32_stages_tc ? tcs : nullptr, tf32_scratch_bytes(n));
     FL_TRY(reduce<float>(ctx, A_dev, n, lda, &w, st));
   }
-  const Arena rest = ar;
   {
     StageTimer t(ctx, kStageTridiagDC, st);
     FL_TRY(stedc_run<float>(ctx, w.d, w.e, n, lambda_dev, Z, n, &ar, st));

@@ -679,6 +679,7 @@ int stage1_take(Arena* ar, int64_t n, int b, int G, Stage1T<T>* s) {
   s->XX = ar->take<T>(s->xx_len);
   s->X = s->XX;
   s->XT = s->XX ? s->XX + x : nullptr;
+  s->XTstore = nullptr;
   s->Mm = ar->take<T>((int64_t)b * b);
   s->gram = ar->take<double>((int64_t)b * b);
   s->partials = ar->take<double>(3 * 2 * (int64_t)b);
@@ -826,7 +827,7 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
     T* A22 = Aw + (j0 + b) + (j0 + b) * lda;
     using D = GemmDescT<T>;
     // XT = V T  (m x b)
-    T* XT = s->XT;
+    T* XT = s->XTstore ? s->XTstore + voff : s->XT;
     FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, Tf, b, XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
     // X = A22 XT (A22 symmetric, lower triangle); narrow products share their
     // long sums by themselves, the TF32 route splits them into a zeroed X
@@ -852,13 +853,19 @@ int sy2sb_run(fraclap_ctx* ctx, T* Aw, int64_t n, int64_t lda, int b, T* band, S
 
 // Back-transformation by Q1 = Q_0 Q_1 ... Q_{p-1}: Z <- Q1 Z (n x ncols).
 // Applied from the last panel to the first: Z(rows_j, :) -= (V_j T_j) (V_j^T Z(rows_j, :)),
-// V_j T_j formed again (its n^2 / 2 entries would cost the memory of larger
-// problems; some 6 us a panel).
+// V_j T_j as the reduction formed it where the caller had room for its n^2 / 2
+// entries, else formed again (some 6 us a panel).
 template <class T>
 int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, int64_t ldz,
                  int64_t ncols, T* W1, cudaStream_t st) {
   int64_t voff = s->vtotal;
   using D = GemmDescT<T>;
+  const auto vt = [&](int64_t p, int64_t m, const T* V, const T** XT) -> int {
+    *XT = s->XTstore ? s->XTstore + voff : s->XT;
+    if (s->XTstore) return 0;
+    return gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, s->Tstore + p * b * b, b, s->XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st);
+  };
+  const T* XT;
   if (sizeof(T) == 4 && ctx->tc_scratch) {
     // tensor-core shapes (tall and wide products): W1^T = Z_r^T V (n x b), Z_r -=
     // (V T) W1 -- the same products, transposed
@@ -869,8 +876,8 @@ int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, 
       T* Zr = Z + (j0 + b);
       FL_CUDA(ctx, cudaMemsetAsync(W1, 0, sizeof(T) * b * ncols, st));
       FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{ncols, b, m, Zr, ldz, V, m, W1, ncols, nullptr, 0, nullptr, 0, 0, 1.0, 1.0}, (int)std::min<int64_t>(cdiv(m, 1024), 16), st));
-      FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, s->Tstore + p * b * b, b, s->XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
-      FL_TRY(gemm<T>(ctx, false, true, kGemmPlain, D{m, ncols, b, s->XT, m, W1, ncols, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
+      FL_TRY(vt(p, m, V, &XT));
+      FL_TRY(gemm<T>(ctx, false, true, kGemmPlain, D{m, ncols, b, XT, m, W1, ncols, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
     }
     return 0;
   }
@@ -885,8 +892,8 @@ int q1_apply_run(fraclap_ctx* ctx, const Stage1T<T>* s, int64_t n, int b, T* Z, 
     if (split) FL_CUDA(ctx, cudaMemsetAsync(W1, 0, sizeof(T) * b * ncols, st));
     FL_TRY(gemm<T>(ctx, true, false, kGemmPlain, D{b, ncols, m, V, m, Zr, ldz, W1, b, nullptr, 0, nullptr, 0, 0, 1.0, split ? 1.0 : 0.0}, split ? (int)std::min<int64_t>(cdiv(m, 1024), 16) : 1, st));
     // Zr -= (V T) W1
-    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, b, b, V, m, s->Tstore + p * b * b, b, s->XT, m, nullptr, 0, nullptr, 0, 0, 1.0, 0.0}, 1, st));
-    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, ncols, b, s->XT, m, W1, b, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
+    FL_TRY(vt(p, m, V, &XT));
+    FL_TRY(gemm<T>(ctx, false, false, kGemmPlain, D{m, ncols, b, XT, m, W1, b, Zr, ldz, nullptr, 0, nullptr, 0, 0, -1.0, 1.0}, 1, st));
   }
   return 0;
 }
