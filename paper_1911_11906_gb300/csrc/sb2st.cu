@@ -659,7 +659,7 @@ struct alignas(sizeof(T) * N) Vec {
 template <class T, int B, int NCB>
 __global__ void __launch_bounds__(Q2Shape<T, B, NCB>::NT)
 q2_block_kernel(const T* __restrict__ refl, const T* __restrict__ ut, int64_t n, int64_t kmax, int64_t N0, int64_t kbeg,
-                int64_t kend, T* Y, int64_t ldy, int64_t ncols) {  // steps kbeg .. kend - 1, whose factors ut holds
+                int64_t kend, T* Y, int64_t ldy, int64_t ncols) {  // steps kbeg .. kend - 1; ut: where block 0's factor would be
   using Sh = Q2Shape<T, B, NCB>;
   using P = Pair2<T>;
   constexpr int RT = Sh::RT, CT = Sh::CT, NT = Sh::NT, LC = Sh::LC, LDV = Sh::LDV;
@@ -727,7 +727,7 @@ q2_block_kernel(const T* __restrict__ refl, const T* __restrict__ ut, int64_t n,
     }
   };
   auto fetch_u = [&](int64_t blk) {
-    const T* src = ut + (blk - q2_block_offset(kbeg, N0)) * (2 * B * B);
+    const T* src = ut + blk * (2 * B * B);
     T* dst = Us;
     constexpr int E = 16 / sizeof(T);
     for (int p = tid * E; p < 2 * B * B; p += NT * E)
@@ -963,7 +963,8 @@ int q2_blocks_launch(fraclap_ctx* ctx, const Stage2T<T>* s, int64_t n, int64_t n
     q2_factor_kernel<T, B><<<(unsigned)(q2_block_offset(e, N0) - first), 256, fsm, st>>>(s->refl, s->rtau, n, s->kmax, N0,
                                                                                         first, ut);
     count_launch(ctx);
-    q2_block_kernel<T, B, NCB><<<(unsigned)cdiv(ncols, NCB), Sh::NT, Sh::SMEM, st>>>(s->refl, ut, n, s->kmax, N0, k, e,
+    const T* block0 = reinterpret_cast<const T*>(reinterpret_cast<uintptr_t>(ut) - sizeof(T) * 2 * B * B * (size_t)first);
+    q2_block_kernel<T, B, NCB><<<(unsigned)cdiv(ncols, NCB), Sh::NT, Sh::SMEM, st>>>(s->refl, block0, n, s->kmax, N0, k, e,
                                                                                      Yt, ldy, ncols);
     count_launch(ctx);
     k = e;
