@@ -169,7 +169,7 @@ int reduce(fraclap_ctx* ctx, const double* A, int64_t n, int64_t lda, EigWork<T>
 template <class T>
 Arena lend_vt(Arena ar, size_t front, EigWork<T>* w) {
   const size_t bytes = align256(sizeof(T) * (size_t)std::max<int64_t>(w->s1.vtotal, 1)), end = ar.cap / 256 * 256;
-  if (end >= ar.off + front + bytes) {
+  if (!w->s1.XTstore && end >= ar.off + front + bytes) {
     ar.cap = end - bytes;
     w->s1.XTstore = reinterpret_cast<T*>(ar.base + ar.cap);
   }

@@ -256,7 +256,7 @@ struct Stage1T {
   double* tau;       // npanel * b
   T* X;              // n * b
   T* XT;             // n * b, V T of the panel in work
-  T* XTstore;        // as Vstore, V T of every panel: null unless the caller has room to lend
+  T* XTstore;        // as Vstore, V T of every panel: null for large n unless the caller has room to lend
   T* XX;             // X and XT as one buffer (xx_len entries, 2 b^2 ceil(n / b) or more)
   int64_t xx_len;
   T* Mm;             // b * b

@@ -679,7 +679,8 @@ int stage1_take(Arena* ar, int64_t n, int b, int G, Stage1T<T>* s) {
   s->XX = ar->take<T>(s->xx_len);
   s->X = s->XX;
   s->XT = s->XX ? s->XX + x : nullptr;
-  s->XTstore = nullptr;
+  // (up to 64 MiB, n = 4096 in FP64, V T of every panel costs no problem its memory)
+  s->XTstore = (sizeof(T) * (size_t)s->vtotal <= ((size_t)64 << 20)) ? ar->take<T>(s->vtotal) : nullptr;
   s->Mm = ar->take<T>((int64_t)b * b);
   s->gram = ar->take<double>((int64_t)b * b);
   s->partials = ar->take<double>(3 * 2 * (int64_t)b);

@@ -26,3 +26,18 @@ def test_blocks_and_single_reflectors_give_the_same_q(n):
     for d, e, Q in out[1:]:
         assert torch.equal(d, out[0][0]) and torch.equal(e, out[0][1])  # the reduction is shared
         assert (Q - out[0][2]).norm() <= 20 * n * eps
+
+
+@pytest.mark.parametrize("band", [32, 64])
+def test_fp64_routes_of_many_columns(band):
+    """Past 4096 columns the first back-transformation splits its sums, past 4256 the
+    second applies reflectors one by one (b = 64): residual and orthogonality of the
+    whole FP64 decomposition, to 10 n eps."""
+    import paper_1911_11906_gb300 as F
+    n, eps = 4300, torch.finfo(torch.float64).eps
+    g = torch.Generator(device="cuda").manual_seed(band)
+    A = torch.randn(n, n, dtype=torch.float64, device="cuda", generator=g)
+    A = A + A.t()
+    lam, V = F.eig_full(A, ctx=F.Context(band_width=band, wait_timeout_s=5.0))[:2]
+    assert (V.t() @ V - torch.eye(n, dtype=torch.float64, device="cuda")).norm() <= 10 * n * eps
+    assert (A @ V - V * lam).norm() <= 10 * n * eps * A.norm()
